@@ -1,9 +1,11 @@
 // C ABI of the AFQMC library: workspace plan, set-up, step sequencing.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "kernels.cuh"
@@ -37,15 +39,57 @@ struct Bump {
 };
 }  // namespace
 
+// Slices of the walkers' operands live in one scratch area of at most about
+// this size: populations that need more are taken in chunks of walkers.
+constexpr size_t kOzScratch = size_t(2) << 30;
+// A state whose workspace would grow above this keeps the float64 kernels,
+// whose workspace is up to 40% smaller (states that fitted a 288 GB GPU
+// before still do).
+constexpr size_t kOzWorkspace = size_t(160) << 30;
+
+// Whether the float64 contractions run on the tensor cores (oz.cuh).  Below,
+// a system is bound by latency and the float64 kernels' fewer launches win.
+// Five steps and an energy (5 M vectors), float64 kernels against tensor
+// cores, us: M = 32, N = 4: 1047 / 1243 at 48 walkers, 1469 / 1512 at 256,
+// 4570 / 2918 at 1024; M = 48, N = 6: 2065 / 1433, 4015 / 1845, 14199 / 4514;
+// M = 20, N = 3: 770 / 1152, 828 / 1325, 1935 / 2395.
+static bool oz_pays(int M, int W) { return M >= 40 || (M >= 28 && W >= 512); }
+
+// V of a walker as row tiles of equal height, and the term's columns.
+static void oz_taylor_operands(size_t M, size_t N, size_t Mp, OzOperand* V, OzOperand* T) {
+  const size_t nt = oz_tiles(M, 128);
+  V->RT = V->rows_per_tile = (int)(((M + nt - 1) / nt + 7) / 8 * 8);
+  T->RT = T->rows_per_tile = oz_term_width((int)N);
+  V->nkb = T->nkb = (int)(2 * Mp / 16);
+  V->batch_stride = (long)oz_bytes(M, V->rows_per_tile, V->RT, 2 * Mp);
+  T->batch_stride = (long)oz_bytes(2 * N, T->rows_per_tile, T->RT, 2 * Mp);
+  V->batch_exp_stride = (long)M;
+  T->batch_exp_stride = (long)(2 * N);
+}
+
+static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz);
+
 size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   Bufs tmp;
   if (!b) b = &tmp;
+  bool oz = p.precision == AFQMC_FP64 && oz_pays(p.M, p.nwalkers);
+  if (oz) {
+    Bufs probe;
+    oz = plan_route(p, &probe, nullptr, true) <= kOzWorkspace;
+  }
+  return plan_route(p, b, base, oz);
+}
+
+static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   // N: orbital columns per walker (N_up + N_dn with two spin blocks)
   const size_t M = p.M, N = p.N + (p.Ndn > 0 ? p.Ndn : 0), G = p.nchol, W = p.nwalkers;
   const size_t P = M * (M + 1) / 2;
   const bool mixed = p.precision != AFQMC_FP64;
   size_t nchunk = (G + exchange_chunk((int)N, p.nchol) - 1) / exchange_chunk((int)N, p.nchol);
   if (mixed) nchunk = G;  // the tensor-core exchange leaves one partial per vector
+  b->oz = oz;
+  b->oz_exch = oz && p.ndet == 0 && N <= 32;
+  if (b->oz_exch) nchunk = oz_tiles(G, oz_exchange_vectors((int)N));
   const size_t lo = (p.precision == AFQMC_MIXED_BF16 || p.precision == AFQMC_MIXED_BF16_F32LU ||
                      p.precision == AFQMC_MIXED_BF16_F64THETA)
                         ? 2
@@ -55,7 +99,7 @@ size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   const size_t Gp = (G + 7) / 8 * 8, Mp = (M + 15) / 16 * 16, Pp = (P + 3) / 4 * 4;
   Bump a{base};
   // constants
-  b->LpT = a.take<double>(P * G);
+  if (!oz) b->LpT = a.take<double>(P * G);
   b->Lh = a.take<double>(G * N * M);
   b->hh = a.take<double>(N * M);
   b->c = a.take<double>(G);
@@ -147,6 +191,39 @@ size_t plan(const afqmc_params& p, Bufs* b, char* base) {
     b->Bh_split = a.take<char>(M * 2 * (size_t)b->Kp1 * lo);
     b->Bh_split_tf = a.take<float>(M * 4 * Mp);
   }
+  size_t oz_need = 0, oz_exps = 0;
+  if (oz) {
+    auto take = [&](OzOperand& o, size_t rows, int rpt, int RT, size_t k) {
+      o.RT = RT;
+      o.rows_per_tile = rpt;
+      o.nkb = (int)((k + 15) / 16);
+      o.data = a.take<char>(oz_bytes(rows, rpt, RT, k));
+      o.exps = a.take<int>(rows);
+    };
+    take(b->ozL, P, 64, 64, G);
+    take(b->ozB, M, 64, 64, M);
+    if (p.ndet == 0) take(b->ozF, G, 64, 64, N * M);
+    if (b->oz_exch) {
+      const int rpt = oz_exchange_vectors((int)N) * (int)N;
+      take(b->ozX, G * N, rpt, (rpt + 7) / 8 * 8, M);
+    }
+    OzOperand V, T;
+    oz_taylor_operands(M, N, Mp, &V, &T);
+    const size_t per = (size_t)(V.batch_stride + T.batch_stride);
+    size_t wc = kOzScratch / per;
+    wc = wc >= W ? W : wc < 64 ? 64 : wc / 64 * 64;
+    if (wc > W) wc = W;
+    b->oz_wc = (int)wc;
+    auto need = [&](size_t bytes, size_t exps) {
+      if (bytes > oz_need) oz_need = bytes;
+      if (exps > oz_exps) oz_exps = exps;
+    };
+    need(per * wc, wc * (M + 2 * N));
+    need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
+    need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
+    if (p.ndet == 0) need(oz_bytes(2 * wc, 128, 128, N * M), 2 * wc);
+    if (b->oz_exch) need(oz_bytes(2 * N * wc, 2 * (int)N * oz_exchange_walkers((int)N), 64, M), 2 * N * wc);
+  }
   // scratch: the set-up and the step never run at the same time
   const size_t scratch_at = (a.off + 255) & ~size_t(255);
   Bump s1{base, scratch_at};
@@ -165,6 +242,10 @@ size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   b->T0 = s1.take<double>(W * 2 * N * M);  // Taylor terms (FP64) / comb copies
   b->T1 = s1.take<double>(W * 2 * N * M);
   b->tmp_ld = s1.take<double>(2 * W);
+  if (oz) {
+    b->oz_mem = s1.take<char>(oz_need);
+    b->oz_exp = s1.take<int>(oz_exps);
+  }
   Bump s2{base, scratch_at};
   b->Lfull = s2.take<double>(G * M * M);
   b->L2 = s2.take<double>(M * M);
@@ -175,6 +256,7 @@ size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   b->red = s2.take<double>(8);
   b->ych = (int)(G < 32 ? G : 32);
   b->Ych = s2.take<double>((size_t)b->ych * M * M);
+  if (oz) b->LpT = s2.take<double>(P * G);  // only the set-up reads it: the step has its slices
   b->P = (int)P;
   b->nchunk = (int)nchunk;
   b->gc = exchange_chunk((int)N, p.nchol);
@@ -427,6 +509,92 @@ void desc_half2(afqmc_state* s, double* phi_out, void* phi_lo_out, TcJobDesc* d)
   d->acc_id = b.acc32;
 }
 
+// C rows = (src rows) B^T, B sliced at set-up, rw rows of k values per walker
+// (contiguous), sliced a chunk of walkers at a time; 2^alpha_log2 the factor.
+static int oz_rows_gemm(afqmc_state* s, const double* src, int rw, int k, const OzOperand& B, double* C,
+                        int n, int alpha_log2, const double* mask) {
+  const Bufs& b = s->b;
+  for (int w0 = 0; w0 < s->p.nwalkers; w0 += b.oz_wc) {
+    const int nw = std::min(b.oz_wc, s->p.nwalkers - w0);
+    OzGemm g;
+    g.A.data = b.oz_mem;
+    g.A.exps = b.oz_exp;
+    g.A.nkb = B.nkb;
+    AFQ_TRY(oz_slice_rows(src + (size_t)w0 * rw * k, (long)nw * rw, k, k, g.A, s->st));
+    g.m = nw * rw;
+    g.n = n;
+    g.B = B;
+    g.C = C + (size_t)w0 * rw * n;
+    g.ldc = n;
+    g.alpha_log2 = alpha_log2;
+    g.mask = mask ? mask + 2 * (size_t)w0 : nullptr;
+    g.mask_rows = rw;
+    g.err = b.status;
+    AFQ_TRY(oz_gemm_store(g, s->st));
+  }
+  return AFQMC_OK;
+}
+
+// acc = T_n(V) t0 with V = i sqrt(dt) Y (packed), a chunk of walkers at a time.
+static int oz_taylor(afqmc_state* s) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  OzTerm t;
+  oz_taylor_operands(p.M, p.N, b.Mp, &t.V, &t.T);
+  const size_t row = (size_t)2 * p.N * p.M;
+  for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
+    const int nw = std::min(b.oz_wc, p.nwalkers - w0);
+    t.V.data = b.oz_mem;
+    t.V.exps = b.oz_exp;
+    t.T.data = b.oz_mem + (size_t)nw * t.V.batch_stride;
+    t.T.exps = b.oz_exp + (size_t)nw * t.V.batch_exp_stride;
+    AFQ_TRY(oz_slice_v(b.Y + (size_t)w0 * 2 * b.P, b.P, nw, p.M, b.Mp, t.V, s->st));
+    t.W = nw;
+    t.M = p.M;
+    t.N = p.N;
+    t.acc = b.acc + w0 * row;
+    t.err = b.status;
+    double* in = b.T0 + w0 * row;
+    double* out = b.T1 + w0 * row;
+    for (int k = 1; k <= p.taylor_order; ++k) {
+      t.k = k;
+      t.scale = s->sdt / k;
+      t.last = k == p.taylor_order;
+      t.tin = in;
+      t.tout = out;
+      AFQ_TRY(oz_slice_term(in, nw, p.N, p.M, b.Mp, t.T, s->st));
+      AFQ_TRY(oz_taylor_term(t, s->st));
+      std::swap(in, out);
+    }
+  }
+  return AFQMC_OK;
+}
+
+// part[w][c] = the exchange sums of the live state's Theta (Eq. localenergy3).
+static int oz_energy_exchange(afqmc_state* s) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  OzExchange x;
+  x.N = p.N;
+  x.G = p.nchol;
+  x.nup = s->nup;
+  x.nchunk = b.nchunk;
+  x.A = b.ozX;
+  x.B.data = b.oz_mem;
+  x.B.exps = b.oz_exp;
+  x.B.RT = 64;
+  x.B.rows_per_tile = 2 * p.N * oz_exchange_walkers(p.N);
+  x.B.nkb = b.ozX.nkb;
+  x.err = b.status;
+  for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
+    x.W = std::min(b.oz_wc, p.nwalkers - w0);
+    AFQ_TRY(oz_slice_rows(b.thetaT + (size_t)w0 * 2 * p.N * p.M, 2L * p.N * x.W, p.M, p.M, x.B, s->st));
+    x.part = b.part + (size_t)w0 * b.nchunk * 2;
+    AFQ_TRY(oz_exchange(x, s->st));
+  }
+  return AFQMC_OK;
+}
+
 int force_bias_gemm(afqmc_state* s) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
@@ -439,6 +607,12 @@ int force_bias_gemm(afqmc_state* s) {
     TcJobDesc d;
     desc_force_bias(s, &d);
     AFQ_TRY(tc_job_launch(d, s->st));
+    s->t_fresh = true;
+    return AFQMC_OK;
+  }
+  if (b.oz) {
+    // (sum over spins: 2 Tr(Lh_g Theta) for the closed-shell block)
+    AFQ_TRY(oz_rows_gemm(s, b.thetaT, 2, p.N * p.M, b.ozF, b.t, p.nchol, s->sf == 2.0 ? 1 : 0, nullptr));
     s->t_fresh = true;
     return AFQMC_OK;
   }
@@ -477,6 +651,8 @@ int energy_eval(afqmc_state* s, bool append, bool record = true) {
     g.tf32 = b.lo_kind == LO_TF32;
     g.err = b.status;
     AFQ_TRY(tc_exchange(g, p.nchol, p.nwalkers, p.N, b.part, b.nchunk, s->st));
+  } else if (b.oz_exch) {
+    AFQ_TRY(oz_energy_exchange(s));
   } else {
     ExchArgs ex{p.nwalkers, p.M, p.N, p.nchol, b.gc, b.nchunk, b.Lh, b.thetaT, b.part, b.wt};
     ex.nup = s->nup;
@@ -513,6 +689,21 @@ int apply_b_f64(afqmc_state* s, const double* phi_in, double* phi_out, const dou
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   const int W = p.nwalkers, N = p.N, M = p.M, G = p.nchol;
+  if (b.oz) {
+    prof_begin(s, AFQMC_PH_V);
+    AFQ_TRY(oz_rows_gemm(s, b.x, 2, G, b.ozL, b.Y, b.P, 0, nullptr));
+    prof_end(s);
+    prof_begin(s, AFQMC_PH_BHALF);
+    AFQ_TRY(oz_rows_gemm(s, phi_in, 2 * N, M, b.ozB, b.T0, M, 0, nullptr));
+    prof_end(s);
+    prof_begin(s, AFQMC_PH_TAYLOR);
+    AFQ_TRY(oz_taylor(s));
+    prof_end(s);
+    prof_begin(s, AFQMC_PH_BHALF);
+    AFQ_TRY(oz_rows_gemm(s, b.acc, 2 * N, M, b.ozB, phi_out, M, 0, mask));
+    prof_end(s);
+    return AFQMC_OK;
+  }
   // Y = sum_g x_g L_g (packed), the dense contraction with K = N_gamma
   prof_begin(s, AFQMC_PH_V);
   GemmF64 g;
@@ -1035,6 +1226,7 @@ static int setup_device(afqmc_state* s, const double* h1, const double* L, const
   }
   // packed, transposed Cholesky vectors for the float64 V contraction
   if (!f32_rot) AFQ_TRY(launch_pack_transpose(b.Lfull, b.LpT, G, M, st));
+  if (b.oz) AFQ_TRY(oz_slice_rows(b.LpT, b.P, G, G, b.ozL, st));
   // half-rotated vectors Lh_g = V_T^T L_g and hh = V_T^T h (Eq. precomputing2)
   {
     GemmF64 g;
@@ -1133,6 +1325,11 @@ static int setup_device(afqmc_state* s, const double* h1, const double* L, const
   AFQ_CUDA(cudaMemcpyAsync(&sumc2, b.red + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
   AFQ_TRY(expm_device(s));  // synchronises once
   s->H0p = p.H0 - 0.5 * sumc2;
+  if (b.oz) {
+    AFQ_TRY(oz_slice_rows(b.Bh, M, M, M, b.ozB, st));
+    if (!md) AFQ_TRY(oz_slice_rows(b.Lh, G, N * M, (long)N * M, b.ozF, st));
+    if (b.oz_exch) AFQ_TRY(oz_slice_rows(b.Lh, (long)G * N, M, M, b.ozX, st));
+  }
   if (b.mixed) {
     // BF16 / TF32 copies of the contraction operands (zero-padded pitches)
     if (f32_rot)

@@ -140,7 +140,7 @@ struct TaylorArgsT {
 using TaylorArgs = TaylorArgsT<double>;
 int launch_taylor_term(const TaylorArgsT<double>& a, cudaStream_t st);
 // the whole series (a.tin, a.tout, a.k and a.scale unset); t0 holds T_0
-constexpr int kTaylorSmallM = 64;  // one block per walker up to this many orbitals
+constexpr int kTaylorSmallM = 64;  // one block per walker up to this many orbitals (V: 64 KB)
 int taylor_series_f64(TaylorArgs a, int order, double sdt, double* t0, double* t1, cudaStream_t st);
 
 // Fused overlap: S = V_T^T Phi, Gauss-Jordan S^-1 and log det, Theta = Phi S^-1.

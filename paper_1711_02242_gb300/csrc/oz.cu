@@ -1,0 +1,758 @@
+// Float64 contractions as exact integer products on the tensor cores: slicing
+// kernels and the contraction (see oz.cuh for the number format).
+#include <vector>
+
+#include "oz.cuh"
+#include "tc.cuh"
+#include "tc_dev.cuh"
+
+namespace afq {
+namespace {
+
+using namespace tc;
+
+constexpr int kS = kOzSlices;
+constexpr long long kDigitBias = 64ll * (1ll + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) +
+                                         (1ll << 35) + (1ll << 42));
+
+// ---------------------------------------------------------------- slicing ---
+// |x| as the high word of its bits without the sign: monotonic in |x|.
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+
+// Row exponent e with 2^e above every element, from the largest abs_hi.
+__device__ __forceinline__ int row_exp(uint32_t hi, bool any) {
+  const int ef = (int)(hi >> 20);
+  if (ef == 0x7ff) return kOzNanExp;
+  if (!any) return kOzZeroExp;
+  return (ef > 0 ? ef : 1) - 1022;
+}
+
+// x in units of 2^(e - 56), rounded to nearest (|X| <= 2^56).
+__device__ __forceinline__ long long fixed57(double x, int e) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)(u >> 52) & 0x7ff;
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (ef) m |= 1ull << 52;
+  const int sh = (ef ? ef : 1) - 1019 - e;  // 3 for the largest element's binade
+  unsigned long long r;
+  if (sh >= 0) {
+    r = m << sh;
+  } else if (sh >= -54) {
+    r = (m + (1ull << (-sh - 1))) >> -sh;
+  } else {
+    r = 0;
+  }
+  return (long long)u < 0 ? -(long long)r : (long long)r;
+}
+
+// Two integers |d| <= 128 as a pair of BF16 (exact).
+__device__ __forceinline__ uint32_t bf16_pair(int lo, int hi) {
+  const uint32_t a = __float_as_uint(__int_as_float(0x4b400000 + lo) - 12582912.0f);
+  const uint32_t b = __float_as_uint(__int_as_float(0x4b400000 + hi) - 12582912.0f);
+  return __byte_perm(a, b, 0x7632);
+}
+
+// Digit i (0 = leading) of X + kDigitBias.
+__device__ __forceinline__ int digit(long long u, int i) {
+  return i == 0 ? (int)(u >> 49) : (int)((u >> (49 - 7 * i)) & 127) - 64;
+}
+
+// Eight values of K of one row (fixed-point, biased) into the 16-byte core
+// matrix rows of the eight slices.
+__device__ __forceinline__ void put_chunk(char* tile_row, int slice_bytes, const long long* u) {
+#pragma unroll
+  for (int i = 0; i < kS; ++i) {
+    uint4 w;
+    w.x = bf16_pair(digit(u[0], i), digit(u[1], i));
+    w.y = bf16_pair(digit(u[2], i), digit(u[3], i));
+    w.z = bf16_pair(digit(u[4], i), digit(u[5], i));
+    w.w = bf16_pair(digit(u[6], i), digit(u[7], i));
+    *reinterpret_cast<uint4*>(tile_row + (long)i * slice_bytes) = w;
+  }
+}
+
+// Byte offset of (row r of the tile, chunk c of 8 values of K) within a row tile.
+__device__ __forceinline__ long chunk_off(int RT, int r, int c) {
+  return (long)(c >> 1) * (kS * RT * 32) + (r >> 3) * 256 + (c & 1) * 128 + (r & 7) * 16;
+}
+
+// Eight rows per block: each warp takes the largest element of a row, then
+// the block writes the rows' chunks, eight rows of a chunk (128 contiguous
+// bytes per slice) by eight neighbouring lanes.  Bound by memory: 8 bytes in
+// (twice, the second time from L2), 16 out per element.
+__global__ void __launch_bounds__(256) k_oz_slice_rows(const double* src, long rows, int k, long ld,
+                                                       OzOperand o) {
+  __shared__ int e_sh[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gpt = (o.rows_per_tile + 7) >> 3;  // groups of eight rows per row tile
+  const long rt = blockIdx.x / gpt;
+  const int g8 = (int)(blockIdx.x - rt * gpt);
+  {
+    const int r = 8 * g8 + warp;
+    const long gr = rt * o.rows_per_tile + r;
+    uint32_t m = 0, any = 0;
+    if (r < o.rows_per_tile && gr < rows) {
+      const double* p = src + gr * ld;
+      for (int c = lane; c < k; c += 32) {
+        const double x = p[c];
+        m = max(m, abs_hi(x));
+        any |= abs_hi(x) | (uint32_t)__double2loint(x);
+      }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    any = __reduce_or_sync(0xffffffffu, any);
+    const int e = row_exp(m, any != 0);
+    if (lane == 0) {
+      e_sh[warp] = e;
+      if (r < o.rows_per_tile && gr < rows) o.exps[gr] = e;
+    }
+  }
+  __syncthreads();
+  const int r = 8 * g8 + (tid & 7);
+  const long gr = rt * o.rows_per_tile + r;
+  if (r >= o.rows_per_tile || gr >= rows) return;
+  const int e = e_sh[tid & 7];
+  const bool fine = e != kOzNanExp && e != kOzZeroExp;
+  const double* p = src + gr * ld;
+  char* base = reinterpret_cast<char*>(o.data) + rt * o.nkb * (long)(kS * o.RT * 32);
+  for (int c = tid >> 3; c < 2 * o.nkb; c += 32) {
+    long long u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int kk = 8 * c + i;
+      u[i] = kDigitBias + (fine && kk < k ? fixed57(p[kk], e) : 0ll);
+    }
+    put_chunk(base + chunk_off(o.RT, r, c), o.RT * 32, u);
+  }
+}
+
+// V / sqrt(dt) = -Im Y + i Re Y of walker blockIdx.y, rows 8 blockIdx.x ..:
+// operand rows p = [-Im Y_p | Re Y_p], segments of Mp (zero past M), from the
+// packed upper triangle.  The rows' largest element first, then the slices;
+// a tile's rows below the diagonal read Y columns, eight rows of a column at
+// a time (64 contiguous bytes).
+__global__ void __launch_bounds__(256) k_oz_slice_v(const double* Y, long ldy, int M, int Mp, OzOperand o) {
+  __shared__ uint32_t m_sh[8], any_sh[8];
+  const int tid = threadIdx.x, w = blockIdx.y;
+  const int gpt = (o.rows_per_tile + 7) >> 3;
+  const int rt = blockIdx.x / gpt, g8 = blockIdx.x - rt * gpt;
+  const int r = 8 * g8 + (tid & 7);
+  const int p = rt * o.rows_per_tile + r;
+  const bool act = r < o.rows_per_tile && p < M;
+  const double* yr = Y + (long)w * 2 * ldy;
+  const double* yi = yr + ldy;
+  if (tid < 8) m_sh[tid] = any_sh[tid] = 0u;
+  __syncthreads();
+  uint32_t m = 0, any = 0;
+  if (act)
+    for (int q = tid >> 3; q < M; q += 32) {
+      const int a = q <= p ? q : p, b = q <= p ? p : q;
+      const long id = (long)a * M - (long)a * (a - 1) / 2 + (b - a);
+      const double vr = yi[id], vi = yr[id];
+      m = max(m, max(abs_hi(vr), abs_hi(vi)));
+      any |= abs_hi(vr) | (uint32_t)__double2loint(vr) | abs_hi(vi) | (uint32_t)__double2loint(vi);
+    }
+  if (m | any) {
+    atomicMax(&m_sh[tid & 7], m);
+    atomicOr(&any_sh[tid & 7], any);
+  }
+  __syncthreads();
+  if (!act) return;
+  const int e = row_exp(m_sh[tid & 7], any_sh[tid & 7] != 0);
+  if (tid < 8) o.exps[(long)w * o.batch_exp_stride + p] = e;
+  const bool fine = e != kOzNanExp && e != kOzZeroExp;
+  char* base = reinterpret_cast<char*>(o.data) + (long)w * o.batch_stride +
+               (long)rt * o.nkb * (long)(kS * o.RT * 32);
+  for (int c = tid >> 3; c < Mp / 8; c += 32) {
+    long long ur[8], ui[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int q = 8 * c + i;
+      ur[i] = ui[i] = kDigitBias;
+      if (fine && q < M) {
+        const int a = q <= p ? q : p, b = q <= p ? p : q;
+        const long id = (long)a * M - (long)a * (a - 1) / 2 + (b - a);
+        ur[i] -= fixed57(yi[id], e);
+        ui[i] += fixed57(yr[id], e);
+      }
+    }
+    put_chunk(base + chunk_off(o.RT, r, c), o.RT * 32, ur);
+    put_chunk(base + chunk_off(o.RT, r, Mp / 8 + c), o.RT * 32, ui);
+  }
+}
+
+// A Taylor term [2][N][M] of walker blockIdx.y as operand rows i = [Re T_i |
+// -Im T_i] and N + i = [Im T_i | Re T_i] (segments of Mp), so that the rows
+// [Re | Im] of V times them give Re and Im of V T.  One warp per orbital i.
+__global__ void __launch_bounds__(128) k_oz_slice_term(const double* t, int N, int M, int Mp,
+                                                       OzOperand o) {
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 4 + (threadIdx.x >> 5), w = blockIdx.y;
+  if (i >= N) return;
+  const double* tr = t + ((long)w * 2 * N + i) * M;
+  const double* ti = tr + (long)N * M;
+  uint32_t m = 0, any = 0;
+  for (int p = lane; p < M; p += 32) {
+    const double x = tr[p], y = ti[p];
+    m = max(m, max(abs_hi(x), abs_hi(y)));
+    any |= abs_hi(x) | (uint32_t)__double2loint(x) | abs_hi(y) | (uint32_t)__double2loint(y);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  any = __reduce_or_sync(0xffffffffu, any);
+  const int e = row_exp(m, any != 0);
+  const bool fine = e != kOzNanExp && e != kOzZeroExp;
+  int* ex = o.exps + (long)w * o.batch_exp_stride;
+  if (lane == 0) ex[i] = ex[N + i] = e;
+  const int rpt = o.rows_per_tile;
+  const long tile_stride = (long)o.nkb * (kS * o.RT * 32);
+  char* base = reinterpret_cast<char*>(o.data) + (long)w * o.batch_stride;
+  char* re_row = base + (i / rpt) * tile_stride;
+  char* im_row = base + ((N + i) / rpt) * tile_stride;
+  const int r0 = i % rpt, r1 = (N + i) % rpt;
+  for (int c = lane; c < Mp / 8; c += 32) {
+    long long ur[8], ui[8], un[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int p = 8 * c + j;
+      const long long xr = fine && p < M ? fixed57(tr[p], e) : 0ll;
+      const long long xi = fine && p < M ? fixed57(ti[p], e) : 0ll;
+      ur[j] = kDigitBias + xr;
+      ui[j] = kDigitBias + xi;
+      un[j] = kDigitBias - xi;
+    }
+    put_chunk(re_row + chunk_off(o.RT, r0, c), o.RT * 32, ur);
+    put_chunk(re_row + chunk_off(o.RT, r0, Mp / 8 + c), o.RT * 32, un);
+    put_chunk(im_row + chunk_off(o.RT, r1, c), o.RT * 32, ui);
+    put_chunk(im_row + chunk_off(o.RT, r1, Mp / 8 + c), o.RT * 32, ur);
+  }
+}
+
+// ------------------------------------------------------------ contraction ---
+// (hi 2^28 + lo) 2^e as float64, rounded to nearest even once.
+__device__ __forceinline__ double round_sum(long long hi, long long lo, int e) {
+  long long h = hi + (lo >> 28);
+  uint32_t l = (uint32_t)lo & 0xfffffffu;
+  const bool neg = h < 0;
+  if (neg) {  // negate the pair
+    l = (0x10000000u - l) & 0xfffffffu;
+    h = ~h + (l == 0 ? 1 : 0);
+  }
+  unsigned long long x;  // leading bit at 63
+  int top;               // weight of the leading bit
+  uint32_t lost = 0;
+  if (h != 0) {
+    const int z = __clzll(h);
+    x = (unsigned long long)h << z;
+    if (z >= 28) {
+      x |= (unsigned long long)l << (z - 28);
+    } else {
+      x |= l >> (28 - z);
+      lost = l & ((1u << (28 - z)) - 1u);
+    }
+    top = 63 - z + 28;
+  } else {
+    if (l == 0) return 0.0;
+    const int z = __clzll((long long)l);
+    x = (unsigned long long)l << z;
+    top = 63 - z;
+  }
+  unsigned long long man = x >> 11;
+  const uint32_t rest = (uint32_t)x & 2047u;
+  if (rest > 1024u || (rest == 1024u && (lost != 0 || (man & 1ull)))) ++man;  // may carry to 2^53
+  const int E = top + e;
+  const unsigned long long sign = neg ? 1ull << 63 : 0ull;
+  if (E > -1022 && E < 1023)
+    return __longlong_as_double((long long)(sign | (((unsigned long long)(E + 1022) << 52) + man)));
+  const double d = __longlong_as_double((long long)(sign | ((1022ull << 52) + man)));  // E = 0
+  return scalbn(d, E < -4000 ? -4000 : (E > 4000 ? 4000 : E));
+}
+
+__device__ __forceinline__ double scaled_sum(long long hi, long long lo, int ea, int eb, int extra) {
+  if (ea == kOzNanExp || eb == kOzNanExp) return __longlong_as_double(0x7ff8000000000000ll);
+  return round_sum(hi, lo, ea + eb - 63 + extra);
+}
+
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
+}
+
+// Contiguous global -> shared copy, completing on an mbarrier.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// Shared-memory matrix descriptor of a K-major operand in core matrices of 8
+// rows x 16 bytes (no swizzle): 128 bytes between the two core matrices of a
+// K step, 256 bytes between groups of eight rows.
+__device__ __forceinline__ uint64_t core_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(128 >> 4) << 16;
+  d |= (uint64_t)(256 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
+struct OzArgs {
+  const char* A;
+  const char* B;
+  long a_batch, b_batch;    // bytes
+  const int* ea;
+  const int* eb;
+  long ea_batch, eb_batch;  // rows
+  int a_rpt, b_rpt;         // rows of a tile that are operand rows
+  int a_bytes;              // bytes of an A tile's K block
+  int RTA;
+  int nkb, nseg;
+  int nmt, nnt, ntiles;     // tiles = batch x nnt x nmt, mt fastest
+  int* err;
+};
+
+constexpr int kEpiWarps = 8;
+constexpr int kOzThreads = 64 + 32 * kEpiWarps;
+
+// Shared memory: a ring of STAGES K blocks (A tile of up to 128 rows, then the
+// B tile), 1 KB in which the last slice's M = 128 rows may end when RTA < 128,
+// the epilogue's buffer, the barriers.
+template <int BN, class Epi>
+struct OzSmem {
+  static constexpr int STAGE = kS * 32 * (BM + BN);
+  static constexpr int STAGES = Epi::kStages;
+  static constexpr int EPI = STAGES * STAGE;
+  static constexpr int BAR = EPI + Epi::kSmemBytes;
+  static constexpr int TOTAL = BAR + 256 + 1024;
+};
+
+// Persistent contraction: one CTA per SM walks 128 x BN tiles.  Warp 0 copies
+// the operands' K blocks (16 values of K, all eight slices: contiguous in
+// memory) into the ring; one thread of warp 1 multiplies: slice i of A against
+// slices 0 .. 7 - i of B, which lie side by side as (8 - i) BN columns, into
+// the accumulator columns of D_i .. D_7, so that one instruction covers several
+// slice pairs and every A slice is read once per 256 columns.  36 of 64 pairs.
+// Eight warps drain the accumulators after every kOzSegBlk blocks (64-bit
+// integer sums in registers) and hand the rounded values to the epilogue.
+// BN = 64 fills tensor memory with one set of accumulators; narrower tiles
+// have two, so that the epilogue overlaps the next segment.
+// Bound by the tensor pipe at large K: 36 x 64 columns take 1152 cycles per
+// K block against 48 KB of operands from L2 (43 B per cycle).  Measured (the
+// float64 pipe's limit is 1.2 TFLOP/s, its kernel reached 1.19): 1024 x 5050 x
+// 500 in 174 us, 29.7 TFLOP/s; 1024 x 4096 x 1800 in 383 us, 39.4 TFLOP/s.
+// Errors against 128-bit sums, relative to the operands' 2-norms (rms over
+// Gaussian rows, K = 16 .. 7500): 1.4e-17 .. 1.4e-18, a float64 FMA chain
+// 3.7e-17 .. 3.2e-17.
+template <int BN, class Epi>
+__global__ void __launch_bounds__(kOzThreads, 1)
+    k_oz_gemm(const OzArgs g, const __grid_constant__ Epi epi) {
+  extern __shared__ uint8_t oz_raw[];
+  using S = OzSmem<BN, Epi>;
+  constexpr int STAGES = S::STAGES;
+  constexpr int NBUF = BN <= 32 ? 2 : 1;
+  constexpr uint32_t DCOLS = kS * BN;
+  constexpr uint32_t TCOLS = NBUF * DCOLS;
+  constexpr int CW = BN / 2;  // columns per epilogue warp
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::BAR);
+  uint64_t* empty = full + STAGES;
+  uint64_t* tfull = empty + STAGES;  // [2]
+  uint64_t* tempty = tfull + 2;      // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&tfull[a], 1);
+      mbar_init(&tempty[a], kEpiWarps);
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(TCOLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int per_batch = g.nmt * g.nnt;
+  constexpr int B_BYTES = kS * BN * 32;
+
+  if (warp == 0 && lane == 0) {
+    int it = 0;
+    for (int t = blockIdx.x; t < g.ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
+      const int b = t / per_batch, rem = t - b * per_batch, nt = rem / g.nmt, mt = rem - nt * g.nmt;
+      const char* a_src = g.A + b * g.a_batch + (long)mt * g.nkb * g.a_bytes;
+      const char* b_src = g.B + b * g.b_batch + (long)nt * g.nkb * B_BYTES;
+      for (int kb = 0; kb < g.nkb; ++kb, ++it) {
+        const int s = it % STAGES;
+        if (it >= STAGES && !mbar_wait(&empty[s], ((it / STAGES) - 1) & 1, g.err, 61)) {
+          *(volatile int*)abort_flag = 1;
+          break;
+        }
+        uint8_t* dst = smem + s * S::STAGE;
+        mbar_expect_tx(&full[s], (uint32_t)(g.a_bytes + B_BYTES));
+        bulk_load(dst, a_src + (long)kb * g.a_bytes, (uint32_t)g.a_bytes, &full[s]);
+        bulk_load(dst + kS * 32 * BM, b_src + (long)kb * B_BYTES, (uint32_t)B_BYTES, &full[s]);
+      }
+    }
+    // given up: no copy may still be in flight when the CTA's memory is released
+    if (*(volatile int*)abort_flag)
+      for (int n = it > STAGES ? it - STAGES : 0; n < it; ++n)
+        mbar_wait(&full[n % STAGES], (n / STAGES) & 1, g.err, 65);
+  } else if (warp == 1 && lane == 0) {
+    int it = 0, j = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.ntiles && ok && !*(volatile int*)abort_flag; t += gridDim.x) {
+      int kb = 0;
+      for (int sg = 0; sg < g.nseg && ok; ++sg, ++j) {
+        const int kend = (int)((long)g.nkb * (sg + 1) / g.nseg);
+        const int buf = NBUF == 2 ? (j & 1) : 0;
+        if (j >= NBUF && !mbar_wait(&tempty[buf], ((j / NBUF) - 1) & 1, g.err, 62)) {
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t d = tmem + (uint32_t)buf * DCOLS;
+        for (bool first = true; kb < kend; ++kb, ++it, first = false) {
+          const int s = it % STAGES;
+          if (!mbar_wait(&full[s], (it / STAGES) & 1, g.err, 63)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const uint32_t a = smem_u32(smem + s * S::STAGE);
+          const uint32_t bb = a + kS * 32 * BM;
+#pragma unroll
+          for (int i = 0; i < kS; ++i) {
+            const uint64_t ad = core_desc(a + (uint32_t)(i * g.RTA * 32));
+            constexpr int kMaxN = 256;
+#pragma unroll
+            for (int c = 0; c < (kS - i) * BN; c += kMaxN) {
+              const int n = (kS - i) * BN - c < kMaxN ? (kS - i) * BN - c : kMaxN;
+              mma<false>(d + (uint32_t)(i * BN + c), ad, core_desc(bb + (uint32_t)(c * 32)),
+                         instr_desc(1u, (uint32_t)n), (first && i == 0) ? 0u : 1u);
+            }
+          }
+          mma_commit(&empty[s]);
+        }
+        mma_commit(&tfull[buf]);
+      }
+    }
+    if (!ok) *(volatile int*)abort_flag = 1;
+  } else if (warp >= 2) {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    int j = 0;
+    for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
+      const int b = t / per_batch, rem = t - b * per_batch, nt = rem / g.nmt, mt = rem - nt * g.nmt;
+      long long hi[CW], lo[CW];
+#pragma unroll
+      for (int c = 0; c < CW; ++c) hi[c] = lo[c] = 0;
+      bool stop = false;
+      for (int sg = 0; sg < g.nseg; ++sg, ++j) {
+        const int buf = NBUF == 2 ? (j & 1) : 0;
+        const bool bad = !mbar_wait_sleep(&tfull[buf], (j / NBUF) & 1, g.err, 64);
+        fence_after();
+        uint32_t out;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
+            "bar.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(out)
+            : "r"((uint32_t)(bad || *(volatile int*)abort_flag)), "n"(32 * kEpiWarps)
+            : "memory");
+        if (out) {
+          *(volatile int*)abort_flag = 1;
+          stop = true;
+          break;
+        }
+        const uint32_t base = tmem + (uint32_t)buf * DCOLS + ((uint32_t)(32 * q) << 16) + (uint32_t)(CW * half);
+#pragma unroll
+        for (int c0 = 0; c0 < CW; c0 += 8) {
+          // pairs D_t 2^7 + D_{t+1} stay below 2^31
+          uint32_t r[4][8];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) tmem_ld8_async(base + (uint32_t)(u * BN + c0), r[u]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const int p0 = __float2int_rn(__uint_as_float(r[0][c])) * 128 + __float2int_rn(__uint_as_float(r[1][c]));
+            const int p1 = __float2int_rn(__uint_as_float(r[2][c])) * 128 + __float2int_rn(__uint_as_float(r[3][c]));
+            hi[c0 + c] += (long long)p0 * 16384 + p1;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) tmem_ld8_async(base + (uint32_t)((4 + u) * BN + c0), r[u]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const int p0 = __float2int_rn(__uint_as_float(r[0][c])) * 128 + __float2int_rn(__uint_as_float(r[1][c]));
+            const int p1 = __float2int_rn(__uint_as_float(r[2][c])) * 128 + __float2int_rn(__uint_as_float(r[3][c]));
+            lo[c0 + c] += (long long)p0 * 16384 + p1;
+          }
+        }
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[buf]);
+      }
+      if (stop) break;
+      epi.template run<CW>(g, b, mt, nt, 32 * q + lane, CW * half, lane, warp - 2, hi, lo, smem + S::EPI);
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
+  }
+}
+
+// -------------------------------------------------------------- epilogues ---
+// C[m][n] = 2^alpha D: each warp passes its 32 rows x 8 columns through 2 KB
+// of shared memory so that a store instruction covers four rows of 64 bytes.
+struct EpiOzStore {
+  static constexpr int kStages = 4;
+  static constexpr int kSmemBytes = kEpiWarps * 32 * 8 * 8;
+  double* C;
+  long ldc;
+  int M, N, alpha;
+  const double* mask;
+  int mask_rows;
+  template <int CW>
+  __device__ __forceinline__ void run(const OzArgs& g, int, int mt, int nt, int r, int c0, int lane, int ew,
+                                      const long long* hi, const long long* lo, uint8_t* sm) const {
+    double* buf = reinterpret_cast<double*>(sm) + ew * 256;
+    const int row = mt * g.a_rpt + r;
+    const int ea = row < M ? g.ea[row] : kOzZeroExp;
+#pragma unroll
+    for (int c = 0; c < CW; c += 8) {
+      const int col = nt * g.b_rpt + c0 + c;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int eb = col + i < N ? g.eb[col + i] : kOzZeroExp;
+        // 16-byte slots permuted by row: row-per-lane writes without conflicts
+        buf[lane * 8 + ((i & 1) | (((i >> 1) ^ (lane & 3)) << 1))] = scaled_sum(hi[c + i], lo[c + i], ea, eb, alpha);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int rr = 4 * k + (lane >> 3), i = lane & 7;
+        const int grow = row - lane + rr, gcol = col + i;
+        if (grow < M && gcol < N && (!mask || walker_alive(mask, grow / mask_rows)))
+          C[(long)grow * ldc + gcol] = buf[rr * 8 + ((i & 1) | (((i >> 1) ^ (rr & 3)) << 1))];
+      }
+      __syncwarp();
+    }
+  }
+};
+
+// A Taylor term: rows p, columns (c, i) of walker b.  A lane owns a row, so
+// the stores along p are contiguous.
+struct EpiOzTerm {
+  static constexpr int kStages = 4;
+  static constexpr int kSmemBytes = 0;
+  int M, N2;  // N2 = 2 N
+  int first, last;
+  double scale;  // sqrt(dt) / k
+  const double* tin;
+  double* tout;
+  double* acc;
+  template <int CW>
+  __device__ __forceinline__ void run(const OzArgs& g, int b, int mt, int nt, int r, int c0, int, int,
+                                      const long long* hi, const long long* lo, uint8_t*) const {
+    const int p = mt * g.a_rpt + r;
+    if (r >= g.a_rpt || p >= M) return;
+    const int ea = g.ea[(long)b * g.ea_batch + p];
+    const int* eb = g.eb + (long)b * g.eb_batch;
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+      const int col = nt * g.b_rpt + c0 + c;
+      if (col >= N2) break;
+      const double v = scaled_sum(hi[c], lo[c], ea, eb[col], 0) * scale;
+      const long at = ((long)b * N2 + col) * M + p;
+      if (!last) tout[at] = v;
+      acc[at] = (first ? tin[at] : acc[at]) + v;
+    }
+  }
+};
+
+// Exchange: the tile of T into shared memory, then sum_ij T_ij T_ji per walker
+// of the tile over the tile's vectors; every unordered pair {i, j} once, at
+// twice its weight (j = i + d mod N), by the lane of row (g, i); nw warps per
+// walker, their sums added in a fixed order.
+struct EpiOzExchange {
+  static constexpr int kStages = 3;
+  static constexpr int LD = 65;
+  static constexpr int kSmemBytes = BM * LD * 8 + 2 * kEpiWarps * 8;
+  int N, W, G, RG, WT, nup, nchunk;  // RG vectors, WT walkers per tile
+  double* part;
+  template <int CW>
+  __device__ __forceinline__ void run(const OzArgs& g, int, int mt, int nt, int r, int c0, int lane, int ew,
+                                      const long long* hi, const long long* lo, uint8_t* smraw) const {
+    double* T = reinterpret_cast<double*>(smraw);
+    double* red = T + BM * LD;
+    const int row = mt * g.a_rpt + r;
+    const bool rv = r < g.a_rpt && row < G * N;
+    const int ea = rv ? g.ea[row] : kOzZeroExp;
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+      const int cc = c0 + c, col = nt * g.b_rpt + cc;
+      const int eb = cc < g.b_rpt && col < 2 * N * W ? g.eb[col] : kOzZeroExp;
+      T[r * LD + cc] = rv && eb != kOzZeroExp ? scaled_sum(hi[c], lo[c], ea, eb, 0) : 0.0;
+    }
+    asm volatile("bar.sync 2, 256;" ::: "memory");
+    const int nw = WT >= kEpiWarps ? 1 : kEpiWarps / WT;
+    const int nrow = RG * N, nd = (N - 1) / 2;
+    for (int w0 = 0; w0 < WT; w0 += kEpiWarps / nw) {
+      const int wl = w0 + ew / nw, sub = ew % nw;
+      const int w = nt * WT + wl;
+      double er = 0.0, ei = 0.0;
+      if (ew < (kEpiWarps / nw) * nw && wl < WT && w < W) {
+        const double* Tw = T + wl * 2 * N;
+        for (int rr = sub * 32 + lane; rr < nrow; rr += 32 * nw) {
+          const int gl = rr / N, i = rr - gl * N;
+          const double* own = Tw + rr * LD;
+          const double* colp = Tw + gl * N * LD + i;
+          const double dr = own[i], di = own[N + i];
+          double pr = 0.0, pi = 0.0;
+          for (int d = 1; d <= nd; ++d) {
+            const int j = i + d < N ? i + d : i + d - N;
+            if (nup > 0 && (i < nup) != (j < nup)) continue;
+            const double ar = own[j], ai = own[N + j], br = colp[j * LD], bi = colp[j * LD + N];
+            pr = fma(ar, br, fma(-ai, bi, pr));
+            pi = fma(ar, bi, fma(ai, br, pi));
+          }
+          double sr = fma(dr, dr, fma(-di, di, 2.0 * pr)), si = fma(2.0 * dr, di, 2.0 * pi);
+          if ((N & 1) == 0) {
+            const int j = i + N / 2 < N ? i + N / 2 : i - N / 2;
+            if (nup <= 0 || (i < nup) == (j < nup)) {
+              const double ar = own[j], ai = own[N + j], br = colp[j * LD], bi = colp[j * LD + N];
+              sr = fma(ar, br, fma(-ai, bi, sr));
+              si = fma(ar, bi, fma(ai, br, si));
+            }
+          }
+          er += sr;
+          ei += si;
+        }
+      }
+      er = warp_sum(er);
+      ei = warp_sum(ei);
+      if (lane == 0) {
+        red[2 * ew] = er;
+        red[2 * ew + 1] = ei;
+      }
+      asm volatile("bar.sync 2, 256;" ::: "memory");
+      if (lane < 2 && sub == 0 && ew < (kEpiWarps / nw) * nw && wl < WT && w < W) {
+        double sum = 0.0;
+        for (int k = 0; k < nw; ++k) sum += red[2 * (ew + k) + lane];
+        part[((long)w * nchunk + mt) * 2 + lane] = sum;
+      }
+      asm volatile("bar.sync 2, 256;" ::: "memory");
+    }
+  }
+};
+
+template <int BN, class Epi>
+int launch_oz(const OzArgs& g, const Epi& e, cudaStream_t st) {
+  static std::atomic<unsigned long long> attr{0};
+  constexpr int smem = OzSmem<BN, Epi>::TOTAL;
+  static_assert(smem <= 227 * 1024, "shared memory");
+  AFQ_TRY(smem_attr_once(k_oz_gemm<BN, Epi>, smem, attr));
+  if (g.ntiles <= 0) return AFQMC_OK;
+  const int sms = tc_sm_count();
+  AFQ_LAUNCH((k_oz_gemm<BN, Epi>), g.ntiles < sms ? g.ntiles : sms, kOzThreads, smem, st, g, e);
+  return AFQMC_OK;
+}
+
+OzArgs oz_args(const OzOperand& A, const OzOperand& B, long m, long n, int batch, int* err) {
+  OzArgs g;
+  g.A = static_cast<const char*>(A.data);
+  g.B = static_cast<const char*>(B.data);
+  g.a_batch = A.batch_stride;
+  g.b_batch = B.batch_stride;
+  g.ea = A.exps;
+  g.eb = B.exps;
+  g.ea_batch = A.batch_exp_stride;
+  g.eb_batch = B.batch_exp_stride;
+  g.a_rpt = A.rows_per_tile;
+  g.b_rpt = B.rows_per_tile;
+  g.RTA = A.RT;
+  g.a_bytes = kS * A.RT * 32;
+  g.nkb = A.nkb;
+  g.nseg = (A.nkb + kOzSegBlk - 1) / kOzSegBlk;
+  g.nmt = (int)oz_tiles(m, A.rows_per_tile);
+  g.nnt = (int)oz_tiles(n, B.rows_per_tile);
+  g.ntiles = g.nmt * g.nnt * batch;
+  g.err = err;
+  return g;
+}
+
+int check_operand(const OzOperand& A, const OzOperand& B, int bn) {
+  if (!A.data || !B.data || !A.exps || !B.exps || A.nkb != B.nkb || A.nkb < 1 || A.RT % 8 || A.RT < A.rows_per_tile ||
+      A.RT > BM || B.RT != bn || B.rows_per_tile > bn || A.rows_per_tile < 1 || B.rows_per_tile < 1) {
+    set_error("sliced contraction: operands do not match");
+    return AFQMC_EINVAL;
+  }
+  return AFQMC_OK;
+}
+
+}  // namespace
+
+int oz_slice_rows(const double* src, long rows, int k, long ld, const OzOperand& o, cudaStream_t st) {
+  if (rows <= 0) return AFQMC_OK;
+  const long groups = (long)oz_tiles(rows, o.rows_per_tile) * ((o.rows_per_tile + 7) / 8);
+  AFQ_LAUNCH(k_oz_slice_rows, (unsigned)groups, 256, 0, st, src, rows, k, ld, o);
+  return AFQMC_OK;
+}
+
+int oz_slice_v(const double* Y, long ldy, int W, int M, int Mp, const OzOperand& o, cudaStream_t st) {
+  dim3 grid((unsigned)(oz_tiles(M, o.rows_per_tile) * ((o.rows_per_tile + 7) / 8)), W);
+  AFQ_LAUNCH(k_oz_slice_v, grid, 256, 0, st, Y, ldy, M, Mp, o);
+  return AFQMC_OK;
+}
+
+int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand& o, cudaStream_t st) {
+  dim3 grid(cdiv(N, 4), W);
+  AFQ_LAUNCH(k_oz_slice_term, grid, 128, 0, st, t, N, M, Mp, o);
+  return AFQMC_OK;
+}
+
+int oz_gemm_store(const OzGemm& g, cudaStream_t st) {
+  AFQ_TRY(check_operand(g.A, g.B, 64));
+  EpiOzStore e{g.C, g.ldc, g.m, g.n, g.alpha_log2, g.mask, g.mask_rows};
+  return launch_oz<64>(oz_args(g.A, g.B, g.m, g.n, 1, g.err), e, st);
+}
+
+int oz_term_width(int N) { return 2 * N <= 16 ? 16 : 2 * N <= 32 ? 32 : 64; }
+
+int oz_taylor_term(const OzTerm& t, cudaStream_t st) {
+  const int bn = oz_term_width(t.N);
+  AFQ_TRY(check_operand(t.V, t.T, bn));
+  EpiOzTerm e{t.M, 2 * t.N, t.k == 1, t.last ? 1 : 0, t.scale, t.tin, t.tout, t.acc};
+  const OzArgs g = oz_args(t.V, t.T, t.M, 2 * t.N, t.W, t.err);
+  if (bn == 16) return launch_oz<16>(g, e, st);
+  if (bn == 32) return launch_oz<32>(g, e, st);
+  return launch_oz<64>(g, e, st);
+}
+
+int oz_exchange_vectors(int N) { return BM / N > 0 ? BM / N : 1; }
+int oz_exchange_walkers(int N) { return 64 / (2 * N); }
+
+int oz_exchange(const OzExchange& x, cudaStream_t st) {
+  AFQ_TRY(check_operand(x.A, x.B, 64));
+  EpiOzExchange e{x.N, x.W, x.G, x.A.rows_per_tile / x.N, x.B.rows_per_tile / (2 * x.N),
+                  x.nup, x.nchunk, x.part};
+  return launch_oz<64>(oz_args(x.A, x.B, (long)x.G * x.N, 2L * x.N * x.W, 1, x.err), e, st);
+}
+
+}  // namespace afq

@@ -1,0 +1,98 @@
+// Float64 contractions on the tcgen05 tensor cores (internal header).
+//
+// GB300 runs float64 at ~1.2 TFLOP/s, so every dense contraction of the float64
+// path is bound by that pipe.  Here an operand row is held as a fixed-point
+// number of 57 bits relative to a power of two above its largest element,
+//   x = 2^(e - 56) X,  X = sum_i v_i 2^(49 - 7 i),  i = 0 .. 7,
+// |v_0| <= 128 and |v_i| <= 64: integers that BF16 holds exactly (the error-free
+// splitting of K. Ozaki, T. Ogita, S. Oishi, S. M. Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix
+// multiplication", Numer. Algorithms 59 (2012), with digits of a common
+// exponent per row).  A product of two rows is then
+//   sum_k a b = 2^(ea + eb - 63) sum_t D_t 2^(7 (7 - t)),
+//   D_t = sum_{i + j = t} sum_k v_i w_j,
+// each D_t an integer below 2^24 over kOzSegK values of k, so the FP32
+// accumulators hold it exactly; the segments are added as 64-bit integers and
+// the result is rounded to float64 once.  Products with i + j > 7 are left
+// out: at most 7 2^-58 of (2^ea 2^eb) per term, with random signs, against the
+// 2^-53 of the running sum that every step of a float64 FMA chain rounds away.
+#pragma once
+
+#include "kernels.cuh"
+
+namespace afq {
+
+constexpr int kOzSlices = 8;
+constexpr int kOzSegBlk = 25;             // K blocks of 16 between two drains of the accumulators
+constexpr int kOzSegK = 16 * kOzSegBlk;   // 400: 10 * 2^12 * 400 < 2^24 (D_7: 2 * 2^13 + 6 * 2^12 per k)
+constexpr int kOzZeroExp = -30000;        // exponent of a row of zeros
+constexpr int kOzNanExp = 30000;          // a row holding an infinity or a NaN: its results are NaN
+
+// Slices of `rows` operand rows as the kernel's shared-memory tiles: row tile
+// rt = r / rows_per_tile holds RT rows (a multiple of 8, >= rows_per_tile), K
+// in blocks of 16.  Tile (rt, kb) is 8 slices x RT rows x 16 BF16, 256 bytes
+// per 8 rows (two 8 x 8 core matrices); rows past rows_per_tile are not
+// written (they only meet output rows or columns that are dropped).
+struct OzOperand {
+  void* data = nullptr;
+  int* exps = nullptr;  // [tiles * rows_per_tile] row exponents e
+  int RT = 128, rows_per_tile = 128;
+  int nkb = 0;          // K blocks of 16
+  long batch_stride = 0;      // bytes between the operands of a batch (0: shared)
+  long batch_exp_stride = 0;  // row exponents between them
+};
+inline size_t oz_tiles(size_t rows, int rows_per_tile) { return (rows + rows_per_tile - 1) / rows_per_tile; }
+inline size_t oz_bytes(size_t rows, int rows_per_tile, int RT, size_t k) {
+  return oz_tiles(rows, rows_per_tile) * ((k + 15) / 16) * (size_t)kOzSlices * RT * 32;
+}
+
+// Rows of a row-major float64 matrix (pitch ld) into an operand.
+int oz_slice_rows(const double* src, long rows, int k, long ld, const OzOperand& o, cudaStream_t st);
+// Taylor operands of W walkers (see oz.cu): the rows of V / sqrt(dt) from the
+// packed Y, and the term's rows.
+int oz_slice_v(const double* Y, long ldy, int W, int M, int Mp, const OzOperand& o, cudaStream_t st);
+int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand& o, cudaStream_t st);
+
+// C[m][n] = 2^alpha_log2 sum_k A[m][k] B[n][k] (float64, pitch ldc); rows of
+// dead walkers (mask, mask_rows rows each) are not stored.
+struct OzGemm {
+  int m = 0, n = 0;
+  OzOperand A, B;  // B: RT = 64
+  double* C = nullptr;
+  long ldc = 0;
+  int alpha_log2 = 0;
+  const double* mask = nullptr;
+  int mask_rows = 1;
+  int* err = nullptr;
+};
+int oz_gemm_store(const OzGemm& g, cudaStream_t st);
+
+// One Taylor term of W walkers: tout = scale (V tin), acc (k == 1: tin) += tout.
+struct OzTerm {
+  int W = 0, M = 0, N = 0, k = 0;
+  double scale = 0.0;  // sqrt(dt) / k
+  bool last = false;  // tout is not needed
+  OzOperand V, T;     // T: RT = oz_term_width(N)
+  const double* tin = nullptr;
+  double* tout = nullptr;
+  double* acc = nullptr;
+  int* err = nullptr;
+};
+int oz_term_width(int N);
+int oz_taylor_term(const OzTerm& t, cudaStream_t st);
+
+// Exchange: part[w][c][2] = sum over the vectors of row tile c of
+// sum_ij T_ij T_ji, T_g = Lh_g Theta_w (same-spin pairs).  A: rows (g, i),
+// rows_per_tile a multiple of N; B: rows (w, c, j), rows_per_tile a multiple
+// of 2 N.
+struct OzExchange {
+  int W = 0, N = 0, G = 0, nup = 0, nchunk = 0;
+  OzOperand A, B;
+  double* part = nullptr;
+  int* err = nullptr;
+};
+int oz_exchange_vectors(int N);  // vectors per row tile
+int oz_exchange_walkers(int N);  // walkers per column tile
+int oz_exchange(const OzExchange& x, cudaStream_t st);
+
+}  // namespace afq

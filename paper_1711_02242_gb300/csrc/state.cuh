@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "oz.cuh"
 
 namespace afq {
 
@@ -50,6 +51,15 @@ struct Bufs {
   float* Bh_split_tf = nullptr;
   int Kp1 = 0;
   int* status = nullptr;  // device status word (tensor-core waits)
+  // float64 path on the tensor cores (oz.cuh): the sliced vectors of V (rows
+  // (p, q)), of the force bias (rows g) and of the exchange (rows (g, i)), and
+  // of B_half; oz_mem / oz_exp: slices and row exponents of oz_wc walkers at a
+  // time, whatever the contraction at hand reads
+  bool oz = false, oz_exch = false;
+  OzOperand ozL, ozF, ozX, ozB;
+  char* oz_mem = nullptr;
+  int* oz_exp = nullptr;
+  int oz_wc = 0;
   // back-propagation window (afqmc_params.bp_steps > 0): recorded fields
   // [bp_steps][W][2][G] float64 (mixed path: operand rows [W][2][Gp]), Psi_n and the back-propagated
   // orbitals [W][2][N][M], BP-PRes factors [W][2], cos dtheta [W], per-walker

@@ -1,6 +1,7 @@
-"""The float64 path's routes by size against the oracle (Secs. 3.2 - 3.4): up to
-64 orbitals the Taylor series runs in one block per walker, above that one
-launch per term.  Sizes at the edges of the routes.  Walkers, weights,
+"""The float64 path's routes by size against the oracle (Secs. 3.2 - 3.4): small
+systems run the Taylor series in one block per walker, the others every
+contraction as exact integer products on the tensor cores.  Sizes at the edges
+of the routes and of the tiles.  Walkers, weights,
 overlaps and energies agree to the 1e-10 of the parity tests (sums of a few
 thousand float64 terms and inverses of well-conditioned overlaps: about 1e-13
 here)."""
@@ -63,12 +64,37 @@ def check(pkg, M, N, G, W, steps, Ndn=0):
 
 
 @pytest.mark.parametrize("M,N,G,W,Ndn", [
-    (5, 5, 7, 3, 0),      # every orbital occupied
-    (33, 9, 40, 5, 0),    # more elements of a term than threads of a block
-    (64, 7, 70, 4, 0),    # the largest one-block series
-    (64, 20, 30, 3, 19),  # two spin blocks, 39 columns: 144 KB of shared memory
-    (64, 64, 20, 2, 0),   # the most orbitals: 192 KB
-    (65, 7, 70, 4, 0),    # the smallest of the other route
+    # float64 kernels, the series in one block per walker
+    (5, 5, 7, 3, 0),       # every orbital occupied
+    (33, 9, 40, 5, 0),     # more elements of a term than threads of a block
+    (39, 20, 30, 3, 19),   # the most orbitals, two spin blocks
+    # tensor cores
+    (40, 5, 57, 4, 0),     # the fewest orbitals; columns of a term: one 16-wide tile
+    (28, 2, 33, 512, 0),   # fewer with many walkers
+    (64, 32, 90, 3, 0),    # a walker fills the exchange's column tile
+    (64, 64, 20, 2, 0),    # every orbital occupied, two column tiles, float64 exchange kernel
+    (70, 1, 30, 130, 0),   # 32 walkers per column tile of the exchange, 128 vectors per row tile
+    (129, 17, 401, 3, 0),  # two row tiles of V; one vector more than a segment of the sum
+    (130, 33, 150, 3, 0),  # the fewest orbitals with two column tiles
+    (150, 13, 300, 3, 10),  # two spin blocks
 ])
 def test_sizes(pkg, M, N, G, W, Ndn):
     check(pkg, M, N, G, W, 3, Ndn)
+
+
+def test_chunks_of_walkers(pkg):
+    """Populations whose sliced operands exceed the scratch area are taken in
+    chunks: the last walkers of 40000 are those of a small population that
+    draws the same fields."""
+    M, N, G, W, n = 40, 2, 50, 40000, 70
+    h1, L, C = inputs(M, N, G)
+    big = pkg.AfqmcRun(h1, L, C, pkg.default_params(M, N, G, W, qr_period=2, energy_period=0))
+    small = pkg.AfqmcRun(h1, L, C, pkg.default_params(M, N, G, n, qr_period=2, energy_period=0, walker0=W - n))
+    for r in (big, small):
+        r.propagate(3)
+    el = big.local_energies()
+    assert np.array_equal(el[-n:], small.local_energies())
+    assert np.array_equal(big.weights()[-n:], small.weights())
+    assert np.all(np.isfinite(el)) and np.unique(el).size == W
+    big.close()
+    small.close()
