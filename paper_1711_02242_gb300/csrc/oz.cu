@@ -183,46 +183,74 @@ __global__ void __launch_bounds__(256) k_oz_slice_v(const double* Y, long ldy, i
 
 // A Taylor term [2][N][M] of walker blockIdx.y as operand rows i = [Re T_i |
 // -Im T_i] and N + i = [Im T_i | Re T_i] (segments of Mp), so that the rows
-// [Re | Im] of V times them give Re and Im of V T.  One warp per orbital i.
-__global__ void __launch_bounds__(128) k_oz_slice_term(const double* t, int N, int M, int Mp,
+// [Re | Im] of V times them give Re and Im of V T.  Eight orbitals per block, a
+// warp each for the largest element; then eight neighbouring lanes write the
+// eight orbitals' rows of a chunk (128 contiguous bytes per slice where the
+// rows share a group of eight).
+__global__ void __launch_bounds__(256) k_oz_slice_term(const double* t, int N, int M, int Mp,
                                                        OzOperand o) {
-  const int lane = threadIdx.x & 31, i = blockIdx.x * 4 + (threadIdx.x >> 5), w = blockIdx.y;
-  if (i >= N) return;
-  const double* tr = t + ((long)w * 2 * N + i) * M;
-  const double* ti = tr + (long)N * M;
-  uint32_t m = 0, any = 0;
-  for (int p = lane; p < M; p += 32) {
-    const double x = tr[p], y = ti[p];
-    m = max(m, max(abs_hi(x), abs_hi(y)));
-    any |= abs_hi(x) | (uint32_t)__double2loint(x) | abs_hi(y) | (uint32_t)__double2loint(y);
+  __shared__ int e_sh[8];
+  const int tid = threadIdx.x, lane = tid & 31, w = blockIdx.y;
+  const double* tw = t + (long)w * 2 * N * M;
+  {
+    const int i = blockIdx.x * 8 + (tid >> 5);
+    uint32_t m = 0, any = 0;
+    if (i < N) {
+      const double* tr = tw + (long)i * M;
+      const double* ti = tr + (long)N * M;
+      for (int p = lane; p < M; p += 32) {
+        const double x = tr[p], y = ti[p];
+        m = max(m, max(abs_hi(x), abs_hi(y)));
+        any |= abs_hi(x) | (uint32_t)__double2loint(x) | abs_hi(y) | (uint32_t)__double2loint(y);
+      }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    any = __reduce_or_sync(0xffffffffu, any);
+    const int e = row_exp(m, any != 0);
+    if (lane == 0) {
+      e_sh[tid >> 5] = e;
+      if (i < N) {
+        int* ex = o.exps + (long)w * o.batch_exp_stride;
+        ex[i] = ex[N + i] = e;
+      }
+    }
   }
-  m = __reduce_max_sync(0xffffffffu, m);
-  any = __reduce_or_sync(0xffffffffu, any);
-  const int e = row_exp(m, any != 0);
+  __syncthreads();
+  const int i = blockIdx.x * 8 + (tid & 7);
+  if (i >= N) return;
+  const int e = e_sh[tid & 7];
   const bool fine = e != kOzNanExp && e != kOzZeroExp;
-  int* ex = o.exps + (long)w * o.batch_exp_stride;
-  if (lane == 0) ex[i] = ex[N + i] = e;
-  const int rpt = o.rows_per_tile;
+  const double* tr = tw + (long)i * M;
+  const double* ti = tr + (long)N * M;
+  const int rpt = o.rows_per_tile, nc = Mp / 8;
   const long tile_stride = (long)o.nkb * (kS * o.RT * 32);
   char* base = reinterpret_cast<char*>(o.data) + (long)w * o.batch_stride;
   char* re_row = base + (i / rpt) * tile_stride;
   char* im_row = base + ((N + i) / rpt) * tile_stride;
   const int r0 = i % rpt, r1 = (N + i) % rpt;
-  for (int c = lane; c < Mp / 8; c += 32) {
-    long long ur[8], ui[8], un[8];
+  // the real and the imaginary part of a chunk are separate items
+  for (int c2 = tid >> 3; c2 < 2 * nc; c2 += 32) {
+    const bool im = c2 >= nc;
+    const int c = im ? c2 - nc : c2;
+    const double* src = im ? ti : tr;
+    long long u[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int p = 8 * c + j;
-      const long long xr = fine && p < M ? fixed57(tr[p], e) : 0ll;
-      const long long xi = fine && p < M ? fixed57(ti[p], e) : 0ll;
-      ur[j] = kDigitBias + xr;
-      ui[j] = kDigitBias + xi;
-      un[j] = kDigitBias - xi;
+      u[j] = fine && p < M ? fixed57(src[p], e) : 0ll;
     }
-    put_chunk(re_row + chunk_off(o.RT, r0, c), o.RT * 32, ur);
-    put_chunk(re_row + chunk_off(o.RT, r0, Mp / 8 + c), o.RT * 32, un);
-    put_chunk(im_row + chunk_off(o.RT, r1, c), o.RT * 32, ui);
-    put_chunk(im_row + chunk_off(o.RT, r1, Mp / 8 + c), o.RT * 32, ur);
+    long long up[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) up[j] = kDigitBias + u[j];
+    if (!im) {
+      put_chunk(re_row + chunk_off(o.RT, r0, c), o.RT * 32, up);
+      put_chunk(im_row + chunk_off(o.RT, r1, nc + c), o.RT * 32, up);
+    } else {
+      put_chunk(im_row + chunk_off(o.RT, r1, c), o.RT * 32, up);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) up[j] = kDigitBias - u[j];
+      put_chunk(re_row + chunk_off(o.RT, r0, nc + c), o.RT * 32, up);
+    }
   }
 }
 
@@ -266,9 +294,10 @@ __device__ __forceinline__ double round_sum(long long hi, long long lo, int e) {
   return scalbn(d, E < -4000 ? -4000 : (E > 4000 ? 4000 : E));
 }
 
-__device__ __forceinline__ double scaled_sum(long long hi, long long lo, int ea, int eb, int extra) {
-  if (ea == kOzNanExp || eb == kOzNanExp) return __longlong_as_double(0x7ff8000000000000ll);
-  return round_sum(hi, lo, ea + eb - 63 + extra);
+// The same for row exponents ea, eb; a row with an infinity or a NaN gives NaN
+// (its exponent is above any sum of two ordinary ones).
+__device__ __forceinline__ double scaled_sum(long long hi, long long lo, int e) {
+  return e > kOzNanExp / 2 ? __longlong_as_double(0x7ff8000000000000ll) : round_sum(hi, lo, e - 63);
 }
 
 __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
@@ -315,12 +344,9 @@ struct OzArgs {
   int* err;
 };
 
-constexpr int kEpiWarps = 8;
-constexpr int kOzThreads = 64 + 32 * kEpiWarps;
-
 // Shared memory: a ring of STAGES K blocks (A tile of up to 128 rows, then the
-// B tile), 1 KB in which the last slice's M = 128 rows may end when RTA < 128,
-// the epilogue's buffer, the barriers.
+// B tile), the epilogue's buffer, the barriers.  (With RTA < 128 the M = 128
+// rows of a slice run into the next one's; the rows past RTA are dropped.)
 template <int BN, class Epi>
 struct OzSmem {
   static constexpr int STAGE = kS * 32 * (BM + BN);
@@ -330,33 +356,66 @@ struct OzSmem {
   static constexpr int TOTAL = BAR + 256 + 1024;
 };
 
+// Epilogue warps: four per TMEM lane quarter (two for the narrowest tile).
+// With two per quarter the drain and the epilogue, a chain of dependent
+// integer operations per value, took as long as 25 K blocks of MMAs.
+template <int BN>
+constexpr int kOzEpiWarps = BN >= 32 ? 16 : 8;
+template <int BN>
+constexpr int kOzThreads = 64 + 32 * kOzEpiWarps<BN>;
+
+// What an epilogue knows about its tile and thread.
+struct OzTile {
+  int b, mt, nt;  // batch entry, row and column tile
+  int r, c0;      // this thread's row of the tile, first of its warp's columns
+  int lane, ew;
+};
+
+// D_t .. D_{t+3} of eight columns as D_t 2^21 + D_{t+1} 2^14 + D_{t+2} 2^7 +
+// D_{t+3}; the pairs stay below 2^31.
+template <int BN>
+__device__ __forceinline__ void drain4(uint32_t base, int t, long long* sum) {
+  int p[8];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t r0[8], r1[8];
+    tmem_ld8_async(base + (uint32_t)((t + 2 * h) * BN), r0);
+    tmem_ld8_async(base + (uint32_t)((t + 2 * h + 1) * BN), r1);
+    tmem_ld_wait();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int q = __float2int_rn(__uint_as_float(r0[c])) * 128 + __float2int_rn(__uint_as_float(r1[c]));
+      if (h == 0)
+        p[c] = q;
+      else
+        sum[c] += (long long)p[c] * 16384 + q;
+    }
+  }
+}
+
 // Persistent contraction: one CTA per SM walks 128 x BN tiles.  Warp 0 copies
 // the operands' K blocks (16 values of K, all eight slices: contiguous in
 // memory) into the ring; one thread of warp 1 multiplies: slice i of A against
 // slices 0 .. 7 - i of B, which lie side by side as (8 - i) BN columns, into
 // the accumulator columns of D_i .. D_7, so that one instruction covers several
 // slice pairs and every A slice is read once per 256 columns.  36 of 64 pairs.
-// Eight warps drain the accumulators after every kOzSegBlk blocks (64-bit
-// integer sums in registers) and hand the rounded values to the epilogue.
+// The epilogue warps drain the accumulators after every kOzSegBlk blocks
+// (MULTI: 64-bit sums kept in registers) and hand the sums to the epilogue.
 // BN = 64 fills tensor memory with one set of accumulators; narrower tiles
 // have two, so that the epilogue overlaps the next segment.
 // Bound by the tensor pipe at large K: 36 x 64 columns take 1152 cycles per
-// K block against 48 KB of operands from L2 (43 B per cycle).  Measured (the
-// float64 pipe's limit is 1.2 TFLOP/s, its kernel reached 1.19): 1024 x 5050 x
-// 500 in 174 us, 29.7 TFLOP/s; 1024 x 4096 x 1800 in 383 us, 39.4 TFLOP/s.
-// Errors against 128-bit sums, relative to the operands' 2-norms (rms over
-// Gaussian rows, K = 16 .. 7500): 1.4e-17 .. 1.4e-18, a float64 FMA chain
-// 3.7e-17 .. 3.2e-17.
-template <int BN, class Epi>
-__global__ void __launch_bounds__(kOzThreads, 1)
+// K block against 48 KB of operands from L2 (43 B per cycle).
+template <int BN, class Epi, bool MULTI>
+__global__ void __launch_bounds__(kOzThreads<BN>, 1)
     k_oz_gemm(const OzArgs g, const __grid_constant__ Epi epi) {
   extern __shared__ uint8_t oz_raw[];
   using S = OzSmem<BN, Epi>;
+  constexpr int EW = kOzEpiWarps<BN>;
   constexpr int STAGES = S::STAGES;
   constexpr int NBUF = BN <= 32 ? 2 : 1;
   constexpr uint32_t DCOLS = kS * BN;
   constexpr uint32_t TCOLS = NBUF * DCOLS;
-  constexpr int CW = BN / 2;  // columns per epilogue warp
+  constexpr int CW = 4 * BN / EW;  // columns per epilogue warp
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::BAR);
   uint64_t* empty = full + STAGES;
@@ -372,7 +431,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], kEpiWarps);
+      mbar_init(&tempty[a], EW);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -453,15 +512,23 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     }
     if (!ok) *(volatile int*)abort_flag = 1;
   } else if (warp >= 2) {
-    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int q = warp & 3;
+    OzTile tl;
+    tl.lane = lane;
+    tl.ew = warp - 2;
+    tl.r = 32 * q + lane;
+    tl.c0 = CW * (tl.ew >> 2);
     int j = 0;
     for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
       const int b = t / per_batch, rem = t - b * per_batch, nt = rem / g.nmt, mt = rem - nt * g.nmt;
-      long long hi[CW], lo[CW];
+      tl.b = b;
+      tl.mt = mt;
+      tl.nt = nt;
+      long long hi[MULTI ? CW : 8], lo[MULTI ? CW : 8];
 #pragma unroll
-      for (int c = 0; c < CW; ++c) hi[c] = lo[c] = 0;
+      for (int c = 0; c < (MULTI ? CW : 8); ++c) hi[c] = lo[c] = 0;
       bool stop = false;
-      for (int sg = 0; sg < g.nseg; ++sg, ++j) {
+      for (int sg = 0; sg < (MULTI ? g.nseg : 1); ++sg, ++j) {
         const int buf = NBUF == 2 ? (j & 1) : 0;
         const bool bad = !mbar_wait_sleep(&tfull[buf], (j / NBUF) & 1, g.err, 64);
         fence_after();
@@ -470,35 +537,26 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
             "bar.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(out)
-            : "r"((uint32_t)(bad || *(volatile int*)abort_flag)), "n"(32 * kEpiWarps)
+            : "r"((uint32_t)(bad || *(volatile int*)abort_flag)), "n"(32 * EW)
             : "memory");
         if (out) {
           *(volatile int*)abort_flag = 1;
           stop = true;
           break;
         }
-        const uint32_t base = tmem + (uint32_t)buf * DCOLS + ((uint32_t)(32 * q) << 16) + (uint32_t)(CW * half);
+        const uint32_t base = tmem + (uint32_t)buf * DCOLS + ((uint32_t)(32 * q) << 16) + (uint32_t)tl.c0;
 #pragma unroll
         for (int c0 = 0; c0 < CW; c0 += 8) {
-          // pairs D_t 2^7 + D_{t+1} stay below 2^31
-          uint32_t r[4][8];
+          if constexpr (MULTI) {
+            drain4<BN>(base + (uint32_t)c0, 0, hi + c0);
+            drain4<BN>(base + (uint32_t)c0, 4, lo + c0);
+          } else {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) tmem_ld8_async(base + (uint32_t)(u * BN + c0), r[u]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const int p0 = __float2int_rn(__uint_as_float(r[0][c])) * 128 + __float2int_rn(__uint_as_float(r[1][c]));
-            const int p1 = __float2int_rn(__uint_as_float(r[2][c])) * 128 + __float2int_rn(__uint_as_float(r[3][c]));
-            hi[c0 + c] += (long long)p0 * 16384 + p1;
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) tmem_ld8_async(base + (uint32_t)((4 + u) * BN + c0), r[u]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const int p0 = __float2int_rn(__uint_as_float(r[0][c])) * 128 + __float2int_rn(__uint_as_float(r[1][c]));
-            const int p1 = __float2int_rn(__uint_as_float(r[2][c])) * 128 + __float2int_rn(__uint_as_float(r[3][c]));
-            lo[c0 + c] += (long long)p0 * 16384 + p1;
+            for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
+            drain4<BN>(base + (uint32_t)c0, 0, hi);
+            drain4<BN>(base + (uint32_t)c0, 4, lo);
+            epi.chunk(g, tl, tl.c0 + c0, hi, lo, smem + S::EPI);
+            __syncwarp();  // the next TMEM loads need the whole warp
           }
         }
         fence_before();
@@ -506,7 +564,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         if (lane == 0) mbar_arrive(&tempty[buf]);
       }
       if (stop) break;
-      epi.template run<CW>(g, b, mt, nt, 32 * q + lane, CW * half, lane, warp - 2, hi, lo, smem + S::EPI);
+      if constexpr (MULTI) {
+#pragma unroll
+        for (int c0 = 0; c0 < CW; c0 += 8) epi.chunk(g, tl, tl.c0 + c0, hi + c0, lo + c0, smem + S::EPI);
+      }
+      epi.template finish<EW>(g, tl, smem + S::EPI);
     }
   }
   fence_before();
@@ -518,46 +580,45 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 }
 
 // -------------------------------------------------------------- epilogues ---
+// chunk(): eight columns from column cc of the tile, row tl.r.
 // C[m][n] = 2^alpha D: each warp passes its 32 rows x 8 columns through 2 KB
 // of shared memory so that a store instruction covers four rows of 64 bytes.
 struct EpiOzStore {
   static constexpr int kStages = 4;
-  static constexpr int kSmemBytes = kEpiWarps * 32 * 8 * 8;
+  static constexpr int kSmemBytes = 16 * 32 * 8 * 8;
   double* C;
   long ldc;
   int M, N, alpha;
   const double* mask;
   int mask_rows;
-  template <int CW>
-  __device__ __forceinline__ void run(const OzArgs& g, int, int mt, int nt, int r, int c0, int lane, int ew,
-                                      const long long* hi, const long long* lo, uint8_t* sm) const {
-    double* buf = reinterpret_cast<double*>(sm) + ew * 256;
-    const int row = mt * g.a_rpt + r;
-    const int ea = row < M ? g.ea[row] : kOzZeroExp;
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
+                                        const long long* lo, uint8_t* sm) const {
+    double* buf = reinterpret_cast<double*>(sm) + tl.ew * 256;
+    const int lane = tl.lane, row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
+    const int ea = (row < M ? g.ea[row] : kOzZeroExp) + alpha;
 #pragma unroll
-    for (int c = 0; c < CW; c += 8) {
-      const int col = nt * g.b_rpt + c0 + c;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int eb = col + i < N ? g.eb[col + i] : kOzZeroExp;
-        // 16-byte slots permuted by row: row-per-lane writes without conflicts
-        buf[lane * 8 + ((i & 1) | (((i >> 1) ^ (lane & 3)) << 1))] = scaled_sum(hi[c + i], lo[c + i], ea, eb, alpha);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int rr = 4 * k + (lane >> 3), i = lane & 7;
-        const int grow = row - lane + rr, gcol = col + i;
-        if (grow < M && gcol < N && (!mask || walker_alive(mask, grow / mask_rows)))
-          C[(long)grow * ldc + gcol] = buf[rr * 8 + ((i & 1) | (((i >> 1) ^ (rr & 3)) << 1))];
-      }
-      __syncwarp();
+    for (int i = 0; i < 8; ++i) {
+      const int eb = col + i < N ? g.eb[col + i] : kOzZeroExp;
+      // 16-byte slots permuted by row: row-per-lane writes without conflicts
+      buf[lane * 8 + ((i & 1) | (((i >> 1) ^ (lane & 3)) << 1))] = scaled_sum(hi[i], lo[i], ea + eb);
     }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int rr = 4 * k + (lane >> 3), i = lane & 7;
+      const int grow = row - lane + rr, gcol = col + i;
+      if (grow < M && gcol < N && (!mask || walker_alive(mask, grow / mask_rows)))
+        C[(long)grow * ldc + gcol] = buf[rr * 8 + ((i & 1) | (((i >> 1) ^ (rr & 3)) << 1))];
+    }
+    __syncwarp();
   }
+  template <int EW>
+  __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
 };
 
 // A Taylor term: rows p, columns (c, i) of walker b.  A lane owns a row, so
-// the stores along p are contiguous.
+// the accesses along p are contiguous; the running sum's eight loads are
+// issued before the values are formed.
 struct EpiOzTerm {
   static constexpr int kStages = 4;
   static constexpr int kSmemBytes = 0;
@@ -567,23 +628,32 @@ struct EpiOzTerm {
   const double* tin;
   double* tout;
   double* acc;
-  template <int CW>
-  __device__ __forceinline__ void run(const OzArgs& g, int b, int mt, int nt, int r, int c0, int, int,
-                                      const long long* hi, const long long* lo, uint8_t*) const {
-    const int p = mt * g.a_rpt + r;
-    if (r >= g.a_rpt || p >= M) return;
-    const int ea = g.ea[(long)b * g.ea_batch + p];
-    const int* eb = g.eb + (long)b * g.eb_batch;
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
+                                        const long long* lo, uint8_t*) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
+    if (tl.r >= g.a_rpt || p >= M || col >= N2) return;
+    const int ea = g.ea[(long)tl.b * g.ea_batch + p];
+    const int* eb = g.eb + (long)tl.b * g.eb_batch + col;
+    const long at = ((long)tl.b * N2 + col) * M + p;
+    const double* src = (first ? tin : acc) + at;
+    double old[8], v[8];
+    int e[8];
 #pragma unroll
-    for (int c = 0; c < CW; ++c) {
-      const int col = nt * g.b_rpt + c0 + c;
-      if (col >= N2) break;
-      const double v = scaled_sum(hi[c], lo[c], ea, eb[col], 0) * scale;
-      const long at = ((long)b * N2 + col) * M + p;
-      if (!last) tout[at] = v;
-      acc[at] = (first ? tin[at] : acc[at]) + v;
+    for (int c = 0; c < 8; ++c) {
+      old[c] = col + c < N2 ? src[(long)c * M] : 0.0;
+      e[c] = col + c < N2 ? ea + eb[c] : kOzZeroExp;
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = scaled_sum(hi[c], lo[c], e[c]) * scale;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      if (col + c >= N2) break;
+      if (!last) tout[at + (long)c * M] = v[c];
+      acc[at + (long)c * M] = old[c] + v[c];
     }
   }
+  template <int EW>
+  __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
 };
 
 // Exchange: the tile of T into shared memory, then sum_ij T_ij T_ji per walker
@@ -593,31 +663,35 @@ struct EpiOzTerm {
 struct EpiOzExchange {
   static constexpr int kStages = 3;
   static constexpr int LD = 65;
-  static constexpr int kSmemBytes = BM * LD * 8 + 2 * kEpiWarps * 8;
+  static constexpr int kSmemBytes = BM * LD * 8 + 2 * 16 * 8;
   int N, W, G, RG, WT, nup, nchunk;  // RG vectors, WT walkers per tile
   double* part;
-  template <int CW>
-  __device__ __forceinline__ void run(const OzArgs& g, int, int mt, int nt, int r, int c0, int lane, int ew,
-                                      const long long* hi, const long long* lo, uint8_t* smraw) const {
-    double* T = reinterpret_cast<double*>(smraw);
-    double* red = T + BM * LD;
-    const int row = mt * g.a_rpt + r;
-    const bool rv = r < g.a_rpt && row < G * N;
-    const int ea = rv ? g.ea[row] : kOzZeroExp;
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
+                                        const long long* lo, uint8_t* sm) const {
+    double* T = reinterpret_cast<double*>(sm) + tl.r * LD + cc;
+    const int row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
+    const bool rv = tl.r < g.a_rpt && row < G * N;
+    const int ea = rv ? g.ea[row] : 0;
 #pragma unroll
-    for (int c = 0; c < CW; ++c) {
-      const int cc = c0 + c, col = nt * g.b_rpt + cc;
-      const int eb = cc < g.b_rpt && col < 2 * N * W ? g.eb[col] : kOzZeroExp;
-      T[r * LD + cc] = rv && eb != kOzZeroExp ? scaled_sum(hi[c], lo[c], ea, eb, 0) : 0.0;
+    for (int c = 0; c < 8; ++c) {
+      const bool in = rv && cc + c < g.b_rpt && col + c < 2 * N * W;
+      T[c] = in ? scaled_sum(hi[c], lo[c], ea + g.eb[col + c]) : 0.0;
     }
-    asm volatile("bar.sync 2, 256;" ::: "memory");
-    const int nw = WT >= kEpiWarps ? 1 : kEpiWarps / WT;
+  }
+  template <int EW>
+  __device__ __forceinline__ void finish(const OzArgs& g, const OzTile& tl, uint8_t* smraw) const {
+    const double* T = reinterpret_cast<const double*>(smraw);
+    double* red = reinterpret_cast<double*>(smraw) + BM * LD;
+    const int ew = tl.ew, lane = tl.lane;
+    asm volatile("bar.sync 2, %0;" ::"n"(32 * EW) : "memory");
+    const int nw = WT >= EW ? 1 : EW / WT, per = EW / nw;  // warps per walker, walkers at a time
     const int nrow = RG * N, nd = (N - 1) / 2;
-    for (int w0 = 0; w0 < WT; w0 += kEpiWarps / nw) {
-      const int wl = w0 + ew / nw, sub = ew % nw;
-      const int w = nt * WT + wl;
+    const int sub = ew % nw;
+    for (int w0 = 0; w0 < WT; w0 += per) {
+      const int wl = w0 + ew / nw, w = tl.nt * WT + wl;
+      const bool mine = ew < per * nw && wl < WT && w < W;
       double er = 0.0, ei = 0.0;
-      if (ew < (kEpiWarps / nw) * nw && wl < WT && w < W) {
+      if (mine) {
         const double* Tw = T + wl * 2 * N;
         for (int rr = sub * 32 + lane; rr < nrow; rr += 32 * nw) {
           const int gl = rr / N, i = rr - gl * N;
@@ -644,34 +718,38 @@ struct EpiOzExchange {
           er += sr;
           ei += si;
         }
+        er = warp_sum(er);
+        ei = warp_sum(ei);
+        if (lane == 0) {
+          red[2 * ew] = er;
+          red[2 * ew + 1] = ei;
+        }
       }
-      er = warp_sum(er);
-      ei = warp_sum(ei);
-      if (lane == 0) {
-        red[2 * ew] = er;
-        red[2 * ew + 1] = ei;
-      }
-      asm volatile("bar.sync 2, 256;" ::: "memory");
-      if (lane < 2 && sub == 0 && ew < (kEpiWarps / nw) * nw && wl < WT && w < W) {
+      asm volatile("bar.sync 2, %0;" ::"n"(32 * EW) : "memory");
+      if (mine && sub == 0 && lane < 2) {
         double sum = 0.0;
         for (int k = 0; k < nw; ++k) sum += red[2 * (ew + k) + lane];
-        part[((long)w * nchunk + mt) * 2 + lane] = sum;
+        part[((long)w * nchunk + tl.mt) * 2 + lane] = sum;
       }
-      asm volatile("bar.sync 2, 256;" ::: "memory");
+      asm volatile("bar.sync 2, %0;" ::"n"(32 * EW) : "memory");
     }
   }
 };
 
-template <int BN, class Epi>
-int launch_oz(const OzArgs& g, const Epi& e, cudaStream_t st) {
+template <int BN, class Epi, bool MULTI>
+int launch_oz_as(const OzArgs& g, const Epi& e, cudaStream_t st) {
   static std::atomic<unsigned long long> attr{0};
   constexpr int smem = OzSmem<BN, Epi>::TOTAL;
   static_assert(smem <= 227 * 1024, "shared memory");
-  AFQ_TRY(smem_attr_once(k_oz_gemm<BN, Epi>, smem, attr));
-  if (g.ntiles <= 0) return AFQMC_OK;
+  AFQ_TRY(smem_attr_once(k_oz_gemm<BN, Epi, MULTI>, smem, attr));
   const int sms = tc_sm_count();
-  AFQ_LAUNCH((k_oz_gemm<BN, Epi>), g.ntiles < sms ? g.ntiles : sms, kOzThreads, smem, st, g, e);
+  AFQ_LAUNCH((k_oz_gemm<BN, Epi, MULTI>), g.ntiles < sms ? g.ntiles : sms, kOzThreads<BN>, smem, st, g, e);
   return AFQMC_OK;
+}
+template <int BN, class Epi>
+int launch_oz(const OzArgs& g, const Epi& e, cudaStream_t st) {
+  if (g.ntiles <= 0) return AFQMC_OK;
+  return g.nseg > 1 ? launch_oz_as<BN, Epi, true>(g, e, st) : launch_oz_as<BN, Epi, false>(g, e, st);
 }
 
 OzArgs oz_args(const OzOperand& A, const OzOperand& B, long m, long n, int batch, int* err) {
@@ -722,8 +800,8 @@ int oz_slice_v(const double* Y, long ldy, int W, int M, int Mp, const OzOperand&
 }
 
 int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand& o, cudaStream_t st) {
-  dim3 grid(cdiv(N, 4), W);
-  AFQ_LAUNCH(k_oz_slice_term, grid, 128, 0, st, t, N, M, Mp, o);
+  dim3 grid(cdiv(N, 8), W);
+  AFQ_LAUNCH(k_oz_slice_term, grid, 256, 0, st, t, N, M, Mp, o);
   return AFQMC_OK;
 }
 

@@ -26,7 +26,7 @@ constexpr int kOzSlices = 8;
 constexpr int kOzSegBlk = 25;             // K blocks of 16 between two drains of the accumulators
 constexpr int kOzSegK = 16 * kOzSegBlk;   // 400: 10 * 2^12 * 400 < 2^24 (D_7: 2 * 2^13 + 6 * 2^12 per k)
 constexpr int kOzZeroExp = -30000;        // exponent of a row of zeros
-constexpr int kOzNanExp = 30000;          // a row holding an infinity or a NaN: its results are NaN
+constexpr int kOzNanExp = 100000;         // a row holding an infinity or a NaN: its results are NaN
 
 // Slices of `rows` operand rows as the kernel's shared-memory tiles: row tile
 // rt = r / rows_per_tile holds RT rows (a multiple of 8, >= rows_per_tile), K
