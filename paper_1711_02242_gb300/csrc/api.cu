@@ -67,12 +67,24 @@ static void oz_taylor_operands(size_t M, size_t N, size_t Mp, OzOperand* V, OzOp
   T->batch_exp_stride = (long)(2 * N);
 }
 
+// Phi of a walker by rows p and the rows of an inverse (K: the 2 N planes).
+static void oz_theta_operands(size_t M, size_t N, OzOperand* A, OzOperand* B) {
+  const size_t nt = oz_tiles(M, 128);
+  A->RT = A->rows_per_tile = (int)(((M + nt - 1) / nt + 7) / 8 * 8);
+  B->RT = B->rows_per_tile = oz_term_width((int)N);
+  A->nkb = B->nkb = (int)((2 * N + 15) / 16);
+  A->batch_stride = (long)oz_bytes(M, A->rows_per_tile, A->RT, 2 * N);
+  B->batch_stride = (long)oz_bytes(2 * N, B->rows_per_tile, B->RT, 2 * N);
+  A->batch_exp_stride = (long)M;
+  B->batch_exp_stride = (long)(2 * N);
+}
+
 static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz);
 
 size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   Bufs tmp;
   if (!b) b = &tmp;
-  bool oz = p.precision == AFQMC_FP64 && oz_pays(p.M, p.nwalkers);
+  bool oz = (p.precision == AFQMC_FP64 || p.ndet > 0) && oz_pays(p.M, p.nwalkers);
   if (oz) {
     Bufs probe;
     oz = plan_route(p, &probe, nullptr, true) <= kOzWorkspace;
@@ -87,8 +99,9 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   const bool mixed = p.precision != AFQMC_FP64;
   size_t nchunk = (G + exchange_chunk((int)N, p.nchol) - 1) / exchange_chunk((int)N, p.nchol);
   if (mixed) nchunk = G;  // the tensor-core exchange leaves one partial per vector
-  b->oz = oz;
-  b->oz_exch = oz && p.ndet == 0 && N <= 32;
+  b->oz = oz && !mixed;
+  b->oz_ov = oz;
+  b->oz_exch = b->oz && p.ndet == 0 && N <= 32;
   if (b->oz_exch) nchunk = oz_tiles(G, oz_exchange_vectors((int)N));
   const size_t lo = (p.precision == AFQMC_MIXED_BF16 || p.precision == AFQMC_MIXED_BF16_F32LU ||
                      p.precision == AFQMC_MIXED_BF16_F64THETA)
@@ -99,7 +112,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   const size_t Gp = (G + 7) / 8 * 8, Mp = (M + 15) / 16 * 16, Pp = (P + 3) / 4 * 4;
   Bump a{base};
   // constants
-  if (!oz) b->LpT = a.take<double>(P * G);
+  if (!b->oz) b->LpT = a.take<double>(P * G);
   b->Lh = a.take<double>(G * N * M);
   b->hh = a.take<double>(N * M);
   b->c = a.take<double>(G);
@@ -200,17 +213,27 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       o.data = a.take<char>(oz_bytes(rows, rpt, RT, k));
       o.exps = a.take<int>(rows);
     };
-    take(b->ozL, P, 64, 64, G);
-    take(b->ozB, M, 64, 64, M);
-    if (p.ndet == 0) take(b->ozF, G, 64, 64, N * M);
+    const size_t nds = p.ndet > 0 ? 2 * (size_t)p.ndet : 1;
+    take(b->ozV, nds * N, 64, 64, M);
+    if (p.ndet > 0) {
+      b->Sx = a.take<double>(W * 2 * N * nds * N);
+      b->md_Sinv = a.take<double>(nds * W * 2 * N * N);
+    }
+    if (b->oz) {
+      take(b->ozL, P, 64, 64, G);
+      take(b->ozB, M, 64, 64, M);
+      if (p.ndet == 0) take(b->ozF, G, 64, 64, N * M);
+    }
     if (b->oz_exch) {
       const int rpt = oz_exchange_vectors((int)N) * (int)N;
       take(b->ozX, G * N, rpt, (rpt + 7) / 8 * 8, M);
     }
     OzOperand V, T;
     oz_taylor_operands(M, N, Mp, &V, &T);
-    const size_t per = (size_t)(V.batch_stride + T.batch_stride);
-    size_t wc = kOzScratch / per;
+    const size_t per = b->oz ? (size_t)(V.batch_stride + T.batch_stride) : 0;
+    oz_theta_operands(M, N, &V, &T);
+    const size_t per_th = (size_t)V.batch_stride + nds * (size_t)T.batch_stride;
+    size_t wc = kOzScratch / std::max(per, per_th);
     wc = wc >= W ? W : wc < 64 ? 64 : wc / 64 * 64;
     if (wc > W) wc = W;
     b->oz_wc = (int)wc;
@@ -218,10 +241,13 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       if (bytes > oz_need) oz_need = bytes;
       if (exps > oz_exps) oz_exps = exps;
     };
-    need(per * wc, wc * (M + 2 * N));
-    need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
+    need(per_th * wc, wc * (M + nds * 2 * N));
     need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
-    if (p.ndet == 0) need(oz_bytes(2 * wc, 128, 128, N * M), 2 * wc);
+    if (b->oz) {
+      need(per * wc, wc * (M + 2 * N));
+      need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
+      if (p.ndet == 0) need(oz_bytes(2 * wc, 128, 128, N * M), 2 * wc);
+    }
     if (b->oz_exch) need(oz_bytes(2 * N * wc, 2 * (int)N * oz_exchange_walkers((int)N), 64, M), 2 * N * wc);
   }
   // scratch: the set-up and the step never run at the same time
@@ -256,7 +282,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   b->red = s2.take<double>(8);
   b->ych = (int)(G < 32 ? G : 32);
   b->Ych = s2.take<double>((size_t)b->ych * M * M);
-  if (oz) b->LpT = s2.take<double>(P * G);  // only the set-up reads it: the step has its slices
+  if (b->oz) b->LpT = s2.take<double>(P * G);  // only the set-up reads it: the step has its slices
   b->P = (int)P;
   b->nchunk = (int)nchunk;
   b->gc = exchange_chunk((int)N, p.nchol);
@@ -396,12 +422,20 @@ int overlap_update(afqmc_state* s, bool into_ld, bool timed) {
     ov.theta32 = b.theta32 ? 1 : 0;
   }
   if (timed) prof_begin(s, AFQMC_PH_OVERLAP);
+  if (b.oz_ov && s->spin2) {
+    AFQ_TRY(oz_trial_overlaps(s, b.S, p.N));
+    ov.Sext = b.S;
+    ov.ldS = p.N;
+  }
   AFQ_TRY(launch_overlap(ov, s->st));
   if (timed) {
     prof_end(s);
     prof_begin(s, AFQMC_PH_THETA);
   }
-  AFQ_TRY(launch_theta(ov, s->st));
+  if (b.oz_ov)
+    AFQ_TRY(oz_theta_rows(s, b.Sinv, 1, b.thetaT, ov.logdet, 2, ov.unit_trial, 0, nullptr));
+  else
+    AFQ_TRY(launch_theta(ov, s->st));
   if (timed) prof_end(s);
   return AFQMC_OK;
 }
@@ -531,6 +565,45 @@ static int oz_rows_gemm(afqmc_state* s, const double* src, int rw, int k, const 
     g.mask_rows = rw;
     g.err = b.status;
     AFQ_TRY(oz_gemm_store(g, s->st));
+  }
+  return AFQMC_OK;
+}
+
+int oz_trial_overlaps(afqmc_state* s, double* dst, int n) {
+  return oz_rows_gemm(s, s->b.phiT, 2 * s->p.N, s->p.M, s->b.ozV, dst, n, 0, nullptr);
+}
+
+int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
+                  int unit, int zero_singular, void* th_lo) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  OzTheta t;
+  oz_theta_operands(p.M, p.N, &t.A, &t.B);
+  t.W = p.nwalkers;
+  t.M = p.M;
+  t.N = p.N;
+  t.nds = nds;
+  t.theta = theta;
+  t.ld = ld;
+  t.ld_w = ld_w;
+  t.wt = b.wt;
+  t.unit = unit;
+  t.zero_singular = zero_singular;
+  t.th_lo = th_lo;
+  t.lo_kind = b.lo_kind;
+  t.Mp = b.Mp;
+  t.err = b.status;
+  for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
+    t.w0 = w0;
+    t.nw = std::min(b.oz_wc, p.nwalkers - w0);
+    t.A.data = b.oz_mem;
+    t.A.exps = b.oz_exp;
+    t.B.data = b.oz_mem + (size_t)t.nw * t.A.batch_stride;
+    t.B.exps = b.oz_exp + (size_t)t.nw * t.A.batch_exp_stride;
+    AFQ_TRY(oz_slice_cols(b.phiT + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, s->st));
+    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(sinv), p.nwalkers, w0, t.nw, nds, p.N, t.B,
+                             s->st));
+    AFQ_TRY(oz_theta(t, s->st));
   }
   return AFQMC_OK;
 }
@@ -1352,6 +1425,8 @@ static int setup_device(afqmc_state* s, const double* h1, const double* L, const
     AFQ_TRY(launch_split_lo(b.Bh, M, M, M, b.Bh_split, b.Kp1, 2, 0x2u, b.lo_kind, st, 1.0));
     AFQ_TRY(launch_split_lo(b.Bh, M, M, M, b.Bh_split_tf, b.Mp, 4, 0xCu, LO_TF32, st, 1.0));
   }
+  if (b.oz_ov)
+    AFQ_TRY(oz_slice_rows(md ? b.md_V : b.VTt, (md ? 2L * p.ndet : 1L) * N, M, M, b.ozV, st));
   // walkers at the trial, their overlaps, and the trial energy
   AFQ_TRY(launch_init_walkers(b.VTt, b.phiT, b.wt, W, N, M, st));
   AFQ_TRY(refresh_phi_lo(s));

@@ -161,6 +161,12 @@ struct OverlapArgs {
   // closed-shell block standing for both spins); sf = spins per block (2 or 1)
   int nup = 0;
   double sf = 2.0;
+  // S formed by a contraction: S[i][j] of (w, ds) at Sext[((2 w + c) N + j) ldS
+  // + ds N + i].  nds > 0: that many overlaps per walker, S^-1 of (ds, w) at
+  // Sinv[(ds W + w) N N], log det at logdet[2 (w nds + ds)]
+  const double* Sext = nullptr;
+  long ldS = 0;
+  int nds = 0;
 };
 // S^-1 and log det (k_overlap), then Theta (k_theta_rows)
 int launch_overlap(const OverlapArgs& a, cudaStream_t st);

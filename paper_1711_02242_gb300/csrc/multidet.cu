@@ -774,6 +774,27 @@ int smw_detect(afqmc_state* s, const double* up, const double* dn) {
 
 static int smw_chunks(const afqmc_params& p) { return (p.nchol + kSmwGC - 1) / kSmwGC; }
 
+// S, log det and Theta of the first nds (d, s) of every walker: S of all
+// determinants as one contraction, the eliminations, Theta as a contraction
+// (k_md_overlap, one block per (d, s) and walker, formed S with N^2 threads
+// summing over M one after another and took the logarithms inside the pivot
+// loop: 606 us a step at M = 100, N = 10, four determinants, 256 walkers).
+static int md_overlaps_tc(afqmc_state* s, int nds, void* th_lo) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  const int n = nds * p.N;
+  AFQ_TRY(oz_trial_overlaps(s, b.Sx, n));
+  OverlapArgs ov{p.nwalkers, p.M, p.N, nullptr, b.phiT, b.md_theta, b.md_ld, b.wt};
+  ov.Sinv = reinterpret_cast<double2*>(b.md_Sinv);
+  ov.nup = p.N;
+  ov.sf = 1.0;
+  ov.Sext = b.Sx;
+  ov.ldS = n;
+  ov.nds = nds;
+  AFQ_TRY(launch_overlap(ov, s->st));
+  return oz_theta_rows(s, b.md_Sinv, nds, b.md_theta, b.md_ld, 2 * nds, 0, 1, th_lo);
+}
+
 static int smw_overlap_update(afqmc_state* s, bool into_ld) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
@@ -782,8 +803,11 @@ static int smw_overlap_update(afqmc_state* s, bool into_ld) {
   AFQ_CUDA(cudaFuncSetAttribute(k_md_overlap, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
   // determinant 0 only: S_0s, log det, Theta_0s (md_ld rows [w][s])
-  AFQ_LAUNCH(k_md_overlap, dim3(2, W), 256, smem, s->st, W, M, N, b.md_V, b.phiT, b.wt,
-             b.md_theta, b.md_ld, nullptr, b.lo_kind, b.Mp);
+  if (b.oz_ov)
+    AFQ_TRY(md_overlaps_tc(s, 2, nullptr));
+  else
+    AFQ_LAUNCH(k_md_overlap, dim3(2, W), 256, smem, s->st, W, M, N, b.md_V, b.phiT, b.wt,
+               b.md_theta, b.md_ld, nullptr, b.lo_kind, b.Mp);
   AFQ_LAUNCH(k_smw_ratio, W, 128, 0, s->st, W, M, N, nd, kSmwMaxK * nd, s->smw_np[0],
              s->smw_np[1], b.smw_tab, b.smw_prow, b.md_V, b.md_theta, b.md_ld, b.md_logA, b.wt,
              b.smw_xi, b.md_w, into_ld ? b.ld : b.ld_new);
@@ -826,8 +850,11 @@ int md_overlap_update(afqmc_state* s, bool into_ld) {
   const size_t smem = sizeof(double2) * (size_t)N * 2 * N;
   AFQ_CUDA(cudaFuncSetAttribute(k_md_overlap, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
-  AFQ_LAUNCH(k_md_overlap, dim3(2 * nd, W), 256, smem, s->st, W, M, N, b.md_V, b.phiT, b.wt,
-             b.md_theta, b.md_ld, b.mixed ? b.md_theta_lo : nullptr, b.lo_kind, b.Mp);
+  if (b.oz_ov)
+    AFQ_TRY(md_overlaps_tc(s, 2 * nd, b.mixed ? b.md_theta_lo : nullptr));
+  else
+    AFQ_LAUNCH(k_md_overlap, dim3(2 * nd, W), 256, smem, s->st, W, M, N, b.md_V, b.phiT, b.wt,
+               b.md_theta, b.md_ld, b.mixed ? b.md_theta_lo : nullptr, b.lo_kind, b.Mp);
   AFQ_LAUNCH(k_md_combine, cdiv(W, 128), 128, 0, s->st, W, nd, b.md_logA, b.md_ld, b.wt,
              into_ld ? b.ld : b.ld_new, b.md_w);
   return AFQMC_OK;

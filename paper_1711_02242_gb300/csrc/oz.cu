@@ -254,6 +254,98 @@ __global__ void __launch_bounds__(256) k_oz_slice_term(const double* t, int N, i
   }
 }
 
+// Rows p = [Re Phi_p | Im Phi_p] of walker blockIdx.y: K runs over the 2 N
+// orbital planes, a lane owns a row, so both the reads along p and the writes
+// (eight rows of a chunk: 128 contiguous bytes per slice) are contiguous.
+__global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N2, int M, OzOperand o) {
+  __shared__ uint32_t m_sh[8][32], any_sh[8][32];
+  const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, w = blockIdx.y;
+  const int p = blockIdx.x * 32 + lane;
+  const double* src = phi + (long)w * N2 * M + p;
+  uint32_t m = 0, any = 0;
+  if (p < M)
+    for (int k = wk; k < N2; k += 8) {
+      const double x = src[(long)k * M];
+      m = max(m, abs_hi(x));
+      any |= abs_hi(x) | (uint32_t)__double2loint(x);
+    }
+  m_sh[wk][lane] = m;
+  any_sh[wk][lane] = any;
+  __syncthreads();
+  if (p >= M) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    m = max(m, m_sh[q][lane]);
+    any |= any_sh[q][lane];
+  }
+  const int e = row_exp(m, any != 0);
+  const bool fine = e != kOzNanExp && e != kOzZeroExp;
+  if (wk == 0) o.exps[(long)w * o.batch_exp_stride + p] = e;
+  const int rt = p / o.rows_per_tile, r = p - rt * o.rows_per_tile;
+  char* base = reinterpret_cast<char*>(o.data) + (long)w * o.batch_stride +
+               (long)rt * o.nkb * (kS * o.RT * 32);
+  for (int c = wk; c < 2 * o.nkb; c += 8) {
+    long long u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * c + i;
+      u[i] = kDigitBias + (fine && k < N2 ? fixed57(src[(long)k * M], e) : 0ll);
+    }
+    put_chunk(base + chunk_off(o.RT, r, c), o.RT * 32, u);
+  }
+}
+
+// The inverse of (ds, w) = (blockIdx.y, blockIdx.x) as operand rows (re, j) =
+// [Re S^-1_j | -Im S^-1_j] and (im, j) = [Im S^-1_j | Re S^-1_j], S^-1_j column j.
+__global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, int W, int w0, int N,
+                                                          OzOperand o) {
+  __shared__ int e_sh[64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int w = blockIdx.x, ds = blockIdx.y;
+  const long batch = (long)ds * gridDim.x + w;
+  const double2* S = sinv + ((long)ds * W + w0 + w) * N * N;
+  int* ex = o.exps + batch * o.batch_exp_stride;
+  for (int j = warp; j < N; j += 8) {
+    uint32_t m = 0, any = 0;
+    for (int i = lane; i < N; i += 32) {
+      const double2 x = S[i * N + j];
+      m = max(m, max(abs_hi(x.x), abs_hi(x.y)));
+      any |= abs_hi(x.x) | (uint32_t)__double2loint(x.x) | abs_hi(x.y) | (uint32_t)__double2loint(x.y);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    any = __reduce_or_sync(0xffffffffu, any);
+    if (lane == 0) {
+      const int e = row_exp(m, any != 0);
+      e_sh[j] = e;
+      ex[j] = ex[N + j] = e;
+    }
+  }
+  __syncthreads();
+  const int rows8 = (2 * N + 7) / 8 * 8;
+  const long tile_stride = (long)o.nkb * (kS * o.RT * 32);
+  char* base = reinterpret_cast<char*>(o.data) + batch * o.batch_stride;
+  for (int it = threadIdx.x; it < rows8 * 2 * o.nkb; it += 256) {
+    const int row = it % rows8, c = it / rows8;
+    if (row >= 2 * N) continue;
+    const int im = row >= N ? 1 : 0, j = row - im * N, e = e_sh[j];
+    const bool fine = e != kOzNanExp && e != kOzZeroExp;
+    long long u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * c + i;
+      u[i] = kDigitBias;
+      if (fine && k < 2 * N) {
+        const int part = k >= N ? 1 : 0;
+        const double2 x = S[(k - part * N) * N + j];
+        const long long f = fixed57(im == part ? x.x : x.y, e);
+        u[i] += (im == 0 && part == 1) ? -f : f;
+      }
+    }
+    put_chunk(base + (row / o.rows_per_tile) * tile_stride + chunk_off(o.RT, row % o.rows_per_tile, c),
+              o.RT * 32, u);
+  }
+}
+
 // ------------------------------------------------------------ contraction ---
 // (hi 2^28 + lo) 2^e as float64, rounded to nearest even once.
 __device__ __forceinline__ double round_sum(long long hi, long long lo, int e) {
@@ -341,6 +433,7 @@ struct OzArgs {
   int RTA;
   int nkb, nseg;
   int nmt, nnt, ntiles;     // tiles = batch x nnt x nmt, mt fastest
+  int a_mod;                // batch entry b reads A of entry b % a_mod
   int* err;
 };
 
@@ -453,7 +546,7 @@ __global__ void __launch_bounds__(kOzThreads<BN>, 1)
     int it = 0;
     for (int t = blockIdx.x; t < g.ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
       const int b = t / per_batch, rem = t - b * per_batch, nt = rem / g.nmt, mt = rem - nt * g.nmt;
-      const char* a_src = g.A + b * g.a_batch + (long)mt * g.nkb * g.a_bytes;
+      const char* a_src = g.A + (b % g.a_mod) * g.a_batch + (long)mt * g.nkb * g.a_bytes;
       const char* b_src = g.B + b * g.b_batch + (long)nt * g.nkb * B_BYTES;
       for (int kb = 0; kb < g.nkb; ++kb, ++it) {
         const int s = it % STAGES;
@@ -656,6 +749,35 @@ struct EpiOzTerm {
   __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
 };
 
+// Theta rows: like a Taylor term's, batch entry b = (ds, w).
+struct EpiOzTheta {
+  static constexpr int kStages = 4;
+  static constexpr int kSmemBytes = 0;
+  OzTheta t;
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
+                                        const long long* lo, uint8_t*) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc, N2 = 2 * t.N;
+    if (tl.r >= g.a_rpt || p >= t.M || col >= N2) return;
+    const int ds = tl.b / t.nw, wl = tl.b - ds * t.nw, w = t.w0 + wl;
+    if (t.wt && !walker_alive(t.wt, w)) return;
+    const bool ok = t.ld[(long)w * t.ld_w + (long)ds * t.ld_ds] > -INFINITY;
+    if (!ok && !t.zero_singular) return;
+    const int ea = g.ea[(long)wl * g.ea_batch + p];
+    const int* eb = g.eb + (long)tl.b * g.eb_batch + col;
+    const long row = ((long)ds * t.W + w) * N2 + col;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      if (col + c >= N2) break;
+      double v = ok ? scaled_sum(hi[c], lo[c], ea + eb[c]) : 0.0;
+      if (t.unit && p < t.N) v = col + c == p ? 1.0 : 0.0;
+      t.theta[(row + c) * t.M + p] = v;
+      if (t.th_lo) store_lo(t.th_lo, t.lo_kind, (row + c) * t.Mp + p, v);
+    }
+  }
+  template <int EW>
+  __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
+};
+
 // Exchange: the tile of T into shared memory, then sum_ij T_ij T_ji per walker
 // of the tile over the tile's vectors; every unordered pair {i, j} once, at
 // twice its weight (j = i + d mod N), by the lane of row (g, i); nw warps per
@@ -771,6 +893,7 @@ OzArgs oz_args(const OzOperand& A, const OzOperand& B, long m, long n, int batch
   g.nmt = (int)oz_tiles(m, A.rows_per_tile);
   g.nnt = (int)oz_tiles(n, B.rows_per_tile);
   g.ntiles = g.nmt * g.nnt * batch;
+  g.a_mod = batch;
   g.err = err;
   return g;
 }
@@ -821,6 +944,28 @@ int oz_taylor_term(const OzTerm& t, cudaStream_t st) {
   if (bn == 16) return launch_oz<16>(g, e, st);
   if (bn == 32) return launch_oz<32>(g, e, st);
   return launch_oz<64>(g, e, st);
+}
+
+int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, 2 * N, M, o);
+  return AFQMC_OK;
+}
+
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,
+                     cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, o);
+  return AFQMC_OK;
+}
+
+int oz_theta(const OzTheta& t, cudaStream_t st) {
+  const int bn = oz_term_width(t.N);
+  AFQ_TRY(check_operand(t.A, t.B, bn));
+  EpiOzTheta e{t};
+  OzArgs g = oz_args(t.A, t.B, t.M, 2 * t.N, t.nds * t.nw, t.err);
+  g.a_mod = t.nw;
+  if (bn == 16) return launch_oz_as<16, EpiOzTheta, false>(g, e, st);
+  if (bn == 32) return launch_oz_as<32, EpiOzTheta, false>(g, e, st);
+  return launch_oz_as<64, EpiOzTheta, false>(g, e, st);
 }
 
 int oz_exchange_vectors(int N) { return BM / N > 0 ? BM / N : 1; }

@@ -81,6 +81,31 @@ struct OzTerm {
 int oz_term_width(int N);
 int oz_taylor_term(const OzTerm& t, cudaStream_t st);
 
+// Theta = Phi S^-1 of nds inverses per walker (see oz.cu for the operands):
+// theta[ds][w][2][N][M]; rows p < N are the identity when unit.  A walker with
+// weight 0 or without an inverse (log det -inf, at ld[w ld_w + ds ld_ds])
+// keeps its rows, or gets zeros (zero_singular, live walkers only).
+struct OzTheta {
+  int W = 0, M = 0, N = 0, nds = 1;
+  int w0 = 0, nw = 0;   // walkers [w0, w0 + nw) of the operands
+  OzOperand A, B;
+  double* theta = nullptr;
+  const double* ld = nullptr;
+  int ld_w = 2, ld_ds = 2;
+  const double* wt = nullptr;
+  int unit = 0, zero_singular = 0;
+  void* th_lo = nullptr;  // BF16/TF32 copy of the rows, pitch Mp
+  int lo_kind = 0, Mp = 0;
+  int* err = nullptr;
+};
+// operand rows p = [Re Phi_p | Im Phi_p] (2 N values) of W walkers
+int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st);
+// operand rows (re, j) = [Re S^-1_j | -Im S^-1_j], (im, j) = [Im | Re] of the
+// inverses sinv[ds W + w0 + w], batch ds nw + w
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,
+                     cudaStream_t st);
+int oz_theta(const OzTheta& t, cudaStream_t st);
+
 // Exchange: part[w][c][2] = sum over the vectors of row tile c of
 // sum_ij T_ij T_ji, T_g = Lh_g Theta_w (same-spin pairs).  A: rows (g, i),
 // rows_per_tile a multiple of N; B: rows (w, c, j), rows_per_tile a multiple

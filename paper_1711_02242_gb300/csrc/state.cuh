@@ -55,8 +55,13 @@ struct Bufs {
   // (p, q)), of the force bias (rows g) and of the exchange (rows (g, i)), and
   // of B_half; oz_mem / oz_exp: slices and row exponents of oz_wc walkers at a
   // time, whatever the contraction at hand reads
-  bool oz = false, oz_exch = false;
-  OzOperand ozL, ozF, ozX, ozB;
+  // oz_ov: Theta = Phi S^-1 and the products V^T Phi that are no gather (ozV:
+  // rows of the trial's orbitals; Sx, md_Sinv: the overlaps of every
+  // determinant and their inverses), also for a multi-determinant trial on
+  // the mixed path, which keeps these in float64
+  bool oz = false, oz_exch = false, oz_ov = false;
+  OzOperand ozL, ozF, ozX, ozB, ozV;
+  double *Sx = nullptr, *md_Sinv = nullptr;
   char* oz_mem = nullptr;
   int* oz_exp = nullptr;
   int oz_wc = 0;
@@ -169,6 +174,11 @@ int md_setup(afqmc_state* s, const double* coef);
 int smw_detect(afqmc_state* s, const double* up, const double* dn);
 // Make the state's stream wait for a pending side-stream Gram-Schmidt.
 int join_side(afqmc_state* s);
+// Theta rows of nds inverses per walker on the tensor cores (b.oz_ov; see
+// OzTheta), and S of every determinant (or of two spin blocks) into dst
+int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
+                  int unit, int zero_singular, void* th_lo);
+int oz_trial_overlaps(afqmc_state* s, double* dst, int n);
 }  // namespace afq
 
 namespace afq {

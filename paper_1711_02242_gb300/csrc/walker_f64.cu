@@ -391,7 +391,7 @@ struct Vec2<float> {
 // order (pos[c] = the column of A holding column c of S^-1), log det stored
 // for live walkers.  Returns true when S is singular (block-uniform).
 template <typename T>
-__device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, bool live,
+__device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, int ds, bool live,
                                              typename Vec2<T>::type* A, int* pos) {
   using T2 = typename Vec2<T>::type;
   __shared__ __align__(16) unsigned char misc_raw[sizeof(T2) * 129];
@@ -403,7 +403,17 @@ __device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, bool l
   __shared__ int order[64];
   const double* fr = a.phiT + (long)w * 2 * N * M;
   const double* fi = fr + (long)N * M;
-  if (a.unit_trial) {
+  if (a.Sext) {
+    // formed beforehand; zero between two spin blocks (see below)
+    const int nup = a.nup > 0 ? a.nup : N;
+    const double* sr = a.Sext + (long)w * 2 * N * a.ldS + (long)ds * N;
+    for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
+      const int j = idx / N, i = idx - j * N;
+      const bool in = (i < nup) == (j < nup);
+      A[i * N + j] = Vec2<T>::make(Vec2<T>::from_f64(in ? sr[j * a.ldS + i] : 0.0),
+                                   Vec2<T>::from_f64(in ? sr[(N + j) * a.ldS + i] : 0.0));
+    }
+  } else if (a.unit_trial) {
     // S[i][j] = Phi[i][j], the top block of the orbitals
     for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
       const int i = idx / N, j = idx % N;
@@ -549,12 +559,13 @@ __device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, bool l
   }
   __syncthreads();
   if (threadIdx.x == 0 && live) {
+    double* ld = a.logdet + 2 * (a.nds > 0 ? (long)w * a.nds + ds : (long)w);
     if (singular) {
-      a.logdet[2L * w] = -INFINITY;
-      a.logdet[2L * w + 1] = 0.0;
+      ld[0] = -INFINITY;
+      ld[1] = 0.0;
     } else {
-      a.logdet[2L * w] = a.sf * (red[0] + red[2]);
-      a.logdet[2L * w + 1] = wrap_pi(a.sf * ((red[1] + red[3]) + 3.141592653589793 * swaps));
+      ld[0] = a.sf * (red[0] + red[2]);
+      ld[1] = wrap_pi(a.sf * ((red[1] + red[3]) + 3.141592653589793 * swaps));
     }
   }
   return singular != 0;
@@ -565,14 +576,14 @@ __global__ void __launch_bounds__(OV_T) k_overlap(OverlapArgs a) {
   using T2 = typename Vec2<T>::type;
   extern __shared__ __align__(16) unsigned char ov_raw[];
   __shared__ int pos[64];
-  const int w = blockIdx.x, N = a.N;
+  const int w = blockIdx.x, ds = blockIdx.y, N = a.N;
   const bool live = !a.wt || walker_alive(a.wt, w);
   T2* A = reinterpret_cast<T2*>(ov_raw);  // [N][N], inverted in place
-  const bool singular = overlap_core<T>(a, w, live, A, pos);
+  const bool singular = overlap_core<T>(a, w, ds, live, A, pos);
   // S^-1 of live, non-singular walkers for the Theta kernel: column c of the
   // inverse is column pos[c] of A (the row interchanges undone)
   if (singular || !live) return;
-  T2* si = Vec2<T>::sinv(a) + (long)w * N * N;
+  T2* si = Vec2<T>::sinv(a) + ((long)ds * a.W + w) * N * N;
   for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
     const int r = idx / N, c = idx - (idx / N) * N;
     si[idx] = A[r * N + pos[c]];
@@ -725,7 +736,7 @@ static int launch_theta_rows(const OverlapArgs& a, cudaStream_t st) {
 
 int launch_overlap(const OverlapArgs& a, cudaStream_t st) {
   const size_t smem = 2ull * a.N * a.N * sizeof(double2);
-  if (!a.Sinv || (!a.unit_trial && (a.Sinv32 || a.nup <= 0 || a.nup > a.N))) {
+  if (!a.Sinv || (!a.unit_trial && !a.Sext && (a.Sinv32 || a.nup <= 0 || a.nup > a.N))) {
     set_error("overlap: S^-1 scratch is required, and a trial other than V_T = [I; 0] only "
               "in float64 with two spin blocks");
     return AFQMC_EINVAL;
@@ -742,7 +753,7 @@ int launch_overlap(const OverlapArgs& a, cudaStream_t st) {
     AFQ_LAUNCH(k_overlap<float>, a.W, OV_T, smem / 2, st, a);
     return AFQMC_OK;
   }
-  AFQ_LAUNCH(k_overlap<double>, a.W, OV_T, smem, st, a);
+  AFQ_LAUNCH(k_overlap<double>, dim3(a.W, a.nds > 0 ? a.nds : 1), OV_T, smem, st, a);
   return AFQMC_OK;
 }
 

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import workloads
-from oracle import afqmc
+from oracle import afqmc, multidet, smw
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +98,50 @@ def test_chunks_of_walkers(pkg):
     assert np.all(np.isfinite(el)) and np.unique(el).size == W
     big.close()
     small.close()
+
+
+@pytest.mark.parametrize("M,N,nd,kind,precision", [
+    (40, 5, 3, "noci", 0),    # the fewest orbitals of the route
+    (70, 33, 2, "noci", 0),   # two column tiles of Theta, 132 rows of the trial's orbitals
+    (130, 6, 2, "noci", 0),   # two row tiles of Phi
+    (44, 6, 4, "ci", 0),      # relative to determinant 0: its overlap alone
+    (44, 6, 3, "noci", 2),    # the mixed path keeps these float64
+])
+def test_determinants(pkg, M, N, nd, kind, precision):
+    """Overlaps and Theta of every determinant, against the oracles' walks.  On
+    the mixed path only the first local energies are compared: the BF16
+    exchange and traces are good to 2^-8 of their terms there."""
+    G, W = 50, 5
+    h1, L, C = inputs(M, N, G)
+    rng = np.random.default_rng(M + nd)
+    full = np.linalg.qr(np.hstack([C, rng.standard_normal((M, M - N))]))[0]
+    ups, dns = [C], [C]
+    for d in range(1, nd):
+        if kind == "ci":
+            u, v = C.copy(), C.copy()
+            u[:, d] = full[:, N + d]
+            v[:, 0] = full[:, N + 2 * d]
+        else:
+            u, v = (np.linalg.qr(C + 0.05 * rng.standard_normal((M, N)))[0] for _ in range(2))
+        ups.append(u)
+        dns.append(v)
+    ups, dns = np.array(ups), np.array(dns)
+    coef = np.array([1.0] + [0.2 / d + 0.1j for d in range(1, nd)])
+    Orc = smw.SMWOracle if kind == "ci" else multidet.MultiDetOracle
+    orc = Orc(h1, L, coef, ups, dns, W, afqmc.Params(qr_period=2, energy_period=1))
+    p = pkg.default_params(M, N, G, W, qr_period=2, energy_period=1, ndet=nd, precision=precision)
+    run = pkg.AfqmcRun(h1, L, (coef, ups, dns), p)
+    if precision:
+        el = orc.local_energies()
+        assert np.max(np.abs(run.local_energies() - el) / np.abs(el)) < 2.0 ** -8
+        return
+    run.propagate(3)
+    orc.run(3)
+    phi, wt, lo = run.get_walkers()
+    assert np.max(np.abs(phi - orc.phi)) < TOL * np.abs(orc.phi).max()
+    assert np.max(np.abs(wt - orc.weight) / orc.weight) < TOL
+    assert np.max(np.abs(lo - orc.logdet)) < TOL * (1 + np.abs(orc.logdet).max())
+    el = orc.local_energies()
+    assert np.max(np.abs(run.local_energies() - el) / np.abs(el)) < TOL
+    assert run.info().status == 0
+    run.close()
