@@ -590,6 +590,149 @@ __global__ void __launch_bounds__(OV_T) k_overlap(OverlapArgs a) {
   }
 }
 
+// The same elimination with a lane per row and floor(32 / N) walkers per warp
+// (N <= 16), the rows in registers: the pivot row comes by shuffle, rows are
+// not moved (each lane keeps the position its row would have), and the columns
+// rotate by one per pivot so that the pivot column is always register 0 and
+// the loop over pivots needs no unrolling.  Same operations on the same
+// values in the same order as k_overlap<double>, so the same results, without
+// its three block barriers per pivot.  Bound by the latency of the float64
+// chain of a pivot (|a|^2, the reciprocal, the factors), 7.4 k cycles at
+// N = 10.  1024 walkers, N = 10: 73.3 us (one block of 256 threads per walker,
+// 100 of them with an element) to 38.7; 128 walkers, N = 2: 15.2 to 12.2.
+// Above 16 rows a warp has one walker and the block's eight warps win: 301
+// walkers, N = 17: 59 us against 72; 512, N = 25: 128.9 us either way.
+namespace {
+constexpr int OW_WARPS = 4;
+}
+template <int N>
+__global__ void __launch_bounds__(32 * OW_WARPS) k_overlap_warp(OverlapArgs a) {
+  constexpr int PER = 32 / N;  // walkers per warp
+  __shared__ int inv_sh[OW_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ds = blockIdx.y, M = a.M;
+  const int seg = lane / N < PER ? lane / N : PER - 1;  // spare lanes follow the last walker
+  const int base = seg * N, r0 = lane - base;           // own row (>= N for spare lanes)
+  const bool row = r0 < N;
+  const long w = ((long)blockIdx.x * OW_WARPS + warp) * PER + seg;
+  const bool in = w < a.W;
+  double xr[N], xi[N];
+  if (a.Sext) {
+    const int nup = a.nup > 0 ? a.nup : N;
+    const double* sr = a.Sext + w * 2 * N * a.ldS + (long)ds * N + r0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const bool ok = in && row && (r0 < nup) == (j < nup);
+      xr[j] = ok ? sr[j * a.ldS] : 0.0;
+      xi[j] = ok ? sr[(N + j) * a.ldS] : 0.0;
+    }
+  } else {
+    const double* fr = a.phiT + w * 2 * N * M + r0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      xr[j] = in && row ? fr[(long)j * M] : 0.0;
+      xi[j] = in && row ? fr[(long)(N + j) * M] : 0.0;
+    }
+  }
+  int pos = r0, swaps = 0;  // the row's position after the interchanges so far
+  bool singular = false;
+  double pvr = 1.0, pvi = 0.0;  // pivot r0, kept for the log det
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) {
+    // pivot: the largest |a_rk|^2 at positions >= k, the first position on ties
+    const double v = xr[0] * xr[0] + xi[0] * xi[0];
+    unsigned long long key = row && pos >= k && v > 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+    int best = row && pos >= k ? pos : N, who = lane;
+#pragma unroll
+    for (int o = 1; o < N; o <<= 1) {
+      // all-to-all over the segment: after the steps every row has seen all
+      const int src = base + (r0 + o) % N;
+      const unsigned long long ok_ = __shfl_sync(0xffffffffu, key, src);
+      const int ob = __shfl_sync(0xffffffffu, best, src), ow = __shfl_sync(0xffffffffu, who, src);
+      if (ok_ > key || (ok_ == key && ob < best)) {
+        key = ok_;
+        best = ob;
+        who = ow;
+      }
+    }
+    if (key == 0ull) singular = true;
+    // 1 / pivot: the real part by even, the imaginary part by odd rows
+    const double pr = __shfl_sync(0xffffffffu, xr[0], who), pi = __shfl_sync(0xffffffffu, xi[0], who);
+    if (r0 == k) {
+      pvr = pr;
+      pvi = pi;
+    }
+    const double den = pr * pr + pi * pi;
+    double rr, ri;
+    if constexpr (N == 1) {
+      rr = pr / den;
+      ri = -pi / den;
+    } else {
+      const double half = ((r0 & 1) ? -pi : pr) / den;
+      rr = __shfl_sync(0xffffffffu, half, base);
+      ri = __shfl_sync(0xffffffffu, half, base + 1);
+    }
+    // the rows at positions k and best change places
+    if (best != k) ++swaps;
+    const bool piv = lane == who;
+    if (piv)
+      pos = k;
+    else if (pos == k)
+      pos = best;
+    // a_rj -= f_r v_j with f_r = a_rk / p; the pivot row becomes v_j / p
+    // (products in k_overlap's order: the one rounded by itself is f_i v_r in
+    // the first case, v_i Re(1 / p) in the second)
+    const double fr_ = xr[0] * rr - xi[0] * ri, fi_ = xr[0] * ri + xi[0] * rr;
+    const double c0 = piv ? rr : -fr_, c1 = piv ? -ri : fi_;
+    const double c2 = piv ? ri : -fr_, c3 = piv ? rr : -fi_;
+    const double nr = piv ? rr : -fr_, ni = piv ? ri : -fi_;
+#pragma unroll
+    for (int j = 1; j < N; ++j) {
+      const double vr = __shfl_sync(0xffffffffu, xr[j], who), vi = __shfl_sync(0xffffffffu, xi[j], who);
+      const double dr = piv ? 0.0 : xr[j], di = piv ? 0.0 : xi[j];
+      xr[j - 1] = fma(c0, vr, fma(c1, vi, dr));
+      xi[j - 1] = fma(c2, piv ? vr : vi, fma(c3, piv ? vi : vr, di));
+    }
+    xr[N - 1] = nr;
+    xi[N - 1] = ni;
+  }
+  const bool live = in && (!a.wt || walker_alive(a.wt, w));
+  // log det = sum_k log |p_k| + i (sum_k arg p_k + pi swaps), the tree of a
+  // 32-lane sum with zeros past N
+  double la = 0.0, ph = 0.0;
+  if (!singular && row) {
+    la = 0.5 * log(pvr * pvr + pvi * pvi);
+    ph = atan2(pvi, pvr);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double b = __shfl_sync(0xffffffffu, la, (lane + o) & 31), c = __shfl_sync(0xffffffffu, ph, (lane + o) & 31);
+    if (r0 < o && r0 + o < N) {
+      la += b;
+      ph += c;
+    }
+  }
+  if (live && r0 == 0) {
+    double* ld = a.logdet + 2 * (a.nds > 0 ? w * a.nds + ds : w);
+    ld[0] = singular ? -INFINITY : a.sf * la;
+    ld[1] = singular ? 0.0 : wrap_pi(a.sf * (ph + 3.141592653589793 * swaps));
+  }
+  // column j of the rows is column inv[j] of S^-1, inv[j] the row that ended
+  // at position j
+  if (row) inv_sh[warp][base + pos] = r0;
+  __syncwarp();
+  if (!live || singular || !row) return;
+  double2* si = a.Sinv + ((long)ds * a.W + w) * N * N + pos * N;
+#pragma unroll
+  for (int j = 0; j < N; ++j) si[inv_sh[warp][base + j]] = make_double2(xr[j], xi[j]);
+}
+
+template <int N>
+static int launch_overlap_warp(const OverlapArgs& a, cudaStream_t st) {
+  const unsigned per = OW_WARPS * (32 / N);
+  AFQ_LAUNCH(k_overlap_warp<N>, dim3(cdiv(a.W, per), a.nds > 0 ? a.nds : 1), 32 * OW_WARPS, 0, st, a);
+  return AFQMC_OK;
+}
+
 // Theta^T[i][p] = sum_j S^-1[j][i] Phi^T[j][p]: block (x, w) takes rows
 // p in [x TH_P, (x + 1) TH_P) of walker w in work items (p, block of IB
 // orbitals i), IB the largest divisor of N up to 8 (no padded lanes), so the
@@ -752,6 +895,17 @@ int launch_overlap(const OverlapArgs& a, cudaStream_t st) {
     AFQ_TRY(smem_attr_once(k_overlap<float>, 200 * 1024, attr32));
     AFQ_LAUNCH(k_overlap<float>, a.W, OV_T, smem / 2, st, a);
     return AFQMC_OK;
+  }
+  // a lane per row while two walkers share a warp and S needs no sums
+  if (a.N <= 16 && (a.unit_trial || a.Sext)) {
+    switch (a.N) {
+#define AFQ_OV(n) \
+  case n:         \
+    return launch_overlap_warp<n>(a, st);
+      AFQ_OV(1) AFQ_OV(2) AFQ_OV(3) AFQ_OV(4) AFQ_OV(5) AFQ_OV(6) AFQ_OV(7) AFQ_OV(8)
+      AFQ_OV(9) AFQ_OV(10) AFQ_OV(11) AFQ_OV(12) AFQ_OV(13) AFQ_OV(14) AFQ_OV(15) AFQ_OV(16)
+#undef AFQ_OV
+    }
   }
   AFQ_LAUNCH(k_overlap<double>, dim3(a.W, a.nds > 0 ? a.nds : 1), OV_T, smem, st, a);
   return AFQMC_OK;
