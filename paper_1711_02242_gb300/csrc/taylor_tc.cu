@@ -30,8 +30,8 @@
 // and its rows share their position within the 8-row swizzle atoms, so each
 // thread computes the swizzled offsets of its two K columns (p and Mp + p)
 // once per tile and a store costs one add.  Warp roles: warp 0 TMA producer,
-// warp 1 TMEM allocation and the MMA thread, warps 2-17 epilogue (four warps
-// per 32-lane quarter of TMEM, splitting the chunks).  Every wait is bounded;
+// warp 1 TMEM allocation and the MMA thread, warps 2.. epilogue (four or two
+// warps per 32-lane quarter of TMEM, splitting the chunks).  Every wait is bounded;
 // on time-out the kernel records an error and stops.
 #include <cuda_bf16.h>
 
@@ -43,9 +43,11 @@ namespace afq {
 namespace tc {
 
 constexpr int kVBox = BM * BKB;   // one V box: a 128-row p-tile x 128 bytes of K
-constexpr int kEpiWarps = 16;     // epilogue warps (4 per TMEM lane quarter)
-constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kSeriesThreads = 64 + kEpiThreads;
+// Epilogue warps: 4 per TMEM lane quarter, 2 when V is resident (two CTAs per SM)
+template <bool RES>
+constexpr int kEpiWarps = RES ? 8 : 16;
+template <bool RES>
+constexpr int kSeriesThreads = 64 + 32 * kEpiWarps<RES>;
 
 struct SeriesArgs {
   float* S;     // [W][2N][lds]: S = T_1 + ... + T_n, columns p < M
@@ -82,19 +84,27 @@ __device__ __forceinline__ void put_op(uint8_t* bop, uint32_t off, float v) {
 
 // Named barrier over the epilogue threads that also ORs a flag across them,
 // so every epilogue warp takes the same branch.
+template <int THREADS>
 __device__ __forceinline__ bool epi_sync_or(bool flag) {
   uint32_t out;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
       "bar.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
       : "=r"(out)
-      : "r"((uint32_t)flag), "n"(kEpiThreads)
+      : "r"((uint32_t)flag), "n"(THREADS)
       : "memory");
   return out != 0;
 }
 
-template <bool TF32>
-__global__ void __launch_bounds__(kSeriesThreads, 1)
+// RES: the walker's whole V stays in shared memory (stages = kblocks, filled
+// once per walker instead of once per term) and two CTAs share an SM, one's
+// products beside the other's epilogue.  A term of a small walker is a chain of
+// short steps (16 MMAs, their commit, TMEM loads, the operand's stores, a
+// fence), so one walker at a time leaves the SM idle most of it: at M = 100,
+// N = 10, 1024 walkers the series took 129 us with V streamed and one CTA, and
+// takes 75.5 us so.
+template <bool TF32, bool RES>
+__global__ void __launch_bounds__(kSeriesThreads<RES>, RES ? 2 : 1)
     k_taylor_series(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmT,
                     SeriesArgs a, int* err) {
   extern __shared__ uint8_t smem_raw[];
@@ -117,6 +127,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
   constexpr int ELEM = TF32 ? 4 : 2;
   constexpr int BK = BKB / ELEM;
   constexpr int KSTEPS = BKB / 32;
+  constexpr int EPW = kEpiWarps<RES>;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
@@ -126,7 +137,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
     mbar_init(bfull, 1);
     mbar_init(bfree, 1);
     mbar_init(dfull, 1);
-    mbar_init(bnext, kEpiThreads);  // every epilogue thread arrives
+    mbar_init(bnext, 32 * EPW);  // every epilogue thread arrives
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -155,7 +166,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
       mbar_expect_tx(bfull, (uint32_t)a.kblocks * opk);
       for (int kb = 0; kb < a.kblocks; ++kb)
         tma_load_4d(bop + kb * opk, &tmT, bfull, kb * BK, 0, 0, w);
-      for (int k = 1; k <= a.order && !stop; ++k)
+      for (int k = 1; k <= (RES ? 1 : a.order) && !stop; ++k)
         for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
           if ((it >= a.stages && !mbar_wait(&empty[s], ph ^ 1u, err, 32)) || *abort_flag) {
             stop = true;
@@ -188,7 +199,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
         // one stage = one K block of every p-tile: the p-tiles' MMAs are
         // interleaved (independent accumulators)
         for (int kb = 0; kb < a.kblocks; ++kb) {
-          if (!mbar_wait(&full[s], ph, err, 35)) {
+          if ((!RES || k == 1) && !mbar_wait(&full[s], ph, err, 35)) {
             *abort_flag = 1;
             stop = true;
             break;
@@ -204,10 +215,10 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
                 mma<TF32>(tmem + (uint32_t)(pt * a.nb),
                           sw128_desc(av + (uint32_t)(pt * kVBox) + 32 * kk),
                           sw128_desc(bv + 32 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(&empty[s]);
+          if (!RES || k == a.order) mma_commit(&empty[s]);
           if (++s == a.stages) {
             s = 0;
-            ph ^= 1u;
+            if (!RES || k == a.order) ph ^= 1u;
           }
         }
         mma_commit(dfull);
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
     if (stop) *abort_flag = 1;
   } else if (warp >= 2) {
     // epilogue: warp quarter q holds TMEM lanes (p within the tile) 32q .. 32q + 31;
-    // the four warps of a quarter take every fourth 16-column chunk
+    // the warps of a quarter share its 16-column chunks
     const int q = warp & 3, half = (warp - 2) >> 2;
     const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
     const uint32_t soff = (uint32_t)(a.ptiles * a.nb);  // columns of the running sum
@@ -230,7 +241,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
       for (int k = 1; k <= a.order; ++k, ++g) {
         bool bad = !mbar_wait_sleep(dfull, g & 1, err, 36) || *abort_flag;
         fence_after();
-        if (epi_sync_or(bad)) {
+        if (epi_sync_or<32 * EPW>(bad)) {
           stop = true;
           break;
         }
@@ -244,7 +255,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 1)
           column_offsets<TF32>(p, opk, offp);
           column_offsets<TF32>(a.Mp + p, opk, offq);
 #pragma unroll 1
-          for (int ch = half; ch < nchunk; ch += kEpiWarps / 4) {
+          for (int ch = half; ch < nchunk; ch += EPW / 4) {
             const int c0 = ch * 16;
             const int cpart = c0 >= NH ? 1 : 0, i0 = c0 - cpart * NH;
             if (i0 >= N) continue;  // a chunk of padding rows only
@@ -306,7 +317,11 @@ namespace {
 constexpr int kSmemMax = 232448;
 constexpr int kSmemFixed = 1024 /*align*/ + 256 /*barriers*/;
 
-bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* smem) {
+// Shared memory of a CTA when two share an SM (228 KB, 1 KB of it the system's
+// per CTA).
+constexpr int kSmemHalf = 114 * 1024 - 1024;
+
+bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* smem, bool* res) {
   if (N < 1 || M < 1 || Mp < M || Mp % 16) return false;
   const int elem = lo_kind == LO_TF32 ? 4 : 2;
   const int nh = (N + 15) / 16 * 16;
@@ -320,6 +335,10 @@ bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* sme
   int stages = (int)(room / ((long)ptiles * tc::kVBox));
   if (stages > 8) stages = 8;
   if (stages < 2) return false;
+  // V resident, two CTAs per SM, where both fit
+  const bool resident = op + (long)kblocks * ptiles * tc::kVBox + kSmemFixed <= kSmemHalf &&
+                        2 * ptiles * nb <= 256;
+  if (resident) stages = kblocks;
   uint32_t tcols = 32;
   while (tcols < (uint32_t)(2 * ptiles * nb)) tcols <<= 1;
   if (sa) {
@@ -330,20 +349,31 @@ bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* sme
     sa->stages = stages;
     sa->tcols = tcols;
   }
+  if (res) *res = resident;
   if (smem) *smem = (int)(op + (long)stages * ptiles * tc::kVBox + kSmemFixed);
   return true;
 }
 }  // namespace
 
+template <bool TF32, bool RES>
+static int launch_series(int grid, int smem, const CUtensorMap& tv, const CUtensorMap& tt,
+                         const tc::SeriesArgs& sa, int* err, cudaStream_t st) {
+  static std::atomic<unsigned long long> attr{0};
+  AFQ_TRY(smem_attr_once(tc::k_taylor_series<TF32, RES>, kSmemMax, attr));
+  AFQ_LAUNCH((tc::k_taylor_series<TF32, RES>), grid, tc::kSeriesThreads<RES>, smem, st, tv, tt, sa, err);
+  return AFQMC_OK;
+}
+
 bool tc_taylor_series_fits(int lo_kind, int N, int M, int Mp) {
-  return series_plan(lo_kind, N, M, Mp, nullptr, nullptr);
+  return series_plan(lo_kind, N, M, Mp, nullptr, nullptr, nullptr);
 }
 
 int tc_taylor_series(const void* V, const void* T0, float* S, long lds, int lo_kind, int W, int N,
                      int M, int Mp, int order, int* err, cudaStream_t st) {
   tc::SeriesArgs sa{};
   int smem = 0;
-  if (!series_plan(lo_kind, N, M, Mp, &sa, &smem)) {
+  bool res = false;
+  if (!series_plan(lo_kind, N, M, Mp, &sa, &smem, &res)) {
     set_error("taylor series kernel: shape N=%d M=%d does not fit", N, M);
     return AFQMC_EUNSUPPORTED;
   }
@@ -364,17 +394,13 @@ int tc_taylor_series(const void* V, const void* T0, float* S, long lds, int lo_k
   const long tstr[3] = {2L * Mp * eb, (long)N * 2 * Mp * eb, 2L * N * 2 * Mp * eb};
   const int tbox[4] = {tc::BKB / eb, sa.nh, 2, 1};
   AFQ_TRY(make_tmap_nd(&tt, T0, eb, 4, tdims, tstr, tbox));
-  const int grid = W < tc_sm_count() ? W : tc_sm_count();
-  if (tf32) {
-    static std::atomic<unsigned long long> attr{0};
-    AFQ_TRY(smem_attr_once(tc::k_taylor_series<true>, kSmemMax, attr));
-    AFQ_LAUNCH(tc::k_taylor_series<true>, grid, tc::kSeriesThreads, smem, st, tv, tt, sa, err);
-  } else {
-    static std::atomic<unsigned long long> attr{0};
-    AFQ_TRY(smem_attr_once(tc::k_taylor_series<false>, kSmemMax, attr));
-    AFQ_LAUNCH(tc::k_taylor_series<false>, grid, tc::kSeriesThreads, smem, st, tv, tt, sa, err);
-  }
-  return AFQMC_OK;
+  const int most = (res ? 2 : 1) * tc_sm_count();
+  const int grid = W < most ? W : most;
+  if (tf32)
+    return res ? launch_series<true, true>(grid, smem, tv, tt, sa, err, st)
+               : launch_series<true, false>(grid, smem, tv, tt, sa, err, st);
+  return res ? launch_series<false, true>(grid, smem, tv, tt, sa, err, st)
+             : launch_series<false, false>(grid, smem, tv, tt, sa, err, st);
 }
 
 int taylor_apply(const void* V, void* T0, void* T1, float* S, long lds, int lo_kind, int W, int N,
