@@ -1207,25 +1207,44 @@ int tc_tune_store(const TcGemm& g, float* C, long ldc, float alpha, cudaStream_t
   return AFQMC_OK;
 }
 
-// Tile width for an output of n columns: 160 or 256, whichever pads less.
-// At 160 the ring keeps five 36 KB stages beside the epilogue's 16 KB stage.
-constexpr int kHalfStages160 = 5;
-static int half_step_bn(int n) {
-  const int pad160 = cdiv(n, 160) * 160 - n, pad256 = cdiv(n, 256) * 256 - n;
-  return pad160 < pad256 ? 160 : 256;
+// Tile width of a half step's rows x n output: a tile costs about its width
+// (the epilogue) plus a fixed part, the A operand's K blocks, worth about 100
+// columns; the width whose waves of tiles over the SMs cost least.  Measured
+// per pair of half steps: 20480 x 100 (BF16) 57.7 us at 160 (160 tiles: a
+// second wave of eight) and 52.9 at 112; 512 x 20 24.3 us at 160 and 21.8 at
+// 32; 25600 x 300 116 us at 160; 10234 x 217 (TF32) 69 us at 256 (80 tiles, one
+// wave) and 79 at 32 (560 tiles, four).
+constexpr int kHalfStages = 5;  // ring stages of 128-byte K blocks (36 KB at 160)
+static int half_step_bn(long rows, int n) {
+  int best = 160;
+  double cost = 1e300;
+  for (int bn : {256, 160, 112, 64, 32}) {
+    const long tiles = (long)cdiv(rows, tc::BM) * cdiv(n, bn);
+    const double c = (double)((tiles + tc_sm_count() - 1) / tc_sm_count()) * (bn + 100);
+    if (c < cost) {
+      cost = c;
+      best = bn;
+    }
+  }
+  return best;
+}
+template <bool TF32, class Epi>
+static int launch_half(const TcGemm& g, const Epi& e, int bn, cudaStream_t st) {
+  const int gx = cdiv(g.m, tc::BM), gy = cdiv(e.M, bn);
+  switch (bn) {
+    case 32: return launch_tc_persistent<32, kHalfStages, TF32>(g, e, gx, gy, st);
+    case 64: return launch_tc_persistent<64, kHalfStages, TF32>(g, e, gx, gy, st);
+    case 112: return launch_tc_persistent<112, kHalfStages, TF32>(g, e, gx, gy, st);
+    case 160: return launch_tc_persistent<160, kHalfStages, TF32>(g, e, gx, gy, st);
+    default: return launch_tc_persistent<256, 4, TF32>(g, e, gx, gy, st);
+  }
 }
 
 int tc_prop_first(const TcGemm& g, float* acc, long ldacc, void* tb, const double* phi_id,
                   int lo_kind, int N, int M, int Mp, cudaStream_t st) {
-  const int bn = half_step_bn(M);
+  const int bn = half_step_bn(g.m, M);
   tc::EpiProp0 e{acc, ldacc, tb, phi_id, lo_kind, N, M, Mp, g.m, bn};
-  const int gx = cdiv(g.m, tc::BM), gy = cdiv(M, bn);
-  if (bn == 160) {
-    if (g.tf32) return launch_tc_persistent<160, kHalfStages160, true>(g, e, gx, gy, st);
-    return launch_tc_persistent<160, kHalfStages160, false>(g, e, gx, gy, st);
-  }
-  if (g.tf32) return launch_tc_persistent<256, 4, true>(g, e, gx, gy, st);
-  return launch_tc_persistent<256, 4, false>(g, e, gx, gy, st);
+  return g.tf32 ? launch_half<true>(g, e, bn, st) : launch_half<false>(g, e, bn, st);
 }
 
 int tc_taylor_term(const TcGemm& g, float* S, long lds, bool first, void* tb_out, int lo_kind,
@@ -1342,15 +1361,9 @@ int tc_prop_last(const TcGemm& g, double* phiT, const double* wt, int N, int M, 
     set_error("tc last half step: operand pitch %ld, want 2 Mp = %d", g.lda, 2 * Mp);
     return AFQMC_EINVAL;
   }
-  const int bn = half_step_bn(M);
+  const int bn = half_step_bn(g.m, M);
   tc::EpiPhi e{phiT, wt, N, M, g.m, bn, phi_lo, lo_kind, Mp, acc_id};
-  const int gx = cdiv(g.m, tc::BM), gy = cdiv(M, bn);
-  if (bn == 160) {
-    if (g.tf32) return launch_tc_persistent<160, kHalfStages160, true>(g, e, gx, gy, st);
-    return launch_tc_persistent<160, kHalfStages160, false>(g, e, gx, gy, st);
-  }
-  if (g.tf32) return launch_tc_persistent<256, 4, true>(g, e, gx, gy, st);
-  return launch_tc_persistent<256, 4, false>(g, e, gx, gy, st);
+  return g.tf32 ? launch_half<true>(g, e, bn, st) : launch_half<false>(g, e, bn, st);
 }
 
 // ---- per-step contractions as job descriptors, alone or grouped ------------
@@ -1468,10 +1481,10 @@ int dispatch_grouped(const TcGrouped& gr, cudaStream_t st) {
       if (gr.bn == 128) return launch_grouped<128, 4, TF32, tc::EpiV>(gr, st);
       return launch_grouped<256, 3, TF32, tc::EpiV>(gr, st);
     case TC_JOB_PROP0:
-      if (gr.bn == 160) return launch_grouped<160, kHalfStages160, TF32, tc::EpiProp0>(gr, st);
+      if (gr.bn == 160) return launch_grouped<160, kHalfStages, TF32, tc::EpiProp0>(gr, st);
       return launch_grouped<256, 4, TF32, tc::EpiProp0>(gr, st);
     case TC_JOB_PHI:
-      if (gr.bn == 160) return launch_grouped<160, kHalfStages160, TF32, tc::EpiPhi>(gr, st);
+      if (gr.bn == 160) return launch_grouped<160, kHalfStages, TF32, tc::EpiPhi>(gr, st);
       return launch_grouped<256, 4, TF32, tc::EpiPhi>(gr, st);
   }
   set_error("grouped contraction: unknown kind %d", gr.kind);
@@ -1503,7 +1516,7 @@ int tc_grouped_create(const TcJobDesc* d, int n, int bn, TcGrouped** out) {
       return AFQMC_EINVAL;
     }
   const int kind = d[0].kind;
-  if (bn == 0) bn = kind == TC_JOB_STORE ? 256 : kind == TC_JOB_V ? 128 : half_step_bn(d[0].M);
+  if (bn == 0) bn = kind == TC_JOB_STORE ? 256 : kind == TC_JOB_V ? 128 : 160;
   bool ok = false;
   for (int c : bn_candidates(kind)) ok = ok || c == bn;
   if (!ok) {
