@@ -126,20 +126,29 @@ __device__ inline void field_pair(uint64_t seed, uint32_t step, uint32_t walker,
   *xb = rad * s;
 }
 
+// uniform53 rounded to FP32, in integer arithmetic (this GPU's float64 pipe is
+// 1/64 of the FP32 one): a + 0.5 is exact below 2^52, else rounds to the even
+// integer of a, a + 1; the result, at most 54 bits, rounds to FP32 once.
+__device__ inline float uniform53_f32(uint32_t hi, uint32_t lo) {
+  const uint64_t a = ((uint64_t)(hi >> 5) << 26) + (uint64_t)(lo >> 6);
+  const uint64_t twice = (a >> 52) ? 2 * (a + (a & 1)) : 2 * a + 1;
+  return __ull2float_rn(twice) * 5.5511151231257827e-17f;  // 2^-54
+}
+
 // The same pair from the same Philox words with the Box-Muller transform taken
 // in FP32 (mixed path: the fields only feed BF16/TF32 contractions, and
 // float64 log/sincos run on GB300's slow FP64 pipe).
 __device__ inline void field_pair_f32(uint64_t seed, uint32_t step, uint32_t walker, uint32_t k,
-                                      double* xa, double* xb) {
+                                      float* xa, float* xb) {
   u32x4 c = {k, walker, step, 0u};
   u32x4 r = philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-  const float u1 = (float)uniform53(r.x, r.y);
-  const float u2 = (float)uniform53(r.z, r.w);
+  const float u1 = uniform53_f32(r.x, r.y);
+  const float u2 = uniform53_f32(r.z, r.w);
   const float rad = sqrtf(-2.f * logf(u1));
   float s, co;
   sincospif(2.f * u2, &s, &co);
-  *xa = (double)(rad * co);
-  *xb = (double)(rad * s);
+  *xa = rad * co;
+  *xb = rad * s;
 }
 
 // ------------------------------------------------------------ reductions --

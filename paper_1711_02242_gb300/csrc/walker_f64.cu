@@ -39,9 +39,12 @@ __global__ void __launch_bounds__(256) k_field(FieldArgs a) {
   const int npair = (a.G + 1) / 2;
   for (int k = threadIdx.x; k < npair; k += blockDim.x) {
     double xa, xb;
-    if (a.x_lo)
-      field_pair_f32(a.seed, (uint32_t)*a.dstep, (uint32_t)(a.w0 + w), (uint32_t)k, &xa, &xb);
-    else
+    if (a.x_lo) {
+      float fa, fb;
+      field_pair_f32(a.seed, (uint32_t)*a.dstep, (uint32_t)(a.w0 + w), (uint32_t)k, &fa, &fb);
+      xa = fa;
+      xb = fb;
+    } else
       field_pair(a.seed, (uint32_t)*a.dstep, (uint32_t)(a.w0 + w), (uint32_t)k, &xa, &xb);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -94,7 +97,9 @@ __global__ void __launch_bounds__(256) k_field(FieldArgs a) {
 // in FP32 (t comes from an FP32 accumulator and x only feeds the BF16/TF32
 // V contraction; float64 hypot and division run on GB300's slow FP64 pipe).
 // Each thread sums its fields in FP32; the six per-walker sums are reduced in
-// float64 in a fixed order (warps, then the block's warps in turn).
+// float64 in a fixed order (warps, then the block's warps in turn).  No other
+// float64 arithmetic: the uniform variates, their conversion and the warp sums
+// on the float64 pipe took most of the 33 us of 1024 walkers x 500 fields.
 __global__ void __launch_bounds__(256) k_field_lo(FieldArgs a) {
   __shared__ double sh[8][6];
   const int w = blockIdx.x;
@@ -109,14 +114,14 @@ __global__ void __launch_bounds__(256) k_field_lo(FieldArgs a) {
   float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const int npair = (a.G + 1) / 2;
   for (int k = threadIdx.x; k < npair; k += blockDim.x) {
-    double xa, xb;
+    float xa, xb;
     field_pair_f32(a.seed, step, (uint32_t)(a.w0 + w), (uint32_t)k, &xa, &xb);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int g = 2 * k + h;
       if (g >= a.G) break;
-      const float xi = (float)(h ? xb : xa);
-      const float cg = (float)a.c[g];
+      const float xi = h ? xb : xa;
+      const float cg = f64_to_f32(a.c[g]);
       float br = 0.f, bi = 0.f;
       if (phaseless) {
         br = sdt * ti[g];
@@ -142,12 +147,30 @@ __global__ void __launch_bounds__(256) k_field_lo(FieldArgs a) {
       s[5] = fmaf(cg, vi, s[5]);
     }
   }
+  // the six warp sums by halving: at each step a lane keeps half of its values
+  // and adds its partner's, 8 float64 additions instead of 30 in the same tree
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double v[6];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const double d = warp_sum((double)s[i]);
-    if (lane == 0) sh[wid][i] = d;
+  for (int i = 0; i < 6; ++i) v[i] = f32_to_f64(s[i]);
+  const bool up1 = lane & 16, up2 = lane & 8, up3 = lane & 4;
+  double h3[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {  // values i (lanes below 16) and i + 3
+    const double keep = up1 ? v[i + 3] : v[i], give = up1 ? v[i] : v[i + 3];
+    h3[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
   }
+  // of h3: 0 and 1, or 2 (its sums are repeated in the lanes that hold no other)
+  const double g0 = __shfl_xor_sync(0xffffffffu, up2 ? h3[0] : h3[2], 8);
+  const double g1 = __shfl_xor_sync(0xffffffffu, h3[1], 8);
+  double a0 = (up2 ? h3[2] : h3[0]) + g0;
+  const double a1 = h3[1] + g1;
+  const bool take1 = up3 && !up2;
+  const double b = __shfl_xor_sync(0xffffffffu, up2 ? a0 : (up3 ? a0 : a1), 4);
+  a0 = (take1 ? a1 : a0) + b;
+  a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+  a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+  if ((lane & 3) == 0 && !(up2 && up3)) sh[wid][(up1 ? 3 : 0) + (up2 ? 2 : (up3 ? 1 : 0))] = a0;
   __syncthreads();
   if (threadIdx.x < 6) {
     double r = 0.0;
