@@ -48,6 +48,7 @@ __device__ __forceinline__ void ld4(const double* p, double* v) {
 // over k in the same order whatever the tile, so results do not depend on it.
 template <typename TA, typename TB, typename TC, typename ACC, bool SPLIT = false, int TM = 4>
 __global__ void __launch_bounds__(TPB) k_gemm_nt(GemmNT<TA, TB, TC> g) {
+  pdl_begin();
   constexpr int BM = 16 * TM, BN = 16 * TM, PAD = TM == 4 ? 4 : 1;
   __shared__ __align__(16) ACC As[BK][BM + PAD];
   __shared__ __align__(16) ACC Bs[BK][BN + PAD];
@@ -171,11 +172,11 @@ static int launch_gemm(const GemmNT<TA, TB, TC>& g, cudaStream_t st) {
   if ((long)grid.x * grid.y * grid.z < 152) {
     dim3 g2(cdiv(g.n, 32), cdiv(g.m, 32), g.batch);
     if (g2.y <= 65535u) {
-      AFQ_LAUNCH((k_gemm_nt<TA, TB, TC, ACC, SPLIT, 2>), g2, TPB, 0, st, g);
+      AFQ_LAUNCH_PDL((k_gemm_nt<TA, TB, TC, ACC, SPLIT, 2>), g2, TPB, 0, st, g);
       return AFQMC_OK;
     }
   }
-  AFQ_LAUNCH((k_gemm_nt<TA, TB, TC, ACC, SPLIT, 4>), grid, TPB, 0, st, g);
+  AFQ_LAUNCH_PDL((k_gemm_nt<TA, TB, TC, ACC, SPLIT, 4>), grid, TPB, 0, st, g);
   return AFQMC_OK;
 }
 

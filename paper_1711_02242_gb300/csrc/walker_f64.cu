@@ -24,6 +24,7 @@ __host__ __device__ inline long packed_index(int p, int q, int M) {
 // Philox; x = xi - xbar.  Per-walker sums for the weight: sum xi xbar,
 // sum xbar^2 (Eq. hybrid-wt) and sum x c (the scalar of B(x - xbar)).
 __global__ void __launch_bounds__(256) k_field(FieldArgs a) {
+  pdl_begin();
   __shared__ double sh[32];
   const int w = blockIdx.x;
   const bool alive = walker_alive(a.wt, w);
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(256) k_field(FieldArgs a) {
 // float64 arithmetic: the uniform variates, their conversion and the warp sums
 // on the float64 pipe took most of the 33 us of 1024 walkers x 500 fields.
 __global__ void __launch_bounds__(256) k_field_lo(FieldArgs a) {
+  pdl_begin();
   __shared__ double sh[8][6];
   const int w = blockIdx.x;
   const bool alive = walker_alive(a.wt, w);
@@ -181,9 +183,9 @@ __global__ void __launch_bounds__(256) k_field_lo(FieldArgs a) {
 
 int launch_field(const FieldArgs& a, cudaStream_t st) {
   if (a.x_lo && a.t32 && !a.x && !a.t) {
-    AFQ_LAUNCH(k_field_lo, a.W, 256, 0, st, a);
+    AFQ_LAUNCH_PDL(k_field_lo, a.W, 256, 0, st, a);
   } else {
-    AFQ_LAUNCH(k_field, a.W, 256, 0, st, a);
+    AFQ_LAUNCH_PDL(k_field, a.W, 256, 0, st, a);
   }
   return AFQMC_OK;
 }
@@ -295,6 +297,7 @@ constexpr int TS_T = 256;
 size_t taylor_small_smem(int M, int N) { return sizeof(double2) * ((size_t)M * M + 2ull * M * N); }
 }
 __global__ void __launch_bounds__(TS_T) k_taylor_small(TaylorArgsT<double> a, int order, double sdt) {
+  pdl_begin();
   extern __shared__ double2 ts_sm[];
   const int w = blockIdx.x, M = a.M, N = a.N, NM = N * M;
   double2* V = ts_sm;  // [q][p] = Y_qp (re, im)
@@ -353,7 +356,7 @@ int taylor_series_f64(TaylorArgs a, int order, double sdt, double* t0, double* t
     static std::atomic<unsigned long long> attr{0};
     AFQ_TRY(smem_attr_once(k_taylor_small, 200 * 1024, attr));
     a.tin = t0;
-    AFQ_LAUNCH(k_taylor_small, a.W, TS_T, smem, st, a, order, sdt);
+    AFQ_LAUNCH_PDL(k_taylor_small, a.W, TS_T, smem, st, a, order, sdt);
     return AFQMC_OK;
   }
   for (int k = 1; k <= order; ++k) {
@@ -630,6 +633,7 @@ constexpr int OW_WARPS = 4;
 }
 template <int N>
 __global__ void __launch_bounds__(32 * OW_WARPS) k_overlap_warp(OverlapArgs a) {
+  pdl_begin();
   constexpr int PER = 32 / N;  // walkers per warp
   __shared__ int inv_sh[OW_WARPS][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ds = blockIdx.y, M = a.M;
@@ -752,7 +756,7 @@ __global__ void __launch_bounds__(32 * OW_WARPS) k_overlap_warp(OverlapArgs a) {
 template <int N>
 static int launch_overlap_warp(const OverlapArgs& a, cudaStream_t st) {
   const unsigned per = OW_WARPS * (32 / N);
-  AFQ_LAUNCH(k_overlap_warp<N>, dim3(cdiv(a.W, per), a.nds > 0 ? a.nds : 1), 32 * OW_WARPS, 0, st, a);
+  AFQ_LAUNCH_PDL(k_overlap_warp<N>, dim3(cdiv(a.W, per), a.nds > 0 ? a.nds : 1), 32 * OW_WARPS, 0, st, a);
   return AFQMC_OK;
 }
 
@@ -766,6 +770,7 @@ constexpr int TH_P = 64, TH_T = 128;
 }
 template <int IB>
 __global__ void __launch_bounds__(TH_T) k_theta_rows(OverlapArgs a) {
+  pdl_begin();
   extern __shared__ double2 th_sinv[];  // [N][N]
   const int w = blockIdx.y, N = a.N, M = a.M;
   if ((a.wt && !walker_alive(a.wt, w)) || !(a.logdet[2L * w] > -INFINITY)) return;
@@ -821,6 +826,7 @@ __global__ void __launch_bounds__(TH_T) k_theta_rows(OverlapArgs a) {
 // broadcasts.  Conversions use the integer-pipe routines.
 template <int TF_IB>
 __global__ void __launch_bounds__(TH_T) k_theta_rows_f32(OverlapArgs a) {
+  pdl_begin();
   extern __shared__ float2 th_sinv32[];  // [N][N], then Phi [2][N][TH_P] (FP32)
   const int w = blockIdx.y, N = a.N, M = a.M;
   if ((a.wt && !walker_alive(a.wt, w)) || !(a.logdet[2L * w] > -INFINITY)) return;
@@ -886,7 +892,7 @@ static int launch_theta_f32(const OverlapArgs& a, cudaStream_t st) {
   AFQ_TRY(smem_attr_once(k_theta_rows_f32<IB>, 100 * 1024, attr));
   dim3 grid(cdiv(a.M, TH_P), a.W);
   const size_t smem = sizeof(float2) * (size_t)a.N * a.N + sizeof(float) * 2 * a.N * TH_P;
-  AFQ_LAUNCH(k_theta_rows_f32<IB>, grid, TH_T, smem, st, a);
+  AFQ_LAUNCH_PDL(k_theta_rows_f32<IB>, grid, TH_T, smem, st, a);
   return AFQMC_OK;
 }
 
@@ -896,7 +902,7 @@ static int launch_theta_rows(const OverlapArgs& a, cudaStream_t st) {
   const size_t smem = sizeof(double2) * (size_t)a.N * a.N;
   AFQ_TRY(smem_attr_once(k_theta_rows<IB>, 100 * 1024, attr));
   dim3 grid(cdiv(a.M, TH_P), a.W);
-  AFQ_LAUNCH(k_theta_rows<IB>, grid, TH_T, smem, st, a);
+  AFQ_LAUNCH_PDL(k_theta_rows<IB>, grid, TH_T, smem, st, a);
   return AFQMC_OK;
 }
 
@@ -977,6 +983,7 @@ int launch_theta(const OverlapArgs& a, cudaStream_t st) {
 //   |I| = exp(Re log R + Re sum xi xbar - Re sum xbar^2 / 2).
 // Free projection (Eq. weight_update): W e^{i theta} <- W e^{i theta} R.
 __global__ void k_weight(WeightArgs a) {
+  pdl_begin();
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w == 0 && a.dstep) *a.dstep += 1;
   if (w >= a.W) return;
@@ -1012,7 +1019,7 @@ __global__ void k_weight(WeightArgs a) {
 }
 
 int launch_weight(const WeightArgs& a, cudaStream_t st) {
-  AFQ_LAUNCH(k_weight, cdiv(a.W, 128), 128, 0, st, a);
+  AFQ_LAUNCH_PDL(k_weight, cdiv(a.W, 128), 128, 0, st, a);
   return AFQMC_OK;
 }
 
@@ -1249,6 +1256,7 @@ int exchange_chunk(int N, int G) {
 }
 
 __global__ void __launch_bounds__(EX_T) k_exchange(ExchArgs a) {
+  pdl_begin();
   extern __shared__ double ex_sm[];
   const int chunk = blockIdx.x, w = blockIdx.y;  // every walker (dead ones too)
   const int M = a.M, N = a.N;
@@ -1336,7 +1344,7 @@ int launch_exchange(const ExchArgs& a, cudaStream_t st) {
     return AFQMC_EUNSUPPORTED;
   }
   dim3 grid(a.nchunk, a.W);
-  AFQ_LAUNCH(k_exchange, grid, EX_T, smem, st, a);
+  AFQ_LAUNCH_PDL(k_exchange, grid, EX_T, smem, st, a);
   return AFQMC_OK;
 }
 
@@ -1347,6 +1355,7 @@ int launch_exchange(const ExchArgs& a, cudaStream_t st) {
 // exchange are the sums over the blocks, E_loc = H0 + Tr(hh Theta) +
 // 1/2 sum_g [t_g^2 - sum_sigma Tr(T_g,sigma T_g,sigma)].
 __global__ void __launch_bounds__(256) k_eloc(ElocArgs a) {
+  pdl_begin();
   __shared__ double sh[32];
   const int w = blockIdx.x;
   const int M = a.M, N = a.N, G = a.G;
@@ -1389,13 +1398,14 @@ __global__ void __launch_bounds__(256) k_eloc(ElocArgs a) {
 }
 
 int launch_eloc(const ElocArgs& a, cudaStream_t st) {
-  AFQ_LAUNCH(k_eloc, a.W, 256, 0, st, a);
+  AFQ_LAUNCH_PDL(k_eloc, a.W, 256, 0, st, a);
   return AFQMC_OK;
 }
 
 // Mixed estimator (Eq. localenergy) over live walkers, Re E_loc clamped to
 // [lo, hi] (Eq. cap) for phaseless walks; one record (step, E, sum W, live).
 __global__ void __launch_bounds__(256) k_record(RecordArgs a) {
+  pdl_begin();
   __shared__ double sh[32];
   double nr = 0.0, ni = 0.0, dr = 0.0, di = 0.0, na = 0.0;
   for (int w = threadIdx.x; w < a.W; w += blockDim.x) {
@@ -1446,7 +1456,7 @@ __global__ void __launch_bounds__(256) k_record(RecordArgs a) {
 }
 
 int launch_record(const RecordArgs& a, cudaStream_t st) {
-  AFQ_LAUNCH(k_record, 1, 256, 0, st, a);
+  AFQ_LAUNCH_PDL(k_record, 1, 256, 0, st, a);
   return AFQMC_OK;
 }
 
@@ -1458,6 +1468,7 @@ int launch_record(const RecordArgs& a, cudaStream_t st) {
 // C_j (the last live walker if rounding puts it past C_{N_w-1}).  Copies land
 // in walker-index order and every new weight is W_tot / N_w.
 __global__ void __launch_bounds__(256) k_comb_plan(CombArgs a) {
+  pdl_begin();
   __shared__ double s_u;
   __shared__ int s_last, s_ok;
   if (threadIdx.x == 0) {
@@ -1494,6 +1505,7 @@ __global__ void __launch_bounds__(256) k_comb_plan(CombArgs a) {
 }
 
 __global__ void __launch_bounds__(256) k_comb_gather(CombArgs a) {
+  pdl_begin();
   const int k = blockIdx.x;
   const int j = a.parent[k];
   if (j < 0) return;
@@ -1513,6 +1525,7 @@ __global__ void __launch_bounds__(256) k_comb_gather(CombArgs a) {
 }
 
 __global__ void __launch_bounds__(256) k_comb_commit(CombArgs a) {
+  pdl_begin();
   const int k = blockIdx.x;
   if (a.parent[k] < 0) return;
   const long n = 2L * a.N * a.M;
@@ -1529,9 +1542,9 @@ __global__ void __launch_bounds__(256) k_comb_commit(CombArgs a) {
 }
 
 int launch_comb(const CombArgs& a, cudaStream_t st) {
-  AFQ_LAUNCH(k_comb_plan, 1, 256, 0, st, a);
-  AFQ_LAUNCH(k_comb_gather, a.W, 256, 0, st, a);
-  AFQ_LAUNCH(k_comb_commit, a.W, 256, 0, st, a);
+  AFQ_LAUNCH_PDL(k_comb_plan, 1, 256, 0, st, a);
+  AFQ_LAUNCH_PDL(k_comb_gather, a.W, 256, 0, st, a);
+  AFQ_LAUNCH_PDL(k_comb_commit, a.W, 256, 0, st, a);
   return AFQMC_OK;
 }
 
@@ -1691,6 +1704,7 @@ int launch_sumsq(const double* v, double* out, int n, cudaStream_t st) {
 namespace afq {
 __global__ void k_convert_lo(const double* src, long rows, long cols, long lds, void* dst,
                              long ldd, int kind, double minus_diag) {
+  pdl_begin();
   const long n = rows * ldd;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long)gridDim.x * blockDim.x) {
@@ -1703,7 +1717,7 @@ __global__ void k_convert_lo(const double* src, long rows, long cols, long lds, 
 int launch_convert_lo(const double* src, long rows, long cols, long lds, void* dst, long ldd,
                       int kind, cudaStream_t st, double minus_diag) {
   if (rows <= 0) return AFQMC_OK;
-  AFQ_LAUNCH(k_convert_lo, 152 * 8, 256, 0, st, src, rows, cols, lds, dst, ldd, kind, minus_diag);
+  AFQ_LAUNCH_PDL(k_convert_lo, 152 * 8, 256, 0, st, src, rows, cols, lds, dst, ldd, kind, minus_diag);
   return AFQMC_OK;
 }
 
