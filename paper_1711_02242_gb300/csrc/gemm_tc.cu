@@ -1104,7 +1104,9 @@ static int launch_tc_pairs(const TcGemm& g, const Epi& epi, int gx, int gy, cuda
   cfg.blockDim = dim3(64 + 32 * Epi::kWarps);
   cfg.dynamicSmemBytes = kTotal;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as AFQ_LAUNCH
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;

@@ -321,6 +321,242 @@ __global__ void __launch_bounds__(kThreads, VEC == 2 ? 4 : 5)
     next_pivot(st, L, dim, apiv, bv, bi, bl, bad, delta, max_vectors, k + 1);
 }
 
+// The whole decomposition in one cooperative launch, for dimensions whose
+// columns fit a block per SM.  Block b owns `cols` consecutive indices and keeps
+// their components of the vectors found so far in shared memory (as many as
+// fit; the rest it reads back from L, where every vector is also written).
+// Per vector the blocks exchange one (value, index, payload) each: a block
+// publishes its maximum in its slot (two slots per block, used in turn) and
+// then the iteration's number with release order; every block waits for all
+// the numbers, reduces the slots itself, and so knows the next pivot without
+// a second exchange.  The sums run over g in the order of k_mcd_step (eight
+// groups g = r + 8 j, four interleaved accumulators), so the results are the
+// same.
+//
+// k_mcd_step is one launch per vector: its latency chain (launch, grid-wide
+// tickets, the gather by one last block) took 22 us a vector at dim = 5050,
+// 516 vectors (11.2 ms), against 2.2 us of float64 work per SM on average,
+// which bounds this kernel beside the exchange; it takes 9.3 us (4.80 ms).
+// Values are compared as integers of the same order (float64 comparisons run
+// on the slow pipe, a dozen of them per vector one after another).
+struct McdSlot {
+  long long key;  // ordered_key of the maximum
+  double l;
+  int32_t i, bad;
+  uint32_t seq;  // iterations published
+  uint32_t pad;
+};
+
+__device__ __forceinline__ long long ordered_key(double x) {
+  const long long b = __double_as_longlong(x + 0.0);  // -0 as +0
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double key_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ void key_argmax(long long& v, int& i, double& l, int& bad, long long ov,
+                                           int oi, double ol, int ob) {
+  bad |= ob;
+  if (ov > v || (ov == v && oi < i)) {
+    v = ov;
+    i = oi;
+    l = ol;
+  }
+}
+__device__ __forceinline__ void warp_key_argmax(long long& v, int& i, double& l, int& bad) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, i, o), ob = __shfl_xor_sync(0xffffffffu, bad, o);
+    const double ol = __shfl_xor_sync(0xffffffffu, l, o);
+    key_argmax(v, i, l, bad, ov, oi, ol, ob);
+  }
+}
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+constexpr int kAllMaxCols = 64, kAllThreads = 8 * kAllMaxCols;
+constexpr int kAllMaxVectors = 4096;
+constexpr uint32_t kAllPolls = 1u << 20;  // bound of a wait for the other blocks (under a second)
+
+__global__ void __launch_bounds__(kAllThreads, 1)
+    k_mcd_all(const double* __restrict__ V, int dim, int cols, double* __restrict__ d, double* L,
+              int32_t* __restrict__ pivots, double delta, double tau, int max_vectors, int cached,
+              McdSlot* slots, int* abort_flag, McdState* st) {
+  extern __shared__ __align__(16) double all_sm[];
+  double* a_sm = all_sm;                  // L[g][piv], g < k
+  double* Ls = all_sm + max_vectors;      // [cached][cols]
+  __shared__ double red[8][kAllMaxCols];
+  __shared__ long long sv[16];
+  __shared__ double sl[16], root_sh;
+  __shared__ int si[16], sb[16], stop_sh;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
+  const int nb = gridDim.x;
+  const int c = tid % cols, r = tid / cols;  // column and group of this thread
+  const bool sum = r < 8;
+  const int mu0 = blockIdx.x * cols;
+  // thread c < cols finishes column c
+  const bool fin = tid < cols && mu0 + tid < dim;
+  double dm = fin ? d[mu0 + tid] : 0.0;
+  int piv = st->piv, done = st->done;
+  double dmax = st->dmax, lpiv = 0.0;
+  int k = 0;
+  while (!done) {
+    // the pivot's components of the earlier vectors (the newest travelled with
+    // the pivot), its row of V, 1 / sqrt(dmax)'s root and the screening
+    for (int g = tid; g < k - 1; g += blockDim.x) a_sm[g] = __ldcg(L + (int64_t)g * dim + piv);
+    if (tid == 0 && k > 0) a_sm[k - 1] = lpiv;
+    double vv = 0.0;
+    bool screened = false;
+    if (fin) {
+      vv = V[(int64_t)piv * dim + mu0 + tid];
+      screened = sqrt(__dmul_rn(fabs(dm), dmax)) <= tau;
+    }
+    if (tid == blockDim.x - 1) root_sh = sqrt(dmax);
+    if (blockIdx.x == 0 && tid == 0 && pivots) pivots[k] = piv;
+    __syncthreads();
+    if (sum) {
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      const double* lc = Ls + c;
+      int g = r;
+      const int kc = k < cached ? k : cached;
+      for (; g + 56 < kc; g += 64) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          acc[u & 3] = fma(lc[(g + 8 * u) * cols], a_sm[g + 8 * u], acc[u & 3]);
+      }
+      const double* gc = L + mu0 + c;
+      const bool in = mu0 + c < dim;
+      for (; g + 56 < k; g += 64) {
+        double x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int gg = g + 8 * u;
+          x[u] = gg < cached ? lc[gg * cols] : in ? gc[(int64_t)gg * dim] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u & 3] = fma(x[u], a_sm[g + 8 * u], acc[u & 3]);
+      }
+      for (; g < k; g += 8) {
+        const double x = g < cached ? lc[g * cols] : in ? gc[(int64_t)g * dim] : 0.0;
+        acc[0] = fma(x, a_sm[g], acc[0]);
+      }
+      red[r][c] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    }
+    __syncthreads();
+    const long long kLeast = ordered_key(-INFINITY);
+    long long bv = kLeast;
+    double bl = 0.0;
+    int bi = INT_MAX, bad = 0;
+    if (tid < cols) {
+      double lv = 0.0;
+      if (fin) {
+        double s = red[0][tid];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) s += red[w][tid];
+        lv = screened ? 0.0 : (vv - s) / root_sh;
+        dm = screened ? 0.0 : __dsub_rn(dm, __dmul_rn(lv, lv));
+        L[(int64_t)k * dim + mu0 + tid] = lv;
+        key_argmax(bv, bi, bl, bad, ordered_key(dm), mu0 + tid, lv, !isfinite(dm));
+      }
+      if (k < cached) Ls[k * cols + tid] = lv;
+    }
+    // the block's maximum (warps past the columns hold none)
+    const int fw = (cols + 31) >> 5;
+    if (wid < fw) {
+      warp_key_argmax(bv, bi, bl, bad);
+      if (lane == 0) {
+        sv[wid] = bv;
+        sl[wid] = bl;
+        si[wid] = bi;
+        sb[wid] = bad;
+      }
+    }
+    __syncthreads();  // also: every write of this vector is before the release below
+    McdSlot* mine = slots + (size_t)(k & 1) * nb;
+    if (tid == 0) {
+      for (int w = 1; w < fw; ++w) key_argmax(bv, bi, bl, bad, sv[w], si[w], sl[w], sb[w]);
+      McdSlot* o = mine + blockIdx.x;
+      o->key = bv;
+      o->l = bl;
+      o->i = bi;
+      o->bad = bad;
+      st_release(&o->seq, (uint32_t)k + 1u);
+      stop_sh = 0;
+    }
+    __syncthreads();
+    // all blocks' maxima, one slot per thread of the first warps; a block that
+    // another one has left behind gives up
+    bv = kLeast;
+    bl = 0.0;
+    bi = INT_MAX;
+    bad = 0;
+    const int rw = (nb + 31) >> 5 < nwarp ? (nb + 31) >> 5 : nwarp;
+    if (wid < rw) {
+      bool lost = false;
+      for (int q = tid; q < nb; q += 32 * rw) {
+        const McdSlot* o = mine + q;
+        uint32_t n = 0;
+        while (ld_acquire(&o->seq) != (uint32_t)k + 1u)
+          if (++n > kAllPolls || ((n & 1023u) == 0u && *(volatile int*)abort_flag)) {
+            lost = true;
+            break;
+          }
+        if (lost) break;
+        const long long ov = __ldcg(&o->key);
+        const double ol = __ldcg(&o->l);
+        const int oi = __ldcg(&o->i), ob = __ldcg(&o->bad);
+        key_argmax(bv, bi, bl, bad, ov, oi, ol, ob);
+      }
+      if (lost) {
+        stop_sh = 1;
+        atomicExch(abort_flag, 1);
+      }
+      __syncwarp();
+      warp_key_argmax(bv, bi, bl, bad);
+      if (lane == 0) {
+        sv[wid] = bv;
+        sl[wid] = bl;
+        si[wid] = bi;
+        sb[wid] = bad;
+      }
+    }
+    __syncthreads();
+    bv = sv[0];
+    bl = sl[0];
+    bi = si[0];
+    bad = sb[0];
+    for (int w = 1; w < rw; ++w) key_argmax(bv, bi, bl, bad, sv[w], si[w], sl[w], sb[w]);
+    const bool stop = stop_sh != 0;
+    __syncthreads();  // sv .. sb and stop_sh are written again next time
+    piv = bi;
+    dmax = key_value(bv);
+    lpiv = bl;
+    ++k;
+    if (stop)
+      done = 4;
+    else if (bad || !isfinite(dmax))
+      done = 3;
+    else if (dmax < delta)
+      done = 1;
+    else if (k >= max_vectors)
+      done = 2;
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    st->dmax = dmax;
+    st->piv = piv;
+    st->n = k;
+    st->done = done;
+  }
+}
+
 struct McdLayout {
   size_t state, part, spart, sticket, d, apiv, total;
 };
@@ -330,6 +566,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 McdLayout mcd_layout(int64_t dim, int32_t max_vectors) {
   McdLayout l;
   const int64_t groups = (dim + 31) / 32;  // blocks of a step launch, at most
+  // (k_mcd_all's slots, two per block of at most 8 indices or one SM, lie here too)
   const int64_t nparts = groups > kInitGrid ? groups : kInitGrid;
   const int64_t nfans = (nparts + kFan - 1) / kFan;
   l.state = 0;
@@ -350,6 +587,20 @@ int mcd_check(int64_t dim, int32_t max_vectors) {
   if (max_vectors < 1 || max_vectors > kMaxVectors) {
     set_error("modified Cholesky: max_vectors %d outside [1, %d]", max_vectors, kMaxVectors);
     return AFQMC_EINVAL;
+  }
+  return AFQMC_OK;
+}
+
+int mcd_result(const McdState& hs, int32_t* nvec, double* residual, const char* who) {
+  *nvec = hs.n;
+  if (residual) *residual = hs.dmax;
+  if (hs.done == 3) {
+    set_error("%s: non-finite residual after %d vectors", who, hs.n);
+    return AFQMC_ENONFINITE;
+  }
+  if (hs.done == 4) {
+    set_error("%s: a wait between the blocks gave up after %d vectors", who, hs.n);
+    return AFQMC_ETIMEOUT;
   }
   return AFQMC_OK;
 }
@@ -384,6 +635,45 @@ int run_mcd(int64_t dim, const double* d_V, double delta, int32_t max_vectors, d
   AFQ_CUDA(cudaMemsetAsync(base + lay.sticket, 0, lay.d - lay.sticket, s));
   AFQ_LAUNCH(k_mcd_init, (unsigned)grid0, kThreads, 0, s, d_V, dim, d, delta, max_vectors, tree,
              st);
+  // One launch for the whole decomposition where a block per SM can own the
+  // columns: the slots of the exchange take the place of the tickets' partials.
+  {
+    int dev = 0, sms = 0, coop = 0;
+    AFQ_CUDA(cudaGetDevice(&dev));
+    AFQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    AFQ_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    int cols = (int)((dim + sms - 1) / sms);
+    cols = cols <= 8 ? 8 : (cols + 3) / 4 * 4;  // whole warps of (column, group) pairs
+    if (coop && cols <= kAllMaxCols && max_vectors <= kAllMaxVectors) {
+      constexpr int kSmemAll = 216 * 1024;
+      const size_t row = sizeof(double) * (size_t)cols, av = sizeof(double) * (size_t)max_vectors;
+      int cached = (int)((kSmemAll - av) / row);
+      if (cached > max_vectors) cached = max_vectors;
+      const size_t smem = av + (size_t)cached * row;
+      static std::atomic<unsigned long long> attr{0};
+      AFQ_TRY(smem_attr_once(k_mcd_all, kSmemAll, attr));
+      const unsigned nb = (unsigned)((dim + cols - 1) / cols);
+      McdSlot* slots = reinterpret_cast<McdSlot*>(base + lay.part);
+      int* abort_flag = reinterpret_cast<int*>(base + lay.sticket);
+      // k_mcd_init's partials were here: no iteration is published yet
+      AFQ_CUDA(cudaMemsetAsync(slots, 0, 2 * sizeof(McdSlot) * (size_t)nb, s));
+      const double* va = d_V;
+      int da = (int)dim;
+      void* args[] = {&va, &da, &cols, &d, &d_L, &d_piv, const_cast<double*>(&delta),
+                      const_cast<double*>(&tau), &max_vectors, &cached, &slots, &abort_flag, &st};
+      const cudaError_t e = cudaLaunchCooperativeKernel(
+          reinterpret_cast<const void*>(k_mcd_all), dim3(nb), dim3((unsigned)(8 * cols)), args, smem, s);
+      ++g_launches;
+      if (e != cudaSuccess) {
+        set_error("launch k_mcd_all: %s", cudaGetErrorString(e));
+        return AFQMC_ECUDA;
+      }
+      McdState hs{};
+      AFQ_CUDA(cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s));
+      AFQ_CUDA(cudaStreamSynchronize(s));
+      return mcd_result(hs, nvec, residual, who);
+    }
+  }
   // Launch iterations in chunks and read the state between chunks; launches
   // after convergence return at once.  A launch after `launched` others
   // finds k <= launched earlier vectors, which sizes its shared memory.
@@ -402,13 +692,7 @@ int run_mcd(int64_t dim, const double* d_V, double delta, int32_t max_vectors, d
       ++launched;
     }
   }
-  *nvec = hs.n;
-  if (residual) *residual = hs.dmax;
-  if (hs.done == 3) {
-    set_error("%s: non-finite residual after %d vectors", who, hs.n);
-    return AFQMC_ENONFINITE;
-  }
-  return AFQMC_OK;
+  return mcd_result(hs, nvec, residual, who);
 }
 
 // Pair index of p <= r: row-major order of the upper triangle.
