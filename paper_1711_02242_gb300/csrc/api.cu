@@ -84,7 +84,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz);
 size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   Bufs tmp;
   if (!b) b = &tmp;
-  bool oz = (p.precision == AFQMC_FP64 || p.ndet > 0) && oz_pays(p.M, p.nwalkers);
+  bool oz = oz_pays(p.M, p.nwalkers);
   if (oz) {
     Bufs probe;
     oz = plan_route(p, &probe, nullptr, true) <= kOzWorkspace;
@@ -99,8 +99,10 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   const bool mixed = p.precision != AFQMC_FP64;
   size_t nchunk = (G + exchange_chunk((int)N, p.nchol) - 1) / exchange_chunk((int)N, p.nchol);
   if (mixed) nchunk = G;  // the tensor-core exchange leaves one partial per vector
+  const bool f32lu = p.precision == AFQMC_MIXED_TF32_F32LU || p.precision == AFQMC_MIXED_BF16_F32LU;
   b->oz = oz && !mixed;
-  b->oz_ov = oz;
+  b->oz_ov = oz && (!mixed || p.ndet > 0);
+  b->oz_qr = oz && !f32lu && N <= 32;
   b->oz_exch = b->oz && p.ndet == 0 && N <= 32;
   if (b->oz_exch) nchunk = oz_tiles(G, oz_exchange_vectors((int)N));
   const size_t lo = (p.precision == AFQMC_MIXED_BF16 || p.precision == AFQMC_MIXED_BF16_F32LU ||
@@ -205,7 +207,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
     b->Bh_split_tf = a.take<float>(M * 4 * Mp);
   }
   size_t oz_need = 0, oz_exps = 0;
-  if (oz) {
+  if (b->oz_ov || b->oz_qr) {
     auto take = [&](OzOperand& o, size_t rows, int rpt, int RT, size_t k) {
       o.RT = RT;
       o.rows_per_tile = rpt;
@@ -214,10 +216,15 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       o.exps = a.take<int>(rows);
     };
     const size_t nds = p.ndet > 0 ? 2 * (size_t)p.ndet : 1;
-    take(b->ozV, nds * N, 64, 64, M);
+    if (b->oz_ov) take(b->ozV, nds * N, 64, 64, M);
     if (p.ndet > 0) {
       b->Sx = a.take<double>(W * 2 * N * nds * N);
       b->md_Sinv = a.take<double>(nds * W * 2 * N * N);
+    }
+    if (b->oz_qr) {
+      b->gram = a.take<double>(W * 4 * N * N);
+      b->Rinv = a.take<double>(W * 2 * N * N);
+      b->qr_done = a.take<int>(W);
     }
     if (b->oz) {
       take(b->ozL, P, 64, 64, G);
@@ -232,8 +239,9 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
     oz_taylor_operands(M, N, Mp, &V, &T);
     const size_t per = b->oz ? (size_t)(V.batch_stride + T.batch_stride) : 0;
     oz_theta_operands(M, N, &V, &T);
-    const size_t per_th = (size_t)V.batch_stride + nds * (size_t)T.batch_stride;
-    size_t wc = kOzScratch / std::max(per, per_th);
+    const size_t per_th = (size_t)V.batch_stride + (b->oz_ov ? nds : 1) * (size_t)T.batch_stride;
+    const size_t per_gram = b->oz_qr ? oz_bytes(2 * N, 2 * (int)N, oz_term_width((int)N), M) : 0;
+    size_t wc = (b->oz_ov ? kOzScratch : kOzScratch / 8) / std::max(per, std::max(per_th, per_gram));
     wc = wc >= W ? W : wc < 64 ? 64 : wc / 64 * 64;
     if (wc > W) wc = W;
     b->oz_wc = (int)wc;
@@ -242,7 +250,8 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       if (exps > oz_exps) oz_exps = exps;
     };
     need(per_th * wc, wc * (M + nds * 2 * N));
-    need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
+    need(per_gram * wc, 2 * N * wc);
+    if (b->oz_ov) need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
     if (b->oz) {
       need(per * wc, wc * (M + 2 * N));
       need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
@@ -268,7 +277,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   b->T0 = s1.take<double>(W * 2 * N * M);  // Taylor terms (FP64) / comb copies
   b->T1 = s1.take<double>(W * 2 * N * M);
   b->tmp_ld = s1.take<double>(2 * W);
-  if (oz) {
+  if (oz_need) {
     b->oz_mem = s1.take<char>(oz_need);
     b->oz_exp = s1.take<int>(oz_exps);
   }
@@ -573,23 +582,16 @@ int oz_trial_overlaps(afqmc_state* s, double* dst, int n) {
   return oz_rows_gemm(s, s->b.phiT, 2 * s->p.N, s->p.M, s->b.ozV, dst, n, 0, nullptr);
 }
 
-int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
-                  int unit, int zero_singular, void* th_lo) {
+// t.theta rows = Phi times the matrices m[ds][w] (N x N, t.nds per walker) for
+// the walkers that t's conditions let through.
+static int oz_rotate(afqmc_state* s, const double* m, OzTheta t, cudaStream_t st) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
-  OzTheta t;
   oz_theta_operands(p.M, p.N, &t.A, &t.B);
   t.W = p.nwalkers;
   t.M = p.M;
   t.N = p.N;
-  t.nds = nds;
-  t.theta = theta;
-  t.ld = ld;
-  t.ld_w = ld_w;
   t.wt = b.wt;
-  t.unit = unit;
-  t.zero_singular = zero_singular;
-  t.th_lo = th_lo;
   t.lo_kind = b.lo_kind;
   t.Mp = b.Mp;
   t.err = b.status;
@@ -600,12 +602,57 @@ int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, co
     t.A.exps = b.oz_exp;
     t.B.data = b.oz_mem + (size_t)t.nw * t.A.batch_stride;
     t.B.exps = b.oz_exp + (size_t)t.nw * t.A.batch_exp_stride;
-    AFQ_TRY(oz_slice_cols(b.phiT + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, s->st));
-    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(sinv), p.nwalkers, w0, t.nw, nds, p.N, t.B,
-                             s->st));
-    AFQ_TRY(oz_theta(t, s->st));
+    AFQ_TRY(oz_slice_cols(b.phiT + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, st));
+    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, t.B, st));
+    AFQ_TRY(oz_theta(t, st));
   }
   return AFQMC_OK;
+}
+
+int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
+                  int unit, int zero_singular, void* th_lo) {
+  OzTheta t;
+  t.nds = nds;
+  t.theta = theta;
+  t.ld = ld;
+  t.ld_w = ld_w;
+  t.unit = unit;
+  t.zero_singular = zero_singular;
+  t.th_lo = th_lo;
+  return oz_rotate(s, sinv, t, s->st);
+}
+
+// Gram-Schmidt of the walkers on stream st: Phi <- Phi R^-1 with R from the
+// Gram matrix for well-conditioned walkers (k_gram_factor), the sweep for the
+// others.  (The scratch is free: nothing that uses it runs beside this.)
+static int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  if (!b.oz_qr) return launch_mgs(m, st);
+  const int N = p.N, M = p.M;
+  const size_t row = (size_t)2 * N * M;
+  OzOperand rows;
+  rows.RT = oz_term_width(N);
+  rows.rows_per_tile = 2 * N;
+  rows.nkb = (M + 15) / 16;
+  rows.data = b.oz_mem;
+  rows.exps = b.oz_exp;
+  rows.batch_stride = (long)oz_bytes(2 * N, 2 * N, rows.RT, M);
+  rows.batch_exp_stride = 2 * N;
+  for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
+    const int nw = std::min(b.oz_wc, p.nwalkers - w0);
+    AFQ_TRY(oz_slice_rows(m.phiT + w0 * row, 2L * N * nw, M, M, rows, st));
+    AFQ_TRY(oz_gram(rows, nw, N, b.gram + (size_t)w0 * 4 * N * N, b.status, st));
+  }
+  GramFactorArgs gf{p.nwalkers, N, m.nup, m.sf, b.gram, b.wt, reinterpret_cast<double2*>(b.Rinv), m.ld, b.qr_done};
+  AFQ_TRY(launch_gram_factor(gf, st));
+  OzTheta t;
+  t.theta = m.phiT;
+  t.flag = b.qr_done;
+  t.th_lo = m.phi_lo;
+  AFQ_TRY(oz_rotate(s, b.Rinv, t, st));
+  m.done = b.qr_done;
+  return launch_mgs(m, st);
 }
 
 // acc = T_n(V) t0 with V = i sqrt(dt) Y (packed), a chunk of walkers at a time.
@@ -984,11 +1031,11 @@ int step_after(afqmc_state* s) {
       // join_side() before the next reader (the next first half step)
       AFQ_CUDA(cudaEventRecord(s->ev_fork, s->st));
       AFQ_CUDA(cudaStreamWaitEvent(s->side, s->ev_fork, 0));
-      AFQ_TRY(launch_mgs(ma, s->side));
+      AFQ_TRY(orthonormalise(s, ma, s->side));
       AFQ_CUDA(cudaEventRecord(s->ev_side, s->side));
       s->side_pending = true;
     } else {
-      AFQ_TRY(launch_mgs(ma, s->st));
+      AFQ_TRY(orthonormalise(s, ma, s->st));
     }
     prof_end(s);
   }

@@ -195,8 +195,21 @@ struct MgsArgs {
   int lo_kind = LO_NONE, Mp = 0;
   int nup = 0;      // spin blocks as in OverlapArgs (0: one block), swept separately
   double sf = 2.0;  // spins per block: log <Psi_T|Psi> drops by sf sum_k log r_kk
+  const int* done = nullptr;  // walkers with done[w] != 0 are left alone
 };
 int launch_mgs(const MgsArgs& a, cudaStream_t st);
+// The factor of Phi = Q R from the Gram matrix, for walkers whose columns are
+// well conditioned (done[w] = 1: R^-1 written, ld lowered; 0: nothing done).
+struct GramFactorArgs {
+  int W, N, nup;
+  double sf;
+  const double* gram;  // [W][2N][2N] products of the rows (c, i)
+  const double* wt;
+  double2* Rinv;       // [W][N][N]
+  double* ld;
+  int* done;
+};
+int launch_gram_factor(const GramFactorArgs& a, cudaStream_t st);
 
 struct ExchArgs {
   int W, M, N, G, gc, nchunk;

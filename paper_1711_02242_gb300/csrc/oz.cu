@@ -760,7 +760,7 @@ struct EpiOzTheta {
     if (tl.r >= g.a_rpt || p >= t.M || col >= N2) return;
     const int ds = tl.b / t.nw, wl = tl.b - ds * t.nw, w = t.w0 + wl;
     if (t.wt && !walker_alive(t.wt, w)) return;
-    const bool ok = t.ld[(long)w * t.ld_w + (long)ds * t.ld_ds] > -INFINITY;
+    const bool ok = t.flag ? t.flag[w] != 0 : t.ld[(long)w * t.ld_w + (long)ds * t.ld_ds] > -INFINITY;
     if (!ok && !t.zero_singular) return;
     const int ea = g.ea[(long)wl * g.ea_batch + p];
     const int* eb = g.eb + (long)tl.b * g.eb_batch + col;
@@ -773,6 +773,26 @@ struct EpiOzTheta {
       t.theta[(row + c) * t.M + p] = v;
       if (t.th_lo) store_lo(t.th_lo, t.lo_kind, (row + c) * t.Mp + p, v);
     }
+  }
+  template <int EW>
+  __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
+};
+
+// Products of a walker's rows with each other (2 N x 2 N per batch entry).
+struct EpiOzGram {
+  static constexpr int kStages = 4;
+  static constexpr int kSmemBytes = 0;
+  int N2;
+  double* gram;
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
+                                        const long long* lo, uint8_t*) const {
+    if (tl.r >= N2 || cc >= N2) return;
+    const int* e = g.ea + (long)tl.b * g.ea_batch;
+    const int ea = e[tl.r];
+    double* out = gram + ((long)tl.b * N2 + tl.r) * N2 + cc;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (cc + c < N2) out[c] = scaled_sum(hi[c], lo[c], ea + e[cc + c]);
   }
   template <int EW>
   __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
@@ -966,6 +986,16 @@ int oz_theta(const OzTheta& t, cudaStream_t st) {
   if (bn == 16) return launch_oz_as<16, EpiOzTheta, false>(g, e, st);
   if (bn == 32) return launch_oz_as<32, EpiOzTheta, false>(g, e, st);
   return launch_oz_as<64, EpiOzTheta, false>(g, e, st);
+}
+
+int oz_gram(const OzOperand& rows, int W, int N, double* gram, int* err, cudaStream_t st) {
+  const int bn = oz_term_width(N);
+  AFQ_TRY(check_operand(rows, rows, bn));
+  EpiOzGram e{2 * N, gram};
+  const OzArgs g = oz_args(rows, rows, 2 * N, 2 * N, W, err);
+  if (bn == 16) return launch_oz<16>(g, e, st);
+  if (bn == 32) return launch_oz<32>(g, e, st);
+  return launch_oz<64>(g, e, st);
 }
 
 int oz_exchange_vectors(int N) { return BM / N > 0 ? BM / N : 1; }

@@ -93,6 +93,7 @@ struct OzTheta {
   const double* ld = nullptr;
   int ld_w = 2, ld_ds = 2;
   const double* wt = nullptr;
+  const int* flag = nullptr;  // instead of ld: walkers with flag 0 keep their rows
   int unit = 0, zero_singular = 0;
   void* th_lo = nullptr;  // BF16/TF32 copy of the rows, pitch Mp
   int lo_kind = 0, Mp = 0;
@@ -105,6 +106,10 @@ int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cu
 int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,
                      cudaStream_t st);
 int oz_theta(const OzTheta& t, cudaStream_t st);
+
+// gram[w][r][c] = sum_k of rows r and c of each walker's 2 N rows (A and B the
+// same operand, one tile per walker, RT = oz_term_width(N), N <= 32).
+int oz_gram(const OzOperand& rows, int W, int N, double* gram, int* err, cudaStream_t st);
 
 // Exchange: part[w][c][2] = sum over the vectors of row tile c of
 // sum_ij T_ij T_ji, T_g = Lh_g Theta_w (same-spin pairs).  A: rows (g, i),

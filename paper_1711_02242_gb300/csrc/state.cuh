@@ -59,7 +59,11 @@ struct Bufs {
   // rows of the trial's orbitals; Sx, md_Sinv: the overlaps of every
   // determinant and their inverses), also for a multi-determinant trial on
   // the mixed path, which keeps these in float64
-  bool oz = false, oz_exch = false, oz_ov = false;
+  // oz_qr: Gram-Schmidt from the Gram matrix (also on the mixed path): its
+  // products, R^-1 and which walkers took it
+  bool oz = false, oz_exch = false, oz_ov = false, oz_qr = false;
+  double *gram = nullptr, *Rinv = nullptr;
+  int* qr_done = nullptr;
   OzOperand ozL, ozF, ozX, ozB, ozV;
   double *Sx = nullptr, *md_Sinv = nullptr;
   char* oz_mem = nullptr;

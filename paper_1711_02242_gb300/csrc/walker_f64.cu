@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(256) k_mgs(MgsArgs a) {
   __shared__ double inv_sh;
   __shared__ double norms[64];  // |v_k|^2, for log det R after the sweep
   const int w = blockIdx.x;
-  if (!walker_alive(a.wt, w)) return;
+  if (!walker_alive(a.wt, w) || (a.done && a.done[w])) return;
   const int M = a.M, N = a.N;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   double* re = a.phiT + (long)w * 2 * N * M;
@@ -1112,6 +1112,126 @@ __global__ void __launch_bounds__(256) k_mgs(MgsArgs a) {
   }
   __syncthreads();
   if (threadIdx.x == 0 && a.ld) a.ld[2L * w] -= a.sf * (sh[0] + sh[1]);
+  // the operand copy (rows (w, c, k), pitch Mp; the pad columns stay zero)
+  if (a.phi_lo)
+    for (int e = threadIdx.x; e < 2 * N * M; e += blockDim.x)
+      store_lo(a.phi_lo, a.lo_kind, ((long)w * 2 * N + e / M) * a.Mp + e % M, re[e]);
+}
+
+// The same Q and R from the Gram matrix G = Phi^+ Phi = R^+ R (Cholesky QR):
+// the 8 M N^2 operations of the sweep become two exact sliced contractions on
+// the tensor cores (G, and Q = Phi R^-1), and what is left on the float64 pipe
+// is N^3.  The error of Q then grows with the square of the columns' condition
+// number instead of its first power, so a walker takes this route only where
+// the columns, scaled to unit norm, have |R^-1|_F^2 <= N + 1: with s_i their
+// singular values (sum s_i^2 = N) that is sum 1 / s_i^2 <= N + 1, which leaves
+// none below 0.57 or so.  The others are left to k_mgs.  Walkers that
+// Gram-Schmidt visits every few steps are well inside.
+//
+// A lane holds row r of G (N <= 32, floor(32 / N) walkers per warp) and the rows
+// are eliminated without pivoting as in k_overlap_warp: G = L D L^+, the row
+// operations that leave U = D L^+ also leave L^-1 in the eliminated columns,
+// and R^-1 = L^-+ D^-1/2.  N = 25, 512 walkers: @GF@ us.
+namespace {
+constexpr int GF_WARPS = 4;
+}
+template <int N>
+__global__ void __launch_bounds__(32 * GF_WARPS) k_gram_factor(GramFactorArgs a) {
+  constexpr int PER = 32 / N;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int seg = lane / N < PER ? lane / N : PER - 1;
+  const int base = seg * N, r = lane - base;
+  const bool row = r < N;
+  const long w = ((long)blockIdx.x * GF_WARPS + warp) * PER + seg;
+  const bool in = w < a.W;
+  const int nup = a.nup > 0 ? a.nup : N;
+  // G_rj = sum conj(v_r) v_j; spin blocks are factored on their own
+  double xr[N], xi[N];
+  const double* P = a.gram + w * 4 * N * N;
+  const bool ld_row = in && row;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const bool ok = ld_row && (r < nup) == (j < nup);
+    xr[j] = ok ? P[j * 2 * N + r] + P[(N + j) * 2 * N + N + r] : 0.0;
+    xi[j] = ok ? P[(N + j) * 2 * N + r] - P[j * 2 * N + N + r] : 0.0;
+  }
+  float own = 0.f;  // |v_r|^2, for the check below
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (j == r) own = (float)xr[j];
+  double d = 1.0;  // D_r
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) {
+    const double dk = __shfl_sync(0xffffffffu, xr[0], base + k);
+    if (r == k) d = dk;
+    const double inv = 1.0 / dk;
+    const bool below = r > k;
+    const double fr = below ? xr[0] * inv : 0.0, fi = below ? xi[0] * inv : 0.0;
+    // rows below lose f times row k, whose eliminated columns hold L^-1 (its own
+    // column: 1, so f changes sign there); the other rows only turn
+    const double keep_r = below ? -fr : xr[0], keep_i = below ? -fi : xi[0];
+#pragma unroll
+    for (int j = 1; j < N; ++j) {
+      const double vr = __shfl_sync(0xffffffffu, xr[j], base + k), vi = __shfl_sync(0xffffffffu, xi[j], base + k);
+      xr[j - 1] = fma(-fr, vr, fma(fi, vi, xr[j]));
+      xi[j - 1] = fma(-fr, vi, fma(-fi, vr, xi[j]));
+    }
+    xr[N - 1] = keep_r;
+    xi[N - 1] = keep_i;
+  }
+  // |column r of R^-1|^2 with its elements scaled by the columns' norms, summed
+  // over r (FP32: a check, not a result); NaN and overflow fail it
+  const double s = 1.0 / sqrt(d);
+  float q = 0.f;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const float gj = __shfl_sync(0xffffffffu, own, base + j);
+    const float lr_ = (float)(xr[j] * s), li_ = (float)(xi[j] * s);
+    if (j < r) q += (lr_ * lr_ + li_ * li_) * gj;
+  }
+  q += (float)s * (float)s * own;
+  float total = q;
+#pragma unroll
+  for (int o = 1; o < N; ++o) total += __shfl_sync(0xffffffffu, q, base + (r + o) % N);
+  const bool fine = total <= (float)N + 1.f;
+  const bool alive = in && walker_alive(a.wt, w);
+  double lr = row && fine ? 0.5 * log(d) : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double b = __shfl_sync(0xffffffffu, lr, (lane + o) & 31);
+    if (r < o && r + o < N) lr += b;
+  }
+  if (!in || !row) return;
+  if (r == 0) {
+    a.done[w] = alive && fine ? 1 : 0;
+    if (alive && fine && a.ld) a.ld[2 * w] -= a.sf * lr;
+  }
+  if (!alive || !fine) return;
+  // column r of R^-1: conj of row r of L^-1 over sqrt(D_r)
+  double2* R = a.Rinv + w * N * N + r;
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    R[(long)j * N] = j < r ? make_double2(xr[j] * s, -xi[j] * s) : make_double2(j == r ? s : 0.0, 0.0);
+}
+
+template <int N>
+static int launch_gram_factor_n(const GramFactorArgs& a, cudaStream_t st) {
+  AFQ_LAUNCH(k_gram_factor<N>, cdiv(a.W, GF_WARPS * (32 / N)), 32 * GF_WARPS, 0, st, a);
+  return AFQMC_OK;
+}
+int launch_gram_factor(const GramFactorArgs& a, cudaStream_t st) {
+  switch (a.N) {
+#define AFQ_GF(n) \
+  case n:         \
+    return launch_gram_factor_n<n>(a, st);
+    AFQ_GF(1) AFQ_GF(2) AFQ_GF(3) AFQ_GF(4) AFQ_GF(5) AFQ_GF(6) AFQ_GF(7) AFQ_GF(8)
+    AFQ_GF(9) AFQ_GF(10) AFQ_GF(11) AFQ_GF(12) AFQ_GF(13) AFQ_GF(14) AFQ_GF(15) AFQ_GF(16)
+    AFQ_GF(17) AFQ_GF(18) AFQ_GF(19) AFQ_GF(20) AFQ_GF(21) AFQ_GF(22) AFQ_GF(23) AFQ_GF(24)
+    AFQ_GF(25) AFQ_GF(26) AFQ_GF(27) AFQ_GF(28) AFQ_GF(29) AFQ_GF(30) AFQ_GF(31) AFQ_GF(32)
+#undef AFQ_GF
+  }
+  set_error("gram factor: N=%d", a.N);
+  return AFQMC_EINVAL;
 }
 
 // Mixed precisions: the same sweep in FP32 with the walker's orbitals resident
@@ -1217,13 +1337,6 @@ int launch_mgs(const MgsArgs& a, cudaStream_t st) {
     AFQ_TRY(smem_attr_once(k_mgs_f32, 200 * 1024, attr32));
     AFQ_LAUNCH(k_mgs_f32, a.W, 256, smem32, st, a);
     return AFQMC_OK;
-  }
-  if (a.phi_lo) {
-    // the float64 sweep, then the operand copy of every walker
-    MgsArgs b = a;
-    b.phi_lo = nullptr;
-    AFQ_TRY(launch_mgs(b, st));
-    return launch_convert_lo(a.phiT, 2L * a.N * a.W, a.M, a.M, a.phi_lo, a.Mp, a.lo_kind, st);
   }
   const size_t smem = sizeof(double2) * (size_t)a.M;
   if (smem > 200 * 1024) {

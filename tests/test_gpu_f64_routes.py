@@ -145,3 +145,38 @@ def test_determinants(pkg, M, N, nd, kind, precision):
     assert np.max(np.abs(run.local_energies() - el) / np.abs(el)) < TOL
     assert run.info().status == 0
     run.close()
+
+
+@pytest.mark.parametrize("M,N,Ndn", [(48, 6, 0), (130, 25, 0), (60, 17, 15)])
+def test_gram_schmidt_routes(pkg, M, N, Ndn):
+    """Gram-Schmidt of well-conditioned walkers (from the Gram matrix) and of
+    walkers with nearly parallel columns (the sweep) in one population: Q is
+    orthonormal to rounding, and walkers, overlaps and weights follow the
+    oracle's modified Gram-Schmidt.  The nearly parallel columns' condition
+    number is about 1e3, so 1e-10 leaves their 1e-13 room."""
+    G, W = 60, 5
+    h1, L, trial = inputs(M, N, G, Ndn)
+    up, dn = trial if Ndn else (trial, None)
+    both = np.hstack([up, dn]) if Ndn else up
+    rng = np.random.default_rng(3 * M)
+    Nt = N + Ndn
+    phi = np.repeat(both[None], W, 0).astype(complex)
+    phi += 0.02 * (rng.standard_normal(phi.shape) + 1j * rng.standard_normal(phi.shape))
+    for w in (1, 4):
+        phi[w, :, N - 1] = phi[w, :, 0] + 1e-3 * phi[w, :, N - 1]
+    orc = afqmc.Oracle(h1, L, up, W, afqmc.Params(qr_period=1, energy_period=0, fb_cap=1.0), trial_dn=dn, phi0=phi)
+    p = pkg.default_params(M, N, G, W, qr_period=1, energy_period=0, Ndn=Ndn)
+    run = pkg.AfqmcRun(h1, L, trial, p)
+    run.set_walkers(phi, np.ones(W))
+    run.propagate(1)
+    orc.run(1)
+    got, wt, lo = run.get_walkers()
+    assert np.all(orc.weight > 0)
+    for a, b in ((0, N), (N, Nt))[:2 if Ndn else 1]:
+        S = np.einsum("wpi,wpj->wij", got[:, :, a:b].conj(), got[:, :, a:b])
+        assert np.abs(S - np.eye(b - a)).max() < 1e-12
+        assert np.abs(S[[0, 2, 3]] - np.eye(b - a)).max() < 1e-14
+    assert np.abs(got - orc.phi).max() < TOL
+    assert np.max(np.abs(wt - orc.weight) / orc.weight) < TOL
+    assert np.max(np.abs(lo - orc.logdet)) < TOL * (1 + np.abs(orc.logdet).max())
+    run.close()
