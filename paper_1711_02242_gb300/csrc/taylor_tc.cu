@@ -43,11 +43,11 @@ namespace afq {
 namespace tc {
 
 constexpr int kVBox = BM * BKB;   // one V box: a 128-row p-tile x 128 bytes of K
-// Epilogue warps: 4 per TMEM lane quarter, 2 when V is resident (two CTAs per SM)
-template <bool RES>
-constexpr int kEpiWarps = RES ? 8 : 16;
-template <bool RES>
-constexpr int kSeriesThreads = 64 + 32 * kEpiWarps<RES>;
+// Epilogue warps: 4 per TMEM lane quarter, 2 when two CTAs share an SM
+template <bool TWO>
+constexpr int kEpiWarps = TWO ? 8 : 16;
+template <bool TWO>
+constexpr int kSeriesThreads = 64 + 32 * kEpiWarps<TWO>;
 
 struct SeriesArgs {
   float* S;     // [W][2N][lds]: S = T_1 + ... + T_n, columns p < M
@@ -96,15 +96,14 @@ __device__ __forceinline__ bool epi_sync_or(bool flag) {
   return out != 0;
 }
 
-// RES: the walker's whole V stays in shared memory (stages = kblocks, filled
-// once per walker instead of once per term) and two CTAs share an SM, one's
-// products beside the other's epilogue.  A term of a small walker is a chain of
-// short steps (16 MMAs, their commit, TMEM loads, the operand's stores, a
-// fence), so one walker at a time leaves the SM idle most of it: at M = 100,
-// N = 10, 1024 walkers the series took 129 us with V streamed and one CTA, and
-// takes 75.5 us so.
-template <bool TF32, bool RES>
-__global__ void __launch_bounds__(kSeriesThreads<RES>, RES ? 2 : 1)
+// TWO: two CTAs share an SM, one's products beside the other's epilogue.  A term
+// is a chain of short steps (the MMAs, their commit, TMEM loads, the operand's
+// stores, a fence), so one walker at a time leaves the SM idle much of it.
+// RES: the walker's whole V also stays in shared memory (stages = kblocks,
+// filled once per walker instead of once per term).  1024 walkers, M = 100,
+// N = 10: 129 us with V streamed and one CTA, 75.5 us so.
+template <bool TF32, bool RES, bool TWO>
+__global__ void __launch_bounds__(kSeriesThreads<TWO>, TWO ? 2 : 1)
     k_taylor_series(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmT,
                     SeriesArgs a, int* err) {
   extern __shared__ uint8_t smem_raw[];
@@ -127,7 +126,7 @@ __global__ void __launch_bounds__(kSeriesThreads<RES>, RES ? 2 : 1)
   constexpr int ELEM = TF32 ? 4 : 2;
   constexpr int BK = BKB / ELEM;
   constexpr int KSTEPS = BKB / 32;
-  constexpr int EPW = kEpiWarps<RES>;
+  constexpr int EPW = kEpiWarps<TWO>;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
@@ -321,7 +320,8 @@ constexpr int kSmemFixed = 1024 /*align*/ + 256 /*barriers*/;
 // per CTA).
 constexpr int kSmemHalf = 114 * 1024 - 1024;
 
-bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* smem, bool* res) {
+bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* smem, bool* res,
+                 bool* two) {
   if (N < 1 || M < 1 || Mp < M || Mp % 16) return false;
   const int elem = lo_kind == LO_TF32 ? 4 : 2;
   const int nh = (N + 15) / 16 * 16;
@@ -335,10 +335,14 @@ bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* sme
   int stages = (int)(room / ((long)ptiles * tc::kVBox));
   if (stages > 8) stages = 8;
   if (stages < 2) return false;
-  // V resident, two CTAs per SM, where both fit
-  const bool resident = op + (long)kblocks * ptiles * tc::kVBox + kSmemFixed <= kSmemHalf &&
-                        2 * ptiles * nb <= 256;
-  if (resident) stages = kblocks;
+  // two CTAs per SM where both fit, with V resident or a ring of two stages at least
+  const long stage = (long)ptiles * tc::kVBox, half = kSmemHalf - kSmemFixed - op;
+  const bool pair = 2 * ptiles * nb <= 256 && half >= 2 * stage;
+  const bool resident = 2 * ptiles * nb <= 256 && half >= kblocks * stage;
+  if (resident)
+    stages = kblocks;
+  else if (pair)
+    stages = (int)(half / stage);
   uint32_t tcols = 32;
   while (tcols < (uint32_t)(2 * ptiles * nb)) tcols <<= 1;
   if (sa) {
@@ -350,30 +354,31 @@ bool series_plan(int lo_kind, int N, int M, int Mp, tc::SeriesArgs* sa, int* sme
     sa->tcols = tcols;
   }
   if (res) *res = resident;
+  if (two) *two = resident || pair;
   if (smem) *smem = (int)(op + (long)stages * ptiles * tc::kVBox + kSmemFixed);
   return true;
 }
 }  // namespace
 
-template <bool TF32, bool RES>
+template <bool TF32, bool RES, bool TWO>
 static int launch_series(int grid, int smem, const CUtensorMap& tv, const CUtensorMap& tt,
                          const tc::SeriesArgs& sa, int* err, cudaStream_t st) {
   static std::atomic<unsigned long long> attr{0};
-  AFQ_TRY(smem_attr_once(tc::k_taylor_series<TF32, RES>, kSmemMax, attr));
-  AFQ_LAUNCH((tc::k_taylor_series<TF32, RES>), grid, tc::kSeriesThreads<RES>, smem, st, tv, tt, sa, err);
+  AFQ_TRY(smem_attr_once(tc::k_taylor_series<TF32, RES, TWO>, kSmemMax, attr));
+  AFQ_LAUNCH((tc::k_taylor_series<TF32, RES, TWO>), grid, tc::kSeriesThreads<TWO>, smem, st, tv, tt, sa, err);
   return AFQMC_OK;
 }
 
 bool tc_taylor_series_fits(int lo_kind, int N, int M, int Mp) {
-  return series_plan(lo_kind, N, M, Mp, nullptr, nullptr, nullptr);
+  return series_plan(lo_kind, N, M, Mp, nullptr, nullptr, nullptr, nullptr);
 }
 
 int tc_taylor_series(const void* V, const void* T0, float* S, long lds, int lo_kind, int W, int N,
                      int M, int Mp, int order, int* err, cudaStream_t st) {
   tc::SeriesArgs sa{};
   int smem = 0;
-  bool res = false;
-  if (!series_plan(lo_kind, N, M, Mp, &sa, &smem, &res)) {
+  bool res = false, two = false;
+  if (!series_plan(lo_kind, N, M, Mp, &sa, &smem, &res, &two)) {
     set_error("taylor series kernel: shape N=%d M=%d does not fit", N, M);
     return AFQMC_EUNSUPPORTED;
   }
@@ -394,13 +399,15 @@ int tc_taylor_series(const void* V, const void* T0, float* S, long lds, int lo_k
   const long tstr[3] = {2L * Mp * eb, (long)N * 2 * Mp * eb, 2L * N * 2 * Mp * eb};
   const int tbox[4] = {tc::BKB / eb, sa.nh, 2, 1};
   AFQ_TRY(make_tmap_nd(&tt, T0, eb, 4, tdims, tstr, tbox));
-  const int most = (res ? 2 : 1) * tc_sm_count();
+  const int most = (two ? 2 : 1) * tc_sm_count();
   const int grid = W < most ? W : most;
   if (tf32)
-    return res ? launch_series<true, true>(grid, smem, tv, tt, sa, err, st)
-               : launch_series<true, false>(grid, smem, tv, tt, sa, err, st);
-  return res ? launch_series<false, true>(grid, smem, tv, tt, sa, err, st)
-             : launch_series<false, false>(grid, smem, tv, tt, sa, err, st);
+    return res   ? launch_series<true, true, true>(grid, smem, tv, tt, sa, err, st)
+           : two ? launch_series<true, false, true>(grid, smem, tv, tt, sa, err, st)
+                 : launch_series<true, false, false>(grid, smem, tv, tt, sa, err, st);
+  return res   ? launch_series<false, true, true>(grid, smem, tv, tt, sa, err, st)
+         : two ? launch_series<false, false, true>(grid, smem, tv, tt, sa, err, st)
+               : launch_series<false, false, false>(grid, smem, tv, tt, sa, err, st);
 }
 
 int taylor_apply(const void* V, void* T0, void* T1, float* S, long lds, int lo_kind, int W, int N,
