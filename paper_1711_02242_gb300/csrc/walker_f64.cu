@@ -402,6 +402,7 @@ struct Vec2<double> {
   __device__ static double from_f64(double x) { return x; }
   __device__ static double to_f64(double x) { return x; }
   __device__ static double2* sinv(const OverlapArgs& a) { return a.Sinv; }
+  __device__ static unsigned long long bits(double x) { return (unsigned long long)__double_as_longlong(x); }
 };
 template <>
 struct Vec2<float> {
@@ -410,6 +411,7 @@ struct Vec2<float> {
   __device__ static float from_f64(double x) { return f64_to_f32(x); }
   __device__ static double to_f64(float x) { return f32_to_f64(x); }
   __device__ static float2* sinv(const OverlapArgs& a) { return a.Sinv32; }
+  __device__ static unsigned long long bits(float x) { return __float_as_uint(x); }
 };
 
 // Steps 1-2 for walker w by the whole block (blockDim >= 64): S into A
@@ -479,19 +481,22 @@ __device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, int ds
   for (int k = 0; k < N; ++k) {
     if (threadIdx.x < 32) {
       // pivot: the largest |a_rk|^2 over rows r >= k, the first such row on ties
+      // (non-negative floats order as their bits: integer comparisons, the
+      // float64 ones run on the narrow pipe)
       int best = k;
-      T bv = -1;
+      unsigned long long bv = 0;
       for (int r = k + threadIdx.x; r < N; r += 32) {
         const T2 x = A[r * N + k];
         const T v = x.x * x.x + x.y * x.y;
-        if (v > bv) {
-          bv = v;
+        const unsigned long long key = v > 0 ? Vec2<T>::bits(v) : 0ull;
+        if (key > bv) {
+          bv = key;
           best = r;
         }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
         const int ob = __shfl_xor_sync(0xffffffffu, best, o);
         if (ov > bv || (ov == bv && ob < best)) {
           bv = ov;
@@ -513,10 +518,12 @@ __device__ __forceinline__ bool overlap_core(const OverlapArgs& a, int w, int ds
           }
           __syncwarp();
         }
-        // 1 / pivot once per lane (a float64 division runs long on the FP64 pipe)
+        // 1 / pivot: the real part by even, the imaginary part by odd lanes
+        // (a float64 division runs long on the FP64 pipe)
         const T2 pv = A[k * N + k];
         const T den = pv.x * pv.x + pv.y * pv.y;
-        const T2 rp = Vec2<T>::make(pv.x / den, -pv.y / den);
+        const T part = ((threadIdx.x & 1) ? -pv.y : pv.x) / den;
+        const T2 rp = Vec2<T>::make(__shfl_sync(0xffffffffu, part, 0), __shfl_sync(0xffffffffu, part, 1));
         for (int r = threadIdx.x; r < N; r += 32) {
           const T2 x = A[r * N + k];
           fac[r] = Vec2<T>::make(x.x * rp.x - x.y * rp.y, x.x * rp.y + x.y * rp.x);
@@ -627,7 +634,7 @@ __global__ void __launch_bounds__(OV_T) k_overlap(OverlapArgs a) {
 // N = 10.  1024 walkers, N = 10: 73.3 us (one block of 256 threads per walker,
 // 100 of them with an element) to 38.7; 128 walkers, N = 2: 15.2 to 12.2.
 // Above 16 rows a warp has one walker and the block's eight warps win: 301
-// walkers, N = 17: 59 us against 72; 512, N = 25: 128.9 us either way.
+// walkers, N = 17: 47 us against 72; 512, N = 25: 109 us against 129.
 namespace {
 constexpr int OW_WARPS = 4;
 }
@@ -1131,7 +1138,7 @@ __global__ void __launch_bounds__(256) k_mgs(MgsArgs a) {
 // A lane holds row r of G (N <= 32, floor(32 / N) walkers per warp) and the rows
 // are eliminated without pivoting as in k_overlap_warp: G = L D L^+, the row
 // operations that leave U = D L^+ also leave L^-1 in the eliminated columns,
-// and R^-1 = L^-+ D^-1/2.  N = 25, 512 walkers: @GF@ us.
+// and R^-1 = L^-+ D^-1/2.  512 walkers, N = 25: 112 us; 1024, N = 10: 27 us.
 namespace {
 constexpr int GF_WARPS = 4;
 }
