@@ -824,65 +824,88 @@ __global__ void __launch_bounds__(TH_T) k_theta_rows(OverlapArgs a) {
 // Mixed precisions: the same rows with FP32 arithmetic.  Theta only feeds the
 // BF16/TF32 contractions (force bias, exchange) and the one-body energy
 // there, so FP32 products (S^-1 and Phi rounded to FP32) lose nothing those do
-// not, and this GPU's FP32 pipe is ~60x its FP64 one: the kernel becomes bound
-// by the traffic of Phi and Theta.  S^-1 comes from the float64 elimination
-// (rounded once to FP32 here), or from the FP32 one of the _F32LU precisions.  The block's TH_P columns of Phi are staged
-// in shared memory as FP32 (all loads in flight at once, converted once);
-// one work item = row p and IB orbitals i, IB = N / ceil(N / 16) rounded up
-// (guarded tail of at most ceil(N / 16) - 1 lanes); S^-1 reads are warp-wide
-// broadcasts.  Conversions use the integer-pipe routines.
-template <int TF_IB>
+// not, and this GPU's FP32 pipe is ~60x its FP64 one: the floor is the traffic
+// of Phi and Theta (137 MB, 20 us at M = 300, 512 walkers).  S^-1 comes from the
+// float64 elimination (rounded once to FP32 here), or from the FP32 one of the
+// _F32LU precisions.  The block's P columns of Phi are staged in shared memory
+// as FP32 and S^-1 in rows padded with zeros, so that an item (row p and IB
+// orbitals i, IB = N / ceil(N / 16) rounded up to even) reads a 16-byte
+// broadcast per two orbitals and needs no guards.  Conversions use the
+// integer-pipe routines.  Bound by issue slots (FMAs, conversions, stores).
+// Against an 8-byte broadcast and a guard per orbital: 1024 walkers, M = 100,
+// N = 10 24.5 -> 16.6 us; 301, M = 217, N = 17 25.1 -> 20.5; 512, M = 300, N = 25
+// 72.3 -> 69.5.  (Packed FMAs over two orbitals with S^-1 as separate real and
+// imaginary rows measured 25.4 us at M = 217.)
+template <int IB, int P>
 __global__ void __launch_bounds__(TH_T) k_theta_rows_f32(OverlapArgs a) {
   pdl_begin();
-  extern __shared__ float2 th_sinv32[];  // [N][N], then Phi [2][N][TH_P] (FP32)
+  extern __shared__ __align__(16) float2 th_sinv32[];  // [N][NP], then Phi [2][N][P] (FP32)
   const int w = blockIdx.y, N = a.N, M = a.M;
   if ((a.wt && !walker_alive(a.wt, w)) || !(a.logdet[2L * w] > -INFINITY)) return;
-  float* ph = reinterpret_cast<float*>(th_sinv32 + N * N);
-  if (a.Sinv32) {
-    const float2* si = a.Sinv32 + (long)w * N * N;
-    for (int idx = threadIdx.x; idx < N * N; idx += TH_T) th_sinv32[idx] = si[idx];
-  } else {
-    const double2* si = a.Sinv + (long)w * N * N;
-    for (int idx = threadIdx.x; idx < N * N; idx += TH_T) {
-      const double2 v = si[idx];
-      th_sinv32[idx] = make_float2(f64_to_f32(v.x), f64_to_f32(v.y));
+  const int nib = (N + IB - 1) / IB, NP = nib * IB;
+  float* ph = reinterpret_cast<float*>(th_sinv32 + N * NP);
+  for (int idx = threadIdx.x; idx < N * NP; idx += TH_T) {
+    const int j = idx / NP, i = idx - j * NP;
+    float2 v = make_float2(0.f, 0.f);
+    if (i < N) {
+      if (a.Sinv32) {
+        v = a.Sinv32[((long)w * N + j) * N + i];
+      } else {
+        const double2 d = a.Sinv[((long)w * N + j) * N + i];
+        v = make_float2(f64_to_f32(d.x), f64_to_f32(d.y));
+      }
     }
+    th_sinv32[idx] = v;
   }
-  const double* phw = a.phiT + (long)w * 2 * N * M;
-  const int pb = blockIdx.x * TH_P, pe = min(M, pb + TH_P), np = pe - pb;
-#pragma unroll 4
-  for (int e = threadIdx.x; e < 2 * N * np; e += TH_T) {
-    const int row = e / np, pl = e - row * np;  // row = plane * N + j
-    ph[row * TH_P + pl] = f64_to_f32(phw[(long)row * M + pb + pl]);
+  const int pb = blockIdx.x * P, np = min(M - pb, P);
+  const double* phw = a.phiT + (long)w * 2 * N * M + pb;
+  // each warp takes whole rows of the tile
+  const int lane = threadIdx.x & 31;
+  for (int row = threadIdx.x >> 5; row < 2 * N; row += TH_T / 32) {
+    double x[P / 32];
+#pragma unroll
+    for (int u = 0; u < P / 32; ++u) x[u] = lane + 32 * u < np ? phw[(long)row * M + lane + 32 * u] : 0.0;
+#pragma unroll
+    for (int u = 0; u < P / 32; ++u) ph[row * P + lane + 32 * u] = f64_to_f32(x[u]);
   }
   __syncthreads();
   double* tr = a.thetaT + (long)w * 2 * N * M;
   double* ti = tr + (long)N * M;
-  const int nib = (N + TF_IB - 1) / TF_IB;
-  for (int item = threadIdx.x; item < np * nib; item += TH_T) {
-    const int pl = item % np, p = pb + pl, i0 = (item / np) * TF_IB;
-    float ar[TF_IB], ai[TF_IB];
+  for (int item = threadIdx.x; item < P * nib; item += TH_T) {
+    const int pl = item % P, p = pb + pl, i0 = (item / P) * IB;
+    if (pl >= np) continue;
+    float ar[IB], ai[IB];
 #pragma unroll
-    for (int u = 0; u < TF_IB; ++u) ar[u] = ai[u] = 0.f;
+    for (int u = 0; u < IB; ++u) ar[u] = ai[u] = 0.f;
     if (a.unit_trial && p < N) {
 #pragma unroll
-      for (int u = 0; u < TF_IB; ++u) ar[u] = (i0 + u == p) ? 1.f : 0.f;
+      for (int u = 0; u < IB; ++u) ar[u] = (i0 + u == p) ? 1.f : 0.f;
     } else {
+#pragma unroll 5
       for (int j = 0; j < N; ++j) {
-        const float xr = ph[j * TH_P + pl], xi = ph[(N + j) * TH_P + pl];
-        const float2* srow = th_sinv32 + j * N + i0;
+        const float xr = ph[j * P + pl], xi = ph[(N + j) * P + pl];
+        const float2* srow = th_sinv32 + j * NP + i0;
 #pragma unroll
-        for (int u = 0; u < TF_IB; ++u) {
-          if (i0 + u < N) {
-            const float2 sv = srow[u];
-            ar[u] = fmaf(xr, sv.x, fmaf(-xi, sv.y, ar[u]));
-            ai[u] = fmaf(xr, sv.y, fmaf(xi, sv.x, ai[u]));
+        for (int u = 0; u < IB; u += 2) {
+          // two orbitals per 16-byte broadcast (IB = 1: one)
+          float4 sv;
+          if constexpr (IB % 2 == 0) {
+            sv = *reinterpret_cast<const float4*>(srow + u);
+          } else {
+            const float2 h = srow[u];
+            sv = make_float4(h.x, h.y, 0.f, 0.f);
+          }
+          ar[u] = fmaf(xr, sv.x, fmaf(-xi, sv.y, ar[u]));
+          ai[u] = fmaf(xr, sv.y, fmaf(xi, sv.x, ai[u]));
+          if (u + 1 < IB) {
+            ar[u + 1] = fmaf(xr, sv.z, fmaf(-xi, sv.w, ar[u + 1]));
+            ai[u + 1] = fmaf(xr, sv.w, fmaf(xi, sv.z, ai[u + 1]));
           }
         }
       }
     }
 #pragma unroll
-    for (int u = 0; u < TF_IB; ++u) {
+    for (int u = 0; u < IB; ++u) {
       const int i = i0 + u;
       if (i >= N) continue;
       tr[(long)i * M + p] = f32_to_f64(ar[u]);
@@ -895,11 +918,20 @@ __global__ void __launch_bounds__(TH_T) k_theta_rows_f32(OverlapArgs a) {
 
 template <int IB>
 static int launch_theta_f32(const OverlapArgs& a, cudaStream_t st) {
-  static std::atomic<unsigned long long> attr{0};
-  AFQ_TRY(smem_attr_once(k_theta_rows_f32<IB>, 100 * 1024, attr));
-  dim3 grid(cdiv(a.M, TH_P), a.W);
-  const size_t smem = sizeof(float2) * (size_t)a.N * a.N + sizeof(float) * 2 * a.N * TH_P;
-  AFQ_LAUNCH_PDL(k_theta_rows_f32<IB>, grid, TH_T, smem, st, a);
+  // one item per thread where a walker's orbitals are one item wide
+  constexpr int P1 = 128, P2 = 64;
+  const int nib = (a.N + IB - 1) / IB, P = nib == 1 ? P1 : P2;
+  const size_t smem = sizeof(float2) * (size_t)a.N * nib * IB + sizeof(float) * 2 * a.N * P;
+  dim3 grid(cdiv(a.M, P), a.W);
+  if (nib == 1) {
+    static std::atomic<unsigned long long> attr{0};
+    AFQ_TRY(smem_attr_once(k_theta_rows_f32<IB, P1>, 100 * 1024, attr));
+    AFQ_LAUNCH_PDL((k_theta_rows_f32<IB, P1>), grid, TH_T, smem, st, a);
+  } else {
+    static std::atomic<unsigned long long> attr{0};
+    AFQ_TRY(smem_attr_once(k_theta_rows_f32<IB, P2>, 100 * 1024, attr));
+    AFQ_LAUNCH_PDL((k_theta_rows_f32<IB, P2>), grid, TH_T, smem, st, a);
+  }
   return AFQMC_OK;
 }
 
@@ -953,15 +985,15 @@ int launch_theta(const OverlapArgs& a, cudaStream_t st) {
       set_error("theta: the FP32 rows need the operand copy");
       return AFQMC_EINVAL;
     }
-    const int nib = (a.N + 15) / 16, ib = (a.N + nib - 1) / nib;
+    const int nib = (a.N + 15) / 16;
+    int ib = (a.N + nib - 1) / nib;
+    if (ib > 1) ib = (ib + 1) / 2 * 2;
     switch (ib) {
 #define AFQ_THETA32(n) \
   case n:              \
     return launch_theta_f32<n>(a, st);
-      AFQ_THETA32(1) AFQ_THETA32(2) AFQ_THETA32(3) AFQ_THETA32(4) AFQ_THETA32(5)
-      AFQ_THETA32(6) AFQ_THETA32(7) AFQ_THETA32(8) AFQ_THETA32(9) AFQ_THETA32(10)
-      AFQ_THETA32(11) AFQ_THETA32(12) AFQ_THETA32(13) AFQ_THETA32(14) AFQ_THETA32(15)
-      AFQ_THETA32(16)
+      AFQ_THETA32(1) AFQ_THETA32(2) AFQ_THETA32(4) AFQ_THETA32(6) AFQ_THETA32(8) AFQ_THETA32(10)
+      AFQ_THETA32(12) AFQ_THETA32(14) AFQ_THETA32(16)
 #undef AFQ_THETA32
       default:
         set_error("theta: IB=%d", ib);
