@@ -334,6 +334,30 @@ struct EpiStore {
   }
 };
 
+// The same for a batch of products of equal shape in one launch: the operands'
+// row blocks of batch entry b start at rows b * bm of A and b * bn_rows of B,
+// its output at C + b * sC.  Tiles are numbered batch entry by batch entry
+// along x, so a launch fills the SMs where one entry's tiles would not.
+struct EpiStoreBatch {
+  static constexpr int kSmemBytes = 0;
+  static constexpr bool kB3D = false;
+  static constexpr int kWarps = 4;
+  static constexpr int kMT = 1;
+  EpiStore one;
+  int gxm;              // row tiles of an entry
+  int bm, bn_rows;      // rows of A and of B per entry
+  long sC;
+  __device__ __forceinline__ int m_origin(int bx, int) const { return (bx / gxm) * bm + (bx % gxm) * BM; }
+  __device__ __forceinline__ int n_origin(int bx, int by) const { return (bx / gxm) * bn_rows + by * one.bn; }
+  template <int BN>
+  __device__ __forceinline__ void run(uint32_t tmem, int q, int lane, int ew, int bx, int by, int, int,
+                                      int, int, float* sm) const {
+    EpiStore e = one;
+    e.C += (bx / gxm) * sC;
+    e.template run<BN>(tmem, q, lane, ew, bx, by, (bx % gxm) * BM, by * one.bn, bm, bn_rows, sm);
+  }
+};
+
 // Exchange part of Eq. localenergy3 fused into the T_g = Lh_g Theta
 // contraction.  Rows of the product are (g, i) = Lh rows, columns (w, c, j)
 // = Theta^T rows (c = re/im plane).  A tile covers RG whole Cholesky vectors
@@ -1172,6 +1196,30 @@ int tc_gemm_store(const TcGemm& g, float* C, long ldc, float alpha, cudaStream_t
     if (it != g_tuned_bn.end()) bn = it->second;
   }
   return launch_store_bn(g, C, ldc, alpha, bn, st);
+}
+
+// C[b] = alpha A_b B_b^T for `batch` products of g.m x g.n x g.k whose operand
+// rows follow one another (batch g.m rows of A, batch g.n rows of B).  The
+// widest tile that still gives every SM one.
+int tc_gemm_store_batch(const TcGemm& g, int batch, float* C, long ldc, long sC, float alpha,
+                        cudaStream_t st) {
+  if (g.m <= 0 || g.n <= 0 || batch <= 0) return AFQMC_OK;
+  const int gxm = cdiv(g.m, tc::BM);
+  int bn = 256;
+  while (bn > 64 && (long)batch * gxm * cdiv(g.n, bn) < tc_sm_count()) bn /= 2;
+  tc::EpiStoreBatch e{tc::EpiStore{C, ldc, alpha, bn}, gxm, g.m, g.n, sC};
+  TcGemm all = g;  // the tensor maps cover the whole batch
+  all.m = batch * g.m;
+  all.n = batch * g.n;
+  const int gx = batch * gxm, gy = cdiv(g.n, bn);
+  if (bn == 64)
+    return g.tf32 ? launch_tc_persistent<64, 8, true>(all, e, gx, gy, st)
+                  : launch_tc_persistent<64, 8, false>(all, e, gx, gy, st);
+  if (bn == 128)
+    return g.tf32 ? launch_tc_persistent<128, 6, true>(all, e, gx, gy, st)
+                  : launch_tc_persistent<128, 6, false>(all, e, gx, gy, st);
+  return g.tf32 ? launch_tc_persistent<256, 4, true>(all, e, gx, gy, st)
+                : launch_tc_persistent<256, 4, false>(all, e, gx, gy, st);
 }
 
 int tc_tune_store(const TcGemm& g, float* C, long ldc, float alpha, cudaStream_t st, int* chosen) {

@@ -25,6 +25,9 @@ struct TcGemm {
 };
 
 int tc_gemm_store(const TcGemm& g, float* C, long ldc, float alpha, cudaStream_t st);
+// The same for a batch whose operand rows and outputs follow one another.
+int tc_gemm_store_batch(const TcGemm& g, int batch, float* C, long ldc, long sC, float alpha,
+                        cudaStream_t st);
 // Time the tile-width candidates for this shape on the given buffers (not
 // under stream capture) and remember the fastest for tc_gemm_store().
 int tc_tune_store(const TcGemm& g, float* C, long ldc, float alpha, cudaStream_t st, int* chosen);
