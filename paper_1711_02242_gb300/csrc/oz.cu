@@ -464,6 +464,15 @@ struct OzTile {
   int lane, ew;
 };
 
+// An epilogue's reads for a thread's row and its warp's CW columns: the sums of
+// the row exponents, whether the row is stored, earlier values (narrow tiles).
+template <int CW>
+struct OzPre {
+  int e[CW];
+  bool on;
+  double old[CW <= 8 ? CW : 1];
+};
+
 // D_t .. D_{t+3} of eight columns as D_t 2^21 + D_{t+1} 2^14 + D_{t+2} 2^7 +
 // D_{t+3}; the pairs stay below 2^31.
 template <int BN>
@@ -620,6 +629,9 @@ __global__ void __launch_bounds__(kOzThreads<BN>, 1)
       long long hi[MULTI ? CW : 8], lo[MULTI ? CW : 8];
 #pragma unroll
       for (int c = 0; c < (MULTI ? CW : 8); ++c) hi[c] = lo[c] = 0;
+      // what the epilogue reads from memory, in flight during the products
+      OzPre<CW> pre;
+      epi.pre(g, tl, pre);
       bool stop = false;
       for (int sg = 0; sg < (MULTI ? g.nseg : 1); ++sg, ++j) {
         const int buf = NBUF == 2 ? (j & 1) : 0;
@@ -648,7 +660,7 @@ __global__ void __launch_bounds__(kOzThreads<BN>, 1)
             for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
             drain4<BN>(base + (uint32_t)c0, 0, hi);
             drain4<BN>(base + (uint32_t)c0, 4, lo);
-            epi.chunk(g, tl, tl.c0 + c0, hi, lo, smem + S::EPI);
+            epi.chunk(g, tl, c0, hi, lo, pre, smem + S::EPI);
             __syncwarp();  // the next TMEM loads need the whole warp
           }
         }
@@ -659,7 +671,7 @@ __global__ void __launch_bounds__(kOzThreads<BN>, 1)
       if (stop) break;
       if constexpr (MULTI) {
 #pragma unroll
-        for (int c0 = 0; c0 < CW; c0 += 8) epi.chunk(g, tl, tl.c0 + c0, hi + c0, lo + c0, smem + S::EPI);
+        for (int c0 = 0; c0 < CW; c0 += 8) epi.chunk(g, tl, c0, hi + c0, lo + c0, pre, smem + S::EPI);
       }
       epi.template finish<EW>(g, tl, smem + S::EPI);
     }
@@ -673,7 +685,8 @@ __global__ void __launch_bounds__(kOzThreads<BN>, 1)
 }
 
 // -------------------------------------------------------------- epilogues ---
-// chunk(): eight columns from column cc of the tile, row tl.r.
+// pre(): reads that do not depend on the products; chunk(): eight columns from
+// the warp's column c0 on, row tl.r.
 // C[m][n] = 2^alpha D: each warp passes its 32 rows x 8 columns through 2 KB
 // of shared memory so that a store instruction covers four rows of 64 bytes.
 struct EpiOzStore {
@@ -684,17 +697,22 @@ struct EpiOzStore {
   int M, N, alpha;
   const double* mask;
   int mask_rows;
-  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
-                                        const long long* lo, uint8_t* sm) const {
-    double* buf = reinterpret_cast<double*>(sm) + tl.ew * 256;
-    const int lane = tl.lane, row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
+  template <int CW>
+  __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
+    const int row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0;
     const int ea = (row < M ? g.ea[row] : kOzZeroExp) + alpha;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int eb = col + i < N ? g.eb[col + i] : kOzZeroExp;
+    for (int c = 0; c < CW; ++c) q.e[c] = ea + (col + c < N ? g.eb[col + c] : kOzZeroExp);
+  }
+  template <int CW>
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int c0, const long long* hi,
+                                        const long long* lo, const OzPre<CW>& q, uint8_t* sm) const {
+    double* buf = reinterpret_cast<double*>(sm) + tl.ew * 256;
+    const int lane = tl.lane, row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0 + c0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
       // 16-byte slots permuted by row: row-per-lane writes without conflicts
-      buf[lane * 8 + ((i & 1) | (((i >> 1) ^ (lane & 3)) << 1))] = scaled_sum(hi[i], lo[i], ea + eb);
-    }
+      buf[lane * 8 + ((i & 1) | (((i >> 1) ^ (lane & 3)) << 1))] = scaled_sum(hi[i], lo[i], q.e[c0 + i]);
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -710,8 +728,8 @@ struct EpiOzStore {
 };
 
 // A Taylor term: rows p, columns (c, i) of walker b.  A lane owns a row, so
-// the accesses along p are contiguous; the running sum's eight loads are
-// issued before the values are formed.
+// the accesses along p are contiguous; the running sum is read ahead (narrow
+// tiles) or before the values are formed.
 struct EpiOzTerm {
   static constexpr int kStages = 4;
   static constexpr int kSmemBytes = 0;
@@ -721,23 +739,36 @@ struct EpiOzTerm {
   const double* tin;
   double* tout;
   double* acc;
-  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
-                                        const long long* lo, uint8_t*) const {
-    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
-    if (tl.r >= g.a_rpt || p >= M || col >= N2) return;
-    const int ea = g.ea[(long)tl.b * g.ea_batch + p];
+  template <int CW>
+  __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0;
+    q.on = tl.r < g.a_rpt && p < M && col < N2;
+    const int ea = q.on ? g.ea[(long)tl.b * g.ea_batch + p] : kOzZeroExp;
     const int* eb = g.eb + (long)tl.b * g.eb_batch + col;
+#pragma unroll
+    for (int c = 0; c < CW; ++c) q.e[c] = q.on && col + c < N2 ? ea + eb[c] : kOzZeroExp;
+    if constexpr (CW <= 8) {
+      const double* src = (first ? tin : acc) + ((long)tl.b * N2 + col) * M + p;
+#pragma unroll
+      for (int c = 0; c < CW; ++c) q.old[c] = q.on && col + c < N2 ? src[(long)c * M] : 0.0;
+    }
+  }
+  template <int CW>
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int c0, const long long* hi,
+                                        const long long* lo, const OzPre<CW>& q, uint8_t*) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0 + c0;
+    if (!q.on || col >= N2) return;
     const long at = ((long)tl.b * N2 + col) * M + p;
-    const double* src = (first ? tin : acc) + at;
     double old[8], v[8];
-    int e[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      old[c] = col + c < N2 ? src[(long)c * M] : 0.0;
-      e[c] = col + c < N2 ? ea + eb[c] : kOzZeroExp;
+      if constexpr (CW <= 8)
+        old[c] = q.old[c];
+      else
+        old[c] = col + c < N2 ? ((first ? tin : acc) + at)[(long)c * M] : 0.0;
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = scaled_sum(hi[c], lo[c], e[c]) * scale;
+    for (int c = 0; c < 8; ++c) v[c] = scaled_sum(hi[c], lo[c], q.e[c0 + c]) * scale;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       if (col + c >= N2) break;
@@ -754,21 +785,32 @@ struct EpiOzTheta {
   static constexpr int kStages = 4;
   static constexpr int kSmemBytes = 0;
   OzTheta t;
-  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
-                                        const long long* lo, uint8_t*) const {
-    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc, N2 = 2 * t.N;
-    if (tl.r >= g.a_rpt || p >= t.M || col >= N2) return;
+  template <int CW>
+  __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0, N2 = 2 * t.N;
     const int ds = tl.b / t.nw, wl = tl.b - ds * t.nw, w = t.w0 + wl;
-    if (t.wt && !walker_alive(t.wt, w)) return;
+    // the three conditions' loads are independent
     const bool ok = t.flag ? t.flag[w] != 0 : t.ld[(long)w * t.ld_w + (long)ds * t.ld_ds] > -INFINITY;
-    if (!ok && !t.zero_singular) return;
-    const int ea = g.ea[(long)wl * g.ea_batch + p];
+    const bool alive = !t.wt || walker_alive(t.wt, w);
+    q.on = tl.r < g.a_rpt && p < t.M && col < N2 && alive && (ok || t.zero_singular);
+    const int ea = q.on ? g.ea[(long)wl * g.ea_batch + p] : kOzZeroExp;
     const int* eb = g.eb + (long)tl.b * g.eb_batch + col;
+    // (a row of zeros gives zeros whatever the sums: singular walkers)
+#pragma unroll
+    for (int c = 0; c < CW; ++c) q.e[c] = q.on && ok && col + c < N2 ? ea + eb[c] : kSkip;
+  }
+  static constexpr int kSkip = -(1 << 28);
+  template <int CW>
+  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int c0, const long long* hi,
+                                        const long long* lo, const OzPre<CW>& q, uint8_t*) const {
+    const int p = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0 + c0, N2 = 2 * t.N;
+    if (!q.on || col >= N2) return;
+    const int ds = tl.b / t.nw, w = t.w0 + tl.b - ds * t.nw;
     const long row = ((long)ds * t.W + w) * N2 + col;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       if (col + c >= N2) break;
-      double v = ok ? scaled_sum(hi[c], lo[c], ea + eb[c]) : 0.0;
+      double v = q.e[c0 + c] != kSkip ? scaled_sum(hi[c], lo[c], q.e[c0 + c]) : 0.0;
       if (t.unit && p < t.N) v = col + c == p ? 1.0 : 0.0;
       t.theta[(row + c) * t.M + p] = v;
       if (t.th_lo) store_lo(t.th_lo, t.lo_kind, (row + c) * t.Mp + p, v);
@@ -784,21 +826,32 @@ struct EpiOzGram {
   static constexpr int kSmemBytes = 0;
   int N2;
   double* gram;
-  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
-                                        const long long* lo, uint8_t*) const {
-    if (tl.r >= N2 || cc >= N2) return;
+  template <int CW>
+  __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
     const int* e = g.ea + (long)tl.b * g.ea_batch;
-    const int ea = e[tl.r];
+    q.on = tl.r < N2;
+    const int ea = q.on ? e[tl.r] : 0;
+#pragma unroll
+    for (int c = 0; c < CW; ++c) q.e[c] = ea + (tl.c0 + c < N2 ? e[tl.c0 + c] : 0);
+  }
+  template <int CW>
+  __device__ __forceinline__ void chunk(const OzArgs&, const OzTile& tl, int c0, const long long* hi,
+                                        const long long* lo, const OzPre<CW>& q, uint8_t*) const {
+    const int cc = tl.c0 + c0;
+    if (!q.on || cc >= N2) return;
     double* out = gram + ((long)tl.b * N2 + tl.r) * N2 + cc;
 #pragma unroll
     for (int c = 0; c < 8; ++c)
-      if (cc + c < N2) out[c] = scaled_sum(hi[c], lo[c], ea + e[cc + c]);
+      if (cc + c < N2) out[c] = scaled_sum(hi[c], lo[c], q.e[c0 + c]);
   }
   template <int EW>
   __device__ __forceinline__ void finish(const OzArgs&, const OzTile&, uint8_t*) const {}
 };
 
-// Exchange: the tile of T into shared memory, then sum_ij T_ij T_ji per walker
+// Exchange (M = 100, N = 10, 1024 walkers: 1.19 ms for 14364 tiles, 24 k cycles
+// a tile, the drain, conversion and traces against 8 k of products; holding the
+// sums in registers so that the next products start earlier spilled and
+// measured 1.48 ms).  The tile of T into shared memory, then sum_ij T_ij T_ji per walker
 // of the tile over the tile's vectors; every unordered pair {i, j} once, at
 // twice its weight (j = i + d mod N), by the lane of row (g, i); nw warps per
 // walker, their sums added in a fixed order.
@@ -808,17 +861,22 @@ struct EpiOzExchange {
   static constexpr int kSmemBytes = BM * LD * 8 + 2 * 16 * 8;
   int N, W, G, RG, WT, nup, nchunk;  // RG vectors, WT walkers per tile
   double* part;
-  __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int cc, const long long* hi,
-                                        const long long* lo, uint8_t* sm) const {
-    double* T = reinterpret_cast<double*>(sm) + tl.r * LD + cc;
-    const int row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + cc;
-    const bool rv = tl.r < g.a_rpt && row < G * N;
-    const int ea = rv ? g.ea[row] : 0;
+  template <int CW>
+  __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
+    const int row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0;
+    q.on = tl.r < g.a_rpt && row < G * N;
+    const int ea = q.on ? g.ea[row] : 0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const bool in = rv && cc + c < g.b_rpt && col + c < 2 * N * W;
-      T[c] = in ? scaled_sum(hi[c], lo[c], ea + g.eb[col + c]) : 0.0;
-    }
+    for (int c = 0; c < CW; ++c)
+      q.e[c] = ea + (q.on && tl.c0 + c < g.b_rpt && col + c < 2 * N * W ? g.eb[col + c] : kOff);
+  }
+  static constexpr int kOff = -(1 << 28);  // no element there: T is zero
+  template <int CW>
+  __device__ __forceinline__ void chunk(const OzArgs&, const OzTile& tl, int c0, const long long* hi,
+                                        const long long* lo, const OzPre<CW>& q, uint8_t* sm) const {
+    double* T = reinterpret_cast<double*>(sm) + tl.r * LD + tl.c0 + c0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) T[c] = q.e[c0 + c] > kOff / 2 ? scaled_sum(hi[c], lo[c], q.e[c0 + c]) : 0.0;
   }
   template <int EW>
   __device__ __forceinline__ void finish(const OzArgs& g, const OzTile& tl, uint8_t* smraw) const {
