@@ -79,6 +79,24 @@ static void oz_theta_operands(size_t M, size_t N, OzOperand* A, OzOperand* B) {
   B->batch_exp_stride = (long)(2 * N);
 }
 
+// The back-propagated densities of groups of walkers: K = 2 N cw of at most one
+// segment of exact sums, so that groups are independent products.
+static void oz_density_operands(size_t M, size_t N, size_t W, OzOperand* A, OzOperand* B, int* cw, int* nz) {
+  *cw = (int)std::max<size_t>(1, kOzSegK / (2 * N));
+  if ((size_t)*cw > W) *cw = (int)W;
+  const size_t K = 2 * N * *cw, nt = oz_tiles(2 * M, 128);
+  A->RT = A->rows_per_tile = (int)(((2 * M + nt - 1) / nt + 7) / 8 * 8);
+  B->RT = B->rows_per_tile = 64;
+  A->nkb = B->nkb = (int)((K + 15) / 16);
+  A->batch_stride = (long)oz_bytes(2 * M, A->rows_per_tile, A->RT, K);
+  B->batch_stride = (long)oz_bytes(2 * M, 64, 64, K);
+  A->batch_exp_stride = B->batch_exp_stride = (long)(2 * M);
+  // groups at a time: their slices and products stay within some 100 MB
+  const size_t per = A->batch_stride + B->batch_stride + 4 * M * M * sizeof(double);
+  const size_t all = (W + *cw - 1) / *cw, fit = std::max<size_t>(1, (size_t(128) << 20) / per);
+  *nz = (int)std::min(all, fit);
+}
+
 static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz);
 
 size_t plan(const afqmc_params& p, Bufs* b, char* base) {
@@ -104,6 +122,10 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   b->oz_ov = oz && (!mixed || p.ndet > 0);
   b->oz_qr = oz && !f32lu && N <= 32;
   b->oz_exch = b->oz && p.ndet == 0 && N <= 32;
+  b->oz_bp = oz && p.bp_steps > 0;
+  OzOperand denA, denB;
+  int den_cw = 0, den_nz = 0;
+  oz_density_operands(M, N, W, &denA, &denB, &den_cw, &den_nz);
   if (b->oz_exch) nchunk = oz_tiles(G, oz_exchange_vectors((int)N));
   const size_t lo = (p.precision == AFQMC_MIXED_BF16 || p.precision == AFQMC_MIXED_BF16_F32LU ||
                      p.precision == AFQMC_MIXED_BF16_F64THETA)
@@ -175,7 +197,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
     b->bp_f = a.take<double>(2 * W);
     b->bp_cos = a.take<double>(W);
     b->bp_part = a.take<double>(4 * W);
-    b->bp_red = a.take<double>((size_t)kBpSlices * 2 * M * M);
+    b->bp_red = a.take<double>((b->oz_bp ? (size_t)den_nz * 4 : (size_t)kBpSlices * 2) * M * M);
     b->bp_R = a.take<double>(4 * M * M);
     b->bp_out = a.take<double>(4 * M * M + 4);
     size_t row = sizeof(double) * 2 * N * M;
@@ -258,6 +280,10 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       if (p.ndet == 0) need(oz_bytes(2 * wc, 128, 128, N * M), 2 * wc);
     }
     if (b->oz_exch) need(oz_bytes(2 * N * wc, 2 * (int)N * oz_exchange_walkers((int)N), 64, M), 2 * N * wc);
+  }
+  if (b->oz_bp) {
+    oz_need = std::max(oz_need, (size_t)den_nz * (denA.batch_stride + denB.batch_stride));
+    oz_exps = std::max(oz_exps, (size_t)den_nz * 4 * M);
   }
   // scratch: the set-up and the step never run at the same time
   const size_t scratch_at = (a.off + 255) & ~size_t(255);
@@ -582,9 +608,9 @@ int oz_trial_overlaps(afqmc_state* s, double* dst, int n) {
   return oz_rows_gemm(s, s->b.phiT, 2 * s->p.N, s->p.M, s->b.ozV, dst, n, 0, nullptr);
 }
 
-// t.theta rows = Phi times the matrices m[ds][w] (N x N, t.nds per walker) for
-// the walkers that t's conditions let through.
-static int oz_rotate(afqmc_state* s, const double* m, OzTheta t, cudaStream_t st) {
+// t.theta rows = the orbitals phi times the matrices m[ds][w] (N x N, t.nds per
+// walker) for the walkers that t's conditions let through.
+static int oz_rotate(afqmc_state* s, const double* phi, const double* m, OzTheta t, cudaStream_t st) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   oz_theta_operands(p.M, p.N, &t.A, &t.B);
@@ -602,7 +628,7 @@ static int oz_rotate(afqmc_state* s, const double* m, OzTheta t, cudaStream_t st
     t.A.exps = b.oz_exp;
     t.B.data = b.oz_mem + (size_t)t.nw * t.A.batch_stride;
     t.B.exps = b.oz_exp + (size_t)t.nw * t.A.batch_exp_stride;
-    AFQ_TRY(oz_slice_cols(b.phiT + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, st));
+    AFQ_TRY(oz_slice_cols(phi + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, st));
     AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, t.B, st));
     AFQ_TRY(oz_theta(t, st));
   }
@@ -619,13 +645,13 @@ int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, co
   t.unit = unit;
   t.zero_singular = zero_singular;
   t.th_lo = th_lo;
-  return oz_rotate(s, sinv, t, s->st);
+  return oz_rotate(s, s->b.phiT, sinv, t, s->st);
 }
 
 // Gram-Schmidt of the walkers on stream st: Phi <- Phi R^-1 with R from the
 // Gram matrix for well-conditioned walkers (k_gram_factor), the sweep for the
 // others.  (The scratch is free: nothing that uses it runs beside this.)
-static int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
+int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   if (!b.oz_qr) return launch_mgs(m, st);
@@ -650,9 +676,34 @@ static int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
   t.theta = m.phiT;
   t.flag = b.qr_done;
   t.th_lo = m.phi_lo;
-  AFQ_TRY(oz_rotate(s, b.Rinv, t, st));
+  AFQ_TRY(oz_rotate(s, m.phiT, b.Rinv, t, st));
   m.done = b.qr_done;
   return launch_mgs(m, st);
+}
+
+// The groups of walkers [*w0, ...) of the back-propagated densities: their
+// products D[z][2 M][2 M] (see oz_slice_densities), *nz of them; *w0 moves on.
+int oz_density_products(afqmc_state* s, const double* thA, const double* thB, int* w0, int* nz, double* D) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  OzGemm g;
+  int cw = 0;
+  oz_density_operands(p.M, p.N, p.nwalkers, &g.A, &g.B, &cw, nz);
+  *nz = std::min(*nz, (p.nwalkers - *w0 + cw - 1) / cw);
+  g.m = g.n = 2 * p.M;
+  g.batch = *nz;
+  g.ldc = 2L * p.M;
+  g.c_batch = 4L * p.M * p.M;
+  g.C = D;
+  g.A.data = b.oz_mem;
+  g.A.exps = b.oz_exp;
+  g.B.data = b.oz_mem + (size_t)*nz * g.A.batch_stride;
+  g.B.exps = b.oz_exp + (size_t)*nz * g.A.batch_exp_stride;
+  g.err = b.status;
+  AFQ_TRY(oz_slice_densities(b.bp_phi, thA, thB, p.nwalkers, p.N, p.M, *w0, *nz, cw, g.A, g.B, s->st));
+  AFQ_TRY(oz_gemm_store(g, s->st));
+  *w0 += *nz * cw;
+  return AFQMC_OK;
 }
 
 // acc = T_n(V) t0 with V = i sqrt(dt) Y (packed), a chunk of walkers at a time.

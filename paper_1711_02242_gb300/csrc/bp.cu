@@ -24,16 +24,17 @@ namespace {
 constexpr int kRhoTile = 32;
 constexpr int kRhoK = 16;
 
-// C = A B^T for M x M float64 matrices.
-int gemm_sq_f64(const double* A, const double* B, double* C, int M, cudaStream_t st) {
+// C = A B^T for M x M and n x M float64 matrices.
+int gemm_sq_f64(const double* A, const double* B, double* C, int M, int n, cudaStream_t st) {
   GemmF64 g;
-  g.m = g.n = g.k = M;
+  g.m = g.k = M;
+  g.n = n;
   g.A = A;
   g.lda = M;
   g.B = B;
   g.ldb = M;
   g.C = C;
-  g.ldc = M;
+  g.ldc = n;
   return gemm_nt_f64(g, st);
 }
 
@@ -296,6 +297,21 @@ __global__ void k_bp_reduce(long n, int Z, const double* red, double* R) {
   }
 }
 
+// The same from the products D[z][2 M][2 M] of groups of walkers (rows (c, p),
+// columns (e, q)), on top of R (add): R[e][c][p][q].
+__global__ void k_bp_reduce_groups(int M, int Z, const double* D, int add, double* R) {
+  const long MM = (long)M * M;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < 4 * MM;
+       t += (long)gridDim.x * blockDim.x) {
+    const long plane = t / MM, p = t % MM / M, q = t % M;
+    const double* d = D + ((plane & 1) * M + p) * 2 * M + (plane >> 1) * M + q;
+    double s = add ? R[t] : 0.0;
+#pragma unroll 4
+    for (int z = 0; z < Z; ++z) s += d[4 * z * MM];
+    R[t] = s;
+  }
+}
+
 // Weight sums over the walkers in order: sums = (sum W f, sum W) re/im.
 __global__ void k_bp_wsum(int W, const double* part, double* sums) {
   __shared__ double sh[32];
@@ -307,15 +323,17 @@ __global__ void k_bp_wsum(int W, const double* part, double* sums) {
   }
 }
 
-// rho = R / A for the complex weight sum A = sums[off], sums[off + 1].
-__global__ void k_bp_scale(long MM, const double* R, const double* sums, int off, double* rho) {
-  const double ar = sums[off], ai = sums[off + 1];
-  const double den = ar * ar + ai * ai;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < MM;
+// rho[e] = R_e / A_e for the complex weight sums A_e = sums[2 e], sums[2 e + 1];
+// R[p][q][e][c].
+__global__ void k_bp_scale(long MM, const double* R, const double* sums, double* rho) {
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < 2 * MM;
        t += (long)gridDim.x * blockDim.x) {
-    const double xr = R[t], xi = R[MM + t];
-    rho[t] = (xr * ar + xi * ai) / den;
-    rho[MM + t] = (xi * ar - xr * ai) / den;
+    const long e = t / MM, pq = t - e * MM;
+    const double ar = sums[2 * e], ai = sums[2 * e + 1];
+    const double den = ar * ar + ai * ai;
+    const double xr = R[4 * pq + 2 * e], xi = R[4 * pq + 2 * e + 1];
+    rho[2 * e * MM + pq] = (xr * ar + xi * ai) / den;
+    rho[(2 * e + 1) * MM + pq] = (xi * ar - xr * ai) / den;
   }
 }
 
@@ -407,9 +425,12 @@ int bp_close(afqmc_state* s) {
     }
     if (p.qr_period && done % p.qr_period == 0) {
       MgsArgs ma{W, M, N, b.bp_phi, b.wt, b.tmp_ld};
-      AFQ_TRY(launch_mgs(ma, st));
-      if (b.mixed)
-        AFQ_TRY(launch_convert_lo(b.bp_phi, 2L * N * W, M, M, b.bp_phi_lo, b.Mp, b.lo_kind, st));
+      if (b.mixed) {
+        ma.phi_lo = b.bp_phi_lo;
+        ma.lo_kind = b.lo_kind;
+        ma.Mp = b.Mp;
+      }
+      AFQ_TRY(orthonormalise(s, ma, st));
     }
   }
   // per-walker (Phi^H Psi)^-1 and the scaled Theta rows (T0: BP-PRes, T1: BP-PhL)
@@ -419,24 +440,32 @@ int bp_close(afqmc_state* s) {
   AFQ_LAUNCH(k_bp_theta, W, 256, smem, st, W, M, N, b.bp_phi, b.bp_psi, b.wt, b.bp_f, b.T0, b.T1,
              b.bp_part);
   AFQ_LAUNCH(k_bp_wsum, 1, 256, 0, st, W, b.bp_part, b.bp_out + 4 * MM);
-  const long K = (long)W * N;
-  const int tiles = (int)cdiv(M, kRhoTile);
-  int Z = (int)((4L * tc_sm_count() + tiles * tiles - 1) / (tiles * tiles));
-  if (Z > kBpSlices) Z = kBpSlices;
-  if (Z > K / kRhoK) Z = (int)(K / kRhoK);
-  if (Z < 1) Z = 1;
-  for (int e = 0; e < 2; ++e) {
-    const double* th = e == 0 ? b.T0 : b.T1;
-    AFQ_LAUNCH(k_bp_rho, dim3(tiles, tiles, Z), 256, 0, st, M, K, NM, N, b.bp_phi, th, b.bp_red);
-    AFQ_LAUNCH(k_bp_reduce, cdiv(2 * MM, 256), 256, 0, st, 2 * MM, Z, b.bp_red, b.bp_R);
-    // rho = Q R Q^T for each plane: Y = Q R^T, then Q Y^T
-    for (int c = 0; c < 2; ++c) {
-      AFQ_TRY(gemm_sq_f64(b.Qb, b.bp_R + c * MM, b.bp_red, M, st));
-      AFQ_TRY(gemm_sq_f64(b.Qb, b.bp_red, b.bp_R + 2 * MM + c * MM, M, st));
+  // R_e (BP-PRes, BP-PhL) as planes (e, re/im).  512 walkers of M = 100, N = 10:
+  // the float64 products take 2 x 707 us, the sliced ones 105 us.
+  if (b.oz_bp) {
+    for (int w0 = 0, nz = 0; w0 < W;) {
+      const int add = w0 > 0;
+      AFQ_TRY(oz_density_products(s, b.T0, b.T1, &w0, &nz, b.bp_red));
+      AFQ_LAUNCH(k_bp_reduce_groups, cdiv(4 * MM, 256), 256, 0, st, M, nz, b.bp_red, add, b.bp_R);
     }
-    AFQ_LAUNCH(k_bp_scale, cdiv(MM, 256), 256, 0, st, MM, b.bp_R + 2 * MM, b.bp_out + 4 * MM,
-               2 * e, b.bp_out + e * 2 * MM);
+  } else {
+    const long K = (long)W * N;
+    const int tiles = (int)cdiv(M, kRhoTile);
+    int Z = (int)((4L * tc_sm_count() + tiles * tiles - 1) / (tiles * tiles));
+    if (Z > kBpSlices) Z = kBpSlices;
+    if (Z > K / kRhoK) Z = (int)(K / kRhoK);
+    if (Z < 1) Z = 1;
+    for (int e = 0; e < 2; ++e) {
+      AFQ_LAUNCH(k_bp_rho, dim3(tiles, tiles, Z), 256, 0, st, M, K, NM, N, b.bp_phi, e == 0 ? b.T0 : b.T1,
+                 b.bp_red);
+      AFQ_LAUNCH(k_bp_reduce, cdiv(2 * MM, 256), 256, 0, st, 2 * MM, Z, b.bp_red, b.bp_R + 2 * e * MM);
+    }
   }
+  // rho = Q R Q^T for each plane: Y = Q R^T for all of them side by side, rows
+  // (q, plane) of M values, then Q Y^T
+  AFQ_TRY(gemm_sq_f64(b.Qb, b.bp_R, b.bp_red, M, 4 * M, st));
+  AFQ_TRY(gemm_sq_f64(b.Qb, b.bp_red, b.bp_R, M, 4 * M, st));
+  AFQ_LAUNCH(k_bp_scale, cdiv(2 * MM, 256), 256, 0, st, MM, b.bp_R, b.bp_out + 4 * MM, b.bp_out);
   return AFQMC_OK;
 }
 

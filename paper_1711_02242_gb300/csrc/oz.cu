@@ -295,6 +295,61 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N2
   }
 }
 
+// Rows of the density sums (oz_slice_densities): group blockIdx.y of cw
+// walkers, whose K values (w, c, i) of a column p lie M apart; blockIdx.z: Phi
+// as it is, Phi times i, thA, thB.  A lane owns a row as in k_oz_slice_cols.
+__global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, const double* thA,
+                                                            const double* thB, int W, int N, int M, int w0,
+                                                            int cw, OzOperand A, OzOperand B) {
+  __shared__ uint32_t m_sh[8][32], any_sh[8][32];
+  const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, z = blockIdx.y, which = blockIdx.z;
+  const int p = blockIdx.x * 32 + lane, first = w0 + z * cw, N2 = 2 * N;
+  const int nk = (W - first < cw ? W - first : cw) * N2;
+  const OzOperand& o = which < 2 ? A : B;
+  const double* src = (which < 2 ? phi : which == 2 ? thA : thB) + (long)first * N2 * M + p;
+  uint32_t m = 0, any = 0;
+  if (p < M)
+#pragma unroll 4
+    for (int k = wk; k < nk; k += 8) {
+      const double x = src[(long)k * M];
+      m = max(m, abs_hi(x));
+      any |= abs_hi(x) | (uint32_t)__double2loint(x);
+    }
+  m_sh[wk][lane] = m;
+  any_sh[wk][lane] = any;
+  __syncthreads();
+  if (p >= M) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    m = max(m, m_sh[q][lane]);
+    any |= any_sh[q][lane];
+  }
+  const int e = row_exp(m, any != 0);
+  const bool fine = e != kOzNanExp && e != kOzZeroExp;
+  const int row = (which & 1) * M + p, rt = row / o.rows_per_tile, r = row - rt * o.rows_per_tile;
+  if (wk == 0) o.exps[(long)z * o.batch_exp_stride + row] = e;
+  char* base = reinterpret_cast<char*>(o.data) + (long)z * o.batch_stride + (long)rt * o.nkb * (kS * o.RT * 32);
+  for (int c = wk; c < 2 * o.nkb; c += 8) {
+    long long u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * c + i;
+      long long v = 0;
+      if (fine && k < nk) {
+        if (which == 1) {  // (re, im) <- (-im, re)
+          const bool re = k % N2 < N;
+          v = fixed57(src[(long)(re ? k + N : k - N) * M], e);
+          if (re) v = -v;
+        } else {
+          v = fixed57(src[(long)k * M], e);
+        }
+      }
+      u[i] = kDigitBias + v;
+    }
+    put_chunk(base + chunk_off(o.RT, r, c), o.RT * 32, u);
+  }
+}
+
 // The inverse of (ds, w) = (blockIdx.y, blockIdx.x) as operand rows (re, j) =
 // [Re S^-1_j | -Im S^-1_j] and (im, j) = [Im S^-1_j | Re S^-1_j], S^-1_j column j.
 __global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, int W, int w0, int N,
@@ -693,16 +748,17 @@ struct EpiOzStore {
   static constexpr int kStages = 4;
   static constexpr int kSmemBytes = 16 * 32 * 8 * 8;
   double* C;
-  long ldc;
+  long ldc, c_batch;
   int M, N, alpha;
   const double* mask;
   int mask_rows;
   template <int CW>
   __device__ __forceinline__ void pre(const OzArgs& g, const OzTile& tl, OzPre<CW>& q) const {
     const int row = tl.mt * g.a_rpt + tl.r, col = tl.nt * g.b_rpt + tl.c0;
-    const int ea = (row < M ? g.ea[row] : kOzZeroExp) + alpha;
+    const int ea = (row < M ? g.ea[(long)tl.b * g.ea_batch + row] : kOzZeroExp) + alpha;
+    const int* eb = g.eb + (long)tl.b * g.eb_batch;
 #pragma unroll
-    for (int c = 0; c < CW; ++c) q.e[c] = ea + (col + c < N ? g.eb[col + c] : kOzZeroExp);
+    for (int c = 0; c < CW; ++c) q.e[c] = ea + (col + c < N ? eb[col + c] : kOzZeroExp);
   }
   template <int CW>
   __device__ __forceinline__ void chunk(const OzArgs& g, const OzTile& tl, int c0, const long long* hi,
@@ -718,8 +774,9 @@ struct EpiOzStore {
     for (int k = 0; k < 8; ++k) {
       const int rr = 4 * k + (lane >> 3), i = lane & 7;
       const int grow = row - lane + rr, gcol = col + i;
-      if (grow < M && gcol < N && (!mask || walker_alive(mask, grow / mask_rows)))
-        C[(long)grow * ldc + gcol] = buf[rr * 8 + ((i & 1) | (((i >> 1) ^ (rr & 3)) << 1))];
+      if (tl.r - lane + rr < g.a_rpt && grow < M && gcol < N && (!mask || walker_alive(mask, grow / mask_rows)))
+        C[(long)tl.b * c_batch + (long)grow * ldc + gcol] =
+            buf[rr * 8 + ((i & 1) | (((i >> 1) ^ (rr & 3)) << 1))];
     }
     __syncwarp();
   }
@@ -1008,8 +1065,8 @@ int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand&
 
 int oz_gemm_store(const OzGemm& g, cudaStream_t st) {
   AFQ_TRY(check_operand(g.A, g.B, 64));
-  EpiOzStore e{g.C, g.ldc, g.m, g.n, g.alpha_log2, g.mask, g.mask_rows};
-  return launch_oz<64>(oz_args(g.A, g.B, g.m, g.n, 1, g.err), e, st);
+  EpiOzStore e{g.C, g.ldc, g.c_batch, g.m, g.n, g.alpha_log2, g.mask, g.mask_rows};
+  return launch_oz<64>(oz_args(g.A, g.B, g.m, g.n, g.batch, g.err), e, st);
 }
 
 int oz_term_width(int N) { return 2 * N <= 16 ? 16 : 2 * N <= 32 ? 32 : 64; }
@@ -1026,6 +1083,12 @@ int oz_taylor_term(const OzTerm& t, cudaStream_t st) {
 
 int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st) {
   AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, 2 * N, M, o);
+  return AFQMC_OK;
+}
+
+int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
+                       int nz, int cw, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, A, B);
   return AFQMC_OK;
 }
 

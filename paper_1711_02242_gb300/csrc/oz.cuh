@@ -54,9 +54,11 @@ int oz_slice_v(const double* Y, long ldy, int W, int M, int Mp, const OzOperand&
 int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand& o, cudaStream_t st);
 
 // C[m][n] = 2^alpha_log2 sum_k A[m][k] B[n][k] (float64, pitch ldc); rows of
-// dead walkers (mask, mask_rows rows each) are not stored.
+// dead walkers (mask, mask_rows rows each) are not stored.  A batch of them
+// with the operands' strides and C c_batch values apart.
 struct OzGemm {
-  int m = 0, n = 0;
+  int m = 0, n = 0, batch = 1;
+  long c_batch = 0;
   OzOperand A, B;  // B: RT = 64
   double* C = nullptr;
   long ldc = 0;
@@ -101,6 +103,13 @@ struct OzTheta {
 };
 // operand rows p = [Re Phi_p | Im Phi_p] (2 N values) of W walkers
 int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st);
+// Operands of sum_k conj(Phi_k[p]) Th_k[q] over the rows k = (w, i) of nz
+// groups of cw walkers from walker w0 on (the last may be short), a batch entry
+// each, K = 2 N cw: A rows p = [Re Phi_p | Im Phi_p] and M + p =
+// [-Im Phi_p | Re Phi_p] per walker (sums with [Re Th | Im Th]: the real and the
+// imaginary part), B rows q of thA and M + q of thB.
+int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
+                       int nz, int cw, const OzOperand& A, const OzOperand& B, cudaStream_t st);
 // operand rows (re, j) = [Re S^-1_j | -Im S^-1_j], (im, j) = [Im | Re] of the
 // inverses sinv[ds W + w0 + w], batch ds nw + w
 int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,

@@ -61,7 +61,8 @@ struct Bufs {
   // the mixed path, which keeps these in float64
   // oz_qr: Gram-Schmidt from the Gram matrix (also on the mixed path): its
   // products, R^-1 and which walkers took it
-  bool oz = false, oz_exch = false, oz_ov = false, oz_qr = false;
+  // oz_bp: the products of the back-propagated densities
+  bool oz = false, oz_exch = false, oz_ov = false, oz_qr = false, oz_bp = false;
   double *gram = nullptr, *Rinv = nullptr;
   int* qr_done = nullptr;
   OzOperand ozL, ozF, ozX, ozB, ozV;
@@ -72,7 +73,8 @@ struct Bufs {
   // back-propagation window (afqmc_params.bp_steps > 0): recorded fields
   // [bp_steps][W][2][G] float64 (mixed path: operand rows [W][2][Gp]), Psi_n and the back-propagated
   // orbitals [W][2][N][M], BP-PRes factors [W][2], cos dtheta [W], per-walker
-  // weights [W][4], estimator slices [kBpSlices][2][M][M], R [4][M][M] and
+  // weights [W][4], estimator slices [kBpSlices][2][M][M] (oz_bp: products of
+  // groups of walkers [2 M][2 M]), R [4][M][M] and
   // the results [2][2][M][M] + 4 weight sums
   double *bp_hist = nullptr, *bp_psi = nullptr, *bp_phi = nullptr, *bp_f = nullptr;
   double *bp_cos = nullptr, *bp_part = nullptr, *bp_red = nullptr, *bp_R = nullptr;
@@ -183,6 +185,8 @@ int join_side(afqmc_state* s);
 int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
                   int unit, int zero_singular, void* th_lo);
 int oz_trial_overlaps(afqmc_state* s, double* dst, int n);
+int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st);
+int oz_density_products(afqmc_state* s, const double* thA, const double* thB, int* w0, int* nz, double* D);
 }  // namespace afq
 
 namespace afq {

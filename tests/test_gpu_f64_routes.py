@@ -180,3 +180,51 @@ def test_gram_schmidt_routes(pkg, M, N, Ndn):
     assert np.max(np.abs(wt - orc.weight) / orc.weight) < TOL
     assert np.max(np.abs(lo - orc.logdet)) < TOL * (1 + np.abs(orc.logdet).max())
     run.close()
+
+
+@pytest.mark.parametrize("M,N,G,W,m,qr", [
+    (40, 5, 57, 41, 3, 2),    # the fewest orbitals; a group of 40 walkers and one of a single walker
+    (65, 13, 70, 15, 2, 0),   # two row tiles of A, the last group full
+    (100, 33, 60, 13, 2, 1),  # rows of the last tile short; K not a multiple of 16, QR by the sweep
+    (44, 5, 50, 6, 0, 5),     # an empty window, fewer walkers than a group
+])
+def test_densities(pkg, M, N, G, W, m, qr):
+    """The back-propagated densities from groups of walkers, against the oracle's window."""
+    h1, L, C = inputs(M, N, G)
+    orc = afqmc.Oracle(h1, L, C, W, afqmc.Params(qr_period=qr, energy_period=0))
+    p = pkg.default_params(M, N, G, W, qr_period=qr, energy_period=0, bp_steps=4)
+    run = pkg.AfqmcRun(h1, L, C, p)
+    orc.run(2)
+    run.propagate(2)
+    orc.bp_begin()
+    run.bp_begin()
+    orc.run(m)
+    run.propagate(m)
+    want, got = orc.bp_end(), run.bp_end()
+    scale = max(1.0, np.abs(want[0]).max(), np.abs(want[1]).max())
+    for a, b in zip(got[:4], want[:4]):
+        assert np.max(np.abs(a - b)) < TOL * max(scale, np.max(np.abs(b)))
+    assert np.count_nonzero(orc.weight) > W // 2
+    run.close()
+
+
+def test_densities_of_chunks(pkg):
+    """More groups than one launch takes: the sums of a population are those of
+    its two halves (which draw the same fields), and bit for bit repeatable."""
+    M, N, G, W = 40, 2, 50, 12000
+    h1, L, C = inputs(M, N, G)
+
+    def densities(n, walker0):
+        p = pkg.default_params(M, N, G, n, qr_period=2, energy_period=0, bp_steps=2, walker0=walker0)
+        run = pkg.AfqmcRun(h1, L, C, p)
+        run.bp_begin()
+        run.propagate(2)
+        out = run.bp_end()
+        run.close()
+        return out
+
+    whole, again, a, b = densities(W, 0), densities(W, 0), densities(7000, 0), densities(5000, 7000)
+    assert np.array_equal(whole[0], again[0]) and np.array_equal(whole[1], again[1])
+    for k in (0, 1):
+        ref = (a[k] * a[2 + k] + b[k] * b[2 + k]) / (a[2 + k] + b[2 + k])
+        assert np.max(np.abs(whole[k] - ref)) < TOL * max(1.0, np.abs(ref).max())
