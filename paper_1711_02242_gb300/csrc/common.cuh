@@ -211,6 +211,15 @@ __device__ inline T block_sum(T v, T* sh /* >= 32 */) {
   return r;
 }
 
+// A float as a double by integer operations: the conversion instruction runs
+// on the float64 pipe, at 1/64 of their rate.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)x;  // zeros, subnormals, infinities, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 __host__ __device__ inline double wrap_pi(double a) {
   // (-pi, pi]
   const double PI = 3.141592653589793, TWO_PI = 6.283185307179586;

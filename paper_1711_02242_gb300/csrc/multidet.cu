@@ -176,74 +176,86 @@ __global__ void __launch_bounds__(256)
 
 // Per walker: log <Psi_T|Psi> = log sum_d exp(log A_d^* + ld_du + ld_dd) in
 // the order of d (largest real part factored out), its phase in (-pi, pi],
-// and the weights w_d.
-__global__ void k_md_combine(int W, int nd, const double* logA, const double* ldds,
-                             const double* wt, double* ldout, double* wd) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+// and the weights w_d.  A warp per walker, a lane per determinant (32 at a
+// time, added in order by shuffles): bound by the chain of an exponential, a
+// sine and cosine, a logarithm and an arctangent in float64.  256 walkers, 4
+// determinants: 24.6 us with a thread per walker, which took the first three
+// eight times one after another, 9.5 now.
+__global__ void __launch_bounds__(32) k_md_combine(int W, int nd, const double* logA, const double* ldds,
+                                                   const double* wt, double* ldout, double* wd) {
+  const int w = blockIdx.x, lane = threadIdx.x;
   if (w >= W || !walker_alive(wt, w)) return;
   const double* l = ldds + (long)w * nd * 4;  // [nd][2 spins][re, im]
+  auto real = [&](int d) { return logA[2 * d] + l[4 * d] + l[4 * d + 2]; };
   double ref = -INFINITY;
-  for (int d = 0; d < nd; ++d) {
-    const double re = logA[2 * d] + l[4 * d] + l[4 * d + 2];
+  for (int d = lane; d < nd; d += 32) {
+    const double re = real(d);
     if (re > ref) ref = re;
   }
-  double tr = 0.0, ti = 0.0;
-  for (int d = 0; d < nd; ++d) {
-    const double re = logA[2 * d] + l[4 * d] + l[4 * d + 2];
-    if (!(re > -INFINITY)) continue;
-    const double m = exp(re - ref);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double other = __shfl_xor_sync(0xffffffffu, ref, o);
+    if (other > ref) ref = other;
+  }
+  // m e^{i phi} of determinant d, zero without an overlap
+  auto term = [&](int d, double* xr, double* xi) {
+    *xr = *xi = 0.0;
+    if (d >= nd || !(real(d) > -INFINITY)) return;
+    const double m = exp(real(d) - ref);
     double sn, cs;
     sincos(logA[2 * d + 1] + l[4 * d + 1] + l[4 * d + 3], &sn, &cs);
-    tr += m * cs;
-    ti += m * sn;
+    *xr = m * cs;
+    *xi = m * sn;
+  };
+  double tr = 0.0, ti = 0.0, xr, xi;
+  for (int d0 = 0; d0 < nd; d0 += 32) {
+    term(d0 + lane, &xr, &xi);
+    const int n = nd - d0 < 32 ? nd - d0 : 32;
+    for (int k = 0; k < n; ++k) {
+      tr += __shfl_sync(0xffffffffu, xr, k);
+      ti += __shfl_sync(0xffffffffu, xi, k);
+    }
   }
   const double den = tr * tr + ti * ti;
-  for (int d = 0; d < nd; ++d) {
-    const double re = logA[2 * d] + l[4 * d] + l[4 * d + 2];
-    double xr = 0.0, xi = 0.0;
-    if (re > -INFINITY) {
-      const double m = exp(re - ref);
-      double sn, cs;
-      sincos(logA[2 * d + 1] + l[4 * d + 1] + l[4 * d + 3], &sn, &cs);
-      // (m e^{i phi}) / (tr + i ti)
-      xr = (m * cs * tr + m * sn * ti) / den;
-      xi = (m * sn * tr - m * cs * ti) / den;
-    }
-    wd[((long)w * nd + d) * 2] = xr;
-    wd[((long)w * nd + d) * 2 + 1] = xi;
+  for (int d = lane; d < nd; d += 32) {
+    if (nd > 32) term(d, &xr, &xi);
+    const bool any = real(d) > -INFINITY;
+    wd[((long)w * nd + d) * 2] = any ? (xr * tr + xi * ti) / den : 0.0;
+    wd[((long)w * nd + d) * 2 + 1] = any ? (xi * tr - xr * ti) / den : 0.0;
   }
-  ldout[2 * w] = ref + 0.5 * log(den);
-  ldout[2 * w + 1] = wrap_pi(atan2(ti, tr));
+  if (lane == 0) ldout[2 * w] = ref + 0.5 * log(den);
+  if (lane == 1) ldout[2 * w + 1] = wrap_pi(atan2(ti, tr));
 }
 
 // t[w][c][g] = sum_(d,s) w_d (C_ds[(w,re)][g] + i C_ds[(w,im)][g]) as re/im planes
-// (float64 traces and t on the float64 path, FP32 on the mixed path).
+// (float64 traces and t on the float64 path, FP32 on the mixed path).  Bound by
+// the float64 pipe, also with FP32 traces (hence no conversions on it): 256
+// walkers, 4 determinants, 500 vectors take 18.2 us, 20.4 with conversions and a
+// division per value.
 template <typename TC>
-__global__ void k_md_fb_combine(int W, int nd, int G, const TC* C, const double* wd,
-                                const double* wt, TC* t) {
-  const long n = (long)W * G;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
-       e += (long)gridDim.x * blockDim.x) {
-    const int w = (int)(e / G), g = (int)(e - (long)w * G);
-    if (!walker_alive(wt, w)) continue;
-    double sr = 0.0, si = 0.0;
-    for (int d = 0; d < nd; ++d) {
-      const double ar = wd[((long)w * nd + d) * 2], ai = wd[((long)w * nd + d) * 2 + 1];
-      double cr = 0.0, ci = 0.0;
-      for (int s = 0; s < 2; ++s) {
-        const TC* Cd = C + (long)(2 * d + s) * 2 * W * G;
-        cr += (double)Cd[(2L * w) * G + g];
-        ci += (double)Cd[(2L * w + 1) * G + g];
-      }
-      sr += ar * cr - ai * ci;
-      si += ar * ci + ai * cr;
-    }
-    t[(2L * w) * G + g] = (TC)sr;
-    t[(2L * w + 1) * G + g] = (TC)si;
+__global__ void __launch_bounds__(256) k_md_fb_combine(int W, int nd, int G, const TC* C, const double* wd,
+                                                       const double* wt, TC* t) {
+  const int w = blockIdx.y, g = blockIdx.x * 256 + threadIdx.x;
+  if (g >= G || !walker_alive(wt, w)) return;
+  const long plane = 2L * W * G;  // traces of one (d, s)
+  const TC* c = C + 2L * w * G + g;
+  const double* a = wd + 2L * w * nd;
+  double sr = 0.0, si = 0.0;
+#pragma unroll 4
+  for (int d = 0; d < nd; ++d, c += 2 * plane) {
+    const double ar = a[2 * d], ai = a[2 * d + 1];
+    const double cr = widen(c[0]) + widen(c[plane]), ci = widen(c[G]) + widen(c[plane + G]);
+    sr += ar * cr - ai * ci;
+    si += ar * ci + ai * cr;
   }
+  t[(2L * w) * G + g] = (TC)sr;
+  t[(2L * w + 1) * G + g] = (TC)si;
 }
 
-// E_loc per walker (one block): sum_d w_d [one-body + Coulomb - exchange / 2] + H0.
+// E_loc per walker (one block): sum_d w_d [one-body + Coulomb - exchange / 2] + H0,
+// each thread's share weighted before the block's one sum.  (A block sum of each
+// of the six parts per determinant took more float64 operations than the parts:
+// 256 walkers, 4 determinants, 76.5 us; 54.8 now.)
 template <typename TC>
 __global__ void __launch_bounds__(256)
     k_md_eloc(int W, int nd, int M, int N, int G, int nchunk, double H0, const double* hh,
@@ -276,22 +288,18 @@ __global__ void __launch_bounds__(256)
       double tr = 0.0, ti = 0.0;
       for (int s = 0; s < 2; ++s) {
         const TC* Cd = C + (long)(2 * d + s) * 2 * W * G;
-        tr += (double)Cd[(2L * w) * G + g];
-        ti += (double)Cd[(2L * w + 1) * G + g];
+        tr += widen(Cd[(2L * w) * G + g]);
+        ti += widen(Cd[(2L * w + 1) * G + g]);
       }
       cr += tr * tr - ti * ti;
       ci += 2.0 * tr * ti;
     }
-    e1r = block_sum(e1r, sh);
-    e1i = block_sum(e1i, sh);
-    cr = block_sum(cr, sh);
-    ci = block_sum(ci, sh);
-    xr = block_sum(xr, sh);
-    xi = block_sum(xi, sh);
     const double edr = e1r + 0.5 * cr - 0.5 * xr, edi = e1i + 0.5 * ci - 0.5 * xi;
     er += ar * edr - ai * edi;
     ei += ar * edi + ai * edr;
   }
+  er = block_sum(er, sh);
+  ei = block_sum(ei, sh);
   if (threadIdx.x == 0) {
     eloc[2 * w] = H0 + er;
     eloc[2 * w + 1] = ei;
@@ -855,7 +863,7 @@ int md_overlap_update(afqmc_state* s, bool into_ld) {
   else
     AFQ_LAUNCH(k_md_overlap, dim3(2 * nd, W), 256, smem, s->st, W, M, N, b.md_V, b.phiT, b.wt,
                b.md_theta, b.md_ld, b.mixed ? b.md_theta_lo : nullptr, b.lo_kind, b.Mp);
-  AFQ_LAUNCH(k_md_combine, cdiv(W, 128), 128, 0, s->st, W, nd, b.md_logA, b.md_ld, b.wt,
+  AFQ_LAUNCH(k_md_combine, W, 32, 0, s->st, W, nd, b.md_logA, b.md_ld, b.wt,
              into_ld ? b.ld : b.ld_new, b.md_w);
   return AFQMC_OK;
 }
@@ -907,7 +915,7 @@ int md_force_bias(afqmc_state* s) {
   if (s->smw) return smw_force_bias(s);
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
-  const unsigned grid = cdiv((size_t)p.nwalkers * p.nchol, 256);
+  const dim3 grid(cdiv(p.nchol, 256), p.nwalkers);
   if (b.mixed) {
     AFQ_TRY(md_traces_lo(s));
     AFQ_LAUNCH(k_md_fb_combine<float>, grid, 256, 0, s->st, p.nwalkers, p.ndet, p.nchol, b.md_C32,

@@ -630,13 +630,15 @@ __global__ void __launch_bounds__(OV_T) k_overlap(OverlapArgs a) {
 // the loop over pivots needs no unrolling.  Same operations on the same
 // values in the same order as k_overlap<double>, so the same results, without
 // its three block barriers per pivot.  Bound by the latency of the float64
-// chain of a pivot (|a|^2, the reciprocal, the factors), 7.4 k cycles at
-// N = 10.  1024 walkers, N = 10: 73.3 us (one block of 256 threads per walker,
-// 100 of them with an element) to 38.7; 128 walkers, N = 2: 15.2 to 12.2.
+// chain of a pivot (|a|^2, the reciprocal, the factors) up to two warps per SM,
+// by the SM's float64 pipe above: a warp per block spreads them evenly.  1024
+// walkers, N = 10: 73.3 us (one block of 256 threads per walker, 100 of them
+// with an element) to 35.3; 128 walkers, N = 2: 15.2 to 8.3; 256 walkers with 8
+// overlaps each, N = 10: 38.9 (54.4 with four warps per block, on fewer SMs).
 // Above 16 rows a warp has one walker and the block's eight warps win: 301
 // walkers, N = 17: 47 us against 72; 512, N = 25: 109 us against 129.
 namespace {
-constexpr int OW_WARPS = 4;
+constexpr int OW_WARPS = 1;
 }
 template <int N>
 __global__ void __launch_bounds__(32 * OW_WARPS) k_overlap_warp(OverlapArgs a) {
@@ -1505,7 +1507,10 @@ int launch_exchange(const ExchArgs& a, cudaStream_t st) {
 // (Eqs. localenergy2/3; the 1/2 is that of H_2 in Eq. bo_ham2) for the
 // closed-shell block; with two spin blocks (sf = 1) the one-body trace and the
 // exchange are the sums over the blocks, E_loc = H0 + Tr(hh Theta) +
-// 1/2 sum_g [t_g^2 - sum_sigma Tr(T_g,sigma T_g,sigma)].
+// 1/2 sum_g [t_g^2 - sum_sigma Tr(T_g,sigma T_g,sigma)].  Bound by the float64
+// pipe: each thread adds its share of the three parts before the block's one
+// sum, and FP32 traces are widened by integer operations.  1024 walkers of
+// M = 100, N = 10, G = 500: 35.5 us with a block sum of each part, 26.1 now.
 __global__ void __launch_bounds__(256) k_eloc(ElocArgs a) {
   pdl_begin();
   __shared__ double sh[32];
@@ -1522,8 +1527,8 @@ __global__ void __launch_bounds__(256) k_eloc(ElocArgs a) {
   for (int g = threadIdx.x; g < G; g += blockDim.x) {
     double re, imv;
     if (a.t32) {
-      re = a.t32[(long)w * 2 * G + g];
-      imv = a.t32[(long)w * 2 * G + G + g];
+      re = widen(a.t32[(long)w * 2 * G + g]);
+      imv = widen(a.t32[(long)w * 2 * G + G + g]);
     } else {
       re = a.t[(long)w * 2 * G + g];
       imv = a.t[(long)w * 2 * G + G + g];
@@ -1537,15 +1542,11 @@ __global__ void __launch_bounds__(256) k_eloc(ElocArgs a) {
     xr += pp[2 * c];
     xi += pp[2 * c + 1];
   }
-  e1r = block_sum(e1r, sh);
-  e1i = block_sum(e1i, sh);
-  cr = block_sum(cr, sh);
-  ci = block_sum(ci, sh);
-  xr = block_sum(xr, sh);
-  xi = block_sum(xi, sh);
+  const double er = block_sum(a.sf * e1r + 0.5 * cr - (0.5 * a.sf) * xr, sh);
+  const double ei = block_sum(a.sf * e1i + 0.5 * ci - (0.5 * a.sf) * xi, sh);
   if (threadIdx.x == 0) {
-    a.eloc[2 * w] = a.H0 + a.sf * e1r + 0.5 * cr - (0.5 * a.sf) * xr;
-    a.eloc[2 * w + 1] = a.sf * e1i + 0.5 * ci - (0.5 * a.sf) * xi;
+    a.eloc[2 * w] = a.H0 + er;
+    a.eloc[2 * w + 1] = ei;
   }
 }
 

@@ -104,6 +104,7 @@ def test_chunks_of_walkers(pkg):
     (40, 5, 3, "noci", 0),    # the fewest orbitals of the route
     (70, 33, 2, "noci", 0),   # two column tiles of Theta, 132 rows of the trial's orbitals
     (130, 6, 2, "noci", 0),   # two row tiles of Phi
+    (40, 3, 33, "noci", 0),   # one determinant more than the lanes of a warp
     (44, 6, 4, "ci", 0),      # relative to determinant 0: its overlap alone
     (44, 6, 3, "noci", 2),    # the mixed path keeps these float64
 ])
