@@ -364,13 +364,26 @@ struct EpiStoreBatch {
 // (RG*N <= 128 rows) and CW whole walkers; the B tile is one 3-D TMA box of
 // CW walkers x NPAD rows (the 2N rows of a walker, zero-padded to a power of
 // two), so walker wl of the tile owns accumulator columns [wl NPAD, wl NPAD +
-// 2N).  The accumulator is copied to this epilogue's own shared memory; the
-// thread of row (g, i) then forms its share of sum_ij T_ij T_ji (complex) from
-// its own row and column i of the block, the N shares of a vector are summed,
-// and part[w][g][2] receives one partial per (g, w) (nchunk = G), summed later
-// in a fixed order.  T never reaches global memory.
+// 2N).  Half the accumulator's columns at a time (CW / 2 walkers) are copied to
+// this epilogue's own shared memory; the thread of row (g, i) then forms its
+// share of sum_ij T_ij T_ji (complex) from its own row and column i of the
+// block, the N shares of a vector are summed, and part[w][g][2] receives one
+// partial per (g, w) (nchunk = G), summed later in a fixed order.  T never
+// reaches global memory.
+//
+// A pitch of 132 floats: 16-byte stores of a row per lane (33 slots of 16 bytes
+// apart), the walk along rows (j = i + d: 133 floats apart) and the walk along
+// columns are all free of bank conflicts.  (With a pitch of 257 for the whole
+// tile the row walk had two-way conflicts, the copy took 4-byte stores and two
+// ring stages were left.)  512 walkers, M = 300, N = 25, 1800 vectors: 1250 us
+// to 1060; 301, M = 217 (TF32): 320 to 250.  Bound by the SM's shared memory,
+// which the operands pass twice (TMA in, MMA out: 3.8 k cycles per tile of
+// 6.7 k at M = 300) and the tile's values twice.  Tried and not kept: CTA pairs
+// sharing B by multicast (1 - 2% either way), sixteen warps (1322 against 1159
+// us for the energy of 512 walkers).
 struct EpiExchange {
-  static constexpr int kSmemBytes = 128 * 257 * 4;  // one 128 x 256 FP32 tile
+  static constexpr int LD = 132;
+  static constexpr int kSmemBytes = 128 * LD * 4;  // 128 x 128 FP32
   static constexpr bool kB3D = true;
   static constexpr int kWarps = 8;  // two per TMEM lane quarter, splitting columns / walkers
   static constexpr int kMT = 1;
@@ -383,25 +396,9 @@ struct EpiExchange {
   template <int BN>
   __device__ __forceinline__ void run(uint32_t tmem, int q, int lane, int ew, int bx, int by, int,
                                       int, int, int, float* sm) const {
-    constexpr int LD = BN + 1;  // odd pitch: row and column walks are conflict-free
-    const int r = 32 * q + lane, half = ew >> 2;
-    const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
-    // the two warps of a lane quarter take alternate 16-column chunks, two
-    // TMEM loads in flight per wait
-#pragma unroll 1
-    for (int c0 = 16 * half; c0 < BN; c0 += 64) {
-      uint32_t ra[16], rb[16];
-      tmem_ld16_async(tq + (uint32_t)c0, ra);
-      if (c0 + 32 < BN) tmem_ld16_async(tq + (uint32_t)(c0 + 32), rb);
-      tmem_ld_wait();
-#pragma unroll
-      for (int i = 0; i < 16; ++i) sm[r * LD + c0 + i] = __uint_as_float(ra[i]);
-      if (c0 + 32 < BN) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[r * LD + c0 + 32 + i] = __uint_as_float(rb[i]);
-      }
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
+    static_assert(BN == 256, "two halves of 128 columns");
+    const int r = 32 * q + lane, side = ew >> 2, hw = CW / 2;
+    const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(64 * side);
     const int gl = r / N, i = r - gl * N;
     const bool rv = gl < RG;
     // sum_ij T_ij T_ji of a vector only enters summed over i, so each unordered
@@ -414,62 +411,94 @@ struct EpiExchange {
     const int nd = (N - 1) / 2;
     float e[kMaxCW];
 #pragma unroll
-    for (int h = 0; h < kMaxCW / 2; ++h) {
-      const int wl = 2 * h + half;
-      float er = 0.f, ei = 0.f;
-      if (wl < CW && rv) {
-        const float* own = sm + r * LD + wl * NPAD;             // T_ij: [j], [N + j]
-        const float* col = sm + (gl * N) * LD + wl * NPAD + i;  // T_ji: [j LD], [j LD + N]
-        const float dr = own[i], di = own[N + i];
-        float pr = 0.f, pi = 0.f;
-#pragma unroll 4
-        for (int d = 1; d <= nd; ++d) {
-          const int j = i + d < N ? i + d : i + d - N;
-          const float ar = own[j], ai = own[N + j];
-          const float br = col[j * LD], bi = col[j * LD + N];
-          pr = fmaf(ar, br, fmaf(-ai, bi, pr));
-          pi = fmaf(ar, bi, fmaf(ai, br, pi));
-        }
-        er = fmaf(dr, dr, fmaf(-di, di, 2.f * pr));
-        ei = fmaf(2.f * dr, di, 2.f * pi);
-        if ((N & 1) == 0) {
-          const int j = i + N / 2 < N ? i + N / 2 : i - N / 2;
-          const float ar = own[j], ai = own[N + j];
-          const float br = col[j * LD], bi = col[j * LD + N];
-          er = fmaf(ar, br, fmaf(-ai, bi, er));
-          ei = fmaf(ar, bi, fmaf(ai, br, ei));
-        }
-      }
-      e[2 * h] = er;
-      e[2 * h + 1] = ei;
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");  // every read of the tile is done
+    for (int hf = 0; hf < 2; ++hf) {
+      // each warp copies 64 columns of its rows, two TMEM loads in flight per wait
 #pragma unroll
-    for (int h = 0; h < kMaxCW / 2; ++h) {
-      const int wl = 2 * h + half;
-      if (wl < CW) {
-        sm[r * LD + 2 * wl] = e[2 * h];
-        sm[r * LD + 2 * wl + 1] = e[2 * h + 1];
+      for (int c = 0; c < 64; c += 32) {
+        uint32_t ra[16], rb[16];
+        tmem_ld16_async(tq + (uint32_t)(128 * hf + c), ra);
+        tmem_ld16_async(tq + (uint32_t)(128 * hf + c + 16), rb);
+        tmem_ld_wait();
+        uint4* dst = reinterpret_cast<uint4*>(sm + r * LD + 64 * side + c);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[k] = make_uint4(ra[4 * k], ra[4 * k + 1], ra[4 * k + 2], ra[4 * k + 3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[4 + k] = make_uint4(rb[4 * k], rb[4 * k + 1], rb[4 * k + 2], rb[4 * k + 3]);
       }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll
+      for (int h = 0; h < kMaxCW / 4; ++h) {
+        const int wl = 2 * h + side;  // walker of the half
+        float er = 0.f, ei = 0.f;
+        if (wl < hw && rv) {
+          const float* own = sm + r * LD + wl * NPAD;             // T_ij: [j], [N + j]
+          const float* col = sm + (gl * N) * LD + wl * NPAD + i;  // T_ji: [j LD], [j LD + N]
+          const float dr = own[i], di = own[N + i];
+          float pr = 0.f, pi = 0.f;
+#pragma unroll 4
+          for (int d = 1; d <= nd; ++d) {
+            const int j = i + d < N ? i + d : i + d - N;
+            const float ar = own[j], ai = own[N + j];
+            const float br = col[j * LD], bi = col[j * LD + N];
+            pr = fmaf(ar, br, fmaf(-ai, bi, pr));
+            pi = fmaf(ar, bi, fmaf(ai, br, pi));
+          }
+          er = fmaf(dr, dr, fmaf(-di, di, 2.f * pr));
+          ei = fmaf(2.f * dr, di, 2.f * pi);
+          if ((N & 1) == 0) {
+            const int j = i + N / 2 < N ? i + N / 2 : i - N / 2;
+            const float ar = own[j], ai = own[N + j];
+            const float br = col[j * LD], bi = col[j * LD + N];
+            er = fmaf(ar, br, fmaf(-ai, bi, er));
+            ei = fmaf(ar, bi, fmaf(ai, br, ei));
+          }
+        }
+        e[(hf * (kMaxCW / 4) + h) * 2] = er;
+        e[(hf * (kMaxCW / 4) + h) * 2 + 1] = ei;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // every read of the half is done
+    }
+#pragma unroll
+    for (int k = 0; k < kMaxCW / 2; ++k) {
+      const int wl = 2 * (k % (kMaxCW / 4)) + side;
+      if (wl < hw)
+        *reinterpret_cast<float2*>(sm + r * LD + 2 * (k / (kMaxCW / 4) * hw + wl)) =
+            make_float2(e[2 * k], e[2 * k + 1]);
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    // one thread per (vector, walker, re/im): the N rows' shares added in
-    // four interleaved partial sums, combined in a fixed order
-    const int g0 = bx * RG, w0 = by * CW;
-    for (int item = r + 128 * half; item < 2 * RG * CW; item += 256) {
+    // per (vector, walker, re/im) the N rows' shares in four interleaved partial
+    // sums, combined in a fixed order: by a thread each, or for many rows by four
+    // neighbouring threads
+    const int g0 = bx * RG, w0 = by * CW, tid = r + 128 * side;
+    const int lanes = N >= 16 ? 4 : 1, items = 2 * RG * CW * lanes;
+    for (int x0 = 0; x0 < items; x0 += 256) {
+      const int x = x0 + tid, item = lanes == 4 ? x >> 2 : x, z = x & 3;
+      const bool on = x < items;
       const int c = item & 1, gw = item >> 1, g = gw / CW, wl = gw - g * CW;
-      if (g0 + g >= G || w0 + wl >= W) continue;
       const float* src = sm + (g * N) * LD + 2 * wl + c;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      int i2 = 0;
-      for (; i2 + 4 <= N; i2 += 4) {
-        s0 += src[i2 * LD];
-        s1 += src[(i2 + 1) * LD];
-        s2 += src[(i2 + 2) * LD];
-        s3 += src[(i2 + 3) * LD];
+      if (lanes == 4) {
+        if (on) {
+          int i2 = z;
+          for (; i2 < (N & ~3); i2 += 4) s0 += src[i2 * LD];
+          if (z == 0)
+            for (; i2 < N; ++i2) s0 += src[i2 * LD];
+        }
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+      } else if (on) {
+        int i2 = 0;
+        for (; i2 + 4 <= N; i2 += 4) {
+          s0 += src[i2 * LD];
+          s1 += src[(i2 + 1) * LD];
+          s2 += src[(i2 + 2) * LD];
+          s3 += src[(i2 + 3) * LD];
+        }
+        for (; i2 < N; ++i2) s0 += src[i2 * LD];
+        s0 = (s0 + s1) + (s2 + s3);
       }
-      for (; i2 < N; ++i2) s0 += src[i2 * LD];
-      part[((long)(w0 + wl) * nchunk + g0 + g) * 2 + c] = (double)((s0 + s1) + (s2 + s3));
+      if (on && (lanes == 1 || z == 0) && g0 + g < G && w0 + wl < W)
+        part[((long)(w0 + wl) * nchunk + g0 + g) * 2 + c] = (double)s0;
     }
     // the next tile's copy into sm must wait until every warp is done reading
     asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -1685,7 +1714,7 @@ void exchange_tile(int N, int* RG, int* CW, int* NPAD) {
 int tc_exchange(const TcGemm& g, int G, int W, int N, double* part, int nchunk, cudaStream_t st) {
   int RG, CW, NPAD;
   exchange_tile(N, &RG, &CW, &NPAD);
-  if (RG < 1 || CW < 1 || CW > tc::EpiExchange::kMaxCW || nchunk != G) {
+  if (RG < 1 || CW < 2 || CW > tc::EpiExchange::kMaxCW || nchunk != G) {
     set_error("tc exchange: N=%d not supported", N);
     return AFQMC_EUNSUPPORTED;
   }
@@ -1694,11 +1723,11 @@ int tc_exchange(const TcGemm& g, int G, int W, int N, double* part, int nchunk, 
   CUtensorMap tb;
   AFQ_TRY(make_tmap_3d(&tb, g.B, eb, W, 2L * N, g.k, g.ldb, 2L * N * g.ldb, NPAD, CW));
   tc::EpiExchange e{part, G, W, N, RG, CW, NPAD, nchunk};
-  // K = M is a few k-blocks of L2-resident operands: a 2-deep ring leaves room
-  // for the epilogue's own 128 KB tile buffer
+  // K = M is a few k-blocks of L2-resident operands: three ring stages beside
+  // the epilogue's own 66 KB buffer
   if (g.tf32)
-    return launch_tc_persistent<256, 2, true>(g, e, cdiv(G, RG), cdiv(W, CW), st, &tb);
-  return launch_tc_persistent<256, 2, false>(g, e, cdiv(G, RG), cdiv(W, CW), st, &tb);
+    return launch_tc_persistent<256, 3, true>(g, e, cdiv(G, RG), cdiv(W, CW), st, &tb);
+  return launch_tc_persistent<256, 3, false>(g, e, cdiv(G, RG), cdiv(W, CW), st, &tb);
 }
 
 }  // namespace afq
