@@ -121,7 +121,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   b->oz = oz && !mixed;
   b->oz_ov = oz && (!mixed || p.ndet > 0);
   b->oz_qr = oz && !f32lu && N <= 32;
-  b->oz_exch = b->oz && p.ndet == 0 && N <= 32;
+  b->oz_exch = b->oz && N <= 32;
   b->oz_bp = oz && p.bp_steps > 0;
   OzOperand denA, denB;
   int den_cw = 0, den_nz = 0;
@@ -253,7 +253,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       take(b->ozB, M, 64, 64, M);
       if (p.ndet == 0) take(b->ozF, G, 64, 64, N * M);
     }
-    if (b->oz_exch) {
+    if (b->oz_exch && p.ndet == 0) {
       const int rpt = oz_exchange_vectors((int)N) * (int)N;
       take(b->ozX, G * N, rpt, (rpt + 7) / 8 * 8, M);
     }
@@ -277,9 +277,15 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
     if (b->oz) {
       need(per * wc, wc * (M + 2 * N));
       need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
-      if (p.ndet == 0) need(oz_bytes(2 * wc, 128, 128, N * M), 2 * wc);
+      // several determinants: with the slices of one determinant's vectors
+      need(oz_bytes(2 * wc, 128, 128, N * M) + (p.ndet > 0 ? oz_bytes(G, 64, 64, N * M) : 0), 2 * wc + G);
     }
-    if (b->oz_exch) need(oz_bytes(2 * N * wc, 2 * (int)N * oz_exchange_walkers((int)N), 64, M), 2 * N * wc);
+    if (b->oz_exch) {
+      const int rpt = oz_exchange_vectors((int)N) * (int)N;
+      need(oz_bytes(2 * N * wc, 2 * (int)N * oz_exchange_walkers((int)N), 64, M) +
+               (p.ndet > 0 ? oz_bytes(G * N, rpt, (rpt + 7) / 8 * 8, M) : 0),
+           2 * N * wc + G * N);
+    }
   }
   if (b->oz_bp) {
     oz_need = std::max(oz_need, (size_t)den_nz * (denA.batch_stride + denB.batch_stride));
@@ -581,13 +587,13 @@ void desc_half2(afqmc_state* s, double* phi_out, void* phi_lo_out, TcJobDesc* d)
 // C rows = (src rows) B^T, B sliced at set-up, rw rows of k values per walker
 // (contiguous), sliced a chunk of walkers at a time; 2^alpha_log2 the factor.
 static int oz_rows_gemm(afqmc_state* s, const double* src, int rw, int k, const OzOperand& B, double* C,
-                        int n, int alpha_log2, const double* mask) {
+                        int n, int alpha_log2, const double* mask, size_t at = 0, size_t at_exp = 0) {
   const Bufs& b = s->b;
   for (int w0 = 0; w0 < s->p.nwalkers; w0 += b.oz_wc) {
     const int nw = std::min(b.oz_wc, s->p.nwalkers - w0);
     OzGemm g;
-    g.A.data = b.oz_mem;
-    g.A.exps = b.oz_exp;
+    g.A.data = b.oz_mem + at;
+    g.A.exps = b.oz_exp + at_exp;
     g.A.nkb = B.nkb;
     AFQ_TRY(oz_slice_rows(src + (size_t)w0 * rw * k, (long)nw * rw, k, k, g.A, s->st));
     g.m = nw * rw;
@@ -742,7 +748,8 @@ static int oz_taylor(afqmc_state* s) {
 }
 
 // part[w][c] = the exchange sums of the live state's Theta (Eq. localenergy3).
-static int oz_energy_exchange(afqmc_state* s) {
+static int oz_exchange_parts(afqmc_state* s, const OzOperand& A, const double* theta, double* part, size_t at,
+                             size_t at_exp) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   OzExchange x;
@@ -750,20 +757,58 @@ static int oz_energy_exchange(afqmc_state* s) {
   x.G = p.nchol;
   x.nup = s->nup;
   x.nchunk = b.nchunk;
-  x.A = b.ozX;
-  x.B.data = b.oz_mem;
-  x.B.exps = b.oz_exp;
+  x.A = A;
+  x.B.data = b.oz_mem + at;
+  x.B.exps = b.oz_exp + at_exp;
   x.B.RT = 64;
   x.B.rows_per_tile = 2 * p.N * oz_exchange_walkers(p.N);
-  x.B.nkb = b.ozX.nkb;
+  x.B.nkb = A.nkb;
   x.err = b.status;
   for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
     x.W = std::min(b.oz_wc, p.nwalkers - w0);
-    AFQ_TRY(oz_slice_rows(b.thetaT + (size_t)w0 * 2 * p.N * p.M, 2L * p.N * x.W, p.M, p.M, x.B, s->st));
-    x.part = b.part + (size_t)w0 * b.nchunk * 2;
+    AFQ_TRY(oz_slice_rows(theta + (size_t)w0 * 2 * p.N * p.M, 2L * p.N * x.W, p.M, p.M, x.B, s->st));
+    x.part = part + (size_t)w0 * b.nchunk * 2;
     AFQ_TRY(oz_exchange(x, s->st));
   }
   return AFQMC_OK;
+}
+
+static int oz_energy_exchange(afqmc_state* s) {
+  return oz_exchange_parts(s, s->b.ozX, s->b.thetaT, s->b.part, 0, 0);
+}
+
+// The exchange sums and the traces of one (determinant, spin): its half-rotated
+// vectors are sliced into the scratch area for each evaluation (24 bytes per
+// value moved, against 16 per value, determinant and spin held for good).
+int oz_md_exchange(afqmc_state* s, int ds) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  const long gn = (long)p.nchol * p.N;
+  OzOperand A;
+  A.rows_per_tile = oz_exchange_vectors(p.N) * p.N;
+  A.RT = (A.rows_per_tile + 7) / 8 * 8;
+  A.nkb = (p.M + 15) / 16;
+  A.data = b.oz_mem;
+  A.exps = b.oz_exp;
+  AFQ_TRY(oz_slice_rows(b.md_Lh + (size_t)ds * gn * p.M, gn, p.M, p.M, A, s->st));
+  return oz_exchange_parts(s, A, b.md_theta + (size_t)ds * p.nwalkers * 2 * p.N * p.M,
+                           b.md_part + (size_t)ds * p.nwalkers * b.nchunk * 2,
+                           oz_bytes(gn, A.rows_per_tile, A.RT, p.M), gn);
+}
+
+int oz_md_traces(afqmc_state* s, int ds) {
+  const afqmc_params& p = s->p;
+  const Bufs& b = s->b;
+  const long k = (long)p.N * p.M;
+  OzOperand F;
+  F.RT = F.rows_per_tile = 64;
+  F.nkb = (int)((k + 15) / 16);
+  F.data = b.oz_mem;
+  F.exps = b.oz_exp;
+  AFQ_TRY(oz_slice_rows(b.md_Lh + (size_t)ds * p.nchol * k, p.nchol, (int)k, k, F, s->st));
+  return oz_rows_gemm(s, b.md_theta + (size_t)ds * p.nwalkers * 2 * k, 2, (int)k, F,
+                      b.md_C + (size_t)ds * 2 * p.nwalkers * p.nchol, p.nchol, 0, nullptr,
+                      oz_bytes(p.nchol, 64, 64, k), p.nchol);
 }
 
 int force_bias_gemm(afqmc_state* s) {
@@ -1499,7 +1544,7 @@ static int setup_device(afqmc_state* s, const double* h1, const double* L, const
   if (b.oz) {
     AFQ_TRY(oz_slice_rows(b.Bh, M, M, M, b.ozB, st));
     if (!md) AFQ_TRY(oz_slice_rows(b.Lh, G, N * M, (long)N * M, b.ozF, st));
-    if (b.oz_exch) AFQ_TRY(oz_slice_rows(b.Lh, (long)G * N, M, M, b.ozX, st));
+    if (b.oz_exch && !md) AFQ_TRY(oz_slice_rows(b.Lh, (long)G * N, M, M, b.ozX, st));
   }
   if (b.mixed) {
     // BF16 / TF32 copies of the contraction operands (zero-padded pitches)

@@ -868,12 +868,18 @@ int md_overlap_update(afqmc_state* s, bool into_ld) {
   return AFQMC_OK;
 }
 
-// Per (d, s): C_ds[(w, c)][g] = Tr(Lh_dsg Theta_ds) for every walker, one
-// batched contraction over K = N M.
+// Per (d, s): C_ds[(w, c)][g] = Tr(Lh_dsg Theta_ds) for every walker: sliced
+// products, or one batched contraction over K = N M.  Four determinants, 1024
+// walkers of M = 100, N = 10, float64: a step 16.0 to 2.7 ms with these and an
+// energy 201 to 11.2 ms with the exchange (the float64 kernels per (d, s)).
 static int md_traces(afqmc_state* s) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   const int W = p.nwalkers, N = p.N, M = p.M, G = p.nchol, nd = p.ndet;
+  if (b.oz) {
+    for (int ds = 0; ds < 2 * nd; ++ds) AFQ_TRY(oz_md_traces(s, ds));
+    return AFQMC_OK;
+  }
   GemmF64 g;
   g.m = 2 * W;
   g.n = G;
@@ -951,6 +957,8 @@ int md_local_energies(afqmc_state* s) {
       g.tf32 = b.lo_kind == LO_TF32;
       g.err = b.status;
       AFQ_TRY(tc_exchange(g, G, W, N, part, b.nchunk, s->st));
+    } else if (b.oz_exch) {
+      AFQ_TRY(oz_md_exchange(s, ds));
     } else {
       ExchArgs ex{W, M, N, G, b.gc, b.nchunk, b.md_Lh + (long)ds * G * NM,
                   b.md_theta + (long)ds * W * 2 * NM, part, b.wt};

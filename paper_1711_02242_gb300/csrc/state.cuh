@@ -186,6 +186,8 @@ int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, co
                   int unit, int zero_singular, void* th_lo);
 int oz_trial_overlaps(afqmc_state* s, double* dst, int n);
 int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st);
+int oz_md_exchange(afqmc_state* s, int ds);
+int oz_md_traces(afqmc_state* s, int ds);
 int oz_density_products(afqmc_state* s, const double* thA, const double* thB, int* w0, int* nz, double* D);
 }  // namespace afq
 
