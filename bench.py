@@ -70,6 +70,9 @@ def peaks():
 # clock x 2 FLOP x 2070 MHz = 1.259 TFLOP/s (a DFMA probe kernel measured
 # 1.198 TFLOP/s on this machine, i.e. 2 FMA/clk/SM at the clock under load).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
+# The float64 path's contractions as exact integer products on the tensor cores
+# take 36 BF16 products each: their peak is 1/36 of the BF16 rate.
+SLICE_PRODUCTS = 36
 # FP32 likewise: 152 SMs x 128 FMA per clock x 2 FLOP x 2070 MHz = 80.5 TFLOP/s.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
@@ -79,38 +82,30 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 # runs that kernel; a figure whose source has changed since, or that belongs
 # to another kernel at this precision, is reported as null.
 GEMM_KERNEL = "__device__ __forceinline__ void gemm_body("
+THETA_F32 = "k_theta_rows_f32(OverlapArgs a)"
 TRAFFIC = {
     "theta": [# k_theta_rows_f32 on the float64 S^-1 (the bf16 default path)
-              {"bytes": (66.846720 + 26.307840) * 1e6, "precisions": ("bf16",),
-               "function": "__global__ void __launch_bounds__(TH_T) k_theta_rows_f32(OverlapArgs a)",
-               "sha": "95b521175a189697f17637210e88c7be80b91f899d89ffb387d05b3e718d9736"},
-              # k_theta_rows (float64 Theta of the -f64theta mixed paths): its own
-              # text is unchanged since this capture (DRAM 64.5 + 30.3 MB per launch)
-              {"bytes": (64.544512 + 30.260480) * 1e6, "precisions": ("bf16-f64theta",),
-               "function": "__global__ void __launch_bounds__(TH_T) k_theta_rows(OverlapArgs a)",
-               "sha": "d7ee3083bab22e614e7aa9c51aff2886d255680c62a6454f637a089a17969ae7"}],
-    # k_overlap<double> and k_mgs (float64, the bf16 default path), pinned to
-    # their own text (captures in profiles/overlap_inverse_m300_bf16.md and
-    # profiles/mgs_m300_bf16.md)
-    "overlap": {"bytes": (8.244992 + 0.0) * 1e6, "precisions": ("bf16",),
+              {"bytes": (66.867200 + 28.362496) * 1e6, "precisions": ("bf16",),
+               "function": THETA_F32,
+               "sha": "b9678066890a60a49ae6cda95e5f206a7535efb51318e664cb17366a0f2b1780"}],
+    # k_overlap<double> (float64, the bf16 default path), pinned to its own text
+    # (capture in profiles/overlap_inverse_m300_bf16.md)
+    "overlap": {"bytes": (8.247296 + 0.0) * 1e6, "precisions": ("bf16",),
                 "function": "__global__ void __launch_bounds__(OV_T) k_overlap(OverlapArgs a)",
-                "sha": "5905df615412e8d5881361e99808acd80656d2a0414eef96dd142e0f6e82e0bc"},
-    "qr": {"bytes": (61.483264 + 34.291200) * 1e6, "precisions": ("bf16",),
-           "function": "__global__ void __launch_bounds__(256) k_mgs(MgsArgs a)",
-           "sha": "4e08b7f77fcd6fee61eeb48c18f47fe8220b9dacfe0af8c3a22f28d76f55f22f"},
+                "sha": "506632bed33ba14c3bb70329e83d9b312f5a2da65241c0a02b13fbcf61b8498e"},
     # the tensor-core kernels: pinned to the kernel's text (and its epilogue's),
     # unchanged since these captures (only their host launchers changed)
-    "taylor": {"bytes": (218.472704 + 19.613440) * 1e6, "precisions": ("bf16", "bf16-f32lu", "bf16-f64theta"),
-               "function": "__global__ void __launch_bounds__(kSeriesThreads, 1)",
-               "sha": "e47766a88bc3d88a860c2cac6a6bb846bd1349fc46fd391771607944c29a3feb"},
+    "taylor": {"bytes": (218.408448 + 19.279872) * 1e6, "precisions": ("bf16", "bf16-f32lu", "bf16-f64theta"),
+               "function": "    k_taylor_series(const __grid_constant__ CUtensorMap tmV",
+               "sha": "0b32a127c5dad0e232a2ad36bb4bb65d9e6ddade8ebd8efd61344dd5a7be1bed"},
     # the V contraction in the form the set-up chooses at M=300 (BN = 256 on
     # 128-row tiles, CTA pairs)
     "v_assembly": {"bytes": (183.425536 + 146.092288) * 1e6, "precisions": ("bf16", "bf16-f32lu", "bf16-f64theta"),
                    "function": [GEMM_KERNEL, "struct EpiVT {"],
                    "sha": "b34ba031fd47ee240c8c32d916b8c0c9eaed95718863e675b9597e6ba39dd815"},
-    "energy": {"bytes": (42.981120 + 0.896512) * 1e6, "precisions": ("bf16", "bf16-f32lu", "bf16-f64theta"),
+    "energy": {"bytes": (42.990336 + 0.588544) * 1e6, "precisions": ("bf16", "bf16-f32lu", "bf16-f64theta"),
                "function": [GEMM_KERNEL, "struct EpiExchange {"],
-               "sha": "a34fa5e7f96ce4c61663388be5935414dd273ca610993974abba5e0154a4a6d8"},
+               "sha": "d5da964dca321ecc31a7eae16de7c775e5f11203f8ded3d592aff68cddb90f59"},
 }
 
 
@@ -278,6 +273,19 @@ KERNEL_OF_PHASE = {"overlap": ("k_overlap", "alu", "walker_f64.cu"),
                               "gemm_tc.cu")}
 
 
+def sliced(w, precision):
+    """Whether the float64 path's contractions run on the tensor cores (the
+    library's rule; smaller systems use the float64 kernels)."""
+    return precision == "fp64" and (w.M >= 40 or (w.M >= 28 and w.nwalkers >= 512))
+
+
+# phases of the float64 path that are sliced products
+SLICED_PHASES = {"taylor": "k_oz_gemm (a Taylor term) and the slicing kernels",
+                 "v_assembly": "k_oz_gemm (V) and the slicing of the fields",
+                 "theta": "k_oz_gemm (Theta) and the slicing kernels",
+                 "energy": "k_oz_gemm (force bias, exchange) + k_eloc"}
+
+
 def source_sha(fname):
     import hashlib
 
@@ -369,6 +377,10 @@ def rooflines(w, phases, precision, K):
             peak, unit, src_peak = FP32_PEAK_TFLOPS, "TFLOP/s", (
                 "derived: 152 SMs x 128 FP32 FMA/clk x 2 x 2070 MHz")
             bound = "alu"
+        elif sliced(w, precision) and ph in SLICED_PHASES:
+            kname, src, bound = SLICED_PHASES[ph], "oz.cu", "tensor"
+            peak, unit = pk["bf16_tflops_sustained"] / SLICE_PRODUCTS, "TFLOP/s"
+            src_peak = f"{pk_kind} bf16 sustained / {SLICE_PRODUCTS} (products of slices)"
         elif bound == "alu" or precision == "fp64":
             peak, unit, src_peak = FP64_PEAK_TFLOPS, "TFLOP/s", (
                 "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2070 MHz")
@@ -386,6 +398,10 @@ def rooflines(w, phases, precision, K):
                     "peak_source": src_peak, "ms_per_launch": ms_launch,
                     "launches_per_step": v["count"] / K,
                     "share_of_step": v["ms"] / sum(x["ms"] for x in phases.values())})
+        if ph == "qr" and kname == "k_mgs" and w.N <= 32 and (precision != "fp64" and w.M >= 40
+                                                              or sliced(w, precision)):
+            out[-1]["note"] = ("from the Gram matrix: two sliced products on the tensor cores and "
+                               "k_gram_factor; k_mgs sweeps the walkers left over")
     out.sort(key=lambda d: -d["share_of_step"])
     return out
 
@@ -579,8 +595,9 @@ def fp64_compare(w, p, h1, L, C, dev, stream, steps):
     torch.cuda.empty_cache()
     return {"value": w.nwalkers * steps / (ms * 1e-3), "unit": "walker-steps/s",
             "ms_per_step": ms / steps, "steps": steps,
-            "note": "the same workload on the FP64 path (every step in float64/complex128), "
-                    "same GPU, kernel by kernel"}
+            "note": "the same workload on the FP64 path (every result to float64 accuracy: "
+                    "contractions as exact products of integer slices on the tensor cores, the "
+                    "rest in float64), same GPU, kernel by kernel"}
 
 
 class OracleSampler:
@@ -941,7 +958,7 @@ def run_serve(args):
     ws_total = sum(r.nwalkers * r.nsteps for r in done)
     lat = latency_stats(done)
     # FP64 one at a time: the first requests timed alone, the rest extrapolated
-    # by algorithmic FLOPs (the FP64 path is bound by the FP64 pipe)
+    # by algorithmic FLOPs
     n_fp = min(3, len(reqs))
     fl = lambda r: flops_per_walker_step(workloads.Workload(  # noqa: E731
         "r", M=r.trial.shape[0], N=r.trial.shape[1], nchol=r.L.shape[0], nwalkers=r.nwalkers,

@@ -12,7 +12,9 @@
 // symmetric) and the vectors found so far, so one iteration streams
 // 8 dim (k + 1) bytes after k vectors: an HBM-bound matrix-vector product.
 //
-// One launch per iteration.  A block owns 32 consecutive indices mu, one
+// Matrices of at most kAllMaxCols columns (and kAllMaxVectors vectors) are
+// decomposed in one cooperative launch (k_mcd_all, below).  The others take one
+// launch per iteration: a block owns 32 consecutive indices mu, one
 // per lane, and its 8 warps split the earlier vectors g: warp w reads
 // L[g][mu0 .. mu0+31] (256 contiguous bytes of the caller's output) for
 // g = w, w+8, ... against the pivot's components L[g][nu0], staged in shared

@@ -10,10 +10,11 @@
 //   t_g = sum_d w_d sum_s Tr(Lh_dsg Theta_ds)                    (force bias),
 //   E_loc = H0 + sum_d w_d [sum_s Tr(hh_ds Theta_ds)
 //           + 1/2 sum_g (sum_s Tr(Lh_dsg Theta_ds))^2 - 1/2 sum_s sum_g Tr(T_dsg T_dsg)],
-//   T_dsg = Lh_dsg Theta_ds (the float64 exchange kernel, once per (d, s)).
+//   T_dsg = Lh_dsg Theta_ds (the exchange contraction, once per (d, s)).
+// The float64 contractions (overlaps, Theta, traces, exchange) are sliced products
+// on the tensor cores where the state takes that route (b.oz_ov, b.oz).
 // On the mixed path the traces and the exchange of each (d, s) run on the
-// tensor cores from BF16/TF32 copies of Lh_ds and Theta_ds (written by the
-// overlap kernel); overlaps, weights and the combinations stay float64.
+// tensor cores from BF16/TF32 copies of Lh_ds and Theta_ds; overlaps, weights and the combinations stay float64.
 // All in the run's orthonormal basis, whose first N vectors are the leading
 // spin-up determinant's orbitals.
 //
