@@ -1437,8 +1437,8 @@ def _case_ci(a):
 
 def run_peaks(args):
     """Dense float64 and float32 matrix-multiply throughput through PyTorch
-    (cuBLAS; TF32 off for float32), the counterpart of the driver's BF16
-    measurement for the FP64 and FP32 pipes: best of 5 after warm-up and 4 s
+    (cuBLAS; TF32 off for float32), the counterpart of the measured BF16
+    rate for the FP64 and FP32 pipes: best of 5 after warm-up and 4 s
     back to back, n^3 with n = 8192 (float64: 16384 for the sustained loop's
     operands would not change the rate; 8192 keeps it short)."""
     import torch

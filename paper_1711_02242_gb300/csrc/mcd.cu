@@ -12,7 +12,7 @@
 // symmetric) and the vectors found so far, so one iteration streams
 // 8 dim (k + 1) bytes after k vectors: an HBM-bound matrix-vector product.
 //
-// Matrices of at most kAllMaxCols columns (and kAllMaxVectors vectors) are
+// Matrices of at most kAllMaxCols columns per SM (and kAllMaxVectors vectors) are
 // decomposed in one cooperative launch (k_mcd_all, below).  The others take one
 // launch per iteration: a block owns 32 consecutive indices mu, one
 // per lane, and its 8 warps split the earlier vectors g: warp w reads
