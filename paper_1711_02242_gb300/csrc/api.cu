@@ -1712,7 +1712,13 @@ static int init_state(const afqmc_params* p, const double* h1, const double* L,
   s->st = static_cast<cudaStream_t>(stream);
   s->ws = static_cast<char*>(d_workspace);
   s->ws_bytes = ws_bytes;
-  plan(s->p, &s->b, s->ws);
+  // (the caller's parameters and these lay out the same workspace: a plan that
+  // told them apart would write past its end)
+  if (plan(s->p, &s->b, s->ws) > ws_bytes) {
+    set_error("workspace layout of two spin blocks differs from its size");
+    delete s;
+    return AFQMC_ENOSPC;
+  }
   s->sdt = std::sqrt(p->dt);
   int r = setup_device(s, h1, L, trial, trial_dn, md_coef, md_up, md_dn);
   if (r != AFQMC_OK) {

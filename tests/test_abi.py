@@ -120,3 +120,12 @@ def test_mcd_pairs_workspace_size_without_gpu(built):
     assert n.value < npair * 8 * (1800 + 1) + 17 * npair + (4 << 20)
     for M, mv in ((0, 10), (2049, 10), (10, 0)):
         assert lib.afqmc_mcd_pairs_workspace_size(M, mv, ctypes.byref(n)) == -1
+
+
+@pytest.mark.parametrize("M,N,Ndn,G,W", [(39, 3, 2, 50, 8), (40, 3, 2, 50, 8), (28, 4, 4, 90, 512),
+                                         (150, 13, 10, 700, 150), (130, 17, 16, 400, 64)])
+def test_spin_block_workspace_on_every_route(built, M, N, Ndn, G, W):
+    """The state lays its buffers out for N + Ndn columns: the size it was given for
+    (N, Ndn) has to be that layout's on every route by size."""
+    split = built.afqmc_workspace_size(built.default_params(M, N, G, W, Ndn=Ndn))
+    assert split == built.afqmc_workspace_size(built.default_params(M, N + Ndn, G, W))
