@@ -271,7 +271,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       if (bytes > oz_need) oz_need = bytes;
       if (exps > oz_exps) oz_exps = exps;
     };
-    need(per_th * wc, wc * (M + nds * 2 * N));
+    need(per_th * wc, wc * (M + nds * 2 * N + N));
     need(per_gram * wc, 2 * N * wc);
     if (b->oz_ov) need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
     if (b->oz) {
@@ -634,8 +634,11 @@ static int oz_rotate(afqmc_state* s, const double* phi, const double* m, OzTheta
     t.A.exps = b.oz_exp;
     t.B.data = b.oz_mem + (size_t)t.nw * t.A.batch_stride;
     t.B.exps = b.oz_exp + (size_t)t.nw * t.A.batch_exp_stride;
-    AFQ_TRY(oz_slice_cols(phi + (size_t)w0 * 2 * p.N * p.M, t.nw, p.N, p.M, t.A, st));
-    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, t.B, st));
+    int* orb = t.B.exps + (size_t)t.nds * t.nw * t.B.batch_exp_stride;
+    const double* from = phi + (size_t)w0 * 2 * p.N * p.M;
+    AFQ_TRY(oz_orbital_exps(from, t.nw, p.N, p.M, orb, st));
+    AFQ_TRY(oz_slice_cols(from, t.nw, p.N, p.M, orb, t.A, st));
+    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, orb, t.B, st));
     AFQ_TRY(oz_theta(t, st));
   }
   return AFQMC_OK;

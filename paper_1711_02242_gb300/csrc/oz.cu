@@ -27,6 +27,15 @@ __device__ __forceinline__ int row_exp(uint32_t hi, bool any) {
   return (ef > 0 ? ef : 1) - 1022;
 }
 
+// The same for one element scaled by 2^-s: a row's exponent is the largest.
+__device__ __forceinline__ int elem_exp(double x, int s) {
+  const uint32_t hi = abs_hi(x);
+  const int ef = (int)(hi >> 20);
+  if (ef == 0x7ff) return kOzNanExp;
+  if ((hi | (uint32_t)__double2loint(x)) == 0u) return kOzZeroExp;
+  return (ef > 0 ? ef : 1) - 1022 - s;
+}
+
 // x in units of 2^(e - 56), rounded to nearest (|X| <= 2^56).
 __device__ __forceinline__ long long fixed57(double x, int e) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -254,31 +263,45 @@ __global__ void __launch_bounds__(256) k_oz_slice_term(const double* t, int N, i
   }
 }
 
-// Rows p = [Re Phi_p | Im Phi_p] of walker blockIdx.y: K runs over the 2 N
-// orbital planes, a lane owns a row, so both the reads along p and the writes
-// (eight rows of a chunk: 128 contiguous bytes per slice) are contiguous.
-__global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N2, int M, OzOperand o) {
-  __shared__ uint32_t m_sh[8][32], any_sh[8][32];
-  const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, w = blockIdx.y;
+// Exponent of each orbital's largest element, a warp per orbital (w, i).  Rows
+// that run over a walker's orbitals are sliced with every orbital divided by
+// 2^exps[w N + i] and the other operand's row i multiplied by it: orbitals of
+// very different norm would otherwise share the largest one's exponent and lose
+// the bits that the inverse's small and large rows need.  Bound by memory.
+__global__ void __launch_bounds__(256) k_oz_orbital_exps(const double* phi, long n, int N, int M, int* exps) {
+  pdl_begin();
+  const long t = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (t >= n) return;
+  const long w = t / N, i = t - w * N;
+  const double* re = phi + (w * 2 * N + i) * M;
+  const double* im = re + (long)N * M;
+  int e = kOzZeroExp;
+  for (int p = threadIdx.x & 31; p < M; p += 32) e = max(e, max(elem_exp(re[p], 0), elem_exp(im[p], 0)));
+  e = __reduce_max_sync(0xffffffffu, e);
+  // (no scale for an orbital of zeros, or one that is not finite)
+  if ((threadIdx.x & 31) == 0) exps[t] = e == kOzZeroExp || e == kOzNanExp ? 0 : e;
+}
+
+// Rows p = [Re Phi_p | Im Phi_p] of walker blockIdx.y, orbitals scaled by their
+// exponents: K runs over the 2 N orbital planes, a lane owns a row, so both the
+// reads along p and the writes (eight rows of a chunk: 128 contiguous bytes per
+// slice) are contiguous.
+__global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N, int M, const int* orb,
+                                                       OzOperand o) {
+  __shared__ int e_sh[8][32], s_sh[64];
+  const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, w = blockIdx.y, N2 = 2 * N;
   const int p = blockIdx.x * 32 + lane;
   const double* src = phi + (long)w * N2 * M + p;
-  uint32_t m = 0, any = 0;
+  if (threadIdx.x < N) s_sh[threadIdx.x] = orb[(long)w * N + threadIdx.x];
+  __syncthreads();
+  int e = kOzZeroExp;
   if (p < M)
-    for (int k = wk; k < N2; k += 8) {
-      const double x = src[(long)k * M];
-      m = max(m, abs_hi(x));
-      any |= abs_hi(x) | (uint32_t)__double2loint(x);
-    }
-  m_sh[wk][lane] = m;
-  any_sh[wk][lane] = any;
+    for (int k = wk; k < N2; k += 8) e = max(e, elem_exp(src[(long)k * M], s_sh[k < N ? k : k - N]));
+  e_sh[wk][lane] = e;
   __syncthreads();
   if (p >= M) return;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    m = max(m, m_sh[q][lane]);
-    any |= any_sh[q][lane];
-  }
-  const int e = row_exp(m, any != 0);
+  for (int q = 0; q < 8; ++q) e = max(e, e_sh[q][lane]);
   const bool fine = e != kOzNanExp && e != kOzZeroExp;
   if (wk == 0) o.exps[(long)w * o.batch_exp_stride + p] = e;
   const int rt = p / o.rows_per_tile, r = p - rt * o.rows_per_tile;
@@ -289,7 +312,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N2
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * c + i;
-      u[i] = kDigitBias + (fine && k < N2 ? fixed57(src[(long)k * M], e) : 0ll);
+      u[i] = kDigitBias + (fine && k < N2 ? fixed57(src[(long)k * M], e + s_sh[k < N ? k : k - N]) : 0ll);
     }
     put_chunk(base + chunk_off(o.RT, r, c), o.RT * 32, u);
   }
@@ -351,26 +374,26 @@ __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, c
 }
 
 // The inverse of (ds, w) = (blockIdx.y, blockIdx.x) as operand rows (re, j) =
-// [Re S^-1_j | -Im S^-1_j] and (im, j) = [Im S^-1_j | Re S^-1_j], S^-1_j column j.
+// [Re S^-1_j | -Im S^-1_j] and (im, j) = [Im S^-1_j | Re S^-1_j], S^-1_j column j
+// with row i scaled by 2^orb[w N + i] (k_oz_orbital_exps).
 __global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, int W, int w0, int N,
-                                                          OzOperand o) {
-  __shared__ int e_sh[64];
+                                                          const int* orb, OzOperand o) {
+  __shared__ int e_sh[64], s_sh[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w = blockIdx.x, ds = blockIdx.y;
   const long batch = (long)ds * gridDim.x + w;
   const double2* S = sinv + ((long)ds * W + w0 + w) * N * N;
   int* ex = o.exps + batch * o.batch_exp_stride;
+  if (threadIdx.x < N) s_sh[threadIdx.x] = -orb[(long)w * N + threadIdx.x];
+  __syncthreads();
   for (int j = warp; j < N; j += 8) {
-    uint32_t m = 0, any = 0;
+    int e = kOzZeroExp;
     for (int i = lane; i < N; i += 32) {
       const double2 x = S[i * N + j];
-      m = max(m, max(abs_hi(x.x), abs_hi(x.y)));
-      any |= abs_hi(x.x) | (uint32_t)__double2loint(x.x) | abs_hi(x.y) | (uint32_t)__double2loint(x.y);
+      e = max(e, max(elem_exp(x.x, s_sh[i]), elem_exp(x.y, s_sh[i])));
     }
-    m = __reduce_max_sync(0xffffffffu, m);
-    any = __reduce_or_sync(0xffffffffu, any);
+    e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) {
-      const int e = row_exp(m, any != 0);
       e_sh[j] = e;
       ex[j] = ex[N + j] = e;
     }
@@ -390,9 +413,9 @@ __global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, i
       const int k = 8 * c + i;
       u[i] = kDigitBias;
       if (fine && k < 2 * N) {
-        const int part = k >= N ? 1 : 0;
-        const double2 x = S[(k - part * N) * N + j];
-        const long long f = fixed57(im == part ? x.x : x.y, e);
+        const int part = k >= N ? 1 : 0, q = k - part * N;
+        const double2 x = S[q * N + j];
+        const long long f = fixed57(im == part ? x.x : x.y, e + s_sh[q]);
         u[i] += (im == 0 && part == 1) ? -f : f;
       }
     }
@@ -1081,8 +1104,14 @@ int oz_taylor_term(const OzTerm& t, cudaStream_t st) {
   return launch_oz<64>(g, e, st);
 }
 
-int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, 2 * N, M, o);
+int oz_orbital_exps(const double* phi, int W, int N, int M, int* exps, cudaStream_t st) {
+  const long n = (long)W * N;
+  AFQ_LAUNCH_PDL(k_oz_orbital_exps, (unsigned)((n + 7) / 8), 256, 0, st, phi, n, N, M, exps);
+  return AFQMC_OK;
+}
+
+int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const OzOperand& o, cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, N, M, orb, o);
   return AFQMC_OK;
 }
 
@@ -1092,9 +1121,9 @@ int oz_slice_densities(const double* phi, const double* thA, const double* thB, 
   return AFQMC_OK;
 }
 
-int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,
-                     cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, o);
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* orb,
+                     const OzOperand& o, cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, orb, o);
   return AFQMC_OK;
 }
 

@@ -101,8 +101,12 @@ struct OzTheta {
   int lo_kind = 0, Mp = 0;
   int* err = nullptr;
 };
-// operand rows p = [Re Phi_p | Im Phi_p] (2 N values) of W walkers
-int oz_slice_cols(const double* phi, int W, int N, int M, const OzOperand& o, cudaStream_t st);
+// The exponents exps[w N + i] of W walkers' orbitals, by whose powers of two the
+// rows over the orbitals are scaled (down in Phi, up in the inverse: exactly), so
+// that the result does not depend on the orbitals' norms.
+int oz_orbital_exps(const double* phi, int W, int N, int M, int* exps, cudaStream_t st);
+// operand rows p = [Re Phi_p | Im Phi_p] (2 N values, N <= 64) of W walkers
+int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const OzOperand& o, cudaStream_t st);
 // Operands of sum_k conj(Phi_k[p]) Th_k[q] over the rows k = (w, i) of nz
 // groups of cw walkers from walker w0 on (the last may be short), a batch entry
 // each, K = 2 N cw: A rows p = [Re Phi_p | Im Phi_p] and M + p =
@@ -112,8 +116,8 @@ int oz_slice_densities(const double* phi, const double* thA, const double* thB, 
                        int nz, int cw, const OzOperand& A, const OzOperand& B, cudaStream_t st);
 // operand rows (re, j) = [Re S^-1_j | -Im S^-1_j], (im, j) = [Im | Re] of the
 // inverses sinv[ds W + w0 + w], batch ds nw + w
-int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const OzOperand& o,
-                     cudaStream_t st);
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* orb,
+                     const OzOperand& o, cudaStream_t st);
 int oz_theta(const OzTheta& t, cudaStream_t st);
 
 // gram[w][r][c] = sum_k of rows r and c of each walker's 2 N rows (A and B the

@@ -183,6 +183,53 @@ def test_gram_schmidt_routes(pkg, M, N, Ndn):
     run.close()
 
 
+@pytest.mark.parametrize("M,N,Ndn,nd,precision", [
+    (48, 12, 0, 0, 0),
+    (60, 17, 15, 0, 0),   # two spin blocks
+    (70, 6, 0, 3, 0),     # three determinants
+    (130, 25, 0, 0, 2),   # the mixed path's Gram-Schmidt
+    (130, 25, 0, 2, 2),   # and its overlaps of several determinants
+])
+def test_orbitals_of_unequal_norm(pkg, M, N, Ndn, nd, precision):
+    """Multiplying a walker's orbitals by powers of two (2^-30 .. 2^30, different for
+    each) scales every product of a step by powers of two and changes nothing else:
+    the same local energies, and after a step and Gram-Schmidt the same walkers,
+    weights and overlaps, to the rounding of the overlaps' logarithms (|log| up to
+    20 N: 1e-13); Q orthonormal to rounding."""
+    G, W = 60, 6
+    h1, L, trial = inputs(M, N, G, Ndn)
+    up, dn = trial if Ndn else (trial, None)
+    both = np.hstack([up, dn]) if Ndn else up
+    Nt = N + Ndn
+    rng = np.random.default_rng(5 * M)
+    if nd:
+        dets = np.array([up] + [np.linalg.qr(up + 0.05 * rng.standard_normal((M, N)))[0] for _ in range(1, nd)])
+        trial = (np.array([1.0] + [0.3] * (nd - 1), complex), dets, dets)
+    phi = np.repeat(both[None], W, 0).astype(complex)
+    phi += 0.02 * (rng.standard_normal(phi.shape) + 1j * rng.standard_normal(phi.shape))
+    scale = 2.0 ** rng.integers(-30, 31, (W, 1, Nt))
+    scale[:, :, 0], scale[:, :, N - 1] = 2.0 ** -30, 2.0 ** 30
+    out = []
+    for ph in (phi, phi * scale):
+        p = pkg.default_params(M, N, G, W, qr_period=1, energy_period=0, Ndn=Ndn, ndet=nd, precision=precision)
+        run = pkg.AfqmcRun(h1, L, trial, p)
+        run.set_walkers(ph, np.ones(W))
+        el = run.local_energies()
+        run.propagate(1)
+        got, wt, lo = run.get_walkers()
+        assert run.info().status == 0 and np.all(np.abs(wt) > 0)
+        for a, b in ((0, N), (N, Nt)):
+            S = np.einsum("wpi,wpj->wij", got[:, :, a:b].conj(), got[:, :, a:b])
+            assert b == a or np.abs(S - np.eye(b - a)).max() < 1e-14
+        out.append((el, got, wt, lo))
+        run.close()
+    (el, got, wt, lo), (el2, got2, wt2, lo2) = out
+    assert np.max(np.abs(el2 - el) / np.abs(el)) < 1e-13
+    assert np.max(np.abs(got2 - got)) < 1e-13
+    assert np.max(np.abs(wt2 - wt) / np.abs(wt)) < 1e-11
+    assert np.max(np.abs(lo2 - lo)) < 1e-11
+
+
 @pytest.mark.parametrize("M,N,G,W,m,qr", [
     (40, 5, 57, 41, 3, 2),    # the fewest orbitals; a group of 40 walkers and one of a single walker
     (65, 13, 70, 15, 2, 0),   # two row tiles of A, the last group full
