@@ -289,7 +289,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   }
   if (b->oz_bp) {
     oz_need = std::max(oz_need, (size_t)den_nz * (denA.batch_stride + denB.batch_stride));
-    oz_exps = std::max(oz_exps, (size_t)den_nz * 4 * M);
+    oz_exps = std::max(oz_exps, (size_t)den_nz * (4 * M + den_cw * N));
   }
   // scratch: the set-up and the step never run at the same time
   const size_t scratch_at = (a.off + 255) & ~size_t(255);
@@ -709,7 +709,8 @@ int oz_density_products(afqmc_state* s, const double* thA, const double* thB, in
   g.B.data = b.oz_mem + (size_t)*nz * g.A.batch_stride;
   g.B.exps = b.oz_exp + (size_t)*nz * g.A.batch_exp_stride;
   g.err = b.status;
-  AFQ_TRY(oz_slice_densities(b.bp_phi, thA, thB, p.nwalkers, p.N, p.M, *w0, *nz, cw, g.A, g.B, s->st));
+  int* orb = g.B.exps + (size_t)*nz * g.B.batch_exp_stride;
+  AFQ_TRY(oz_slice_densities(b.bp_phi, thA, thB, p.nwalkers, p.N, p.M, *w0, *nz, cw, orb, g.A, g.B, s->st));
   AFQ_TRY(oz_gemm_store(g, s->st));
   *w0 += *nz * cw;
   return AFQMC_OK;

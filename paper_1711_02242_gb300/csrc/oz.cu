@@ -320,34 +320,33 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N,
 
 // Rows of the density sums (oz_slice_densities): group blockIdx.y of cw
 // walkers, whose K values (w, c, i) of a column p lie M apart; blockIdx.z: Phi
-// as it is, Phi times i, thA, thB.  A lane owns a row as in k_oz_slice_cols.
+// as it is, Phi times i, thA, thB.  A lane owns a row as in k_oz_slice_cols, and
+// the orbitals of Phi are scaled down and Theta's up by 2^orb[(walker - w0) N + i]
+// as there: a row runs over walkers whose orbitals' norms may differ widely.
 __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, const double* thA,
                                                             const double* thB, int W, int N, int M, int w0,
-                                                            int cw, OzOperand A, OzOperand B) {
-  __shared__ uint32_t m_sh[8][32], any_sh[8][32];
+                                                            int cw, const int* orb, OzOperand A, OzOperand B) {
+  __shared__ int e_sh[8][32], s_sh[kOzSegK / 2];  // K = 2 N cw of at most one segment
   const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, z = blockIdx.y, which = blockIdx.z;
   const int p = blockIdx.x * 32 + lane, first = w0 + z * cw, N2 = 2 * N;
   const int nk = (W - first < cw ? W - first : cw) * N2;
   const OzOperand& o = which < 2 ? A : B;
   const double* src = (which < 2 ? phi : which == 2 ? thA : thB) + (long)first * N2 * M + p;
-  uint32_t m = 0, any = 0;
+  for (int t = threadIdx.x; t < nk / 2; t += 256) {
+    const int s = orb[(long)z * cw * N + t];
+    s_sh[t] = which < 2 ? s : -s;
+  }
+  __syncthreads();
+  auto shift = [&](int k) { return s_sh[k / N2 * N + k % N]; };
+  int e = kOzZeroExp;
   if (p < M)
 #pragma unroll 4
-    for (int k = wk; k < nk; k += 8) {
-      const double x = src[(long)k * M];
-      m = max(m, abs_hi(x));
-      any |= abs_hi(x) | (uint32_t)__double2loint(x);
-    }
-  m_sh[wk][lane] = m;
-  any_sh[wk][lane] = any;
+    for (int k = wk; k < nk; k += 8) e = max(e, elem_exp(src[(long)k * M], shift(k)));
+  e_sh[wk][lane] = e;
   __syncthreads();
   if (p >= M) return;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    m = max(m, m_sh[q][lane]);
-    any |= any_sh[q][lane];
-  }
-  const int e = row_exp(m, any != 0);
+  for (int q = 0; q < 8; ++q) e = max(e, e_sh[q][lane]);
   const bool fine = e != kOzNanExp && e != kOzZeroExp;
   const int row = (which & 1) * M + p, rt = row / o.rows_per_tile, r = row - rt * o.rows_per_tile;
   if (wk == 0) o.exps[(long)z * o.batch_exp_stride + row] = e;
@@ -361,10 +360,10 @@ __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, c
       if (fine && k < nk) {
         if (which == 1) {  // (re, im) <- (-im, re)
           const bool re = k % N2 < N;
-          v = fixed57(src[(long)(re ? k + N : k - N) * M], e);
+          v = fixed57(src[(long)(re ? k + N : k - N) * M], e + shift(k));
           if (re) v = -v;
         } else {
-          v = fixed57(src[(long)k * M], e);
+          v = fixed57(src[(long)k * M], e + shift(k));
         }
       }
       u[i] = kDigitBias + v;
@@ -1116,8 +1115,10 @@ int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const 
 }
 
 int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
-                       int nz, int cw, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, A, B);
+                       int nz, int cw, int* orb, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
+  const int n = W - w0 < nz * cw ? W - w0 : nz * cw;
+  AFQ_TRY(oz_orbital_exps(phi + (long)w0 * 2 * N * M, n, N, M, orb, st));
+  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, orb, A, B);
   return AFQMC_OK;
 }
 

@@ -111,9 +111,10 @@ int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const 
 // groups of cw walkers from walker w0 on (the last may be short), a batch entry
 // each, K = 2 N cw: A rows p = [Re Phi_p | Im Phi_p] and M + p =
 // [-Im Phi_p | Re Phi_p] per walker (sums with [Re Th | Im Th]: the real and the
-// imaginary part), B rows q of thA and M + q of thB.
+// imaginary part), B rows q of thA and M + q of thB, orbitals scaled as above
+// (orb: room for the exponents of nz cw walkers).
 int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
-                       int nz, int cw, const OzOperand& A, const OzOperand& B, cudaStream_t st);
+                       int nz, int cw, int* orb, const OzOperand& A, const OzOperand& B, cudaStream_t st);
 // operand rows (re, j) = [Re S^-1_j | -Im S^-1_j], (im, j) = [Im | Re] of the
 // inverses sinv[ds W + w0 + w], batch ds nw + w
 int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* orb,
