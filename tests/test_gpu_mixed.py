@@ -60,9 +60,7 @@ def test_trial_energy_mixed_vs_fp64(pkg, prec, tol):
 def test_one_step_mixed_vs_fp64(pkg, prec, tol_phi, tol_e, nwalkers):
     """One full step of the 12-orbital workload on identical Philox fields;
     200 walkers put field rows in both halves of a 256-row V tile and in a
-    ragged last tile.  With an even number of 256-row V tiles (200, 400
-    walkers) the V contraction runs on CTA pairs sharing the Cholesky tile by
-    multicast, with an odd number (32, 520) on single CTAs."""
+    ragged last tile; even (200, 400 walkers) and odd numbers of 256-row tiles."""
     w = workloads.config("c0")
     r = runs(pkg, w, [0, prec], nwalkers=nwalkers, energy_period=1)
     for x in r.values():
