@@ -175,6 +175,10 @@ __device__ __forceinline__ void gemm_body(const JobTable<Epi, GROUPED>& tab, int
           tma_load_2d(a + S::A_BYTES, v.tmB, &full[s], kb * BK, n0);
       }
     }
+    // given up: no copy may still be in flight when the CTA's memory is released
+    if (*(volatile int*)abort_flag)
+      for (int n = it > STAGES ? it - STAGES : 0; n < it; ++n)
+        mbar_wait(&full[n % STAGES], (n / STAGES) & 1, tab.at(0).err, 15);
   } else if (warp == 1 && lane == 0) {
     constexpr uint32_t idesc = instr_desc(TF32 ? 2u : 1u, (uint32_t)BN);
     int it = 0, j = 0;

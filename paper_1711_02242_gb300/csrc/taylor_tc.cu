@@ -181,6 +181,12 @@ __global__ void __launch_bounds__(kSeriesThreads<TWO>, TWO ? 2 : 1)
         }
     }
     if (stop) *abort_flag = 1;
+    // given up: no copy may still be in flight when the CTA's memory is released
+    if (*abort_flag) {
+      if (j > 0) mbar_wait(bfull, (j - 1) & 1, err, 37);
+      for (int n = it > a.stages ? it - a.stages : 0; n < it; ++n)
+        mbar_wait(&full[n % a.stages], (n / a.stages) & 1, err, 38);
+    }
   } else if (warp == 1 && lane == 0) {
     // MMA thread
     const uint32_t idesc = instr_desc(TF32 ? 2u : 1u, (uint32_t)a.nb);
