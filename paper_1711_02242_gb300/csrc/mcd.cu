@@ -386,12 +386,11 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
 
 constexpr int kAllMaxCols = 64, kAllThreads = 8 * kAllMaxCols;
 constexpr int kAllMaxVectors = 4096;
-constexpr uint32_t kAllPolls = 1u << 20;  // bound of a wait for the other blocks (under a second)
 
 __global__ void __launch_bounds__(kAllThreads, 1)
     k_mcd_all(const double* __restrict__ V, int dim, int cols, double* __restrict__ d, double* L,
               int32_t* __restrict__ pivots, double delta, double tau, int max_vectors, int cached,
-              McdSlot* slots, int* abort_flag, McdState* st) {
+              long long wait_cycles, McdSlot* slots, int* abort_flag, McdState* st) {
   extern __shared__ __align__(16) double all_sm[];
   double* a_sm = all_sm;                  // L[g][piv], g < k
   double* Ls = all_sm + max_vectors;      // [cached][cols]
@@ -505,12 +504,17 @@ __global__ void __launch_bounds__(kAllThreads, 1)
       bool lost = false;
       for (int q = tid; q < nb; q += 32 * rw) {
         const McdSlot* o = mine + q;
-        uint32_t n = 0;
-        while (ld_acquire(&o->seq) != (uint32_t)k + 1u)
-          if (++n > kAllPolls || ((n & 1023u) == 0u && *(volatile int*)abort_flag)) {
+        // every 256th failed poll looks at the clock and at the others' flag
+        long long t0 = 0;
+        for (uint32_t n = 0; ld_acquire(&o->seq) != (uint32_t)k + 1u; ++n) {
+          if (n & 255u) continue;
+          const long long t = clock64();
+          if (n == 0u) t0 = t;
+          if (t - t0 > wait_cycles || (n > 0u && *(volatile int*)abort_flag)) {
             lost = true;
             break;
           }
+        }
         if (lost) break;
         const long long ov = __ldcg(&o->key);
         const double ol = __ldcg(&o->l);
@@ -563,6 +567,13 @@ struct McdLayout {
   size_t state, part, spart, sticket, d, apiv, total;
 };
 
+// Bound of a wait for the other blocks (two seconds at 2 GHz), and the SMs the
+// blocks may count on (0: the device's).
+struct McdOptions {
+  long long wait_cycles = 4000000000ll;
+  int sms = 0;
+};
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 McdLayout mcd_layout(int64_t dim, int32_t max_vectors) {
@@ -607,11 +618,61 @@ int mcd_result(const McdState& hs, int32_t* nvec, double* residual, const char* 
   return AFQMC_OK;
 }
 
+// One launch for the whole decomposition where a block per SM can own the
+// columns (*launched): the slots of the exchange take the place of the tickets'
+// partials.  Where its blocks cannot all run at once (a context with fewer SMs or
+// less shared memory than the device), nothing is launched and a launch per vector
+// does the same.
+int launch_mcd_all(const double* d_V, int64_t dim64, double* d, double* d_L, int32_t* d_piv, double delta, double tau,
+                   int max_vectors, char* base, const McdLayout& lay, const McdOptions& opt, cudaStream_t s,
+                   bool* launched) {
+  int dev = 0, sms = 0, coop = 0;
+  AFQ_CUDA(cudaGetDevice(&dev));
+  AFQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  AFQ_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  const int64_t per = (dim64 + sms - 1) / sms;
+  if (!coop || per > kAllMaxCols || max_vectors > kAllMaxVectors) return AFQMC_OK;
+  int dim = (int)dim64;
+  int cols = per <= 8 ? 8 : (int)(per + 3) / 4 * 4;  // whole warps of (column, group) pairs
+  constexpr int kSmemAll = 216 * 1024;
+  const size_t row = sizeof(double) * (size_t)cols, av = sizeof(double) * (size_t)max_vectors;
+  int cached = (int)((kSmemAll - av) / row);
+  if (cached > max_vectors) cached = max_vectors;
+  const size_t smem = av + (size_t)cached * row;
+  static std::atomic<unsigned long long> attr{0};
+  AFQ_TRY(smem_attr_once(k_mcd_all, kSmemAll, attr));
+  const unsigned nb = (unsigned)((dim + cols - 1) / cols);
+  int fit = 0;
+  AFQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_mcd_all, 8 * cols, smem));
+  if ((int64_t)fit * (opt.sms > 0 ? opt.sms : sms) < (int64_t)nb) return AFQMC_OK;
+  McdState* st = reinterpret_cast<McdState*>(base + lay.state);
+  McdSlot* slots = reinterpret_cast<McdSlot*>(base + lay.part);
+  int* abort_flag = reinterpret_cast<int*>(base + lay.sticket);
+  // k_mcd_init's partials were here: no iteration is published yet
+  AFQ_CUDA(cudaMemsetAsync(slots, 0, 2 * sizeof(McdSlot) * (size_t)nb, s));
+  long long wait_cycles = opt.wait_cycles;
+  void* args[] = {&d_V,         &dim,    &cols,    &d,     &d_L,        &d_piv, &delta,
+                  &tau,         &max_vectors, &cached, &wait_cycles, &slots, &abort_flag, &st};
+  const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_mcd_all), dim3(nb),
+                                                    dim3((unsigned)(8 * cols)), args, smem, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    (void)cudaGetLastError();  // refused, not failed
+    return AFQMC_OK;
+  }
+  if (e != cudaSuccess) {
+    set_error("launch k_mcd_all: %s", cudaGetErrorString(e));
+    return AFQMC_ECUDA;
+  }
+  ++g_launches;
+  *launched = true;
+  return AFQMC_OK;
+}
+
 // The decomposition of the dim x dim matrix V into the rows of L (pitch
 // dim), with the workspace laid out by mcd_layout(dim, max_vectors) at base.
 int run_mcd(int64_t dim, const double* d_V, double delta, int32_t max_vectors, double* d_L,
             int32_t* d_piv, int32_t* nvec, double* residual, char* base, const McdLayout& lay,
-            cudaStream_t s, const char* who) {
+            cudaStream_t s, const char* who, const McdOptions& opt = {}) {
   McdState* st = reinterpret_cast<McdState*>(base + lay.state);
   McdTree tree{reinterpret_cast<McdPartial*>(base + lay.part),
                reinterpret_cast<McdPartial*>(base + lay.spart),
@@ -637,45 +698,8 @@ int run_mcd(int64_t dim, const double* d_V, double delta, int32_t max_vectors, d
   AFQ_CUDA(cudaMemsetAsync(base + lay.sticket, 0, lay.d - lay.sticket, s));
   AFQ_LAUNCH(k_mcd_init, (unsigned)grid0, kThreads, 0, s, d_V, dim, d, delta, max_vectors, tree,
              st);
-  // One launch for the whole decomposition where a block per SM can own the
-  // columns: the slots of the exchange take the place of the tickets' partials.
-  {
-    int dev = 0, sms = 0, coop = 0;
-    AFQ_CUDA(cudaGetDevice(&dev));
-    AFQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    AFQ_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-    int cols = (int)((dim + sms - 1) / sms);
-    cols = cols <= 8 ? 8 : (cols + 3) / 4 * 4;  // whole warps of (column, group) pairs
-    if (coop && cols <= kAllMaxCols && max_vectors <= kAllMaxVectors) {
-      constexpr int kSmemAll = 216 * 1024;
-      const size_t row = sizeof(double) * (size_t)cols, av = sizeof(double) * (size_t)max_vectors;
-      int cached = (int)((kSmemAll - av) / row);
-      if (cached > max_vectors) cached = max_vectors;
-      const size_t smem = av + (size_t)cached * row;
-      static std::atomic<unsigned long long> attr{0};
-      AFQ_TRY(smem_attr_once(k_mcd_all, kSmemAll, attr));
-      const unsigned nb = (unsigned)((dim + cols - 1) / cols);
-      McdSlot* slots = reinterpret_cast<McdSlot*>(base + lay.part);
-      int* abort_flag = reinterpret_cast<int*>(base + lay.sticket);
-      // k_mcd_init's partials were here: no iteration is published yet
-      AFQ_CUDA(cudaMemsetAsync(slots, 0, 2 * sizeof(McdSlot) * (size_t)nb, s));
-      const double* va = d_V;
-      int da = (int)dim;
-      void* args[] = {&va, &da, &cols, &d, &d_L, &d_piv, const_cast<double*>(&delta),
-                      const_cast<double*>(&tau), &max_vectors, &cached, &slots, &abort_flag, &st};
-      const cudaError_t e = cudaLaunchCooperativeKernel(
-          reinterpret_cast<const void*>(k_mcd_all), dim3(nb), dim3((unsigned)(8 * cols)), args, smem, s);
-      ++g_launches;
-      if (e != cudaSuccess) {
-        set_error("launch k_mcd_all: %s", cudaGetErrorString(e));
-        return AFQMC_ECUDA;
-      }
-      McdState hs{};
-      AFQ_CUDA(cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s));
-      AFQ_CUDA(cudaStreamSynchronize(s));
-      return mcd_result(hs, nvec, residual, who);
-    }
-  }
+  bool whole = false;
+  AFQ_TRY(launch_mcd_all(d_V, dim, d, d_L, d_piv, delta, tau, max_vectors, base, lay, opt, s, &whole));
   // Launch iterations in chunks and read the state between chunks; launches
   // after convergence return at once.  A launch after `launched` others
   // finds k <= launched earlier vectors, which sizes its shared memory.
@@ -684,7 +708,7 @@ int run_mcd(int64_t dim, const double* d_V, double delta, int32_t max_vectors, d
   for (;;) {
     AFQ_CUDA(cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s));
     AFQ_CUDA(cudaStreamSynchronize(s));
-    if (hs.done || launched >= max_vectors) break;
+    if (hs.done || whole || launched >= max_vectors) break;
     int chunk = launched < 64 ? 16 : 64;
     if (chunk > max_vectors - launched) chunk = max_vectors - launched;
     for (int c = 0; c < chunk; ++c) {
@@ -768,6 +792,16 @@ extern "C" AFQMC_API int afqmc_modified_cholesky(int64_t dim, const double* d_V,
                  static_cast<char*>(d_work), lay, static_cast<cudaStream_t>(stream),
                  "afqmc_modified_cholesky");
 }
+
+// The decomposition with a wait bound and an SM count of the caller's (tests).
+namespace afq {
+int mcd_bounded(int64_t dim, const double* d_V, double delta, int32_t max_vectors, double* d_L, int32_t* d_piv,
+                int32_t* nvec, double* residual, void* d_work, long long wait_cycles, int sms, cudaStream_t s) {
+  const McdOptions opt{wait_cycles, sms};
+  return run_mcd(dim, d_V, delta, max_vectors, d_L, d_piv, nvec, residual, static_cast<char*>(d_work),
+                 mcd_layout(dim, max_vectors), s, "mcd_bounded", opt);
+}
+}  // namespace afq
 
 extern "C" AFQMC_API int afqmc_mcd_pairs_workspace_size(int32_t M, int32_t max_vectors,
                                                         size_t* bytes) {

@@ -1,7 +1,10 @@
-// The sliced contractions by themselves, for test_gpu_sliced_products.py: linked
-// with the library's object files.  Every pointer is a device pointer; ws holds
-// the slices and row exponents, 256-byte aligned.
+// Parts of the library by themselves, for the tests: linked with its object files.
 #include "../paper_1711_02242_gb300/csrc/oz.cuh"
+
+namespace afq {
+int mcd_bounded(int64_t dim, const double* d_V, double delta, int32_t max_vectors, double* d_L, int32_t* d_piv,
+                int32_t* nvec, double* residual, void* d_work, long long wait_cycles, int sms, cudaStream_t s);
+}
 
 namespace {
 struct Carve {
@@ -25,6 +28,8 @@ struct Carve {
 };
 }  // namespace
 
+// Sliced contractions: every pointer is a device pointer; ws holds the slices and
+// row exponents, 256-byte aligned.
 // D[z][2 M][2 M] of groups of cw walkers (see oz_slice_densities).
 extern "C" __attribute__((visibility("default"))) int sp_densities(
     const double* phi, const double* thA, const double* thB, int W, int N, int M, int cw, double* D, char* ws,
@@ -48,4 +53,14 @@ extern "C" __attribute__((visibility("default"))) int sp_densities(
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   AFQ_TRY(oz_slice_densities(phi, thA, thB, W, N, M, 0, nz, cw, orb, g.A, g.B, st));
   return oz_gemm_store(g, st);
+}
+
+// The modified Cholesky decomposition whose waits end after wait_cycles, on a
+// device of `sms` SMs (0: as it is).
+extern "C" __attribute__((visibility("default"))) int in_mcd(long long dim, const double* V, double delta,
+                                                              int max_vectors, double* L, int* piv, int* nvec,
+                                                              double* residual, void* work, long long wait_cycles,
+                                                              int sms, void* stream) {
+  return afq::mcd_bounded(dim, V, delta, max_vectors, L, piv, nvec, residual, work, wait_cycles, sms,
+                          static_cast<cudaStream_t>(stream));
 }

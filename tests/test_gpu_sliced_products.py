@@ -1,33 +1,11 @@
 """The float64 contractions as products of integer slices (oz.cuh) by
-themselves, through a small entry linked with the library's object files."""
+themselves (internal.cu)."""
 import ctypes
-import glob
-import os
-import subprocess
 
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
-
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-
-
-@pytest.fixture(scope="module")
-def env(tmp_path_factory):
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_1711_02242_gb300 import build as b
-
-    b.build()
-    torch.zeros(1, device="cuda")
-    so = str(tmp_path_factory.mktemp("sliced") / "sliced_products.so")
-    subprocess.run([b._nvcc(), *b.ARCH, *b.FLAGS, "-I", os.path.join(ROOT, "include"), "-shared", "-cudart", "shared",
-                    "-o", so, os.path.join(ROOT, "tests", "sliced_products.cu"),
-                    *sorted(glob.glob(os.path.join(b.BUILD, "*.o")))], check=True, capture_output=True)
-    return torch, ctypes.CDLL(so)
-
 
 def call(torch, fn, *args):
     """fn(*args, ws, ws_bytes, status, stream); device arrays by their pointers."""
@@ -41,12 +19,12 @@ def call(torch, fn, *args):
 
 
 @pytest.mark.parametrize("M,N,W,cw", [(40, 5, 41, 40), (65, 13, 15, 15), (33, 64, 4, 3), (30, 1, 250, 200)])
-def test_densities_of_unequal_norms(env, M, N, W, cw):
+def test_densities_of_unequal_norms(internal, M, N, W, cw):
     """sum_k conj(Phi_k[p]) Th_k[q] over the walkers and orbitals k of a group: with
     Phi_k times and Th_k divided by a power of two of its own the same bits, and
     within the slices' bound, 2.8 K 2^-56 of the row maxima with those powers taken
     out (maxima below 8 here), of NumPy's sum (K 2^-53)."""
-    torch, lib = env
+    torch, lib = internal
     rng = np.random.default_rng(M)
     phi, thA, thB = rng.standard_normal((3, W, 2, N, M))
     scale = 2.0 ** rng.integers(-60, 61, (W, 1, N, 1))
