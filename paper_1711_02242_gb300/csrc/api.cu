@@ -239,6 +239,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
     };
     const size_t nds = p.ndet > 0 ? 2 * (size_t)p.ndet : 1;
     if (b->oz_ov) take(b->ozV, nds * N, 64, 64, M);
+    b->phi_exp = a.take<int>(W * 2 * N);
     if (p.ndet > 0) {
       b->Sx = a.take<double>(W * 2 * N * nds * N);
       b->md_Sinv = a.take<double>(nds * W * 2 * N * N);
@@ -271,9 +272,9 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
       if (bytes > oz_need) oz_need = bytes;
       if (exps > oz_exps) oz_exps = exps;
     };
-    need(per_th * wc, wc * (M + nds * 2 * N + N));
-    need(per_gram * wc, 2 * N * wc);
-    if (b->oz_ov) need(oz_bytes(2 * N * wc, 128, 128, M), 2 * N * wc);
+    need(per_th * wc, wc * (M + nds * 2 * N + 2 * N));
+    need(per_gram * wc, 0);
+    if (b->oz_ov) need(oz_bytes(2 * N * wc, 128, 128, M), 0);
     if (b->oz) {
       need(per * wc, wc * (M + 2 * N));
       need(oz_bytes(2 * wc, 128, 128, G), 2 * wc);
@@ -289,7 +290,7 @@ static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
   }
   if (b->oz_bp) {
     oz_need = std::max(oz_need, (size_t)den_nz * (denA.batch_stride + denB.batch_stride));
-    oz_exps = std::max(oz_exps, (size_t)den_nz * (4 * M + den_cw * N));
+    oz_exps = std::max(oz_exps, (size_t)den_nz * (4 * M + den_cw * 2 * N));
   }
   // scratch: the set-up and the step never run at the same time
   const size_t scratch_at = (a.off + 255) & ~size_t(255);
@@ -474,7 +475,7 @@ int overlap_update(afqmc_state* s, bool into_ld, bool timed) {
     prof_begin(s, AFQMC_PH_THETA);
   }
   if (b.oz_ov)
-    AFQ_TRY(oz_theta_rows(s, b.Sinv, 1, b.thetaT, ov.logdet, 2, ov.unit_trial, 0, nullptr));
+    AFQ_TRY(oz_theta_rows(s, b.Sinv, 1, b.thetaT, ov.logdet, 2, ov.unit_trial, 0, nullptr, s->spin2));
   else
     AFQ_TRY(launch_theta(ov, s->st));
   if (timed) prof_end(s);
@@ -586,14 +587,17 @@ void desc_half2(afqmc_state* s, double* phi_out, void* phi_lo_out, TcJobDesc* d)
 
 // C rows = (src rows) B^T, B sliced at set-up, rw rows of k values per walker
 // (contiguous), sliced a chunk of walkers at a time; 2^alpha_log2 the factor.
+// at, at_exp: the slices' place in the scratch area; exps: all rows' exponents,
+// kept, instead.
 static int oz_rows_gemm(afqmc_state* s, const double* src, int rw, int k, const OzOperand& B, double* C,
-                        int n, int alpha_log2, const double* mask, size_t at = 0, size_t at_exp = 0) {
+                        int n, int alpha_log2, const double* mask, size_t at = 0, size_t at_exp = 0,
+                        int* exps = nullptr) {
   const Bufs& b = s->b;
   for (int w0 = 0; w0 < s->p.nwalkers; w0 += b.oz_wc) {
     const int nw = std::min(b.oz_wc, s->p.nwalkers - w0);
     OzGemm g;
     g.A.data = b.oz_mem + at;
-    g.A.exps = b.oz_exp + at_exp;
+    g.A.exps = exps ? exps + (size_t)w0 * rw : b.oz_exp + at_exp;
     g.A.nkb = B.nkb;
     AFQ_TRY(oz_slice_rows(src + (size_t)w0 * rw * k, (long)nw * rw, k, k, g.A, s->st));
     g.m = nw * rw;
@@ -611,12 +615,14 @@ static int oz_rows_gemm(afqmc_state* s, const double* src, int rw, int k, const 
 }
 
 int oz_trial_overlaps(afqmc_state* s, double* dst, int n) {
-  return oz_rows_gemm(s, s->b.phiT, 2 * s->p.N, s->p.M, s->b.ozV, dst, n, 0, nullptr);
+  return oz_rows_gemm(s, s->b.phiT, 2 * s->p.N, s->p.M, s->b.ozV, dst, n, 0, nullptr, 0, 0, s->b.phi_exp);
 }
 
 // t.theta rows = the orbitals phi times the matrices m[ds][w] (N x N, t.nds per
-// walker) for the walkers that t's conditions let through.
-static int oz_rotate(afqmc_state* s, const double* phi, const double* m, OzTheta t, cudaStream_t st) {
+// walker) for the walkers that t's conditions let through; exps: the exponents
+// of phi's planes where its rows have been sliced.
+static int oz_rotate(afqmc_state* s, const double* phi, const int* exps, const double* m, OzTheta t,
+                     cudaStream_t st) {
   const afqmc_params& p = s->p;
   const Bufs& b = s->b;
   oz_theta_operands(p.M, p.N, &t.A, &t.B);
@@ -634,18 +640,22 @@ static int oz_rotate(afqmc_state* s, const double* phi, const double* m, OzTheta
     t.A.exps = b.oz_exp;
     t.B.data = b.oz_mem + (size_t)t.nw * t.A.batch_stride;
     t.B.exps = b.oz_exp + (size_t)t.nw * t.A.batch_exp_stride;
-    int* orb = t.B.exps + (size_t)t.nds * t.nw * t.B.batch_exp_stride;
     const double* from = phi + (size_t)w0 * 2 * p.N * p.M;
-    AFQ_TRY(oz_orbital_exps(from, t.nw, p.N, p.M, orb, st));
-    AFQ_TRY(oz_slice_cols(from, t.nw, p.N, p.M, orb, t.A, st));
-    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, orb, t.B, st));
+    const int* planes = exps ? exps + (size_t)w0 * 2 * p.N : nullptr;
+    if (!planes) {
+      int* own = t.B.exps + (size_t)t.nds * t.nw * t.B.batch_exp_stride;
+      AFQ_TRY(oz_row_exps(from, 2L * p.N * t.nw, p.M, own, st));
+      planes = own;
+    }
+    AFQ_TRY(oz_slice_cols(from, t.nw, p.N, p.M, planes, t.A, st));
+    AFQ_TRY(oz_slice_inverse(reinterpret_cast<const double2*>(m), p.nwalkers, w0, t.nw, t.nds, p.N, planes, t.B, st));
     AFQ_TRY(oz_theta(t, st));
   }
   return AFQMC_OK;
 }
 
 int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
-                  int unit, int zero_singular, void* th_lo) {
+                  int unit, int zero_singular, void* th_lo, bool sliced) {
   OzTheta t;
   t.nds = nds;
   t.theta = theta;
@@ -654,7 +664,7 @@ int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, co
   t.unit = unit;
   t.zero_singular = zero_singular;
   t.th_lo = th_lo;
-  return oz_rotate(s, s->b.phiT, sinv, t, s->st);
+  return oz_rotate(s, s->b.phiT, sliced ? s->b.phi_exp : nullptr, sinv, t, s->st);
 }
 
 // Gram-Schmidt of the walkers on stream st: Phi <- Phi R^-1 with R from the
@@ -671,11 +681,11 @@ int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
   rows.rows_per_tile = 2 * N;
   rows.nkb = (M + 15) / 16;
   rows.data = b.oz_mem;
-  rows.exps = b.oz_exp;
   rows.batch_stride = (long)oz_bytes(2 * N, 2 * N, rows.RT, M);
   rows.batch_exp_stride = 2 * N;
   for (int w0 = 0; w0 < p.nwalkers; w0 += b.oz_wc) {
     const int nw = std::min(b.oz_wc, p.nwalkers - w0);
+    rows.exps = b.phi_exp + (size_t)w0 * 2 * N;
     AFQ_TRY(oz_slice_rows(m.phiT + w0 * row, 2L * N * nw, M, M, rows, st));
     AFQ_TRY(oz_gram(rows, nw, N, b.gram + (size_t)w0 * 4 * N * N, b.status, st));
   }
@@ -685,7 +695,7 @@ int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st) {
   t.theta = m.phiT;
   t.flag = b.qr_done;
   t.th_lo = m.phi_lo;
-  AFQ_TRY(oz_rotate(s, m.phiT, b.Rinv, t, st));
+  AFQ_TRY(oz_rotate(s, m.phiT, b.phi_exp, b.Rinv, t, st));
   m.done = b.qr_done;
   return launch_mgs(m, st);
 }
@@ -709,8 +719,8 @@ int oz_density_products(afqmc_state* s, const double* thA, const double* thB, in
   g.B.data = b.oz_mem + (size_t)*nz * g.A.batch_stride;
   g.B.exps = b.oz_exp + (size_t)*nz * g.A.batch_exp_stride;
   g.err = b.status;
-  int* orb = g.B.exps + (size_t)*nz * g.B.batch_exp_stride;
-  AFQ_TRY(oz_slice_densities(b.bp_phi, thA, thB, p.nwalkers, p.N, p.M, *w0, *nz, cw, orb, g.A, g.B, s->st));
+  int* planes = g.B.exps + (size_t)*nz * g.B.batch_exp_stride;
+  AFQ_TRY(oz_slice_densities(b.bp_phi, thA, thB, p.nwalkers, p.N, p.M, *w0, *nz, cw, planes, g.A, g.B, s->st));
   AFQ_TRY(oz_gemm_store(g, s->st));
   *w0 += *nz * cw;
   return AFQMC_OK;

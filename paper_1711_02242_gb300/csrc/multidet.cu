@@ -801,7 +801,7 @@ static int md_overlaps_tc(afqmc_state* s, int nds, void* th_lo) {
   ov.ldS = n;
   ov.nds = nds;
   AFQ_TRY(launch_overlap(ov, s->st));
-  return oz_theta_rows(s, b.md_Sinv, nds, b.md_theta, b.md_ld, 2 * nds, 0, 1, th_lo);
+  return oz_theta_rows(s, b.md_Sinv, nds, b.md_theta, b.md_ld, 2 * nds, 0, 1, th_lo, true);
 }
 
 static int smw_overlap_update(afqmc_state* s, bool into_ld) {

@@ -263,40 +263,62 @@ __global__ void __launch_bounds__(256) k_oz_slice_term(const double* t, int N, i
   }
 }
 
-// Exponent of each orbital's largest element, a warp per orbital (w, i).  Rows
-// that run over a walker's orbitals are sliced with every orbital divided by
-// 2^exps[w N + i] and the other operand's row i multiplied by it: orbitals of
-// very different norm would otherwise share the largest one's exponent and lose
-// the bits that the inverse's small and large rows need.  Bound by memory.
-__global__ void __launch_bounds__(256) k_oz_orbital_exps(const double* phi, long n, int N, int M, int* exps) {
+// Exponents of n rows of M values (as k_oz_slice_rows leaves them), four rows per
+// warp so that enough loads are in flight.  Bound by memory: 20480 rows of 100
+// 6.5 us (10.3 with a row per warp).
+__global__ void __launch_bounds__(256) k_oz_row_exps(const double* src, long n, int M, int* exps) {
   pdl_begin();
-  const long t = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (t >= n) return;
-  const long w = t / N, i = t - w * N;
-  const double* re = phi + (w * 2 * N + i) * M;
-  const double* im = re + (long)N * M;
-  int e = kOzZeroExp;
-  for (int p = threadIdx.x & 31; p < M; p += 32) e = max(e, max(elem_exp(re[p], 0), elem_exp(im[p], 0)));
-  e = __reduce_max_sync(0xffffffffu, e);
-  // (no scale for an orbital of zeros, or one that is not finite)
-  if ((threadIdx.x & 31) == 0) exps[t] = e == kOzZeroExp || e == kOzNanExp ? 0 : e;
+  const long t0 = 4 * ((long)blockIdx.x * 8 + (threadIdx.x >> 5));
+  const int lane = threadIdx.x & 31;
+  int e[4] = {kOzZeroExp, kOzZeroExp, kOzZeroExp, kOzZeroExp};
+  for (int p = lane; p < M; p += 32) {
+    double x[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) x[r] = t0 + r < n ? src[(t0 + r) * M + p] : 0.0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) e[r] = max(e[r], elem_exp(x[r], 0));
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) e[r] = __reduce_max_sync(0xffffffffu, e[r]);
+  if (lane < 4 && t0 + lane < n) exps[t0 + lane] = lane == 0 ? e[0] : lane == 1 ? e[1] : lane == 2 ? e[2] : e[3];
+}
+
+// Exponent of orbital i of a walker from those of its 2 N planes; none for an
+// orbital of zeros, or one that is not finite.  Rows that run over a walker's
+// orbitals are sliced with every orbital divided by 2^s and the other operand's
+// row i multiplied by it: orbitals of very different norm would otherwise share
+// the largest one's exponent and lose the bits that the inverse's small and large
+// rows need.
+__device__ __forceinline__ int orbital_exp(const int* planes, int N, int i) {
+  const int e = max(planes[i], planes[N + i]);
+  return e == kOzZeroExp || e == kOzNanExp ? 0 : e;
 }
 
 // Rows p = [Re Phi_p | Im Phi_p] of walker blockIdx.y, orbitals scaled by their
 // exponents: K runs over the 2 N orbital planes, a lane owns a row, so both the
 // reads along p and the writes (eight rows of a chunk: 128 contiguous bytes per
-// slice) are contiguous.
-__global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N, int M, const int* orb,
+// slice) are contiguous.  1024 walkers, M = 100, N = 10 23 us; 512, M = 300, N = 25
+// 47 us (20 and 44 with one scale for all orbitals).
+__global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N, int M, const int* planes,
                                                        OzOperand o) {
   __shared__ int e_sh[8][32], s_sh[64];
   const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, w = blockIdx.y, N2 = 2 * N;
   const int p = blockIdx.x * 32 + lane;
   const double* src = phi + (long)w * N2 * M + p;
-  if (threadIdx.x < N) s_sh[threadIdx.x] = orb[(long)w * N + threadIdx.x];
+  // the first values are on their way while the exponents arrive
+  double x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) x[j] = p < M && wk + 8 * j < N2 ? src[(long)(wk + 8 * j) * M] : 0.0;
+  if (threadIdx.x < N) s_sh[threadIdx.x] = orbital_exp(planes + (long)w * N2, N, threadIdx.x);
   __syncthreads();
   int e = kOzZeroExp;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = wk + 8 * j;
+    if (k < N2) e = max(e, elem_exp(x[j], s_sh[k < N ? k : k - N]));
+  }
   if (p < M)
-    for (int k = wk; k < N2; k += 8) e = max(e, elem_exp(src[(long)k * M], s_sh[k < N ? k : k - N]));
+    for (int k = wk + 64; k < N2; k += 8) e = max(e, elem_exp(src[(long)k * M], s_sh[k < N ? k : k - N]));
   e_sh[wk][lane] = e;
   __syncthreads();
   if (p >= M) return;
@@ -321,11 +343,11 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N,
 // Rows of the density sums (oz_slice_densities): group blockIdx.y of cw
 // walkers, whose K values (w, c, i) of a column p lie M apart; blockIdx.z: Phi
 // as it is, Phi times i, thA, thB.  A lane owns a row as in k_oz_slice_cols, and
-// the orbitals of Phi are scaled down and Theta's up by 2^orb[(walker - w0) N + i]
-// as there: a row runs over walkers whose orbitals' norms may differ widely.
+// the orbitals of Phi are scaled down and Theta's up by their exponents as there
+// (planes: of the walkers from w0 on): a row runs over walkers whose orbitals' norms may differ widely.
 __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, const double* thA,
                                                             const double* thB, int W, int N, int M, int w0,
-                                                            int cw, const int* orb, OzOperand A, OzOperand B) {
+                                                            int cw, const int* planes, OzOperand A, OzOperand B) {
   __shared__ int e_sh[8][32], s_sh[kOzSegK / 2];  // K = 2 N cw of at most one segment
   const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, z = blockIdx.y, which = blockIdx.z;
   const int p = blockIdx.x * 32 + lane, first = w0 + z * cw, N2 = 2 * N;
@@ -333,7 +355,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, c
   const OzOperand& o = which < 2 ? A : B;
   const double* src = (which < 2 ? phi : which == 2 ? thA : thB) + (long)first * N2 * M + p;
   for (int t = threadIdx.x; t < nk / 2; t += 256) {
-    const int s = orb[(long)z * cw * N + t];
+    const int s = orbital_exp(planes + ((long)z * cw + t / N) * N2, N, t % N);
     s_sh[t] = which < 2 ? s : -s;
   }
   __syncthreads();
@@ -374,16 +396,16 @@ __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, c
 
 // The inverse of (ds, w) = (blockIdx.y, blockIdx.x) as operand rows (re, j) =
 // [Re S^-1_j | -Im S^-1_j] and (im, j) = [Im S^-1_j | Re S^-1_j], S^-1_j column j
-// with row i scaled by 2^orb[w N + i] (k_oz_orbital_exps).
+// with row i scaled by the exponent of orbital i (planes: of Phi, walker by walker).
 __global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, int W, int w0, int N,
-                                                          const int* orb, OzOperand o) {
+                                                          const int* planes, OzOperand o) {
   __shared__ int e_sh[64], s_sh[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w = blockIdx.x, ds = blockIdx.y;
   const long batch = (long)ds * gridDim.x + w;
   const double2* S = sinv + ((long)ds * W + w0 + w) * N * N;
   int* ex = o.exps + batch * o.batch_exp_stride;
-  if (threadIdx.x < N) s_sh[threadIdx.x] = -orb[(long)w * N + threadIdx.x];
+  if (threadIdx.x < N) s_sh[threadIdx.x] = -orbital_exp(planes + (long)w * 2 * N, N, threadIdx.x);
   __syncthreads();
   for (int j = warp; j < N; j += 8) {
     int e = kOzZeroExp;
@@ -1103,28 +1125,27 @@ int oz_taylor_term(const OzTerm& t, cudaStream_t st) {
   return launch_oz<64>(g, e, st);
 }
 
-int oz_orbital_exps(const double* phi, int W, int N, int M, int* exps, cudaStream_t st) {
-  const long n = (long)W * N;
-  AFQ_LAUNCH_PDL(k_oz_orbital_exps, (unsigned)((n + 7) / 8), 256, 0, st, phi, n, N, M, exps);
+int oz_row_exps(const double* src, long n, int M, int* exps, cudaStream_t st) {
+  AFQ_LAUNCH_PDL(k_oz_row_exps, (unsigned)((n + 31) / 32), 256, 0, st, src, n, M, exps);
   return AFQMC_OK;
 }
 
-int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const OzOperand& o, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, N, M, orb, o);
+int oz_slice_cols(const double* phi, int W, int N, int M, const int* planes, const OzOperand& o, cudaStream_t st) {
+  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, N, M, planes, o);
   return AFQMC_OK;
 }
 
 int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
-                       int nz, int cw, int* orb, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
+                       int nz, int cw, int* planes, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
   const int n = W - w0 < nz * cw ? W - w0 : nz * cw;
-  AFQ_TRY(oz_orbital_exps(phi + (long)w0 * 2 * N * M, n, N, M, orb, st));
-  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, orb, A, B);
+  AFQ_TRY(oz_row_exps(phi + (long)w0 * 2 * N * M, 2L * N * n, M, planes, st));
+  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, planes, A, B);
   return AFQMC_OK;
 }
 
-int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* orb,
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* planes,
                      const OzOperand& o, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, orb, o);
+  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, planes, o);
   return AFQMC_OK;
 }
 

@@ -101,23 +101,24 @@ struct OzTheta {
   int lo_kind = 0, Mp = 0;
   int* err = nullptr;
 };
-// The exponents exps[w N + i] of W walkers' orbitals, by whose powers of two the
-// rows over the orbitals are scaled (down in Phi, up in the inverse: exactly), so
-// that the result does not depend on the orbitals' norms.
-int oz_orbital_exps(const double* phi, int W, int N, int M, int* exps, cudaStream_t st);
+// Row exponents of n rows of M values, as oz_slice_rows gives them.  Those of the
+// planes (w, c, i) of Phi scale the rows over the orbitals by a power of two per
+// orbital (down in Phi, up in the inverse: exactly), so that a result does not
+// depend on the orbitals' norms.
+int oz_row_exps(const double* src, long n, int M, int* exps, cudaStream_t st);
 // operand rows p = [Re Phi_p | Im Phi_p] (2 N values, N <= 64) of W walkers
-int oz_slice_cols(const double* phi, int W, int N, int M, const int* orb, const OzOperand& o, cudaStream_t st);
+int oz_slice_cols(const double* phi, int W, int N, int M, const int* planes, const OzOperand& o, cudaStream_t st);
 // Operands of sum_k conj(Phi_k[p]) Th_k[q] over the rows k = (w, i) of nz
 // groups of cw walkers from walker w0 on (the last may be short), a batch entry
 // each, K = 2 N cw: A rows p = [Re Phi_p | Im Phi_p] and M + p =
 // [-Im Phi_p | Re Phi_p] per walker (sums with [Re Th | Im Th]: the real and the
 // imaginary part), B rows q of thA and M + q of thB, orbitals scaled as above
-// (orb: room for the exponents of nz cw walkers).
+// (planes: room for 2 N exponents of nz cw walkers).
 int oz_slice_densities(const double* phi, const double* thA, const double* thB, int W, int N, int M, int w0,
-                       int nz, int cw, int* orb, const OzOperand& A, const OzOperand& B, cudaStream_t st);
+                       int nz, int cw, int* planes, const OzOperand& A, const OzOperand& B, cudaStream_t st);
 // operand rows (re, j) = [Re S^-1_j | -Im S^-1_j], (im, j) = [Im | Re] of the
 // inverses sinv[ds W + w0 + w], batch ds nw + w
-int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* orb,
+int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* planes,
                      const OzOperand& o, cudaStream_t st);
 int oz_theta(const OzTheta& t, cudaStream_t st);
 

@@ -65,6 +65,7 @@ struct Bufs {
   bool oz = false, oz_exch = false, oz_ov = false, oz_qr = false, oz_bp = false;
   double *gram = nullptr, *Rinv = nullptr;
   int* qr_done = nullptr;
+  int* phi_exp = nullptr;  // exponents of the rows (w, c, i) of Phi, last sliced
   OzOperand ozL, ozF, ozX, ozB, ozV;
   double *Sx = nullptr, *md_Sinv = nullptr;
   char* oz_mem = nullptr;
@@ -181,9 +182,10 @@ int smw_detect(afqmc_state* s, const double* up, const double* dn);
 // Make the state's stream wait for a pending side-stream Gram-Schmidt.
 int join_side(afqmc_state* s);
 // Theta rows of nds inverses per walker on the tensor cores (b.oz_ov; see
-// OzTheta), and S of every determinant (or of two spin blocks) into dst
+// OzTheta; sliced: oz_trial_overlaps has just sliced the same Phi), and S of every
+// determinant (or of two spin blocks) into dst
 int oz_theta_rows(afqmc_state* s, const double* sinv, int nds, double* theta, const double* ld, int ld_w,
-                  int unit, int zero_singular, void* th_lo);
+                  int unit, int zero_singular, void* th_lo, bool sliced);
 int oz_trial_overlaps(afqmc_state* s, double* dst, int n);
 int orthonormalise(afqmc_state* s, MgsArgs m, cudaStream_t st);
 int oz_md_exchange(afqmc_state* s, int ds);

@@ -42,8 +42,8 @@ extern "C" __attribute__((visibility("default"))) int sp_densities(
   g.B.RT = g.B.rows_per_tile = 64;
   if (!c.operand(g.A, 2 * (size_t)M, 2 * (size_t)N * cw, nz) || !c.operand(g.B, 2 * (size_t)M, 2 * (size_t)N * cw, nz))
     return AFQMC_ENOSPC;
-  int* orb = static_cast<int*>(c.take(sizeof(int) * (size_t)nz * cw * N));
-  if (!orb) return AFQMC_ENOSPC;
+  int* planes = static_cast<int*>(c.take(sizeof(int) * (size_t)nz * cw * 2 * N));
+  if (!planes) return AFQMC_ENOSPC;
   g.m = g.n = 2 * M;
   g.batch = nz;
   g.ldc = 2L * M;
@@ -51,7 +51,7 @@ extern "C" __attribute__((visibility("default"))) int sp_densities(
   g.C = D;
   g.err = status;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  AFQ_TRY(oz_slice_densities(phi, thA, thB, W, N, M, 0, nz, cw, orb, g.A, g.B, st));
+  AFQ_TRY(oz_slice_densities(phi, thA, thB, W, N, M, 0, nz, cw, planes, g.A, g.B, st));
   return oz_gemm_store(g, st);
 }
 
