@@ -47,13 +47,41 @@ constexpr size_t kOzScratch = size_t(2) << 30;
 // before still do).
 constexpr size_t kOzWorkspace = size_t(160) << 30;
 
-// Whether the float64 contractions run on the tensor cores (oz.cuh).  Below,
-// a system is bound by latency and the float64 kernels' fewer launches win.
-// Five steps and an energy (5 M vectors), float64 kernels against tensor
-// cores, us: M = 32, N = 4: 1047 / 1243 at 48 walkers, 1469 / 1512 at 256,
-// 4570 / 2918 at 1024; M = 48, N = 6: 2065 / 1433, 4015 / 1845, 14199 / 4514;
-// M = 20, N = 3: 770 / 1152, 828 / 1325, 1935 / 2395.
-static bool oz_pays(int M, int W) { return M >= 40 || (M >= 28 && W >= 512); }
+// Which products run as sliced contractions (oz.cuh).  The lines depend on the
+// system alone, not on the number of walkers, so that a population does the same
+// arithmetic whole or split over states; each lies where the two sides cross for
+// some number of walkers.  Other side's time / sliced:
+//  f64  five steps and an energy (5 M vectors), 32, 128, 300, 512, 1024 walkers:
+//       M = 28, N = 2 0.82 0.80 0.89 1.09 1.46; M = 28, N = 4 0.91 0.91 1.07 1.41
+//       1.84; M = 32, N = 2 0.84 0.85 1.12 1.30 1.58; M = 32, N = 4 0.98 1.00 1.34
+//       1.61 1.91; M = 36, N = 2 0.96 1.18 1.28 2.12 2.16; M = 36, N = 7 1.37 1.71
+//       2.21 3.23 3.61.  (Below, launches bound a step: M = 24, N = 3 0.81 at 32.)
+//  ov   five steps of two determinants, 32, 128, 512 walkers: M = 36, N = 5 0.89
+//       0.89 1.18; M = 64, N = 5 0.93 0.96 1.28; M = 64, N = 12 1.17 1.51 2.28
+//       (five determinants 0.93 1.25 1.51 and 1.37 2.26 2.70).
+//  qr   ten steps with two visits, 32, 301, 1024 walkers (mixed path, where the
+//       sweep hides behind the next step's products): M = 100, N = 4 0.96 0.96
+//       0.97; M = 100, N = 10 1.00 0.99 1.04; M = 100, N = 12 1.03 1.00 1.07;
+//       M = 200, N = 6 1.00 1.00 1.00; M = 200, N = 16 1.06 1.06 1.11; float64:
+//       M = 100, N = 4 0.99, N = 8 1.00, N = 18 1.01; M = 150, N = 25 1.01.
+//  bp   a window of ten steps, 64, 128, 512 walkers: M = 30, N = 2 0.99 1.00 1.10;
+//       M = 30, N = 5 1.03 1.07 1.33; M = 80, N = 8 1.04 1.12 1.32.
+struct Sliced {
+  bool f64 = false;  // every contraction of the float64 path
+  bool ov = false;   // overlaps and Theta that are no gather (see Bufs)
+  bool qr = false;   // Gram-Schmidt from the Gram matrix
+  bool bp = false;   // back-propagated densities
+};
+static Sliced sliced_route(const afqmc_params& p, int N) {
+  const bool mixed = p.precision != AFQMC_FP64;
+  const bool f32lu = p.precision == AFQMC_MIXED_TF32_F32LU || p.precision == AFQMC_MIXED_BF16_F32LU;
+  Sliced r;
+  r.f64 = !mixed && (p.M >= 36 || (p.M >= 28 && (long)p.M * p.M * N >= 2500));
+  r.ov = mixed ? p.ndet > 0 && p.M >= 36 : r.f64;
+  r.qr = !f32lu && N <= 32 && (long)p.M * N * N >= 10000;
+  r.bp = p.bp_steps > 0 && p.M >= 28;
+  return r;
+}
 
 // V of a walker as row tiles of equal height, and the term's columns.
 static void oz_taylor_operands(size_t M, size_t N, size_t Mp, OzOperand* V, OzOperand* T) {
@@ -97,32 +125,29 @@ static void oz_density_operands(size_t M, size_t N, size_t W, OzOperand* A, OzOp
   *nz = (int)std::min(all, fit);
 }
 
-static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz);
+static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, const Sliced& route);
 
 size_t plan(const afqmc_params& p, Bufs* b, char* base) {
   Bufs tmp;
   if (!b) b = &tmp;
-  bool oz = oz_pays(p.M, p.nwalkers);
-  if (oz) {
-    Bufs probe;
-    oz = plan_route(p, &probe, nullptr, true) <= kOzWorkspace;
-  }
-  return plan_route(p, b, base, oz);
+  Sliced route = sliced_route(p, p.N + (p.Ndn > 0 ? p.Ndn : 0));
+  Bufs probe;
+  if (plan_route(p, &probe, nullptr, route) > kOzWorkspace) route = Sliced{};
+  return plan_route(p, b, base, route);
 }
 
-static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, bool oz) {
+static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, const Sliced& route) {
   // N: orbital columns per walker (N_up + N_dn with two spin blocks)
   const size_t M = p.M, N = p.N + (p.Ndn > 0 ? p.Ndn : 0), G = p.nchol, W = p.nwalkers;
   const size_t P = M * (M + 1) / 2;
   const bool mixed = p.precision != AFQMC_FP64;
   size_t nchunk = (G + exchange_chunk((int)N, p.nchol) - 1) / exchange_chunk((int)N, p.nchol);
   if (mixed) nchunk = G;  // the tensor-core exchange leaves one partial per vector
-  const bool f32lu = p.precision == AFQMC_MIXED_TF32_F32LU || p.precision == AFQMC_MIXED_BF16_F32LU;
-  b->oz = oz && !mixed;
-  b->oz_ov = oz && (!mixed || p.ndet > 0);
-  b->oz_qr = oz && !f32lu && N <= 32;
+  b->oz = route.f64;
+  b->oz_ov = route.ov;
+  b->oz_qr = route.qr;
   b->oz_exch = b->oz && N <= 32;
-  b->oz_bp = oz && p.bp_steps > 0;
+  b->oz_bp = route.bp;
   OzOperand denA, denB;
   int den_cw = 0, den_nz = 0;
   oz_density_operands(M, N, W, &denA, &denB, &den_cw, &den_nz);
@@ -1112,11 +1137,14 @@ int step_after(afqmc_state* s) {
   const bool qr_due = p.qr_period && n % p.qr_period == 0;
   const bool pc_due = p.pc_period && n % p.pc_period == 0;
   const bool e_due = p.energy_period && n % p.energy_period == 0;
-  // Gram-Schmidt on the side stream when nothing of this step after it reads
-  // the orbitals before the next first half step (no comb due): then the
+  // The sweep of Gram-Schmidt on the side stream when nothing of this step after
+  // it reads the orbitals before the next first half step (no comb due): then the
   // energy evaluation, which reads neither Phi nor ld, is enqueued first so
-  // that its persistent contraction takes the SMs and the sweep fills in
-  const bool side = qr_due && !pc_due && s->side && !s->prof.on && !s->bp_on;
+  // that its persistent contraction takes the SMs and the sweep fills in.  (The
+  // products of the Gram matrix are persistent contractions too and take the SMs
+  // from the step's own: 301 walkers, M = 100, N = 10, ten steps with two visits
+  // 1456 us by the sweep, 1556 with them on the side stream, 1467 in line.)
+  const bool side = qr_due && !pc_due && s->side && !s->prof.on && !s->bp_on && !b.oz_qr;
   if (side && e_due) {
     prof_begin(s, AFQMC_PH_ENERGY);
     AFQ_TRY(energy_eval(s, true));

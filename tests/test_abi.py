@@ -123,6 +123,7 @@ def test_mcd_pairs_workspace_size_without_gpu(built):
 
 
 @pytest.mark.parametrize("M,N,Ndn,G,W", [(39, 3, 2, 50, 8), (40, 3, 2, 50, 8), (28, 4, 4, 90, 512),
+                                         (28, 2, 1, 50, 8), (28, 2, 2, 50, 8), (35, 1, 1, 50, 8),
                                          (150, 13, 10, 700, 150), (130, 17, 16, 400, 64)])
 def test_spin_block_workspace_on_every_route(built, M, N, Ndn, G, W):
     """The state lays its buffers out for N + Ndn columns: the size it was given for

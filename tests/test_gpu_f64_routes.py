@@ -67,10 +67,13 @@ def check(pkg, M, N, G, W, steps, Ndn=0):
     # float64 kernels, the series in one block per walker
     (5, 5, 7, 3, 0),       # every orbital occupied
     (33, 9, 40, 5, 0),     # more elements of a term than threads of a block
-    (39, 20, 30, 3, 19),   # the most orbitals, two spin blocks
+    (39, 20, 30, 3, 19),   # two spin blocks
+    (35, 2, 30, 3, 0),     # the most orbitals
+    (28, 2, 33, 512, 0),   # with many walkers
     # tensor cores
-    (40, 5, 57, 4, 0),     # the fewest orbitals; columns of a term: one 16-wide tile
-    (28, 2, 33, 512, 0),   # fewer with many walkers
+    (28, 4, 57, 4, 0),     # the fewest orbitals
+    (36, 1, 30, 3, 0),     # the fewest for a single column
+    (40, 5, 57, 4, 0),     # columns of a term: one 16-wide tile
     (64, 32, 90, 3, 0),    # a walker fills the exchange's column tile
     (64, 64, 20, 2, 0),    # every orbital occupied, two column tiles, float64 exchange kernel
     (70, 1, 30, 130, 0),   # 32 walkers per column tile of the exchange, 128 vectors per row tile
@@ -80,6 +83,23 @@ def check(pkg, M, N, G, W, steps, Ndn=0):
 ])
 def test_sizes(pkg, M, N, G, W, Ndn):
     check(pkg, M, N, G, W, 3, Ndn)
+
+
+@pytest.mark.parametrize("M,N,precision,qr", [(32, 2, 0, 5), (32, 4, 0, 2), (36, 2, 0, 5), (32, 4, 2, 2), (100, 10, 2, 2)])
+def test_population_whole_or_split(pkg, M, N, precision, qr):
+    """The arithmetic does not depend on the number of walkers: a state of 520 and
+    two of 460 and 60 that draw its fields walk the same walk, bit for bit."""
+    G = 40
+    h1, L, C = inputs(M, N, G)
+    out = []
+    for n, w0 in ((520, 0), (460, 0), (60, 460)):
+        p = pkg.default_params(M, N, G, n, qr_period=qr, energy_period=0, walker0=w0, precision=precision)
+        run = pkg.AfqmcRun(h1, L, C, p)
+        run.propagate(5)
+        out.append((*run.get_walkers(), run.local_energies()))
+        run.close()
+    for whole, a, b in zip(*out):
+        assert np.array_equal(whole, np.concatenate([a, b]))
 
 
 def test_chunks_of_walkers(pkg):
@@ -101,7 +121,7 @@ def test_chunks_of_walkers(pkg):
 
 
 @pytest.mark.parametrize("M,N,nd,kind,precision", [
-    (40, 5, 3, "noci", 0),    # the fewest orbitals of the route
+    (40, 5, 3, "noci", 0),    # one 16-wide column tile
     (70, 33, 2, "noci", 0),   # two column tiles of Theta, 132 rows of the trial's orbitals
     (130, 6, 2, "noci", 0),   # two row tiles of Phi
     (40, 3, 33, "noci", 0),   # one determinant more than the lanes of a warp
@@ -231,7 +251,7 @@ def test_orbitals_of_unequal_norm(pkg, M, N, Ndn, nd, precision):
 
 
 @pytest.mark.parametrize("M,N,G,W,m,qr", [
-    (40, 5, 57, 41, 3, 2),    # the fewest orbitals; a group of 40 walkers and one of a single walker
+    (40, 5, 57, 41, 3, 2),    # a group of 40 walkers and one of a single walker
     (65, 13, 70, 15, 2, 0),   # two row tiles of A, the last group full
     (100, 33, 60, 13, 2, 1),  # rows of the last tile short; K not a multiple of 16, QR by the sweep
     (44, 5, 50, 6, 0, 5),     # an empty window, fewer walkers than a group
