@@ -25,8 +25,9 @@
  *     read (and copied) during the call; the caller keeps ownership.
  *   - Device memory is owned by the caller: the library never allocates
  *     device memory.  afqmc_workspace_size() says how many bytes one state
- *     needs; the caller passes a buffer of at least that size (256-byte
- *     aligned) to afqmc_init() and keeps it alive until afqmc_destroy().
+ *     uses; the caller passes a buffer of that size (256-byte aligned; at
+ *     least afqmc_workspace_size_min()) to afqmc_init() and keeps it alive
+ *     until afqmc_destroy().
  *   - Every kernel of a state runs on the CUDA stream given to afqmc_init()
  *     (a cudaStream_t passed as void*, NULL = legacy default stream).
  *     Calls that return results to the host synchronise that stream.
@@ -60,7 +61,7 @@ extern "C" {
 typedef enum afqmc_status {
   AFQMC_OK = 0,
   AFQMC_EINVAL = -1,      /* bad argument, shape or parameter              */
-  AFQMC_ENOSPC = -2,      /* workspace smaller than afqmc_workspace_size() */
+  AFQMC_ENOSPC = -2,      /* workspace smaller than a state can do with    */
   AFQMC_ENONFINITE = -3,  /* non-finite value in a host input              */
   AFQMC_ECUDA = -4,       /* a CUDA runtime call failed                    */
   AFQMC_ETIMEOUT = -5,    /* a bounded device-side wait gave up            */
@@ -149,6 +150,11 @@ AFQMC_API void afqmc_default_params(afqmc_params* p);
 
 /* Bytes of device workspace one state needs for *p (sizes and precision). */
 AFQMC_API int afqmc_workspace_size(const afqmc_params* p, size_t* bytes);
+/* Bytes it can do with: in a workspace of at least these but fewer than
+ * afqmc_workspace_size() the contractions that need room for slices of their
+ * operands (see AFQMC_FP64) run on kernels without, slower and with other
+ * rounding. */
+AFQMC_API int afqmc_workspace_size_min(const afqmc_params* p, size_t* bytes);
 
 typedef struct afqmc_state afqmc_state; /* opaque */
 

@@ -31,7 +31,7 @@ AFQMC_PHASELESS, AFQMC_FREE = 0, 1
 STATUS = {0: "OK", -1: "EINVAL", -2: "ENOSPC", -3: "ENONFINITE", -4: "ECUDA",
           -5: "ETIMEOUT", -6: "ESTATE", -7: "EUNSUPPORTED"}
 
-EXPORTED = ["afqmc_default_params", "afqmc_workspace_size", "afqmc_init", "afqmc_propagate",
+EXPORTED = ["afqmc_default_params", "afqmc_workspace_size", "afqmc_workspace_size_min", "afqmc_init", "afqmc_propagate",
             "afqmc_energy", "afqmc_local_energies", "afqmc_get_walkers", "afqmc_set_walkers",
             "afqmc_get_energy_log", "afqmc_get_info", "afqmc_save", "afqmc_load",
             "afqmc_destroy", "afqmc_last_error", "afqmc_launch_count",
@@ -90,6 +90,7 @@ def lib():
     sig = {
         "afqmc_default_params": (None, [P(Params)]),
         "afqmc_workspace_size": (ctypes.c_int, [P(Params), P(ctypes.c_size_t)]),
+        "afqmc_workspace_size_min": (ctypes.c_int, [P(Params), P(ctypes.c_size_t)]),
         "afqmc_init": (ctypes.c_int, [P(Params), dp, dp, dp, dp, vp, ctypes.c_size_t, vp,
                                       P(vp)]),
         "afqmc_propagate": (ctypes.c_int, [vp, ctypes.c_int32]),
@@ -178,6 +179,13 @@ def default_params(M=0, N=0, nchol=0, nwalkers=0, **kw) -> Params:
 def afqmc_workspace_size(p: Params) -> int:
     n = ctypes.c_size_t(0)
     _check(lib().afqmc_workspace_size(ctypes.byref(p), ctypes.byref(n)))
+    return n.value
+
+
+def afqmc_workspace_size_min(p: Params) -> int:
+    """Bytes a state can do with (slower kernels that need less room)."""
+    n = ctypes.c_size_t(0)
+    _check(lib().afqmc_workspace_size_min(ctypes.byref(p), ctypes.byref(n)))
     return n.value
 
 
@@ -301,7 +309,13 @@ class AfqmcRun:
         self.device = torch.device(device)
         nbytes = afqmc_workspace_size(params)
         if workspace is None:
-            workspace = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
+            try:
+                workspace = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                least = afqmc_workspace_size_min(params)
+                if least == nbytes:
+                    raise
+                workspace = torch.empty(least + 256, dtype=torch.uint8, device=self.device)
         self.ws = workspace
         base = workspace.data_ptr()
         off = (-base) % 256

@@ -1,6 +1,7 @@
 // C ABI of the AFQMC library: workspace plan, set-up, step sequencing.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
@@ -42,9 +43,10 @@ struct Bump {
 // Slices of the walkers' operands live in one scratch area of at most about
 // this size: populations that need more are taken in chunks of walkers.
 constexpr size_t kOzScratch = size_t(2) << 30;
-// A state whose workspace would grow above this keeps the float64 kernels,
-// whose workspace is up to 40% smaller (states that fitted a 288 GB GPU
-// before still do).
+// A state whose workspace would grow above this, or above what the caller has,
+// takes the kernels without slices, whose workspace is smaller: a quarter of it at
+// M = 100, N = 10, 1024 walkers (200 against 720 MB), half at M = 300, N = 25, 512
+// (2.1 against 4.3 GB; mixed path 215 against 290 MB and 2.38 against 2.39 GB).
 constexpr size_t kOzWorkspace = size_t(160) << 30;
 
 // Which products run as sliced contractions (oz.cuh).  The lines depend on the
@@ -127,12 +129,12 @@ static void oz_density_operands(size_t M, size_t N, size_t W, OzOperand* A, OzOp
 
 static size_t plan_route(const afqmc_params& p, Bufs* b, char* base, const Sliced& route);
 
-size_t plan(const afqmc_params& p, Bufs* b, char* base) {
+size_t plan(const afqmc_params& p, Bufs* b, char* base, size_t limit) {
   Bufs tmp;
   if (!b) b = &tmp;
   Sliced route = sliced_route(p, p.N + (p.Ndn > 0 ? p.Ndn : 0));
   Bufs probe;
-  if (plan_route(p, &probe, nullptr, route) > kOzWorkspace) route = Sliced{};
+  if (plan_route(p, &probe, nullptr, route) > std::min(limit, kOzWorkspace)) route = Sliced{};
   return plan_route(p, b, base, route);
 }
 
@@ -1698,7 +1700,13 @@ int afqmc_workspace_size(const afqmc_params* p, size_t* bytes) {
     set_error("bytes is NULL");
     return AFQMC_EINVAL;
   }
-  *bytes = plan(*p, nullptr, nullptr);
+  *bytes = plan(*p, nullptr, nullptr, SIZE_MAX);
+  return AFQMC_OK;
+}
+
+int afqmc_workspace_size_min(const afqmc_params* p, size_t* bytes) {
+  AFQ_TRY(afqmc_workspace_size(p, bytes));
+  *bytes = std::min(*bytes, plan(*p, nullptr, nullptr, 0));
   return AFQMC_OK;
 }
 
@@ -1719,7 +1727,7 @@ static int init_state(const afqmc_params* p, const double* h1, const double* L,
     set_error("use_graph needs a stream created by the caller (default streams cannot be captured)");
     return AFQMC_EINVAL;
   }
-  const size_t need = plan(*p, nullptr, nullptr);
+  const size_t need = plan(*p, nullptr, nullptr, ws_bytes);
   if (ws_bytes < need) {
     set_error("workspace %zu bytes < %zu needed", ws_bytes, need);
     return AFQMC_ENOSPC;
@@ -1756,7 +1764,7 @@ static int init_state(const afqmc_params* p, const double* h1, const double* L,
   s->ws_bytes = ws_bytes;
   // (the caller's parameters and these lay out the same workspace: a plan that
   // told them apart would write past its end)
-  if (plan(s->p, &s->b, s->ws) > ws_bytes) {
+  if (plan(s->p, &s->b, s->ws, ws_bytes) > ws_bytes) {
     set_error("workspace layout of two spin blocks differs from its size");
     delete s;
     return AFQMC_ENOSPC;

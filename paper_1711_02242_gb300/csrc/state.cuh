@@ -109,7 +109,7 @@ constexpr int kSmwGC = 8;     // Cholesky vectors per block of the low-rank kern
 
 constexpr int kBpSlices = 8;
 
-size_t plan(const afqmc_params& p, Bufs* b, char* base);
+size_t plan(const afqmc_params& p, Bufs* b, char* base, size_t limit);
 
 }  // namespace afq
 

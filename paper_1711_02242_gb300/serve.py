@@ -17,7 +17,7 @@ import time
 
 import numpy as np
 
-from . import AfqmcRun, afqmc_workspace_size, default_params
+from . import AfqmcRun, afqmc_workspace_size, afqmc_workspace_size_min, default_params
 
 
 class DevicePool:
@@ -99,7 +99,11 @@ class Server:
                               max_records=max(1, r.nsteps // max(1, r.energy_period)))
 
     def footprint(self, r: Request) -> int:
-        return afqmc_workspace_size(self.params(r)) + 256
+        """Bytes a request takes: what its state uses, or if only that is more than
+        the whole pool what it can do with."""
+        p = self.params(r)
+        n = afqmc_workspace_size(p) + 256
+        return n if n <= self.pool.size else afqmc_workspace_size_min(p) + 256
 
     def run(self, requests, realtime: bool = True):
         """Serve `requests` (sorted by arrival).  With realtime, arrivals are

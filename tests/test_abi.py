@@ -130,3 +130,14 @@ def test_spin_block_workspace_on_every_route(built, M, N, Ndn, G, W):
     (N, Ndn) has to be that layout's on every route by size."""
     split = built.afqmc_workspace_size(built.default_params(M, N, G, W, Ndn=Ndn))
     assert split == built.afqmc_workspace_size(built.default_params(M, N + Ndn, G, W))
+
+
+@pytest.mark.parametrize("M,N,G,W,kw", [(100, 10, 500, 1024, {}), (300, 25, 1800, 512, {}), (100, 10, 500, 1024, {"precision": 2}),
+                                        (100, 10, 500, 256, {"precision": 2, "ndet": 4}), (40, 5, 200, 64, {"bp_steps": 4}),
+                                        (150, 13, 700, 150, {"Ndn": 10}), (12, 3, 48, 32, {})])
+def test_least_workspace(built, M, N, G, W, kw):
+    """What a state can do with is less than what it uses wherever products run as
+    slices, and the same elsewhere."""
+    p = built.default_params(M, N, G, W, **kw)
+    least, size = built.afqmc_workspace_size_min(p), built.afqmc_workspace_size(p)
+    assert least % 256 == 0 and (least < size if M > 12 else least == size)

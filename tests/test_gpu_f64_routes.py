@@ -85,6 +85,44 @@ def test_sizes(pkg, M, N, G, W, Ndn):
     check(pkg, M, N, G, W, 3, Ndn)
 
 
+@pytest.mark.parametrize("M,N,W,Ndn,nd,precision", [
+    (40, 5, 6, 0, 0, 0), (60, 17, 6, 15, 0, 0), (70, 6, 6, 0, 2, 0), (100, 10, 200, 0, 0, 2), (70, 6, 6, 0, 2, 2)])
+def test_least_workspace(pkg, M, N, W, Ndn, nd, precision):
+    """A state in the least workspace it can do with walks the same walk to rounding
+    (float64: a few hundred products a sum, 1e-10; mixed: the float64 overlaps and
+    Gram-Schmidt differ by 1e-14, which a BF16 operand may round to another
+    neighbour, 2^-8 of its size), and a byte less is refused."""
+    import torch
+
+    G = 60
+    h1, L, trial = inputs(M, N, G, Ndn)
+    if nd:
+        rng = np.random.default_rng(M)
+        dets = np.array([trial] + [np.linalg.qr(trial + 0.05 * rng.standard_normal((M, N)))[0] for _ in range(1, nd)])
+        trial = (np.array([1.0] + [0.3] * (nd - 1), complex), dets, dets)
+    p = pkg.default_params(M, N, G, W, qr_period=2, energy_period=0, Ndn=Ndn, ndet=nd, precision=precision,
+                           bp_steps=0 if Ndn or nd else 2)
+    size, least = pkg.afqmc_workspace_size(p), pkg.afqmc_workspace_size_min(p)
+    assert least < size
+    out = []
+    for n in (size, size - 256, least):
+        run = pkg.AfqmcRun(h1, L, trial, p, workspace=torch.empty(n, dtype=torch.uint8, device="cuda"))
+        run.propagate(3)
+        phi, wt, lo = run.get_walkers()
+        out.append([phi, wt, lo, run.local_energies()])
+        if p.bp_steps:
+            run.bp_begin()
+            run.propagate(2)
+            out[-1] += list(run.bp_end()[:2])
+        assert run.info().status == 0
+        run.close()
+    for a, b, c in zip(*out):
+        assert np.array_equal(b, c)  # a little too small for the slices, or by all of them
+        assert np.max(np.abs(a - c)) < (TOL if precision == 0 else 2.0 ** -8) * (1 + np.abs(a).max())
+    with pytest.raises(pkg.AfqmcError, match="ENOSPC"):
+        pkg.AfqmcRun(h1, L, trial, p, workspace=torch.empty(least - 1, dtype=torch.uint8, device="cuda"))
+
+
 @pytest.mark.parametrize("M,N,precision,qr", [(32, 2, 0, 5), (32, 4, 0, 2), (36, 2, 0, 5), (32, 4, 2, 2), (100, 10, 2, 2)])
 def test_population_whole_or_split(pkg, M, N, precision, qr):
     """The arithmetic does not depend on the number of walkers: a state of 520 and

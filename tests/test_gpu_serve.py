@@ -56,6 +56,21 @@ def test_results_alone_equal_results_in_the_mix(pkg, prec):
         assert alone.energies.shape[0] == 4
 
 
+def test_pool_below_what_a_request_uses(pkg):
+    """A request whose state uses more than the whole pool, but can do with it, is served."""
+    from paper_1711_02242_gb300.serve import Server
+
+    r = requests()[3]
+    p = Server(1 << 20, precision=0).params(r)
+    least, size = pkg.afqmc_workspace_size_min(p), pkg.afqmc_workspace_size(p)
+    assert least + 1024 < size
+    a = Server(least + 1024, precision=0).run([r], realtime=False)[0].energies.copy()
+    b = Server(size + 1024, precision=0).run([requests()[3]], realtime=False)[0].energies
+    assert np.max(np.abs(a - b)) < 1e-8 * np.abs(b).max()
+    with pytest.raises(ValueError):
+        Server(least // 2, precision=0).run([requests()[3]], realtime=False)
+
+
 def test_pool_first_fit_reuses_memory(pkg):
     from paper_1711_02242_gb300.serve import DevicePool
 
