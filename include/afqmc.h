@@ -71,10 +71,11 @@ typedef enum afqmc_status {
 
 /* Arithmetic of the step. */
 enum {
-  AFQMC_FP64 = 0,       /* every result to float64 accuracy: the per-walker     */
-                        /* steps in float64 / complex128, the contractions of   */
-                        /* larger systems as exact products of integer slices   */
-                        /* on the tensor cores, rounded to float64 once         */
+  AFQMC_FP64 = 0,       /* float64 / complex128; the contractions of larger     */
+                        /* systems on the tensor cores, as products of 57-bit   */
+                        /* integer slices of their operands, rounded to float64 */
+                        /* once: within 2^-53 of the result + 1.4 K 2^-53 of    */
+                        /* the product of its rows' largest elements (K terms)  */
   AFQMC_MIXED_TF32 = 1, /* contractions on tcgen05 tensor cores, TF32 inputs,   */
                         /* FP32 accumulation; the overlap S = V_T^T Phi, its    */
                         /* LU / inverse S^-1 and log det, the overlap ratios,   */

@@ -13,9 +13,20 @@
 //   D_t = sum_{i + j = t} sum_k v_i w_j,
 // each D_t an integer below 2^24 over kOzSegK values of k, so the FP32
 // accumulators hold it exactly; the segments are added as 64-bit integers and
-// the result is rounded to float64 once.  Products with i + j > 7 are left
-// out: at most 7 2^-58 of (2^ea 2^eb) per term, with random signs, against the
-// 2^-53 of the running sum that every step of a float64 FMA chain rounds away.
+// the result is rounded to float64 once.
+//
+// What is lost, against the row maxima (2^(ea - 1) <= max |a| < 2^ea, or ea =
+// -1021 in a row of subnormals): an element more than three binades below its
+// row's largest is rounded to 2^(e - 57), the products with i + j > 7 are left out
+// (7.1 2^-58 per term at most, of either sign), and so
+//   |C - A B^T| <= 2^-53 |C| + 2.8 K 2^(ea + eb - 56),
+// at most 1.4 K 2^-53 max |a| max |b| beside the rounding of C.  A float64 FMA
+// chain's bound is K 2^-53 sum |a b|: the same kind where a sum is of the size of
+// its largest elements' product, as in a step's, in which one operand's elements
+// are of a size (the fields, Theta's and the orbitals' rows; orbitals against each
+// other are made so by a power of two each, oz_row_exps).  A sum whose large
+// elements meet only small ones loses what the chain would keep.  A row that holds
+// an infinity or a NaN gives NaN.
 #pragma once
 
 #include "kernels.cuh"
@@ -24,7 +35,7 @@ namespace afq {
 
 constexpr int kOzSlices = 8;
 constexpr int kOzSegBlk = 25;             // K blocks of 16 between two drains of the accumulators
-constexpr int kOzSegK = 16 * kOzSegBlk;   // 400: 10 * 2^12 * 400 < 2^24 (D_7: 2 * 2^13 + 6 * 2^12 per k)
+constexpr int kOzSegK = 16 * kOzSegBlk;   // 400: 40960 * 400 < 2^24 (D_7: 2 * 2^13 + 6 * 2^12 per k)
 constexpr int kOzZeroExp = -30000;        // exponent of a row of zeros
 constexpr int kOzNanExp = 100000;         // a row holding an infinity or a NaN: its results are NaN
 

@@ -30,6 +30,27 @@ struct Carve {
 
 // Sliced contractions: every pointer is a device pointer; ws holds the slices and
 // row exponents, 256-byte aligned.
+// C[m][n] = 2^alpha A B^T, rows of k values.
+extern "C" __attribute__((visibility("default"))) int sp_gemm(const double* A, const double* B, int m, int n, int k,
+                                                               double* C, int alpha, char* ws, size_t ws_bytes,
+                                                               int* status, void* stream) {
+  using namespace afq;
+  Carve c{ws, ws + ws_bytes};
+  OzGemm g;
+  g.B.RT = g.B.rows_per_tile = 64;
+  if (!c.operand(g.A, m, k, 1) || !c.operand(g.B, n, k, 1)) return AFQMC_ENOSPC;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  AFQ_TRY(oz_slice_rows(A, m, k, k, g.A, st));
+  AFQ_TRY(oz_slice_rows(B, n, k, k, g.B, st));
+  g.m = m;
+  g.n = n;
+  g.C = C;
+  g.ldc = n;
+  g.alpha_log2 = alpha;
+  g.err = status;
+  return oz_gemm_store(g, st);
+}
+
 // D[z][2 M][2 M] of groups of cw walkers (see oz_slice_densities).
 extern "C" __attribute__((visibility("default"))) int sp_densities(
     const double* phi, const double* thA, const double* thB, int W, int N, int M, int cw, double* D, char* ws,
