@@ -273,17 +273,31 @@ KERNEL_OF_PHASE = {"overlap": ("k_overlap", "alu", "walker_f64.cu"),
                               "gemm_tc.cu")}
 
 
-def sliced(w, precision):
-    """Whether the float64 path's contractions run on the tensor cores (the
-    library's rule; smaller systems use the float64 kernels)."""
-    return precision == "fp64" and (w.M >= 40 or (w.M >= 28 and w.nwalkers >= 512))
-
-
 # phases of the float64 path that are sliced products
 SLICED_PHASES = {"taylor": "k_oz_gemm (a Taylor term) and the slicing kernels",
                  "v_assembly": "k_oz_gemm (V) and the slicing of the fields",
                  "theta": "k_oz_gemm (Theta) and the slicing kernels",
                  "energy": "k_oz_gemm (force bias, exchange) + k_eloc"}
+
+
+def kernels_taken(w, precision, routes):
+    """Phase -> (kernel, bound, source file) for a state whose sliced routes are
+    `routes` (afqmc_sliced_routes)."""
+    import paper_1711_02242_gb300 as pkg
+
+    k = kernel_of_phase(precision)
+    if not precision.endswith("f32lu") and w.N <= 16:
+        k["overlap"] = (f"k_overlap_warp<{w.N}>", "alu", "walker_f64.cu")
+    if routes & pkg.AFQMC_SLICED_F64:
+        for ph, name in SLICED_PHASES.items():
+            k[ph] = (name, "sliced", "oz.cu")
+        if not routes & pkg.AFQMC_SLICED_EXCHANGE:
+            k["energy"] = ("k_oz_gemm (force bias) + k_exchange + k_eloc", "alu", "walker_f64.cu")
+    if routes & pkg.AFQMC_SLICED_QR:
+        # slices and products on the tensor cores, k_gram_factor on the float64
+        # pipe: no one rate bounds the phase
+        k["qr"] = ("k_oz_gemm (Gram matrix, Q) + k_gram_factor + the slicing kernels", "mixed", "oz.cu")
+    return k
 
 
 def source_sha(fname):
@@ -348,20 +362,28 @@ def traffic_of(phase, src, precision):
     return None
 
 
-def rooflines(w, phases, precision, K):
+def rooflines(w, phases, precision, K, routes=0):
     """Roofline entry per timed phase that is one kernel family: algorithmic
     work per launch / device time per launch (CUDA events on the state's
-    stream) against the peak of the pipe that bounds it."""
+    stream) against the peak of the pipe that bounds it; no fraction for a phase
+    of kernels bound by different ones.  routes: afqmc_sliced_routes of the state."""
     pk, pk_kind = peaks()
     per = algorithmic_per_walker(w)
     per_bytes = bytes_per_walker(w, precision)
     out = []
-    for ph, (kname, bound, src) in kernel_of_phase(precision).items():
+    for ph, (kname, bound, src) in kernels_taken(w, precision, routes).items():
         v = phases[ph]
         if v["count"] == 0 or v["ms"] <= 0:
             continue
         ms_launch = v["ms"] / v["count"]
         work = per[ph] * w.nwalkers
+        if bound == "mixed":
+            out.append({"phase": ph, "kernel": kname, "bound": bound, "achieved": None,
+                        "peak": None, "unit": None, "frac": None, "traffic": None,
+                        "peak_source": None, "ms_per_launch": ms_launch,
+                        "launches_per_step": v["count"] / K,
+                        "share_of_step": v["ms"] / sum(x["ms"] for x in phases.values())})
+            continue
         if bound == "hbm":
             # bytes per launch / time, against the measured copy bandwidth
             peak, unit, src_peak = pk["hbm_gbs"], "GB/s", f"{pk_kind} HBM copy bandwidth"
@@ -377,8 +399,8 @@ def rooflines(w, phases, precision, K):
             peak, unit, src_peak = FP32_PEAK_TFLOPS, "TFLOP/s", (
                 "derived: 152 SMs x 128 FP32 FMA/clk x 2 x 2070 MHz")
             bound = "alu"
-        elif sliced(w, precision) and ph in SLICED_PHASES:
-            kname, src, bound = SLICED_PHASES[ph], "oz.cu", "tensor"
+        elif bound == "sliced":
+            bound = "tensor"
             peak, unit = pk["bf16_tflops_sustained"] / SLICE_PRODUCTS, "TFLOP/s"
             src_peak = f"{pk_kind} bf16 sustained / {SLICE_PRODUCTS} (products of slices)"
         elif bound == "alu" or precision == "fp64":
@@ -398,10 +420,6 @@ def rooflines(w, phases, precision, K):
                     "peak_source": src_peak, "ms_per_launch": ms_launch,
                     "launches_per_step": v["count"] / K,
                     "share_of_step": v["ms"] / sum(x["ms"] for x in phases.values())})
-        if ph == "qr" and kname == "k_mgs" and w.N <= 32 and (precision != "fp64" and w.M >= 40
-                                                              or sliced(w, precision)):
-            out[-1]["note"] = ("from the Gram matrix: two sliced products on the tensor cores and "
-                               "k_gram_factor; k_mgs sweeps the walkers left over")
     out.sort(key=lambda d: -d["share_of_step"])
     return out
 
@@ -528,6 +546,7 @@ def run_gpu(args, w: workloads.Workload):
     s_energy = (time.perf_counter() - t0) / n_e
     ms_total = max_over_ranks(ms_total, device=dev)
     info = run.info()
+    routes = run.sliced_routes()
     if pop is not None:
         E, wsum = pop.energy()  # the whole population's estimator
     else:
@@ -565,7 +584,7 @@ def run_gpu(args, w: workloads.Workload):
                 clocks=clk.summary(), e2e_s=t_e2e, trial_converged=conv, trial_grad=grad,
                 h2d_bytes=h1.nbytes + L.nbytes + C.nbytes, world=ws, rank=rank, warmup=Wm,
                 ms_profiled=ms_profiled, s_energy=s_energy, graph=not args.no_graph,
-                sharded=sharded, pc_period=pc,
+                sharded=sharded, pc_period=pc, routes=routes,
                 precision_report=prec_rep, fp64=fp64, bias=bias)
 
 
@@ -1567,7 +1586,7 @@ def main():
     value = job_throughput(w.nwalkers, K, r["ms_total"], N)
     fl = flops_per_walker_step(w)
     # the dominant kernel (largest share of the profiled step) and the others
-    roofs = rooflines(w, r["phases"], args.precision, K)
+    roofs = rooflines(w, r["phases"], args.precision, K, r["routes"])
     top = roofs[0]
     roof = {k: top[k] for k in ("bound", "achieved", "peak", "unit", "frac", "traffic")}
     roof.update(kernel=top["kernel"], peak_source=top["peak_source"],

@@ -290,6 +290,18 @@ typedef struct afqmc_info {
 /* State summary; synchronises the stream. */
 AFQMC_API int afqmc_get_info(afqmc_state* s, afqmc_info* info);
 
+/* Which of a state's products run as integer slices on the tensor cores (it
+ * depends on the sizes, the precision and the workspace): the sum of */
+enum {
+  AFQMC_SLICED_F64 = 1,      /* every contraction of the float64 path           */
+  AFQMC_SLICED_EXCHANGE = 2, /* its exchange among them                         */
+  AFQMC_SLICED_OVERLAP = 4,  /* overlaps and Theta (with AFQMC_SLICED_F64, or   */
+                             /* of several determinants on the mixed path)      */
+  AFQMC_SLICED_QR = 8,       /* Gram-Schmidt from the Gram matrix               */
+  AFQMC_SLICED_BP = 16       /* back-propagated densities                       */
+};
+AFQMC_API int afqmc_sliced_routes(const afqmc_state* s, int32_t* routes);
+
 /*
  * Checkpoint: serialise walkers, weights, overlaps, the step counter and the
  * energy log into host memory.  With buf == NULL, *bytes receives the size

@@ -28,12 +28,14 @@ AFQMC_MIXED_TF32_F32LU, AFQMC_MIXED_BF16_F32LU = 3, 4
 # the mixed paths with Theta = Phi S^-1 also in float64
 AFQMC_MIXED_TF32_F64THETA, AFQMC_MIXED_BF16_F64THETA = 5, 6
 AFQMC_PHASELESS, AFQMC_FREE = 0, 1
+# which products a state runs as integer slices (AfqmcRun.sliced_routes)
+AFQMC_SLICED_F64, AFQMC_SLICED_EXCHANGE, AFQMC_SLICED_OVERLAP, AFQMC_SLICED_QR, AFQMC_SLICED_BP = 1, 2, 4, 8, 16
 STATUS = {0: "OK", -1: "EINVAL", -2: "ENOSPC", -3: "ENONFINITE", -4: "ECUDA",
           -5: "ETIMEOUT", -6: "ESTATE", -7: "EUNSUPPORTED"}
 
 EXPORTED = ["afqmc_default_params", "afqmc_workspace_size", "afqmc_workspace_size_min", "afqmc_init", "afqmc_propagate",
             "afqmc_energy", "afqmc_local_energies", "afqmc_get_walkers", "afqmc_set_walkers",
-            "afqmc_get_energy_log", "afqmc_get_info", "afqmc_save", "afqmc_load",
+            "afqmc_get_energy_log", "afqmc_get_info", "afqmc_sliced_routes", "afqmc_save", "afqmc_load",
             "afqmc_destroy", "afqmc_last_error", "afqmc_launch_count",
             "afqmc_philox4x32_10", "afqmc_gaussian_fields", "afqmc_contract",
             "afqmc_profile_start", "afqmc_profile_stop", "afqmc_local_energies_noalloc",
@@ -100,6 +102,7 @@ def lib():
         "afqmc_set_walkers": (ctypes.c_int, [vp, dp, dp]),
         "afqmc_get_energy_log": (ctypes.c_int, [vp, dp, ctypes.c_int32, P(ctypes.c_int32)]),
         "afqmc_get_info": (ctypes.c_int, [vp, P(Info)]),
+        "afqmc_sliced_routes": (ctypes.c_int, [vp, P(ctypes.c_int32)]),
         "afqmc_save": (ctypes.c_int, [vp, vp, P(ctypes.c_size_t)]),
         "afqmc_load": (ctypes.c_int, [vp, vp, ctypes.c_size_t]),
         "afqmc_destroy": (ctypes.c_int, [vp]),
@@ -431,6 +434,12 @@ class AfqmcRun:
         i = Info()
         _check(lib().afqmc_get_info(self.s, ctypes.byref(i)))
         return i
+
+    def sliced_routes(self) -> int:
+        """Sum of the AFQMC_SLICED_* flags of this state."""
+        r = ctypes.c_int32(0)
+        _check(lib().afqmc_sliced_routes(self.s, ctypes.byref(r)))
+        return r.value
 
     def save(self) -> bytes:
         n = ctypes.c_size_t(0)

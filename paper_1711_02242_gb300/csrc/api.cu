@@ -2088,6 +2088,17 @@ int afqmc_get_energy_log(afqmc_state* s, double* rec, int32_t cap, int32_t* n) {
   return AFQMC_OK;
 }
 
+int afqmc_sliced_routes(const afqmc_state* s, int32_t* routes) {
+  if (!s || !routes) {
+    set_error("afqmc_sliced_routes: NULL argument");
+    return AFQMC_EINVAL;
+  }
+  const Bufs& b = s->b;
+  *routes = (b.oz ? AFQMC_SLICED_F64 : 0) | (b.oz_exch ? AFQMC_SLICED_EXCHANGE : 0) |
+            (b.oz_ov ? AFQMC_SLICED_OVERLAP : 0) | (b.oz_qr ? AFQMC_SLICED_QR : 0) | (b.oz_bp ? AFQMC_SLICED_BP : 0);
+  return AFQMC_OK;
+}
+
 int afqmc_get_info(afqmc_state* s, afqmc_info* info) {
   AFQ_STATE(s);
   if (!info) {

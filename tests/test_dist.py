@@ -54,6 +54,30 @@ def test_job_throughput_counts_all_ranks():
     assert bench.max_over_ranks(7.5) == 7.5  # no process group: local value
 
 
+def test_rooflines_name_the_kernels_that_ran():
+    """Sliced routes (afqmc_sliced_routes) and sizes choose the kernel of a phase; a
+    phase of kernels bound by different pipes has no fraction."""
+    import bench
+    import paper_1711_02242_gb300 as pkg
+    import workloads
+
+    ph = {name: {"ms": 1.0, "count": 1, "kernels": 1} for name in bench.PHASES}
+    by = lambda w, prec, routes: {r["phase"]: r for r in bench.rooflines(w, ph, prec, 10, routes)}  # noqa: E731
+    c2, c1 = workloads.config("c2"), workloads.config("c1")  # 25 and 10 orbitals
+    r = by(c2, "bf16", pkg.AFQMC_SLICED_QR)
+    assert "k_gram_factor" in r["qr"]["kernel"] and r["qr"]["frac"] is None and r["qr"]["ms_per_launch"] == 1.0
+    assert r["overlap"]["kernel"] == "k_overlap" and r["taylor"]["kernel"] == "k_taylor_series"
+    assert by(c1, "bf16", 0)["overlap"]["kernel"] == "k_overlap_warp<10>"
+    assert by(c1, "bf16-f32lu", 0)["overlap"]["kernel"] == "k_overlap<float>"
+    f64 = pkg.AFQMC_SLICED_F64 | pkg.AFQMC_SLICED_OVERLAP
+    r = by(c2, "fp64", f64)
+    peak = bench.peaks()[0]["bf16_tflops_sustained"] / bench.SLICE_PRODUCTS
+    assert r["taylor"]["bound"] == "tensor" and r["taylor"]["peak"] == peak
+    assert "k_exchange" in r["energy"]["kernel"] and r["energy"]["peak"] == bench.FP64_PEAK_TFLOPS
+    assert by(c2, "fp64", f64 | pkg.AFQMC_SLICED_EXCHANGE)["energy"]["peak"] == peak
+    assert by(c2, "fp64", 0)["taylor"]["peak"] == bench.FP64_PEAK_TFLOPS
+
+
 def test_l2_note_states_whether_the_inputs_fit_in_l2():
     """The bench line says whether a step's inputs exceed the 129 MB L2 (no
     flush between steps is needed then) or are L2-resident."""

@@ -107,6 +107,7 @@ def test_least_workspace(pkg, M, N, W, Ndn, nd, precision):
     out = []
     for n in (size, size - 256, least):
         run = pkg.AfqmcRun(h1, L, trial, p, workspace=torch.empty(n, dtype=torch.uint8, device="cuda"))
+        assert bool(run.sliced_routes()) == (n == size)
         run.propagate(3)
         phi, wt, lo = run.get_walkers()
         out.append([phi, wt, lo, run.local_energies()])
