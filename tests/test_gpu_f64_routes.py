@@ -168,9 +168,11 @@ def test_chunks_of_walkers(pkg):
     (44, 6, 3, "noci", 2),    # the mixed path keeps these float64
 ])
 def test_determinants(pkg, M, N, nd, kind, precision):
-    """Overlaps and Theta of every determinant, against the oracles' walks.  On
-    the mixed path only the first local energies are compared: the BF16
-    exchange and traces are good to 2^-8 of their terms there."""
+    """Overlaps and Theta of every determinant, against the oracles' walks.  The
+    mixed path against the float64 one from the same perturbed walkers: overlaps to
+    the 1e-10 of float64, local energies (BF16 exchange and traces) to 2^-8 of their
+    terms, three steps' walkers to a few 2^-9 and weights to some more (sums of
+    products of rounded fields and vectors)."""
     G, W = 50, 5
     h1, L, C = inputs(M, N, G)
     rng = np.random.default_rng(M + nd)
@@ -192,8 +194,23 @@ def test_determinants(pkg, M, N, nd, kind, precision):
     p = pkg.default_params(M, N, G, W, qr_period=2, energy_period=1, ndet=nd, precision=precision)
     run = pkg.AfqmcRun(h1, L, (coef, ups, dns), p)
     if precision:
-        el = orc.local_energies()
-        assert np.max(np.abs(run.local_energies() - el) / np.abs(el)) < 2.0 ** -8
+        ref = pkg.AfqmcRun(h1, L, (coef, ups, dns), pkg.default_params(M, N, G, W, qr_period=2, energy_period=1, ndet=nd))
+        phi = orc.phi + 0.02 * (rng.standard_normal(orc.phi.shape) + 1j * rng.standard_normal(orc.phi.shape))
+        for steps in (0, 3):
+            for r in (run, ref):
+                r.set_walkers(phi, np.ones(W))
+                r.propagate(steps)
+            (p1, w1, l1), (p2, w2, l2) = run.get_walkers(), ref.get_walkers()
+            e1, e2 = run.local_energies(), ref.local_energies()
+            assert np.max(np.abs(e1 - e2) / np.abs(e2)) < 2.0 ** -8
+            if steps == 0:
+                assert np.max(np.abs(l1 - l2)) < TOL * (1 + np.abs(l2).max())
+            else:
+                assert np.max(np.abs(p1 - p2)) < 2.0 ** -6 * np.abs(p2).max()
+                assert np.max(np.abs(w1 - w2) / np.abs(w2)) < 2.0 ** -5
+        assert run.info().status == 0
+        run.close()
+        ref.close()
         return
     run.propagate(3)
     orc.run(3)
