@@ -70,6 +70,7 @@ def check(pkg, M, N, G, W, steps, Ndn=0):
     (39, 20, 30, 3, 19),   # two spin blocks
     (35, 2, 30, 3, 0),     # the most orbitals
     (28, 2, 33, 512, 0),   # with many walkers
+    (27, 20, 30, 3, 0),    # Gram-Schmidt alone from the Gram matrix
     # tensor cores
     (28, 4, 57, 4, 0),     # the fewest orbitals
     (36, 1, 30, 3, 0),     # the fewest for a single column
@@ -224,10 +225,11 @@ def test_determinants(pkg, M, N, nd, kind, precision):
     run.close()
 
 
-@pytest.mark.parametrize("M,N,Ndn", [(48, 6, 0), (130, 25, 0), (60, 17, 15)])
+@pytest.mark.parametrize("M,N,Ndn", [(48, 6, 0), (60, 13, 0), (130, 25, 0), (60, 17, 15)])
 def test_gram_schmidt_routes(pkg, M, N, Ndn):
     """Gram-Schmidt of well-conditioned walkers (from the Gram matrix) and of
-    walkers with nearly parallel columns (the sweep) in one population: Q is
+    walkers with nearly parallel columns (the sweep) in one population, and the sweep
+    alone for few columns: Q is
     orthonormal to rounding, and walkers, overlaps and weights follow the
     oracle's modified Gram-Schmidt.  The nearly parallel columns' condition
     number is about 1e3, so 1e-10 leaves their 1e-13 room."""
@@ -260,7 +262,8 @@ def test_gram_schmidt_routes(pkg, M, N, Ndn):
 
 
 @pytest.mark.parametrize("M,N,Ndn,nd,precision", [
-    (48, 12, 0, 0, 0),
+    (48, 12, 0, 0, 0),    # Gram-Schmidt by the sweep
+    (70, 16, 0, 0, 0),    # and from the Gram matrix
     (60, 17, 15, 0, 0),   # two spin blocks
     (70, 6, 0, 3, 0),     # three determinants
     (130, 25, 0, 0, 2),   # the mixed path's Gram-Schmidt
