@@ -99,11 +99,13 @@ class Server:
                               max_records=max(1, r.nsteps // max(1, r.energy_period)))
 
     def footprint(self, r: Request) -> int:
-        """Bytes a request takes: what its state uses, or if only that is more than
-        the whole pool what it can do with."""
-        p = self.params(r)
-        n = afqmc_workspace_size(p) + 256
-        return n if n <= self.pool.size else afqmc_workspace_size_min(p) + 256
+        return afqmc_workspace_size(self.params(r)) + 256
+
+    def room(self, r: Request) -> int:
+        """Bytes of the pool given to a request: its footprint, or if that is more than
+        the whole pool what its state can do with."""
+        n = self.footprint(r)
+        return n if n <= self.pool.size else afqmc_workspace_size_min(self.params(r)) + 256
 
     def run(self, requests, realtime: bool = True):
         """Serve `requests` (sorted by arrival).  With realtime, arrivals are
@@ -113,7 +115,7 @@ class Server:
 
         pending = sorted(requests, key=lambda r: r.arrival)
         for r in pending:
-            if self.footprint(r) > self.pool.size:
+            if self.room(r) > self.pool.size:
                 raise ValueError(f"request {r.rid} needs more than the whole pool")
         queue, active, done = [], [], []
         t0 = time.perf_counter()
@@ -125,7 +127,7 @@ class Server:
             # admission in arrival order while a slot is free and the footprint fits
             while queue and (self.max_active is None or len(active) < self.max_active):
                 r = queue[0]
-                blk = self.pool.alloc(self.footprint(r))
+                blk = self.pool.alloc(self.room(r))
                 if blk is None:
                     break
                 queue.pop(0)

@@ -125,6 +125,27 @@ def test_least_workspace(pkg, M, N, W, Ndn, nd, precision):
         pkg.AfqmcRun(h1, L, trial, p, workspace=torch.empty(least - 1, dtype=torch.uint8, device="cuda"))
 
 
+def test_allocation_that_fails(pkg, monkeypatch):
+    """Where the workspace a state uses cannot be allocated, one it can do with is."""
+    import torch
+
+    h1, L, C = inputs(40, 5, 60)
+    p = pkg.default_params(40, 5, 60, 6, energy_period=0)
+    size, least, empty = pkg.afqmc_workspace_size(p), pkg.afqmc_workspace_size_min(p), torch.empty
+
+    def bounded(n, *a, **kw):
+        if isinstance(n, int) and n >= size:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return empty(n, *a, **kw)
+
+    monkeypatch.setattr(torch, "empty", bounded)
+    run = pkg.AfqmcRun(h1, L, C, p)
+    assert run.ws.numel() == least + 256 and run.sliced_routes() == 0
+    run.propagate(2)
+    assert run.info().status == 0
+    run.close()
+
+
 @pytest.mark.parametrize("M,N,precision,qr", [(32, 2, 0, 5), (32, 4, 0, 2), (36, 2, 0, 5), (32, 4, 2, 2), (100, 10, 2, 2)])
 def test_population_whole_or_split(pkg, M, N, precision, qr):
     """The arithmetic does not depend on the number of walkers: a state of 520 and

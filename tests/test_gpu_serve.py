@@ -64,6 +64,8 @@ def test_pool_below_what_a_request_uses(pkg):
     p = Server(1 << 20, precision=0).params(r)
     least, size = pkg.afqmc_workspace_size_min(p), pkg.afqmc_workspace_size(p)
     assert least + 1024 < size
+    # whatever the pool, a footprint is what the state uses
+    assert Server(1, precision=0).footprint(r) == Server(size + 1024, precision=0).footprint(r) == size + 256
     a = Server(least + 1024, precision=0).run([r], realtime=False)[0].energies.copy()
     b = Server(size + 1024, precision=0).run([requests()[3]], realtime=False)[0].energies
     assert np.max(np.abs(a - b)) < 1e-8 * np.abs(b).max()
