@@ -52,7 +52,7 @@ constexpr size_t kOzWorkspace = size_t(160) << 30;
 // Which products run as sliced contractions (oz.cuh).  The lines depend on the
 // system alone, not on the number of walkers, so that a population does the same
 // arithmetic whole or split over states; each lies where the two sides cross for
-// some number of walkers.  Other side's time / sliced:
+// some number of walkers.  Other side's time / sliced, in a graph:
 //  f64  five steps and an energy (5 M vectors), 32, 128, 300, 512, 1024 walkers:
 //       M = 28, N = 2 0.82 0.80 0.89 1.09 1.46; M = 28, N = 4 0.91 0.91 1.07 1.41
 //       1.84; M = 32, N = 2 0.84 0.85 1.12 1.30 1.58; M = 32, N = 4 0.98 1.00 1.34

@@ -91,6 +91,7 @@ __device__ __forceinline__ long chunk_off(int RT, int r, int c) {
 // (twice, the second time from L2), 16 out per element.
 __global__ void __launch_bounds__(256) k_oz_slice_rows(const double* src, long rows, int k, long ld,
                                                        OzOperand o) {
+  pdl_begin();
   __shared__ int e_sh[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gpt = (o.rows_per_tile + 7) >> 3;  // groups of eight rows per row tile
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_rows(const double* src, long r
 // a tile's rows below the diagonal read Y columns, eight rows of a column at
 // a time (64 contiguous bytes).
 __global__ void __launch_bounds__(256) k_oz_slice_v(const double* Y, long ldy, int M, int Mp, OzOperand o) {
+  pdl_begin();
   __shared__ uint32_t m_sh[8], any_sh[8];
   const int tid = threadIdx.x, w = blockIdx.y;
   const int gpt = (o.rows_per_tile + 7) >> 3;
@@ -198,6 +200,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_v(const double* Y, long ldy, i
 // rows share a group of eight).
 __global__ void __launch_bounds__(256) k_oz_slice_term(const double* t, int N, int M, int Mp,
                                                        OzOperand o) {
+  pdl_begin();
   __shared__ int e_sh[8];
   const int tid = threadIdx.x, lane = tid & 31, w = blockIdx.y;
   const double* tw = t + (long)w * 2 * N * M;
@@ -301,6 +304,7 @@ __device__ __forceinline__ int orbital_exp(const int* planes, int N, int i) {
 // 47 us (20 and 44 with one scale for all orbitals).
 __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N, int M, const int* planes,
                                                        OzOperand o) {
+  pdl_begin();
   __shared__ int e_sh[8][32], s_sh[64];
   const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, w = blockIdx.y, N2 = 2 * N;
   const int p = blockIdx.x * 32 + lane;
@@ -348,6 +352,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(const double* phi, int N,
 __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, const double* thA,
                                                             const double* thB, int W, int N, int M, int w0,
                                                             int cw, const int* planes, OzOperand A, OzOperand B) {
+  pdl_begin();
   __shared__ int e_sh[8][32], s_sh[kOzSegK / 2];  // K = 2 N cw of at most one segment
   const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5, z = blockIdx.y, which = blockIdx.z;
   const int p = blockIdx.x * 32 + lane, first = w0 + z * cw, N2 = 2 * N;
@@ -399,6 +404,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_densities(const double* phi, c
 // with row i scaled by the exponent of orbital i (planes: of Phi, walker by walker).
 __global__ void __launch_bounds__(256) k_oz_slice_inverse(const double2* sinv, int W, int w0, int N,
                                                           const int* planes, OzOperand o) {
+  pdl_begin();
   __shared__ int e_sh[64], s_sh[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w = blockIdx.x, ds = blockIdx.y;
@@ -1088,22 +1094,36 @@ int check_operand(const OzOperand& A, const OzOperand& B, int bn) {
 
 }  // namespace
 
+// The slicing kernels of a few blocks per SM overlap their predecessor's tail (see
+// AFQ_LAUNCH_PDL): launched one by one, five steps and an energy of 32 and 300
+// walkers take at M = 36, N = 4 1366 -> 1151 and 1586 -> 1398 us, at M = 100, N = 10
+// 2109 -> 1950 and 3739 -> 3554 us.  In a graph larger ones gain nothing and lose up
+// to 0.5 %.
+#define OZ_LAUNCH(kernel, grid, ...)                                          \
+  do {                                                                        \
+    const dim3 g_(grid);                                                      \
+    if ((long)g_.x * g_.y * g_.z <= 4L * tc_sm_count())                       \
+      AFQ_LAUNCH_PDL(kernel, g_, __VA_ARGS__);                                \
+    else                                                                      \
+      AFQ_LAUNCH(kernel, g_, __VA_ARGS__);                                    \
+  } while (0)
+
 int oz_slice_rows(const double* src, long rows, int k, long ld, const OzOperand& o, cudaStream_t st) {
   if (rows <= 0) return AFQMC_OK;
   const long groups = (long)oz_tiles(rows, o.rows_per_tile) * ((o.rows_per_tile + 7) / 8);
-  AFQ_LAUNCH(k_oz_slice_rows, (unsigned)groups, 256, 0, st, src, rows, k, ld, o);
+  OZ_LAUNCH(k_oz_slice_rows, (unsigned)groups, 256, 0, st, src, rows, k, ld, o);
   return AFQMC_OK;
 }
 
 int oz_slice_v(const double* Y, long ldy, int W, int M, int Mp, const OzOperand& o, cudaStream_t st) {
   dim3 grid((unsigned)(oz_tiles(M, o.rows_per_tile) * ((o.rows_per_tile + 7) / 8)), W);
-  AFQ_LAUNCH(k_oz_slice_v, grid, 256, 0, st, Y, ldy, M, Mp, o);
+  OZ_LAUNCH(k_oz_slice_v, grid, 256, 0, st, Y, ldy, M, Mp, o);
   return AFQMC_OK;
 }
 
 int oz_slice_term(const double* t, int W, int N, int M, int Mp, const OzOperand& o, cudaStream_t st) {
   dim3 grid(cdiv(N, 8), W);
-  AFQ_LAUNCH(k_oz_slice_term, grid, 256, 0, st, t, N, M, Mp, o);
+  OZ_LAUNCH(k_oz_slice_term, grid, 256, 0, st, t, N, M, Mp, o);
   return AFQMC_OK;
 }
 
@@ -1131,7 +1151,7 @@ int oz_row_exps(const double* src, long n, int M, int* exps, cudaStream_t st) {
 }
 
 int oz_slice_cols(const double* phi, int W, int N, int M, const int* planes, const OzOperand& o, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, N, M, planes, o);
+  OZ_LAUNCH(k_oz_slice_cols, dim3(cdiv(M, 32), W), 256, 0, st, phi, N, M, planes, o);
   return AFQMC_OK;
 }
 
@@ -1139,13 +1159,13 @@ int oz_slice_densities(const double* phi, const double* thA, const double* thB, 
                        int nz, int cw, int* planes, const OzOperand& A, const OzOperand& B, cudaStream_t st) {
   const int n = W - w0 < nz * cw ? W - w0 : nz * cw;
   AFQ_TRY(oz_row_exps(phi + (long)w0 * 2 * N * M, 2L * N * n, M, planes, st));
-  AFQ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, planes, A, B);
+  OZ_LAUNCH(k_oz_slice_densities, dim3(cdiv(M, 32), nz, 4), 256, 0, st, phi, thA, thB, W, N, M, w0, cw, planes, A, B);
   return AFQMC_OK;
 }
 
 int oz_slice_inverse(const double2* sinv, int W, int w0, int nw, int nds, int N, const int* planes,
                      const OzOperand& o, cudaStream_t st) {
-  AFQ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, planes, o);
+  OZ_LAUNCH(k_oz_slice_inverse, dim3(nw, nds), 256, 0, st, sinv, W, w0, N, planes, o);
   return AFQMC_OK;
 }
 
