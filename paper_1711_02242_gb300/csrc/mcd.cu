@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, VEC == 2 ? 4 : 5)
 // k_mcd_step is one launch per vector: its latency chain (launch, grid-wide
 // tickets, the gather by one last block) took 22 us a vector at dim = 5050,
 // 516 vectors (11.2 ms), against 2.2 us of float64 work per SM on average,
-// which bounds this kernel beside the exchange; it takes 9.3 us (4.80 ms).
+// which bounds this kernel beside the exchange; it takes 8.9 us (4.58 ms).
 // Values are compared as integers of the same order (float64 comparisons run
 // on the slow pipe, a dozen of them per vector one after another).
 struct McdSlot {
